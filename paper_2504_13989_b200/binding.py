@@ -3,6 +3,9 @@
 Argument marshalling only: every step of the path runs in the library's CUDA kernels.
 PyTorch is used for device memory and streams.  There is no CPU fallback: if the shared
 library is missing or a call fails, a GbsError is raised.
+
+Plan's per-call methods go through _native.so (csrc/gbs_torch.cpp), which does the regular call's checks,
+allocations and marshalling in C and answers None for every other call; those take the functions below.
 """
 from __future__ import annotations
 
@@ -124,6 +127,22 @@ def lib() -> ctypes.CDLL:
         L.gbs_status_string.restype = ctypes.c_char_p
         _lib = L
     return _lib
+
+
+_native_module = None
+
+
+def native():
+    """Load _native.so (built beside libgbs.so); fail loudly if absent."""
+    global _native_module
+    if _native_module is None:
+        lib()
+        try:
+            from . import _native
+        except ImportError as e:
+            raise GbsErrorMissing("_native.so does not load (%s) -- run `python -m paper_2504_13989_b200.build`" % e) from e
+        _native_module = _native
+    return _native_module
 
 
 class GbsErrorMissing(RuntimeError):
@@ -397,6 +416,7 @@ class Plan:
     def __init__(self, d: int, d_pad: int | None = None, m: int = 1, bits: int = 4, group: int = 0,
                  alpha: float = 1.0, asymmetric: bool = False):
         d_pad = d if d_pad is None else d_pad
+        self._native = native()
         self.handle = gbs_plan_create_ex(d, d_pad, m, bits, group, alpha, GBS_PLAN_ASYMMETRIC if asymmetric else 0)
         self.info = gbs_plan_info(self.handle)
 
@@ -427,6 +447,9 @@ class Plan:
         return codes, scales, y
 
     def rotate_quantize(self, x: torch.Tensor, want_y: bool = False, out=None, stream=None):
+        done = self._native.rotate_quantize(self.handle, x, want_y, out, stream)
+        if done is not None:
+            return done
         n_rows = x.numel() // self.info.d
         codes, scales, y = out if out is not None else self.alloc_outputs(n_rows, x.device, want_y)
         gbs_rotate_quantize(self.handle, x, codes, scales, y, stream)
@@ -434,6 +457,9 @@ class Plan:
 
     def dequantize(self, codes: torch.Tensor, scales: torch.Tensor, inverse: bool = False,
                    dtype=torch.float32, out=None, stream=None) -> torch.Tensor:
+        done = self._native.dequantize(self.handle, codes, scales, inverse, dtype, out, stream)
+        if done is not None:
+            return done
         n_rows = codes.shape[0]
         width = self.info.d if inverse else self.info.d_pad
         if out is None:
@@ -442,6 +468,10 @@ class Plan:
         return out
 
     def clip_error(self, x: torch.Tensor, alphas, want_rows: bool = False, err_sum=None, stream=None):
+        if err_sum is None and not want_rows:
+            done = self._native.clip_error(self.handle, x, alphas, stream)
+            if done is not None:
+                return done
         n_rows = x.numel() // self.info.d
         K = len(alphas)
         if err_sum is None:
@@ -460,6 +490,9 @@ class Plan:
     def quantized_matmul(self, codes_x, scales_x, plan_w: "Plan", codes_w, scales_w, dtype=torch.float32, out=None,
                          stream=None) -> torch.Tensor:
         """The layer's output from the packed codes of activations (this plan) and weights (plan_w)."""
+        done = self._native.quantized_matmul(self.handle, codes_x, scales_x, plan_w.handle, codes_w, scales_w, dtype, out, stream)
+        if done is not None:
+            return done
         if out is None:
             out = torch.empty((codes_x.shape[0], codes_w.shape[0]), dtype=dtype, device=codes_x.device)
         gbs_quantized_matmul(self.handle, codes_x, scales_x, plan_w.handle, codes_w, scales_w, out, stream)

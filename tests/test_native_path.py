@@ -1,0 +1,62 @@
+"""The native call path of Plan's methods (_native.so) against the functions it stands in for: the regular call gives the
+same bytes, and every other call (views, strides, wrong buffers, CPU tensors) is handed on to the Python path."""
+import pytest
+import torch
+
+from paper_2504_13989_b200 import Plan, binding, synth
+from paper_2504_13989_b200 import build as gbs_build
+
+DEV = "cuda:0"
+
+
+def test_irregular_calls_are_handed_on():
+    gbs_build.build()
+    nat = binding.native()
+    x = torch.zeros(2, 128)
+    assert nat.rotate_quantize(None, x, False, None, None) is None          # no plan
+    assert nat.rotate_quantize(0, x, False, None, None) is None             # null plan
+    assert nat.dequantize(0, x, x, False, torch.float32, None, None) is None
+    assert nat.quantized_matmul(0, x, x, 0, x, x, torch.float32, None, None) is None
+    assert nat.clip_error(0, x, [0.5], None) is None
+
+
+@pytest.mark.gpu
+def test_native_and_python_paths_agree():
+    gbs_build.build()
+    w = synth.WORKLOADS["llama4096"]
+    x = synth.make_host("llama4096", 8).to(DEV)
+    wide = torch.zeros(8, 2 * w.d, dtype=torch.bfloat16, device=DEV)
+    wide[:, :w.d] = x
+    with Plan(w.d, w.d_pad, w.m, 4, 0, w.alpha) as plan:
+        ref = plan.alloc_outputs(8, DEV, True)
+        binding.gbs_rotate_quantize(plan.handle, x, *ref)
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        for args in (dict(x=x), dict(x=x.view(2, 4, w.d)), dict(x=wide[:, :w.d]), dict(x=x, want_y=True), dict(x=x, stream=s),
+                     dict(x=x, out=plan.alloc_outputs(8, DEV)), dict(x=wide.view(2, 4, -1)[..., :w.d]), dict(x=x[0])):
+            codes, scales, y = plan.rotate_quantize(**args)
+            torch.cuda.synchronize()
+            n = codes.shape[0]
+            assert torch.equal(codes, ref[0][:n]) and torch.equal(scales, ref[1][:n])
+            assert (y is None) == (not args.get("want_y", False)) and (y is None or torch.equal(y, ref[2]))
+        want = torch.empty((8, w.d), dtype=torch.bfloat16, device=DEV)
+        binding.gbs_dequantize(plan.handle, ref[0], ref[1], 8, want, binding.GBS_INVERSE_ROTATE)
+        assert torch.equal(plan.dequantize(ref[0], ref[1], inverse=True, dtype=torch.bfloat16), want)
+        mm = torch.empty((8, 8), device=DEV)
+        binding.gbs_quantized_matmul(plan.handle, ref[0], ref[1], plan.handle, ref[0], ref[1], mm)
+        assert torch.equal(plan.quantized_matmul(ref[0], ref[1], plan, ref[0], ref[1]), mm)
+        padded = torch.empty((8, 12), device=DEV)
+        assert torch.equal(plan.quantized_matmul(ref[0], ref[1], plan, ref[0], ref[1], out=padded[:, :8]), mm)
+        err = torch.zeros(3, dtype=torch.float64, device=DEV)
+        plan.clip_error(x, [0.5, 0.75, 1.0], err_sum=err)
+        # per-CTA fp64 totals are added in any order
+        assert torch.allclose(plan.clip_error(x, torch.tensor([0.5, 0.75, 1.0])), err, rtol=1e-12)
+        # errors are the Python path's
+        for bad, exc in ((dict(x=x.cpu()), ValueError), (dict(x=x.half()), TypeError), (dict(x=x[:, :64]), ValueError),
+                         (dict(x=x, out=plan.alloc_outputs(7, DEV)), ValueError)):
+            with pytest.raises(exc):
+                plan.rotate_quantize(**bad)
+        with pytest.raises(TypeError):
+            plan.dequantize(ref[0], ref[1], dtype=torch.float16)
+        with pytest.raises(binding.GbsError):
+            plan.clip_error(x, [1.5])
