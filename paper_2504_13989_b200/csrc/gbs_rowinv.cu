@@ -1,0 +1,134 @@
+// Inverse path of gbs_dequantize for d' = 128 rows (KV entries) with one scale per row (group 0 or 128), symmetric or
+// asymmetric quantizer:
+//     xhat = (H_128^T yhat / sqrt(128))[0:d],   yhat = q * Delta   or   code * Delta + lo
+// (Section 2.1 / 5.1; inverse by the transpose, Section 2.3; H_128 of Eq. (1) is symmetric).
+//
+// One thread owns one row.  A packed field k, masked into the low bits of a 16-bit half, IS the subnormal half-precision
+// number k * 2^-24, and sums of 128 fields of at most 15 stay below 2048 * 2^-24: every one of the seven butterfly stages
+// is exact in packed half arithmetic, two coordinates per instruction, with no conversion before and one to fp32 after.
+// Symmetric codes are stored as q + 2^(b-1); the offset adds 128 * 2^(b-1) to coordinate 0 and nothing elsewhere, where
+// one exact subtraction removes it.  The only rounding is the product with Delta / sqrt(128) (and the output type's).
+//
+// What bounds it: HBM (48 or 64 bytes read and 256 or 512 written per row).  About 7 issue slots per value without any
+// shared memory, barrier or tensor-core round trip; the tensor-core form this replaces waited on that round trip with 16
+// warps per SM.  262 144 rows, 4 bits, asymmetric -> bf16: 33.2 us before.
+#include <string.h>
+
+#include "gbs_internal.h"
+#include "gbs_tc_inv.cuh"
+
+namespace {
+
+constexpr int DP = 128;
+constexpr int RI_THREADS = 128;
+constexpr int RI_BLOCKS = 5;          // per SM: 102 registers per thread, of which 64 hold the row
+
+struct RowInvParams {
+    long long n_rows;
+    int d;                            // output width, a multiple of 32
+    int wide;                         // output rows start on 32-byte boundaries: 32-byte stores
+    float norm;                       // 1 / sqrt(128)
+    const unsigned char* codes;
+    const float* scales;              // Delta per row, or (Delta, lo) per row
+    void* out;
+};
+
+template <int BITS, bool ASYM, typename OutT>
+__global__ void __launch_bounds__(RI_THREADS, RI_BLOCKS) k_row_inv(const __grid_constant__ RowInvParams P)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long long row = (long long)blockIdx.x * RI_THREADS + threadIdx.x;
+    if (row >= P.n_rows) return;
+    constexpr int NW = DP * BITS / 32;                       // packed words of a row
+    unsigned w[NW];
+    const uint4* src = reinterpret_cast<const uint4*>(P.codes + row * (NW * 4));
+#pragma unroll
+    for (int i = 0; i < NW / 4; ++i) {
+        const uint4 v = __ldg(src + i);
+        w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+    }
+    float delta, lo = 0.f;
+    if (ASYM) {
+        const float2 sl = __ldg(reinterpret_cast<const float2*>(P.scales) + row);
+        delta = sl.x; lo = sl.y;
+    } else {
+        delta = __ldg(P.scales + row);
+    }
+    // h[4 o + i] = (coordinate 8 o + i, coordinate 8 o + 4 + i)
+    unsigned h[64];
+#pragma unroll
+    for (int o = 0; o < 16; ++o) unpack_octet<BITS, ASYM, NW>(w, o, h + 4 * o);
+#pragma unroll
+    for (int i = 0; i < 64; ++i) h[i] = hpair(h[i]);
+#pragma unroll
+    for (int s = 1; s < 64; s <<= 1)
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+            if ((i & s) == 0) {
+                const unsigned a = h[i], b = h[i + s];
+                h[i] = hadd2(a, b);
+                h[i + s] = hsub2(a, b);
+            }
+    const float sc = delta * P.norm * 16777216.f;            // the halves are integers times 2^-24
+    const float add0 = ASYM ? 128.f * lo * P.norm : 0.f;
+    constexpr float OFF0 = (ASYM ? 0.f : 128.f * (float)(1 << (BITS - 1))) / 16777216.f;
+    OutT* dst = reinterpret_cast<OutT*>(P.out) + row * (long long)P.d;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {                            // sixteen coordinates each
+        if (c * 16 >= P.d) break;
+        float f[16];
+#pragma unroll
+        for (int o = 0; o < 2; ++o)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&h[8 * c + 4 * o + i]));
+                f[8 * o + i] = v.x;
+                f[8 * o + 4 + i] = v.y;
+            }
+        if (c == 0) f[0] -= OFF0;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) f[e] = (c == 0 && e == 0) ? fmaf(f[0], sc, add0) : f[e] * sc;
+        store_values<16>(dst + 16 * c, f, P.wide != 0);
+    }
+}
+
+typedef void (*RowInvKernel)(const RowInvParams);
+
+}  // namespace
+
+// The plans this path serves: d' = 128 (the ROW family) with one scale (pair) per row and whole 32-value output chunks.
+bool gbs_rowinv_supported(const gbs_plan* p, const float* scales)
+{
+    if (p->variant != GBS_VARIANT_TC_ROW || !(p->group == 0 || p->group == DP) || p->d % 32 != 0) return false;
+    return !(p->asym && (reinterpret_cast<uintptr_t>(scales) & 7u));        // (Delta, lo) pairs are read as one 8-byte word
+}
+
+int gbs_rowinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
+                          int out_dtype, cudaStream_t stream)
+{
+    static const RowInvKernel table[2][2][2] = {
+        {{k_row_inv<3, false, float>, k_row_inv<3, false, __nv_bfloat16>}, {k_row_inv<3, true, float>, k_row_inv<3, true, __nv_bfloat16>}},
+        {{k_row_inv<4, false, float>, k_row_inv<4, false, __nv_bfloat16>}, {k_row_inv<4, true, float>, k_row_inv<4, true, __nv_bfloat16>}}};
+    const long long blocks = (n_rows + RI_THREADS - 1) / RI_THREADS;
+    if (blocks > 0x7fffffff) return (int)cudaErrorInvalidValue;
+    RowInvParams P;
+    memset(&P, 0, sizeof(P));
+    P.n_rows = n_rows;
+    P.d = p->d;
+    P.wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
+    P.norm = p->norm;
+    P.codes = (const unsigned char*)codes;
+    P.scales = scales;
+    P.out = out;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(RI_THREADS);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p->pdl ? 1 : 0;
+    return (int)cudaLaunchKernelEx(&cfg, table[p->bits - 3][p->asym ? 1 : 0][out_dtype == GBS_DTYPE_F32 ? 0 : 1], P);
+}

@@ -1,22 +1,31 @@
-// Tensor-core inverse path of gbs_dequantize for the UV family's shapes with one scale per token:
-//     xhat = (H^T yhat / sqrt(d'))[0:d],  yhat = q * Delta          (Section 2.1; inverse by the transpose,
-//                                                                     Section 2.3)
-// With H = A (x) H_32 (A = H_m (x) H_{2^j}, U x U) the transpose is A^T (x) H_32, and Delta is one number per
-// token, so xhat = (Delta / sqrt(d')) * (A^T Q H_32) with Q the U x 32 matrix of the token's integer codes.
-//   * The codes are unpacked by the epilogue warps straight into the bf16 operand tile the MMA reads
-//     (same [token][u][v] layout and 64-byte swizzle the forward kernel gets from TMA).  No conversion
-//     instruction is needed: the 16-bit pattern 0x4300 | k is the bf16 number 128 + k, so a field f is stored
-//     as 128 + (f ^ 2^(b-1)) = q + OFF with OFF = 128 + 2^(b-1), built with shifts and masks only.
-//   * A^T (Q + OFF) = A^T Q + OFF * rowsum(A^T): the second term is the same in all 32 columns of a TMEM lane,
-//     so after the H_32 butterflies it sits in coordinate 0 alone (32 * OFF * rowsum) and one subtraction
-//     removes it.  Every intermediate is an integer below 2^24: the rotation of the codes is exact in fp32,
-//     and the only rounding is the final multiplication by Delta / sqrt(d').
-//   * tcgen05.mma with the plan's image of A^T, accumulators in TMEM, H_32 in registers, 64 or 128 contiguous
-//     bytes stored per thread: the kernel is bound by the output write.
-// Roles: warp 0 loads the A^T image, warp 1 issues the MMAs, warps 2..17 unpack (two tiles ahead) and run
-// the epilogue; warp (q, t) owns TMEM lane quadrant q and token t of every tile.  Every wait is bounded.
+// Tensor-core inverse path of gbs_dequantize:  xhat = (H^T yhat / sqrt(d'))[0:d],  yhat = q * Delta, one scale per token
+// or per group of a power of two coordinates (Section 2.1; inverse by the transpose, Section 2.3).
+//
+// The rotated row is a U x V matrix of codes Q[u][v] (flat index u V + v; V = 32 for d' <= 4096, 64 up to 8192), and
+// H = A (x) H_V with A = H_m (x) H_{2^j}, U <= 128.  A group is at least V wide, so its scale is constant along v:
+//
+//        xhat = A^T diag(Delta_u) (Q H_V) / sqrt(d').
+//
+//   * Q H_V in registers, exactly: a code field masked into the low bits of a 16-bit half IS the subnormal half-precision
+//     number k * 2^-24, and the sums of V fields stay below 2048 * 2^-24, so the butterflies run in packed half arithmetic
+//     (two coordinates per instruction) without a conversion.  Codes are stored as q + 2^(b-1); after H_V the offset sits
+//     in coordinate v = 0 alone, where one exact subtraction removes it.
+//   * One scale per token: the integers are the fp16 operand as they are, and Delta multiplies once at the end.
+//   * Group scales: the operand is Delta_u n, split into two fp16 numbers hi + lo (22 significant bits, relative to the
+//     token's largest scale): with s = sh + sl the scale in two halves, hi = rn(n sh), lo = rn(n sl + (n sh - hi)), where
+//     n sh - hi is exact in an fma.  A^T then contracts both planes into the same fp32 accumulators.
+//   * tcgen05.mma with the plan's fp16 image of A^T, N = 128 columns (128 / V tokens) per tile, accumulators in TMEM; lane
+//     u' then holds V consecutive output coordinates of a token: scale, round, 32-byte stores.
+// What bounds it: instruction issue of the unpacking (about 290 slots per 32 values with group scales, 230 without)
+// against 48 - 100 bytes of HBM traffic per 32 values.  Doing H_V before the contraction in packed halves takes 80
+// instructions per 32 values where the fp32 form after the contraction took 124 packed (248 slots).
+// 8192 x 3584, 3 bits, groups of 128 -> bf16: 118.5 us on the shared-memory kernel this replaces for group scales.
+// Roles: warp 0 loads the image, warp 1 issues the MMAs, warps 2..17 unpack (ahead) and run the epilogue; warp (q, t) owns
+// TMEM lane quadrant q and token t; with V = 64 two groups of eight warps take alternate tiles.  Every wait is bounded.
 #include <math.h>
 #include <string.h>
+
+#include <mutex>
 
 #include "gbs_internal.h"
 #include "gbs_tc_common.cuh"
@@ -24,22 +33,30 @@
 
 namespace {
 
-constexpr int V = 32;
 constexpr int UMAX = 128;
-constexpr int TOK = 4;                            // tokens per tile (MMA N = 128)
-constexpr int STAGES = 4;
-constexpr int STAGE_COLS = TOK * V;
-constexpr int TMEM_COLS = STAGES * STAGE_COLS;
+constexpr int STAGE_COLS = 128;                   // MMA N: 128 / V tokens of V columns
+constexpr int ACCS = 4;                           // TMEM accumulators of 128 columns
+constexpr int TMEM_COLS = ACCS * STAGE_COLS;
 constexpr int A_BYTES = UMAX * UMAX * 2;
-constexpr int B_STAGE_BYTES = TOK * UMAX * V * 2;
+constexpr int PLANE_BYTES = UMAX * STAGE_COLS * 2;      // one operand plane of a tile at U = 128
 constexpr int EPI_WARPS = 16;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
-constexpr int AHEAD = 2;                          // tiles unpacked ahead of the one in the epilogue
 
-struct __align__(1024) Smem {
-    unsigned char a[A_BYTES];
-    unsigned char b[STAGES][B_STAGE_BYTES];
-    unsigned long long full[STAGES], empty[STAGES], tfull[STAGES], tempty[STAGES];
+// V = 32: all sixteen warps work on every tile.  V = 64: a thread owns 64 codes, so eight warps fill a tile and two groups
+// take alternate tiles; a stage must belong to one group, or a group would wait on barrier phases it took no part in.
+template <int V, bool SPLIT> struct Shape {
+    static constexpr int GROUPS = V / 32;
+    static constexpr int TOK = STAGE_COLS / V;
+    static constexpr int WARPS = EPI_WARPS / GROUPS;            // warps per tile
+    static constexpr int PLANES = SPLIT ? 2 : 1;
+    static constexpr int STAGES = SPLIT ? (V == 32 ? 3 : 2) : 4;
+    static constexpr int AHEAD = V == 32 ? 2 : 1;               // tiles (of its group) a warp unpacks ahead
+    static constexpr int SMEM = 1024 + A_BYTES + STAGES * PLANES * PLANE_BYTES + 256;
+    static_assert(STAGES % GROUPS == 0 && ACCS % GROUPS == 0, "a stage belongs to one group");
+};
+
+struct Bars {
+    unsigned long long full[4], empty[4], tfull[ACCS], tempty[ACCS];
     unsigned long long abar;
     unsigned tmem_base;
     volatile int abort_flag;
@@ -47,112 +64,206 @@ struct __align__(1024) Smem {
 
 struct InvParams {
     long long n_rows;
-    int n_groups;                 // ceil(n_rows / TOK)
+    int n_tiles;                  // ceil(n_rows / TOK)
     int U, Upad, ksteps;
-    int d;                        // output width (multiple of 32)
+    int d;                        // output width, a multiple of V
     int code_row_bytes;
+    int spr;                      // scales per row
+    int glog;                     // log2 of the u-rows per group (group scales)
+    int wide;                     // output rows start on 32-byte boundaries
     float norm;                   // 1 / sqrt(d')
-    const unsigned char* at_img;  // image of A^T
+    const unsigned char* at_img;  // fp16 image of A^T
     const unsigned char* codes;
     const float* scales;
     void* out;
     int* status;
-    float corr[UMAX];             // 32 * OFF * sum_u A[u][u']  (what the offset of the stored codes adds to coordinate 0)
 };
+
+// V codes of one row u -> V/2 packed halves h[4 o + i] = (8 o + i, 8 o + 4 + i), times 2^-24, after H_V; offset removed.
+template <int BITS, int V>
+__device__ __forceinline__ void unpack_rotate(const unsigned* w, unsigned h[V / 2])
+{
+    constexpr int NW = V * BITS / 32;
+#pragma unroll
+    for (int o = 0; o < V / 8; ++o) unpack_octet<BITS, false, NW>(w, o, h + 4 * o);
+#pragma unroll
+    for (int i = 0; i < V / 2; ++i) h[i] = hpair(h[i]);
+#pragma unroll
+    for (int s = 1; s < V / 2; s <<= 1)
+#pragma unroll
+        for (int i = 0; i < V / 2; ++i)
+            if ((i & s) == 0) {
+                const unsigned a = h[i], b = h[i + s];
+                h[i] = hadd2(a, b);
+                h[i + s] = hsub2(a, b);
+            }
+    h[0] = hsub2(h[0], (unsigned)(V << (BITS - 1)));        // low half: V * 2^(b-1) * 2^-24
+}
 
 // ---------------------------------------------------------------------------------------------
 // kernel
 // ---------------------------------------------------------------------------------------------
-template <int BITS, typename OutT>
+template <int BITS, int V, bool SPLIT, typename OutT>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant__ InvParams P)
 {
+    typedef Shape<V, SPLIT> SH;
+    constexpr int TOK = SH::TOK, STAGES = SH::STAGES, GROUPS = SH::GROUPS, AHEAD = SH::AHEAD;
+    constexpr int STAGE_BYTES = SH::PLANES * PLANE_BYTES;
+    constexpr int NW = V * BITS / 32;                       // packed words of V codes
     extern __shared__ unsigned char smem_raw[];
-    Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* sm_a = base;
+    unsigned char* sm_b = base + A_BYTES;
+    Bars* S = reinterpret_cast<Bars*>(base + A_BYTES + STAGES * STAGE_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned tok_bytes = (unsigned)(P.Upad * V * 2);
+    const unsigned slab_bytes = (unsigned)(P.Upad * V * 2);       // a token's operand rows: U lines of V halves
 
     if (threadIdx.x == 0) {
         mbar_init(&S->abar, 1);
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&S->full[s], EPI_WARPS);
+            mbar_init(&S->full[s], SH::WARPS);
             mbar_init(&S->empty[s], 1);
+        }
+        for (int s = 0; s < ACCS; ++s) {
             mbar_init(&S->tfull[s], 1);
-            mbar_init(&S->tempty[s], EPI_WARPS);
+            mbar_init(&S->tempty[s], SH::WARPS);
         }
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         mbar_arrive_expect_tx(&S->abar, A_BYTES);
-        bulk_load(S->a, P.at_img, A_BYTES, &S->abar);         // plan-owned, immutable: needs no ordering
-        // programmatic dependent launch: the codes and scales may still be being written until this returns;
-        // the block barrier below orders every other thread of the CTA behind it
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        bulk_load(sm_a, P.at_img, A_BYTES, &S->abar);         // plan-owned, immutable: needs no ordering
     }
     if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // programmatic dependent launch: the codes and scales may still be being written until this returns
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned tmem_base = S->tmem_base;
+    const int n_mine = (P.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
 
     if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0) {
-            constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS);
-            const unsigned a_base = smem_u32(S->a);
-            const unsigned long long ad0 = smem_desc(a_base, 16, 1024, 2);
-            const unsigned long long bd0 = smem_desc(smem_u32(S->b[0]), tok_bytes, 512, 4);
+            // fp16 operands: the two type fields of instr_desc (bf16) cleared
+            constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS) & ~((1u << 7) | (1u << 10));
+            constexpr unsigned KSTEP = (16 * V * 2) >> 4;          // sixteen u-lines of V halves
+            const unsigned long long ad0 = smem_desc(smem_u32(sm_a), 16, 1024, 2);
+            const unsigned long long bd0 = smem_desc(smem_u32(sm_b), slab_bytes, 8 * V * 2, V == 32 ? 4 : 2);
             const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
             const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
             bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
-            int it = 0;
-            for (int g = blockIdx.x; ok && g < P.n_groups; g += gridDim.x, ++it) {
-                const int s = it % STAGES;
-                const unsigned ph = (it / STAGES) & 1;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
+            for (int it = 0; ok && it < n_mine; ++it) {
+                const int s = it % STAGES, c = it % ACCS;
+                if (!mbar_wait(&S->abort_flag, &S->full[s], (unsigned)(it / STAGES) & 1u, P.status, 2)) break;
+                if (!mbar_wait(&S->abort_flag, &S->tempty[c], ((unsigned)(it / ACCS) & 1u) ^ 1u, P.status, 3)) break;
                 tc_fence_after();
                 // only the address fields (bytes >> 4, low words) of the descriptors change between k-steps
-                unsigned a_lo = ad_lo0, b_lo = bd_lo0 + (unsigned)s * (B_STAGE_BYTES >> 4);
-                const unsigned d_tmem = tmem_base + s * STAGE_COLS;
-                umma_f16_words<false>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
-                for (int ks = 1; ks < P.ksteps; ++ks) {
-                    a_lo += (ks & 3) ? 2u : (unsigned)((UMAX * 128 - 96) >> 4);
-                    b_lo += 1024u >> 4;
-                    umma_f16_words<true>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
+                const unsigned d_tmem = tmem_base + c * STAGE_COLS;
+#pragma unroll
+                for (int pl = 0; pl < SH::PLANES; ++pl) {
+                    unsigned a_lo = ad_lo0, b_lo = bd_lo0 + (unsigned)(s * STAGE_BYTES + pl * PLANE_BYTES) / 16u;
+                    if (pl == 0) umma_f16_words<false>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
+                    else umma_f16_words<true>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
+                    for (int ks = 1; ks < P.ksteps; ++ks) {
+                        a_lo += (ks & 3) ? 2u : (unsigned)((UMAX * 128 - 96) >> 4);
+                        b_lo += KSTEP;
+                        umma_f16_words<true>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
+                    }
                 }
                 umma_commit(&S->empty[s]);
-                umma_commit(&S->tfull[s]);
+                umma_commit(&S->tfull[c]);
             }
         }
     } else if (warp >= 2) {
         // ------------------------------ unpack + epilogue ------------------------------
-        const int t = (warp - 2) >> 2;            // token slot inside every tile
-        const int q = warp & 3;                   // TMEM lane quadrant this warp may access
-        const int up = q * 32 + lane;             // row u of the operand tile it writes; output row u' it reads
+        const int grp = (warp - 2) / SH::WARPS;                    // group of warps: tiles grp, grp + GROUPS, ..
+        const int t = ((warp - 2) % SH::WARPS) >> 2;               // token slot inside its tiles
+        const int q = warp & 3;                                    // TMEM lane quadrant this warp may access
+        const int up = q * 32 + lane;                              // row u of the operand it writes; row u' it reads
         const unsigned taddr0 = tmem_base + ((unsigned)(q * 32) << 16) + t * V;
-        const unsigned row_off = (unsigned)t * tok_bytes + (unsigned)up * 64u;
-        const unsigned swz = (unsigned)((up >> 1) & 3);
-        const float corr = P.corr[up];
-        const long long row_step = (long long)gridDim.x * TOK;
-        const int n_mine = (P.n_groups - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
+        const unsigned row_addr = smem_u32(sm_b) + (unsigned)t * slab_bytes + (unsigned)up * (V * 2);
+        const unsigned swz = V == 32 ? (unsigned)((up >> 1) & 3) : (unsigned)(up & 7);
+        const int n_grp = (n_mine - grp + GROUPS - 1) / GROUPS;    // tiles of this group
+        const long long row_first = ((long long)blockIdx.x + (long long)grp * gridDim.x) * TOK + t;
+        const long long row_step = (long long)GROUPS * gridDim.x * TOK;
+        const bool live_u = up < P.U;
 
-        // codes of tile j of this CTA -> operand tile, stage j % STAGES
-        auto unpack_tile = [&](int j) -> bool {
-            const int s = j % STAGES;
-            if (!mbar_wait(&S->abort_flag, &S->empty[s], ((j / STAGES) & 1) ^ 1, P.status, 1)) return false;
-            const long long row = ((long long)blockIdx.x + (long long)j * gridDim.x) * TOK + t;
-            if (up < P.Upad) {
-                uint4 chunk[4];
-                if (up < P.U && row < P.n_rows) {
-                    unpack_row<BITS, false>(P.codes + row * P.code_row_bytes + up * (V * BITS / 8), chunk);
-                } else {
-                    // rows that pad U to a multiple of 16 and tokens beyond the last: bf16 zeros (A^T has zero
-                    // columns for the former, the latter are never stored)
-                    chunk[0] = chunk[1] = chunk[2] = chunk[3] = make_uint4(0u, 0u, 0u, 0u);
-                }
-                const unsigned base = smem_u32(S->b[s]) + row_off;
+        // packed codes and scales of one tile, one tile ahead of their unpacking
+        unsigned raw[NW];
+        float my_scale = 0.f;
+        unsigned all_scales = 0u;
+        auto fetch = [&](int n) {
+            const long long row = row_first + (long long)n * row_step;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) st_shared_v4(base + ((c ^ swz) << 4), chunk[c]);
+            for (int i = 0; i < NW; ++i) raw[i] = 0u;
+            my_scale = 0.f;
+            all_scales = 0u;
+            if (n >= n_grp || row >= P.n_rows) return;
+            const float* sp = P.scales + row * P.spr;
+            if (SPLIT) {
+                if (live_u) my_scale = __ldg(sp + (up >> P.glog));
+                for (int i = lane; i < P.spr; i += 32) all_scales = max(all_scales, __float_as_uint(__ldg(sp + i)) & 0x7fffffffu);
+            } else {
+                my_scale = __ldg(sp);
+            }
+            if (live_u) {
+                const unsigned char* src = P.codes + row * P.code_row_bytes + up * (V * BITS / 8);
+                if (BITS == 4) {
+#pragma unroll
+                    for (int i = 0; i < NW / 4; ++i) {
+                        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + i);
+                        raw[4 * i] = v.x; raw[4 * i + 1] = v.y; raw[4 * i + 2] = v.z; raw[4 * i + 3] = v.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < NW; ++i) raw[i] = __ldg(reinterpret_cast<const unsigned*>(src) + i);
+                }
+            }
+        };
+
+        // the fetched codes -> operand planes of the n-th tile of this group; returns the factor of its epilogue in `fac`
+        auto unpack_tile = [&](int n, float& fac) -> bool {
+            const int it = n * GROUPS + grp, s = it % STAGES;
+            unsigned h[V / 2];
+            unpack_rotate<BITS, V>(raw, h);
+            unsigned sh2 = 0u, sl2 = 0u;
+            if (SPLIT) {
+                // scales relative to 2^e, the power of two below the token's largest: s = Delta 2^(14-e) in (0, 2^15)
+                const unsigned E = max(__reduce_max_sync(0xffffffffu, all_scales) >> 23, 15u);
+                const float sf = my_scale * __uint_as_float((268u - E) << 23);
+                const __half sh = __float2half_rn(sf), sl = __float2half_rn(sf - __half2float(sh));
+                sh2 = __half_as_ushort(sh) * 0x10001u;
+                sl2 = __half_as_ushort(sl) * 0x10001u;
+                fac = P.norm * __uint_as_float((E - 4u) << 23);            // 2^(e-14), and 2^10 of the integers' scaling below
+            } else {
+                fac = my_scale * P.norm * 16777216.f;                      // the halves are integers times 2^-24
+            }
+            // a warp leaves as one
+            const bool ok = mbar_wait(&S->abort_flag, &S->empty[s], ((unsigned)(it / STAGES) & 1u) ^ 1u, P.status, 1);
+            if (!__all_sync(0xffffffffu, ok)) return false;
+            if (up < P.Upad) {
+                const unsigned dst = row_addr + (unsigned)(s * STAGE_BYTES);
+#pragma unroll
+                for (int c = 0; c < V / 8; ++c) {
+                    // rows that pad U to a multiple of 16 hold zero codes: A^T has zero columns there, any finite value will do
+                    uint4 hi, lo;
+                    unsigned* ph = reinterpret_cast<unsigned*>(&hi);
+                    unsigned* pl = reinterpret_cast<unsigned*>(&lo);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (SPLIT) {
+                            const unsigned n1 = hmul2(h[4 * c + e], 0x74007400u);          // times 2^14: n * 2^-10
+                            ph[e] = hmul2(n1, sh2);
+                            pl[e] = hfma2(n1, sl2, hfma2(n1, sh2, ph[e] ^ 0x80008000u));
+                        } else {
+                            ph[e] = h[4 * c + e];
+                        }
+                    }
+                    st_shared_v4(dst + ((c ^ swz) << 4), hi);
+                    if (SPLIT) st_shared_v4(dst + PLANE_BYTES + ((c ^ swz) << 4), lo);
+                }
             }
             // make the generic-proxy writes visible to the tensor cores' (async proxy) reads, then signal
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -161,29 +272,49 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
             return true;
         };
 
+        float fac[AHEAD + 1];
         bool alive = true;
-        for (int j = 0; alive && j < AHEAD && j < n_mine; ++j) alive = unpack_tile(j);
-        long long row = (long long)blockIdx.x * TOK + t;
-        for (int it = 0; alive && it < n_mine; ++it, row += row_step) {
-            if (it + AHEAD < n_mine) {
-                alive = unpack_tile(it + AHEAD);
+        fetch(0);
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            if (alive && j < n_grp) alive = unpack_tile(j, fac[j]);
+            fetch(j + 1);
+        }
+        long long row = row_first;
+        for (int n = 0; alive && n < n_grp; ++n, row += row_step) {
+            if (n + AHEAD < n_grp) {
+                alive = unpack_tile(n + AHEAD, fac[AHEAD]);
                 if (!alive) break;
+                fetch(n + AHEAD + 1);
             }
-            const int s = it % STAGES;
-            if (!mbar_wait(&S->abort_flag, &S->tfull[s], (it / STAGES) & 1, P.status, 4)) break;
-            unsigned r[32];
+            const int it = n * GROUPS + grp, c = it % ACCS;
+            const bool ok = mbar_wait(&S->abort_flag, &S->tfull[c], (unsigned)(it / ACCS) & 1u, P.status, 4);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            const bool store = row < P.n_rows && up * V < P.d;
+            OutT* dst = reinterpret_cast<OutT*>(P.out) + row * (long long)P.d + up * V;
             tc_fence_after();
-            tmem_ld32_issue(taddr0 + s * STAGE_COLS, r);
-            tmem_ld_wait(r);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S->tempty[s]);
-            (void)fwht32_absmax(r);
-            r[0] = __float_as_uint(__uint_as_float(r[0]) - corr);      // the offset of the stored codes
-            if (row < P.n_rows && up * V < P.d) {
-                const float sc = __ldg(P.scales + row) * P.norm;
-                store_row32<OutT>(reinterpret_cast<OutT*>(P.out) + row * (long long)P.d + up * V, r, sc, 0.f);
+#pragma unroll
+            for (int half = 0; half < V / 32; ++half) {
+                unsigned r[32];
+                tmem_ld32_issue(taddr0 + c * STAGE_COLS + half * 32, r);
+                tmem_ld_wait(r);
+                if (half == V / 32 - 1) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&S->tempty[c]);
+                }
+                if (store) {
+                    // column 8 o + 2 i + b of the accumulator is coordinate 8 o + i + 4 b
+                    float f[32];
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) f[8 * o + (e >> 1) + 4 * (e & 1)] = __uint_as_float(r[8 * o + e]) * fac[0];
+                    store_values<32>(dst + half * 32, f, P.wide != 0);
+                }
             }
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j) fac[j] = fac[j + 1];
         }
     }
 
@@ -196,65 +327,84 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
     }
 }
 
-template <typename KernelT>
-cudaError_t launch(KernelT kernel, int grid, int smem, cudaStream_t stream, bool pdl, const InvParams& P)
+template <int V, bool SPLIT>
+cudaError_t launch(const gbs_plan* p, InvParams& P, int out_dtype, cudaStream_t stream)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    typedef void (*Kernel)(const InvParams);
+    static const Kernel table[2][2] = {
+        {k_tc_uv_inv<3, V, SPLIT, float>, k_tc_uv_inv<3, V, SPLIT, __nv_bfloat16>},
+        {k_tc_uv_inv<4, V, SPLIT, float>, k_tc_uv_inv<4, V, SPLIT, __nv_bfloat16>}};
+    typedef Shape<V, SPLIT> SH;
+    {
+        // opt in to the large dynamic shared memory once per device (not a stream operation)
+        static std::mutex mu;
+        static bool done[64] = {false};
+        std::lock_guard<std::mutex> lock(mu);
+        if (!(p->device >= 0 && p->device < 64 && done[p->device])) {
+            for (int i = 0; i < 4; ++i) {
+                const cudaError_t e = cudaFuncSetAttribute(table[i >> 1][i & 1], cudaFuncAttributeMaxDynamicSharedMemorySize, SH::SMEM);
+                if (e != cudaSuccess) return e;
+            }
+            if (p->device >= 0 && p->device < 64) done[p->device] = true;
+        }
+    }
+    P.n_tiles = (int)((P.n_rows + SH::TOK - 1) / SH::TOK);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = dim3((unsigned)(P.n_tiles < p->sm_count ? P.n_tiles : p->sm_count));
     cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.dynamicSmemBytes = (size_t)SH::SMEM;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, P);
+    cfg.numAttrs = p->pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, table[p->bits - 3][out_dtype == GBS_DTYPE_F32 ? 0 : 1], P);
 }
 
 }  // namespace
 
-// The plans this path serves: the UV family's shapes with one symmetric scale per token.
-bool gbs_tc_uvinv_supported(const gbs_plan* p)
+// The in-register factor V of the inverse path for this shape, or 0: the smallest of 32 and 64 that leaves U <= 128, where
+// a scale is constant over V coordinates.
+int gbs_tc_uvinv_v(const gbs_plan* p)
 {
-    return p->variant == GBS_VARIANT_TC_UV && p->group == 0 && !p->asym && p->d_aimg_t != nullptr &&
-           p->smem_optin >= (int)(sizeof(Smem) + 1024);
+    if (p->asym) return 0;
+    for (int V = 32, lv = 5; V <= 64; V *= 2, ++lv) {
+        if (p->k < lv || p->d_pad % V != 0) return 0;
+        const int U = p->d_pad / V;
+        if (U > UMAX) continue;
+        if (U < 16 || p->d % V != 0 || (p->group != 0 && p->group < V)) return 0;
+        return p->smem_optin >= Shape<32, true>::SMEM ? V : 0;
+    }
+    return 0;
 }
+
+// The plans this path serves: those that got an image of A^T.
+bool gbs_tc_uvinv_supported(const gbs_plan* p) { return p->inv_v != 0 && p->d_aimg_t != nullptr; }
 
 int gbs_tc_uvinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
                             int out_dtype, cudaStream_t stream)
 {
-    if (n_rows > (int64_t)0x7fffffff - TOK) return (int)cudaErrorInvalidValue;
+    if (n_rows > (int64_t)0x7fffffff - 4) return (int)cudaErrorInvalidValue;
+    const int V = p->inv_v;
     InvParams P;
     memset(&P, 0, sizeof(P));
-    const int U = p->d_pad / V;
     P.n_rows = n_rows;
-    P.n_groups = (int)((n_rows + TOK - 1) / TOK);
-    P.U = U;
-    P.Upad = (U + 15) & ~15;
+    P.U = p->d_pad / V;
+    P.Upad = (P.U + 15) & ~15;
     P.ksteps = P.Upad / 16;
     P.d = p->d;
     P.code_row_bytes = p->d_pad * p->bits / 8;
+    P.spr = p->group ? p->d_pad / p->group : 1;
+    while (p->group && (V << P.glog) < p->group) ++P.glog;
+    P.wide = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
     P.norm = p->norm;
     P.at_img = p->d_aimg_t;
     P.codes = (const unsigned char*)codes;
     P.scales = scales;
     P.out = out;
     P.status = p->d_status;
-    const float off = 128.f + (float)(1 << (p->bits - 1));
-    for (int u = 0; u < UMAX; ++u) P.corr[u] = u < U ? 32.f * off * (float)p->a_colsum[u] : 0.f;
-    const int smem = (int)sizeof(Smem) + 1024;
-    const int grid = P.n_groups < p->sm_count ? P.n_groups : p->sm_count;
-    const bool pdl = p->pdl != 0;
-    cudaError_t e;
-    if (out_dtype == GBS_DTYPE_F32) {
-        if (p->bits == 3) e = launch(k_tc_uv_inv<3, float>, grid, smem, stream, pdl, P);
-        else e = launch(k_tc_uv_inv<4, float>, grid, smem, stream, pdl, P);
-    } else {
-        if (p->bits == 3) e = launch(k_tc_uv_inv<3, __nv_bfloat16>, grid, smem, stream, pdl, P);
-        else e = launch(k_tc_uv_inv<4, __nv_bfloat16>, grid, smem, stream, pdl, P);
-    }
+    const cudaError_t e = V == 32 ? (p->group ? launch<32, true>(p, P, out_dtype, stream) : launch<32, false>(p, P, out_dtype, stream))
+                                  : (p->group ? launch<64, true>(p, P, out_dtype, stream) : launch<64, false>(p, P, out_dtype, stream));
     return (int)e;
 }
