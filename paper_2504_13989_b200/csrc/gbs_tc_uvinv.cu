@@ -190,23 +190,28 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
         const long long row_step = (long long)GROUPS * gridDim.x * TOK;
         const bool live_u = up < P.U;
 
-        // packed codes and scales of one tile, one tile ahead of their unpacking
-        unsigned raw[NW];
-        float my_scale = 0.f;
-        unsigned all_scales = 0u;
-        auto fetch = [&](int n) {
+        // Packed codes and scales of one tile, fetched two tiles ahead of their unpacking (one tile is less than the latency
+        // of a DRAM read).  Nothing here looks at a loaded value: that would stall the warp at the fetch.
+        struct Fetched {
+            unsigned raw[NW];
+            float my_scale, all[SPLIT ? 4 : 1];
+        } buf[2];
+        auto fetch = [&](int n, Fetched& B) {
             const long long row = row_first + (long long)n * row_step;
 #pragma unroll
-            for (int i = 0; i < NW; ++i) raw[i] = 0u;
-            my_scale = 0.f;
-            all_scales = 0u;
+            for (int i = 0; i < NW; ++i) B.raw[i] = 0u;
+            B.my_scale = 0.f;
+#pragma unroll
+            for (int i = 0; i < (SPLIT ? 4 : 1); ++i) B.all[i] = 0.f;
             if (n >= n_grp || row >= P.n_rows) return;
             const float* sp = P.scales + row * P.spr;
             if (SPLIT) {
-                if (live_u) my_scale = __ldg(sp + (up >> P.glog));
-                for (int i = lane; i < P.spr; i += 32) all_scales = max(all_scales, __float_as_uint(__ldg(sp + i)) & 0x7fffffffu);
+                if (live_u) B.my_scale = __ldg(sp + (up >> P.glog));
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (lane + 32 * i < P.spr) B.all[i] = __ldg(sp + lane + 32 * i);
             } else {
-                my_scale = __ldg(sp);
+                B.my_scale = __ldg(sp);
             }
             if (live_u) {
                 const unsigned char* src = P.codes + row * P.code_row_bytes + up * (V * BITS / 8);
@@ -214,31 +219,33 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
 #pragma unroll
                     for (int i = 0; i < NW / 4; ++i) {
                         const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + i);
-                        raw[4 * i] = v.x; raw[4 * i + 1] = v.y; raw[4 * i + 2] = v.z; raw[4 * i + 3] = v.w;
+                        B.raw[4 * i] = v.x; B.raw[4 * i + 1] = v.y; B.raw[4 * i + 2] = v.z; B.raw[4 * i + 3] = v.w;
                     }
                 } else {
 #pragma unroll
-                    for (int i = 0; i < NW; ++i) raw[i] = __ldg(reinterpret_cast<const unsigned*>(src) + i);
+                    for (int i = 0; i < NW; ++i) B.raw[i] = __ldg(reinterpret_cast<const unsigned*>(src) + i);
                 }
             }
         };
 
         // the fetched codes -> operand planes of the n-th tile of this group; returns the factor of its epilogue in `fac`
-        auto unpack_tile = [&](int n, float& fac) -> bool {
+        auto unpack_tile = [&](int n, const Fetched& B, float& fac) -> bool {
             const int it = n * GROUPS + grp, s = it % STAGES;
             unsigned h[V / 2];
-            unpack_rotate<BITS, V>(raw, h);
+            unpack_rotate<BITS, V>(B.raw, h);
             unsigned sh2 = 0u, sl2 = 0u;
             if (SPLIT) {
                 // scales relative to 2^e, the power of two below the token's largest: s = Delta 2^(14-e) in (0, 2^15)
-                const unsigned E = max(__reduce_max_sync(0xffffffffu, all_scales) >> 23, 15u);
-                const float sf = my_scale * __uint_as_float((268u - E) << 23);
+                const float big = fmaxf(fmaxf(fabsf(B.all[0]), fabsf(B.all[SPLIT ? 1 : 0])),
+                                        fmaxf(fabsf(B.all[SPLIT ? 2 : 0]), fabsf(B.all[SPLIT ? 3 : 0])));
+                const unsigned E = max(__reduce_max_sync(0xffffffffu, __float_as_uint(big)) >> 23, 15u);
+                const float sf = B.my_scale * __uint_as_float((268u - E) << 23);
                 const __half sh = __float2half_rn(sf), sl = __float2half_rn(sf - __half2float(sh));
                 sh2 = __half_as_ushort(sh) * 0x10001u;
                 sl2 = __half_as_ushort(sl) * 0x10001u;
                 fac = P.norm * __uint_as_float((E - 4u) << 23);            // 2^(e-14), and 2^10 of the integers' scaling below
             } else {
-                fac = my_scale * P.norm * 16777216.f;                      // the halves are integers times 2^-24
+                fac = B.my_scale * P.norm * 16777216.f;                      // the halves are integers times 2^-24
             }
             // a warp leaves as one
             const bool ok = mbar_wait(&S->abort_flag, &S->empty[s], ((unsigned)(it / STAGES) & 1u) ^ 1u, P.status, 1);
@@ -274,22 +281,23 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
 
         float fac[AHEAD + 1];
         bool alive = true;
-        fetch(0);
+        fetch(0, buf[0]);
+        fetch(1, buf[1]);
 #pragma unroll
         for (int j = 0; j < AHEAD; ++j) {
-            if (alive && j < n_grp) alive = unpack_tile(j, fac[j]);
-            fetch(j + 1);
+            if (alive && j < n_grp) alive = unpack_tile(j, buf[j & 1], fac[j]);
+            fetch(j + 2, buf[j & 1]);
         }
         long long row = row_first;
-        for (int n = 0; alive && n < n_grp; ++n, row += row_step) {
+        // one tile: unpack the one AHEAD of it from buffer B, then finish it; false = leave
+        auto tile = [&](int n, Fetched& B) -> bool {
             if (n + AHEAD < n_grp) {
-                alive = unpack_tile(n + AHEAD, fac[AHEAD]);
-                if (!alive) break;
-                fetch(n + AHEAD + 1);
+                if (!unpack_tile(n + AHEAD, B, fac[AHEAD])) return false;
+                fetch(n + AHEAD + 2, B);
             }
             const int it = n * GROUPS + grp, c = it % ACCS;
             const bool ok = mbar_wait(&S->abort_flag, &S->tfull[c], (unsigned)(it / ACCS) & 1u, P.status, 4);
-            if (!__all_sync(0xffffffffu, ok)) break;
+            if (!__all_sync(0xffffffffu, ok)) return false;
             const bool store = row < P.n_rows && up * V < P.d;
             OutT* dst = reinterpret_cast<OutT*>(P.out) + row * (long long)P.d + up * V;
             tc_fence_after();
@@ -315,6 +323,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
             }
 #pragma unroll
             for (int j = 0; j < AHEAD; ++j) fac[j] = fac[j + 1];
+            row += row_step;
+            return true;
+        };
+        for (int n = 0; alive && n < n_grp; n += 2) {
+            if (!tile(n, buf[AHEAD & 1])) break;
+            if (n + 1 < n_grp && !tile(n + 1, buf[(AHEAD + 1) & 1])) break;
         }
     }
 
