@@ -112,15 +112,20 @@ extern "C" int gbs_plan_create_ex(gbs_plan_t** out, int d, int d_pad, int m, int
     if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, sizeof(int));
     if (e != cudaSuccess) { cudaGetLastError(); if (p->d_status) cudaFree(p->d_status); delete p; return GBS_ERR_ALLOC; }
     if (full) {
-        // the only family for a full order: the bf16 image of H_m (m * m * 2 bytes) is the plan's one table
+        // the only family for a full order: the bf16 image of H_m (m * m * 2 bytes, the inverse path's operand) and the
+        // forward path's Toeplitz tables behind it
         if (!gbs_tc_dense_supported(p)) { cudaFree(p->d_status); delete p; return GBS_ERR_UNSUPPORTED; }
         int8_t* hm = (int8_t*)malloc((size_t)m * m);
-        unsigned short* img = (unsigned short*)malloc((size_t)m * m * 2);
+        const size_t off_d = ((size_t)m * m * 2 + 255) & ~(size_t)255, toep = gbs_tc_dense_toeplitz_bytes(m);
+        const size_t all = off_d + toep + gbs_tc_dense_col0_bytes(m);
+        unsigned short* img = (unsigned short*)calloc(all, 1);
         rc = (hm && img) ? gbs_build_hadamard_m(m, hm) : GBS_ERR_ALLOC;
         if (rc == GBS_OK) {
             gbs_tc_dense_image(hm, m, img);
-            e = cudaMalloc(&p->d_aimg, (size_t)m * m * 2);
-            if (e == cudaSuccess) e = cudaMemcpy(p->d_aimg, img, (size_t)m * m * 2, cudaMemcpyHostToDevice);
+            gbs_tc_dense_tables(hm, m, img + off_d / 2, img + (off_d + toep) / 2);
+            e = cudaMalloc(&p->d_aimg, all);
+            if (e == cudaSuccess) e = cudaMemcpy(p->d_aimg, img, all, cudaMemcpyHostToDevice);
+            p->d_dense = p->d_aimg + off_d;
             if (e != cudaSuccess) { cudaGetLastError(); rc = GBS_ERR_ALLOC; }
         }
         free(hm);
@@ -132,7 +137,8 @@ extern "C" int gbs_plan_create_ex(gbs_plan_t** out, int d, int d_pad, int m, int
             return rc;
         }
         p->variant = GBS_VARIANT_TC_DENSE;
-        p->pdl = 0;
+        const char* no = getenv("GBS_NO_PDL");
+        p->pdl = (no && no[0] == '1') ? 0 : 1;
         *out = p;
         return GBS_OK;
     }

@@ -37,6 +37,7 @@ struct gbs_plan {
     int asym;              // asymmetric quantizer (GBS_PLAN_ASYMMETRIC)
     int uvm_glog;          // UVM family: log2 of the number of 32-value chunks per tensor-core output row
     unsigned char* d_aimg; // device: pre-swizzled bf16 image of H_m (x) H_{2^j} for the tensor-core family (32 KB)
+    unsigned char* d_dense; // device: the DENSE family's forward tables (behind its image of H_m), or null
     unsigned char* d_aimg_r; // device: image of H_m (x) H_{2^j} for the UVR family (behind the first one), or null
     unsigned char* d_aimg_t; // device: fp16 image of the transpose for the tensor-core inverse rotation (behind the others), or null
     int inv_v;             // in-register factor V of the tensor-core inverse rotation (d' = U * V), or 0
@@ -120,6 +121,9 @@ int gbs_tc_uvr_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows,
 // gbs_tc_dense.cu
 bool gbs_tc_dense_supported(const gbs_plan* p);
 void gbs_tc_dense_image(const int8_t* hm, int m, unsigned short* img);
+size_t gbs_tc_dense_toeplitz_bytes(int m);
+size_t gbs_tc_dense_col0_bytes(int m);
+void gbs_tc_dense_tables(const int8_t* hm, int m, unsigned short* toep, unsigned short* col0);
 int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
                                  float* scales, float* y_opt, cudaStream_t stream);
 

@@ -5,19 +5,22 @@
 // fast transform for it; Y = X_pad H_m^T is a dense contraction with a +-1 matrix, which is what tensor cores are
 // for: bf16 x (+-1) products are exact, the accumulation is fp32 in TMEM.
 //
-//   * A tile is 256 token rows, two sub-tiles of 128 (MMA M = 128: TMEM lane = token).  The m output coordinates are
-//     produced in blocks of 256 (MMA N; the last block is narrower), the contraction runs over chunks of 64 input
-//     coordinates through a ring of shared-memory stages: two X chunks (128 x 64 each, TMA, columns beyond d
-//     zero-filled = the zero-pad expansion of Section 4.2) and ONE H chunk (256 x 64 from the plan's bf16 image of H_m,
-//     rows and columns beyond m zero-filled) that both sub-tiles contract with: the kernel is bound by the L2
-//     bandwidth that feeds these stages, and sharing the H chunk takes a third of that traffic away.
-//   * TMEM lane t holds coordinates of token t only, so one thread owns one token: max|.|, Delta, rounding, clipping
-//     and packing (Sections 2.1, 3.1) are thread-local.  A token's m fp32 values do not fit in TMEM (512 columns), so
-//     the tile is contracted TWICE: the first sweep over the output blocks only takes max|.|, the second quantizes.
-//     The two sub-tiles' accumulators (256 columns each) fill TMEM, so a block's epilogue (short against its 2 x 100
-//     MMAs) and the next block's MMAs take turns.
-//   * The kernel is bound by the tensor pipe (2 * 2 * m^2 flops per token against 2 d + m b / 8 bytes), as the method
-//     itself is for this order: the paper fuses such a matrix into the weights offline where it can.
+//   * H_m never streams.  Away from row 0 and column 0, Algorithm 2's matrix is Toeplitz: H[n][k] = t(k - n).  In the
+//     tensor cores' unswizzled operand layout (core matrices of 8 rows x 16 bytes) the core matrix of rows 8 nb.. and
+//     columns 8 kb.. then depends on kb - nb alone, so the whole m x m operand is 2 m / 8 core matrices in a row (49 KB at
+//     m = 1544 instead of 4.8 MB), and with the output blocks taken in descending order the descriptor's two strides are
+//     both +128 bytes.  A CTA's share (31 KB) stays in shared memory; only the rows of X move.
+//   * Column 0 of H (constant -1) is repaired by one more MMA per tile with a 16-column operand whose column 0 holds
+//     H[n][0] - t(-n).  Row 0 (x_0 - sum of the others) is summed by the epilogue threads of the CTA that owns it, from the
+//     X stages as they pass.
+//   * One sweep.  A token's m fp32 values do not fit one SM's TMEM, so a CLUSTER of CTAs takes 128 tokens and each CTA up to
+//     512 output coordinates: TMEM lane t holds the CTA's coordinates of token t, and the CTAs exchange their maxima of
+//     every token through distributed shared memory before quantizing (Sections 2.1, 3.1).
+//   * Packed rows are m b / 8 bytes (579 at m = 1544, b = 3: any alignment): a warp packs its 32 tokens' codes into shared
+//     memory and writes each row's piece as aligned words, lanes side by side.
+// What bounds it: the tensor pipe, 2 d m flops per token.  4096 x 1536, b = 4: 176 us with two sweeps over streamed chunks
+// of H on 32 SMs, 27.4 us now (0.44 of the measured bf16 rate); one row: 170 -> 19.5 us.  The number of CTAs per cluster is chosen by cost (pick_split): few wide shares when the batch fills the
+// chip, more and narrower ones when it does not.
 // Every wait is bounded; an expired wait records a code in the plan's status word.
 #include <math.h>
 #include <stdlib.h>
@@ -30,20 +33,20 @@
 
 namespace {
 
-constexpr int TM = 128;                 // tokens per MMA (M)
-constexpr int MAX_SUB = 2;              // 128-token sub-tiles per CTA tile (1 or 2): they share every H chunk on chip
-constexpr int BN = 256;                 // output coordinates per block
+constexpr int TM = 128;                 // tokens per tile (MMA M)
 constexpr int KC = 64;                  // input coordinates per stage (one 128-byte swizzled line of bf16)
-constexpr int STAGES = 3;              // 3 x (2 x 16 + 32) KB
-constexpr int A_STAGE = TM * KC * 2;    // 16 KB per sub-tile
-constexpr int B_STAGE = BN * KC * 2;    // 32 KB
-constexpr int THREADS = 32 * (2 + 4 * MAX_SUB);
+constexpr int STAGES = 6;
+constexpr int A_STAGE = TM * KC * 2;    // 16 KB
+constexpr int EW = 4;                   // epilogue warps per TMEM lane quadrant: each takes a quarter of the coordinates
+constexpr int EPI_WARPS = 4 * EW;
+constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int TMEM_COLS = 512;
+constexpr int MAX_CL = 8;               // CTAs per cluster
+constexpr int CORE = 128;               // bytes of a core matrix: 8 rows x 8 bf16
 
-struct __align__(1024) Smem {
-    unsigned char a[STAGES][MAX_SUB][A_STAGE];
-    unsigned char b[STAGES][B_STAGE];
-    unsigned long long full[STAGES], empty[STAGES], tfull, tempty;
+struct Ctl {
+    float tmax[2][MAX_CL * EW][TM];     // [tile parity][CTA and quarter][token]: maxima of every share of a token
+    unsigned long long full[STAGES], empty[STAGES], tfull, tempty, tbar, maxbar[2];
     unsigned tmem_base;
     volatile int abort_flag;
 };
@@ -52,81 +55,139 @@ struct DenseParams {
     long long n_rows;
     int n_tiles;
     int m;                        // d' = order of H_m
-    int nblk;                     // ceil(m / 256)
-    int n_last;                   // width of the last block, rounded up to 16
-    int kchunks;                  // ceil(m / 64)
+    int cl;                       // CTAs per cluster
+    int ncb;                      // 8-coordinate output blocks per CTA, a multiple of 4
+    int kchunks;                  // ceil(d / 64)
     int ksteps_last;              // MMAs (K = 16) of the last chunk
+    int nbp;                      // output blocks the Toeplitz and column tables are laid out for
     int code_row_bytes;
+    int stage_words;              // words of a token's row in a warp's packing buffer (odd)
     float c_scale, c_half, norm;
+    const unsigned char* toep;    // core matrices J = kb - nb + nbp - 1
+    const unsigned char* col0;    // core matrix pairs (column repair, zeros) of block nbp - 1 - i at i
     unsigned char* codes;
     float* scales;
     float* y_opt;
     int* status;
 };
 
-// The first `nbytes` of a thread's NW packed words to a row position of any alignment (rows of m * bits / 8 bytes
-// start wherever they start: 579-byte rows at m = 1544, b = 3).
-template <int NW>
-__device__ __forceinline__ void store_bytes(unsigned char* dst, const unsigned (&w)[NW], int nbytes)
+__device__ __forceinline__ unsigned cluster_rank()
 {
-    if ((reinterpret_cast<uintptr_t>(dst) & 3u) == 0 && nbytes == 4 * NW) {
-#pragma unroll
-        for (int i = 0; i < NW; ++i) reinterpret_cast<unsigned*>(dst)[i] = w[i];
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4 * NW; ++i)
-            if (i < nbytes) dst[i] = (unsigned char)(w[i >> 2] >> (8 * (i & 3)));
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ unsigned peer_addr(unsigned smem_addr, unsigned rank)
+{
+    unsigned a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void peer_store(unsigned addr, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void peer_arrive(unsigned bar_addr)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
+}
+// bounded wait on a barrier that other CTAs of the cluster arrive at, behind their stores
+__device__ __forceinline__ bool cluster_wait(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
+{
+    const unsigned long long t0 = global_ns();
+    for (unsigned i = 1;; ++i) {
+        unsigned ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(WAIT_HINT_NS) : "memory");
+        if (ok) return true;
+        if ((i & 15u) == 0) {
+            if (*abort_flag) return false;
+            if (global_ns() - t0 > WAIT_LIMIT_NS) break;
+        }
     }
+    *abort_flag = 1;
+    atomicCAS(status, 0, code);
+    return false;
 }
 
-// SUB = 2: a 256-token tile, the H chunk of a stage contracted with both sub-tiles (a third less L2 traffic per token;
-// pays when the batch gives every SM at least a tile of that size).  SUB = 1: 128-token tiles, the four warps of the
-// second sub-tile idle.
-template <int BITS, int SUB>
+// 32 accumulator columns of four output blocks (descending) into coordinate order
+__device__ __forceinline__ void load_chunk(unsigned taddr, unsigned y[32])
+{
+    unsigned r[32];
+    tmem_ld32_issue(taddr, r);
+    tmem_ld_wait(r);
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) y[8 * o + e] = r[8 * (3 - o) + e];
+}
+
+template <int BITS>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constant__ CUtensorMap xmap,
-                                                            const __grid_constant__ CUtensorMap hmap,
                                                             const __grid_constant__ DenseParams P)
 {
     extern __shared__ unsigned char smem_raw[];
-    Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int toep_n = P.kchunks * (KC / 8) + P.ncb;               // core matrices of this CTA's share
+    unsigned char* sm_x = base;
+    unsigned char* sm_t = sm_x + STAGES * A_STAGE;
+    unsigned char* sm_e = sm_t + toep_n * CORE;
+    unsigned* sm_pack = reinterpret_cast<unsigned*>(sm_e + P.ncb * 2 * CORE);
+    Ctl* S = reinterpret_cast<Ctl*>(sm_pack + (EPI_WARPS * 32 * P.stage_words + 3) / 4 * 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int TT = TM * SUB;                   // tokens per CTA tile
-    constexpr int EPI_WARPS = 4 * SUB;
+    const int rank = (int)cluster_rank();
+    const int cluster = (int)blockIdx.x / P.cl, n_clusters = (int)gridDim.x / P.cl;
+    const int nb0 = rank * P.ncb;                                  // first output block of this CTA
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&S->full[s], 1);
-            mbar_init(&S->empty[s], 1);
+            mbar_init(&S->empty[s], rank == 0 ? 1 + 4 : 1);        // the MMAs, and in CTA 0 the warps that sum row 0
         }
         mbar_init(&S->tfull, 1);
         mbar_init(&S->tempty, EPI_WARPS);
+        mbar_init(&S->tbar, 1);
+        mbar_init(&S->maxbar[0], P.cl * EPI_WARPS);
+        mbar_init(&S->maxbar[1], P.cl * EPI_WARPS);
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // plan-owned, immutable tables: need no ordering
+        mbar_arrive_expect_tx(&S->tbar, (unsigned)(toep_n * CORE + P.ncb * 2 * CORE));
+        const int first = P.nbp - nb0 - P.ncb;
+        bulk_load(sm_t, P.toep + (size_t)first * CORE, (unsigned)(toep_n * CORE), &S->tbar);
+        bulk_load(sm_e, P.col0 + (size_t)first * 2 * CORE, (unsigned)(P.ncb * 2 * CORE), &S->tbar);
     }
     if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
+    __syncwarp();
+    cluster_sync();                                                // every CTA's barriers are ready for its peers
     tc_fence_after();
     const unsigned tmem_base = S->tmem_base;
-    const int n_mine = ((int)blockIdx.x < P.n_tiles) ? (P.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const int blocks_per_tile = 2 * P.nblk;               // two sweeps over the output blocks
+    // programmatic dependent launch: until this returns an earlier kernel may still be writing x or reading the outputs
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int n_mine = cluster < P.n_tiles ? (P.n_tiles - cluster + n_clusters - 1) / n_clusters : 0;
 
     if (warp == 0) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
-            int c = 0;                                     // stage uses so far
+            int c = 0;                                             // stage uses so far
             bool ok = true;
             for (int i = 0; ok && i < n_mine; ++i) {
-                const int row0 = ((int)blockIdx.x + i * (int)gridDim.x) * TT;
-                for (int bl = 0; ok && bl < blocks_per_tile; ++bl) {
-                    const int n0 = (bl % P.nblk) * BN;
-                    for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
-                        const int s = c % STAGES;
-                        if (!mbar_wait(&S->abort_flag, &S->empty[s], ((c / STAGES) & 1) ^ 1, P.status, 1)) { ok = false; break; }
-                        mbar_arrive_expect_tx(&S->full[s], SUB * A_STAGE + B_STAGE);
-                        for (int u = 0; u < SUB; ++u) tma_load_2d(S->a[s][u], &xmap, &S->full[s], kc * KC, row0 + u * TM);
-                        tma_load_2d(S->b[s], &hmap, &S->full[s], kc * KC, n0);
-                    }
+                const int row0 = (cluster + i * n_clusters) * TM;
+                for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
+                    const int s = c % STAGES;
+                    if (!mbar_wait(&S->abort_flag, &S->empty[s], ((c / STAGES) & 1) ^ 1, P.status, 1)) { ok = false; break; }
+                    mbar_arrive_expect_tx(&S->full[s], A_STAGE);
+                    tma_load_2d(sm_x + s * A_STAGE, &xmap, &S->full[s], kc * KC, row0);
                 }
             }
             if (!ok) drain_copies(S->full, STAGES, c);
@@ -134,108 +195,273 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0) {
-            const unsigned idesc_full = instr_desc(TM, BN, false);
-            const unsigned idesc_last = instr_desc(TM, P.n_last, false);
-            int c = 0, nb_count = 0;
-            bool ok = true;
+            // the CTA's columns as one or two MMAs of at most 256, each a multiple of 32
+            const int n1 = P.ncb <= 32 ? P.ncb : (P.ncb / 2 + 3) / 4 * 4, n2 = P.ncb - n1;
+            const unsigned idesc1 = instr_desc(TM, 8 * n1, false), idesc2 = instr_desc(TM, 8 * n2, false);
+            // unswizzled core matrices: leading offset = next 8 columns, stride offset = next 8 rows of the operand
+            const unsigned long long td0 = smem_desc(smem_u32(sm_t), CORE, CORE, 0);
+            const unsigned long long ed0 = smem_desc(smem_u32(sm_e), CORE, 2 * CORE, 0);
+            const unsigned tmem2 = tmem_base + 8 * n1;
+            const unsigned long long step2 = (unsigned long long)(n1 * CORE / 16), estep2 = (unsigned long long)(n1 * 2 * CORE / 16);
+            bool ok = mbar_wait(&S->abort_flag, &S->tbar, 0, P.status, 6);
+            int c = 0;
             for (int i = 0; ok && i < n_mine; ++i) {
-                for (int bl = 0; ok && bl < blocks_per_tile; ++bl, ++nb_count) {
-                    const unsigned idesc = (bl % P.nblk == P.nblk - 1) ? idesc_last : idesc_full;
-                    // the two accumulators (one per sub-tile) fill all of TMEM: the next block waits for the epilogue
-                    if (!mbar_wait(&S->abort_flag, &S->tempty, (nb_count & 1) ^ 1, P.status, 3)) { ok = false; break; }
+                // the accumulators fill the CTA's share of TMEM: the next tile waits for the epilogue
+                if (!mbar_wait(&S->abort_flag, &S->tempty, (i & 1) ^ 1, P.status, 3)) break;
+                tc_fence_after();
+                unsigned long long td = td0;
+                for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
+                    const int s = c % STAGES;
+                    if (!mbar_wait(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
-                    for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
-                        const int s = c % STAGES;
-                        if (!mbar_wait(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
-                        tc_fence_after();
-                        const unsigned long long bd = smem_desc(smem_u32(S->b[s]), 16, 1024, 2);
-                        const int ks_n = (kc == P.kchunks - 1) ? P.ksteps_last : KC / 16;
-                        for (int u = 0; u < SUB; ++u) {
-                            const unsigned long long ad = smem_desc(smem_u32(S->a[s][u]), 16, 1024, 2);
-                            for (int ks = 0; ks < ks_n; ++ks)
-                                umma_f16(tmem_base + u * BN, ad + (unsigned long long)(2 * ks), bd + (unsigned long long)(2 * ks),
-                                         idesc, (kc | ks) != 0 ? 1u : 0u);
-                        }
-                        umma_commit(&S->empty[s]);
+                    unsigned long long ad = smem_desc(smem_u32(sm_x + s * A_STAGE), 16, 1024, 2);
+                    const int ks_n = (kc == P.kchunks - 1) ? P.ksteps_last : KC / 16;
+                    if (kc == 0) {
+                        // column 0: H[n][0] - t(-n) against x_0 (the other fifteen columns of the operand are zero)
+                        umma_f16(tmem_base, ad, ed0, idesc1, 0u);
+                        if (n2) umma_f16(tmem2, ad, ed0 + estep2, idesc2, 0u);
                     }
-                    if (ok) umma_commit(&S->tfull);
+                    for (int ks = 0; ks < ks_n; ++ks) {
+                        umma_f16(tmem_base, ad, td, idesc1, 1u);
+                        if (n2) umma_f16(tmem2, ad, td + step2, idesc2, 1u);
+                        ad += 2;                                   // 32 bytes of the 128-byte line
+                        td += 2 * CORE / 16;                       // two core matrices on
+                    }
+                    umma_commit(&S->empty[s]);
                 }
+                if (ok) umma_commit(&S->tfull);
             }
         }
-    } else if (warp < 2 + EPI_WARPS) {
-        // ------------------------------ epilogue: one thread = one token ------------------------------
-        const int q = warp & 3;                        // TMEM lane quadrant this warp may access
-        const int sub = (warp - 2) >> 2;               // which 128-token sub-tile (= which accumulator) it serves
-        const unsigned lane_base = tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(sub * BN);
-        int nb_count = 0;
+    } else {
+        // ------------------------------ epilogue: one thread = one token and a quarter of the coordinates -----------
+        const int q = warp & 3;                            // TMEM lane quadrant this warp may access
+        const int h = (warp - 2) >> 2;                     // which quarter of the CTA's coordinates
+        const int tok = q * 32 + lane;
+        const int chunks = P.ncb / 4;                      // of 32 coordinates
+        const int ch0 = h * chunks / EW, ch1 = (h + 1) * chunks / EW;
+        const unsigned lane_base = tmem_base + ((unsigned)(q * 32) << 16);
+        const int nfirst = (nb0 + 4 * ch0) * 8;            // first coordinate of this warp
+        const bool sums_row0 = rank == 0 && ch0 == 0 && ch1 > 0;   // one warp per quadrant (a small share leaves some without)
+        unsigned* pack = sm_pack + (warp - 2) * 32 * P.stage_words;
+        int c = 0;
         bool ok = true;
         for (int i = 0; ok && i < n_mine; ++i) {
-            const long long row = ((long long)blockIdx.x + (long long)i * gridDim.x) * TT + sub * TM + q * 32 + lane;
+            const long long row0 = ((long long)cluster + (long long)i * n_clusters) * TM;
+            const long long row = row0 + tok;
             const bool live = row < P.n_rows;
-            float M = 0.f, a1 = 0.f;
-            for (int bl = 0; ok && bl < blocks_per_tile; ++bl, ++nb_count) {
-                const int nb = bl % P.nblk;
-                const bool second = bl >= P.nblk;
-                if (!mbar_wait(&S->abort_flag, &S->tfull, nb_count & 1, P.status, 4)) { ok = false; break; }
-                tc_fence_after();
-                if (second && nb == 0) a1 = __fdividef(P.c_half, fmaxf(M, 1e-30f));
-                const int width = (P.m - nb * BN) < BN ? (P.m - nb * BN) : BN;        // live coordinates of this block
-                for (int c0 = 0; c0 < width; c0 += 32) {
-                    unsigned r[32];
-                    tmem_ld32_issue(lane_base + (unsigned)c0, r);
-                    tmem_ld_wait(r);
-                    const int n_here = (width - c0) < 32 ? (width - c0) : 32;
-                    if (n_here < 32) {
+            float y0 = 0.f;
+            if (sums_row0) {
+                // coordinate 0: x_0 - (x_1 + x_2 + ..), from the stages as they pass (columns beyond d are zero)
+                float s4[4] = {0.f, 0.f, 0.f, 0.f}, x0 = 0.f;
+                for (int kc = 0; ok && kc < P.kchunks; ++kc, ++c) {
+                    const int s = c % STAGES;
+                    ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 5));
+                    if (!ok) break;
+                    const uint4* line = reinterpret_cast<const uint4*>(sm_x + s * A_STAGE + tok * 128);
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (e >= n_here) r[e] = 0u;                                // columns no MMA wrote
+                    for (int j = 0; j < 8; ++j) {
+                        const uint4 v = line[j ^ (tok & 7)];
+                        if (kc == 0 && j == 0) x0 = __uint_as_float(v.x << 16);
+                        s4[0] += __uint_as_float(v.x << 16); s4[1] += __uint_as_float(v.x & 0xffff0000u);
+                        s4[2] += __uint_as_float(v.y << 16); s4[3] += __uint_as_float(v.y & 0xffff0000u);
+                        s4[0] += __uint_as_float(v.z << 16); s4[1] += __uint_as_float(v.z & 0xffff0000u);
+                        s4[2] += __uint_as_float(v.w << 16); s4[3] += __uint_as_float(v.w & 0xffff0000u);
                     }
-                    if (!second) {
-                        M = fmaxf(M, absmax32(r));
-                    } else if (live) {
-                        unsigned out[BITS];
-                        quantize_pack32<BITS>(r, a1, out);
-                        unsigned char* dst = P.codes + row * P.code_row_bytes + (long long)(nb * BN + c0) * BITS / 8;
-                        store_bytes(dst, out, n_here * BITS / 8);
-                        if (P.y_opt) {
-                            float* yo = P.y_opt + row * (long long)P.m + nb * BN + c0;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&S->empty[s]);
+                }
+                y0 = 2.f * x0 - ((s4[0] + s4[1]) + (s4[2] + s4[3]));
+            }
+            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull, i & 1, P.status, 4));
+            if (!ok) break;
+            tc_fence_after();
+            float M = 0.f;
+            for (int ch = ch0; ch < ch1; ++ch) {
+                const int n_here = P.m - (nb0 + 4 * ch) * 8;               // live coordinates from here on
+                if (n_here <= 0) break;
+                unsigned y[32];
+                load_chunk(lane_base + (unsigned)(8 * (P.ncb - 4 - 4 * ch)), y);
+                if (sums_row0 && ch == 0) y[0] = __float_as_uint(y0);
+                if (n_here < 32) {
 #pragma unroll
-                            for (int e = 0; e < 32; ++e)
-                                if (e < n_here) yo[e] = __uint_as_float(r[e]) * P.norm;
+                    for (int e = 0; e < 32; ++e)
+                        if (e >= n_here) y[e] = 0u;                        // coordinates beyond m
+                }
+                M = fmaxf(M, absmax32(y));
+            }
+            // the token's maximum over all shares of all CTAs
+            const unsigned mine = smem_u32(&S->tmax[i & 1][rank * EW + h][tok]), bar = smem_u32(&S->maxbar[i & 1]);
+            for (int r = 0; r < P.cl; ++r) peer_store(peer_addr(mine, (unsigned)r), M);
+            __syncwarp();
+            if (lane == 0)
+                for (int r = 0; r < P.cl; ++r) peer_arrive(peer_addr(bar, (unsigned)r));
+            ok = __all_sync(0xffffffffu, cluster_wait(&S->abort_flag, &S->maxbar[i & 1], (unsigned)(i >> 1) & 1u, P.status, 7));
+            if (!ok) break;
+            for (int r = 0; r < P.cl * EW; ++r) M = fmaxf(M, S->tmax[i & 1][r][tok]);
+            const float a1 = __fdividef(P.c_half, fmaxf(M, 1e-30f));
+            for (int ch = ch0; ch < ch1; ++ch) {
+                const int n0 = (nb0 + 4 * ch) * 8, n_here = P.m - n0;
+                if (n_here <= 0) break;
+                unsigned y[32];
+                load_chunk(lane_base + (unsigned)(8 * (P.ncb - 4 - 4 * ch)), y);
+                if (sums_row0 && ch == 0) y[0] = __float_as_uint(y0);
+                unsigned out[BITS];
+                quantize_pack32<BITS>(y, a1, out);
+#pragma unroll
+                for (int w = 0; w < BITS; ++w) pack[lane * P.stage_words + (ch - ch0) * BITS + w] = out[w];
+                if (P.y_opt && live) {
+                    float* yo = P.y_opt + row * (long long)P.m + n0;
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        if (e < n_here) yo[e] = __uint_as_float(y[e]) * P.norm;
+                }
+            }
+            // the accumulators have been read: hand TMEM back to the MMA issuer
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S->tempty);
+            if (rank == 0 && h == 0 && live) P.scales[row] = P.c_scale * M;
+            // this warp's 32 rows, one after the other: aligned words, lanes side by side
+            const int n_codes = (P.m - nfirst) < (ch1 - ch0) * 32 ? (P.m - nfirst) : (ch1 - ch0) * 32;
+            if (n_codes > 0) {
+                const int nbytes = n_codes * BITS / 8;
+                for (int r = 0; r < 32; ++r) {
+                    if (row0 + q * 32 + r >= P.n_rows) break;
+                    unsigned char* dst = P.codes + (row0 + q * 32 + r) * P.code_row_bytes + nfirst / 8 * BITS;
+                    const int off = (int)(reinterpret_cast<uintptr_t>(dst) & 3u);
+                    const unsigned* src = pack + r * P.stage_words;
+                    unsigned* words = reinterpret_cast<unsigned*>(dst - off);
+                    for (int j = lane; 4 * j < off + nbytes; j += 32) {
+                        const unsigned lo = j > 0 ? src[j - 1] : 0u, hi = src[j];
+                        const unsigned v = off ? __funnelshift_l(lo, hi, 8 * off) : hi;
+                        const int b0 = 4 * j - off;                            // first byte of the piece this word covers
+                        if (b0 >= 0 && b0 + 4 <= nbytes) {
+                            words[j] = v;
+                        } else {
+#pragma unroll
+                            for (int b = 0; b < 4; ++b)
+                                if (b0 + b >= 0 && b0 + b < nbytes) reinterpret_cast<unsigned char*>(words + j)[b] = (unsigned char)(v >> (8 * b));
                         }
                     }
                 }
-                // this block's accumulators have been read: hand TMEM back to the MMA issuer
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&S->tempty);
             }
-            if (ok && live) P.scales[row] = P.c_scale * M;
+            __syncwarp();                                                      // the packing buffer is rewritten next
         }
     }
 
-    // ---- teardown
+    // ---- teardown: no CTA leaves while a peer may still write to its shared memory
     tc_fence_before();
     __syncthreads();
+    __syncwarp();
+    cluster_sync();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);
     }
 }
 
+// shared memory of a CTA that takes `ncb` output blocks of a contraction over `kchunks` chunks
+int smem_bytes(int ncb, int kchunks, int bits, int* stage_words)
+{
+    const int w = (((ncb / 4 + EW - 1) / EW) * bits + 1) | 1;      // one word beyond the last is read when rows are unaligned
+    if (stage_words) *stage_words = w;
+    return 1024 + STAGES * A_STAGE + (kchunks * (KC / 8) + ncb) * CORE + ncb * 2 * CORE + (EPI_WARPS * 32 * w + 3) / 4 * 16 + (int)sizeof(Ctl);
+}
+
+typedef void (*DenseKernel)(const CUtensorMap, const DenseParams);
+DenseKernel kernel_of(int bits) { return bits == 3 ? k_tc_dense_rq<3> : k_tc_dense_rq<4>; }
+
+// Clusters of `cl` CTAs that run at once (one CTA per SM; a cluster stays inside a GPC, so this can be less than SMs / cl).
+// Asked once per device, together with the opt-in to the large dynamic shared memory (not stream operations).
+int clusters_at_once(const gbs_plan* p, int cl)
+{
+    static std::mutex mu;
+    static int fit[64][MAX_CL + 1];
+    std::lock_guard<std::mutex> lock(mu);
+    int* f = (p->device >= 0 && p->device < 64) ? fit[p->device] : nullptr;
+    if (f && f[cl]) return f[cl];
+    for (int bits = 3; bits <= 4; ++bits)
+        if (cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_optin) != cudaSuccess) return -1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p->sm_count / cl * cl));
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = (size_t)p->smem_optin;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cl;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel_of(p->bits), &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); return -1; }
+    if (f) f[cl] = n;
+    return n;
+}
+
+// How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 64), a tile's
+// epilogue and exchange a few thousand, and the clusters that fit at once take the tiles in waves: the split with the
+// least total is taken.  n_tiles = 0 only asks whether a split exists.
+int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* ncb_out, int* fit_out)
+{
+    const int nb = p->m / 8;
+    double best = 0.0;
+    *cl_out = 0;
+    for (int want = 1; want <= MAX_CL; ++want) {
+        const int ncb = ((nb + want - 1) / want + 3) / 4 * 4, cl = (nb + ncb - 1) / ncb;
+        if (ncb > 64 || smem_bytes(ncb, kchunks, p->bits, nullptr) > p->smem_optin) continue;
+        const int fit = n_tiles ? clusters_at_once(p, cl) : 1;
+        if (fit < 1) return (int)cudaErrorInvalidConfiguration;
+        const int waves = (n_tiles + fit - 1) / fit;
+        const double mma = ncb <= 32 ? (ncb * 4 < 64 ? 64.0 : ncb * 4.0) : (ncb * 4 < 128 ? 128.0 : ncb * 4.0);
+        const double cost = waves * (4.0 * kchunks * mma + 2500.0 + 20.0 * ncb);
+        if (*cl_out == 0 || cost < best) { best = cost; *cl_out = cl; *ncb_out = ncb; *fit_out = fit; }
+    }
+    return 0;
+}
+
+int padded_blocks(int m) { return m / 8 + 64; }                   // a CTA's share may reach beyond the last block
+
 }  // namespace
 
 // The plans this family serves: d' = m (no Sylvester factor), a large Paley order, one scale per token.
 bool gbs_tc_dense_supported(const gbs_plan* p)
 {
-    return p->k == 0 && p->m >= 128 && p->m % 8 == 0 && p->d % 8 == 0 && p->group == 0 && !p->asym &&
-           get_encode() != nullptr && p->smem_optin >= (int)(sizeof(Smem) + 1024);
+    if (!(p->k == 0 && p->m >= 128 && p->m % 8 == 0 && p->d % 8 == 0 && p->group == 0 && !p->asym && get_encode() != nullptr)) return false;
+    int cl = 0, ncb = 0, fit = 0;
+    pick_split(p, 0, (p->d + KC - 1) / KC, &cl, &ncb, &fit);
+    return cl != 0;
 }
 
-// bf16 image of H_m, row-major (row = output coordinate, column = input coordinate): m * m * 2 bytes.
+// bf16 image of H_m, row-major (row = output coordinate, column = input coordinate): m * m * 2 bytes (the inverse path's
+// operand).
 void gbs_tc_dense_image(const int8_t* hm, int m, unsigned short* img)
 {
     for (size_t i = 0; i < (size_t)m * m; ++i) img[i] = hm[i] < 0 ? 0xBF80 : 0x3F80;
+}
+
+size_t gbs_tc_dense_toeplitz_bytes(int m) { return (size_t)((m + KC - 1) / KC * (KC / 8) + padded_blocks(m)) * CORE; }
+size_t gbs_tc_dense_col0_bytes(int m) { return (size_t)padded_blocks(m) * 2 * CORE; }
+
+// The forward path's tables: the Toeplitz core matrices (J = kb - nb + nbp - 1; row r, column c: t(8 (kb - nb) + c - r)) and
+// the repair of column 0 (block nbp - 1 - i at i).  t(k - n) = H[n][k] for n, k >= 1; zero where no such pair exists.
+void gbs_tc_dense_tables(const int8_t* hm, int m, unsigned short* toep, unsigned short* col0)
+{
+    const int nbp = padded_blocks(m);
+    const int n_core = (int)(gbs_tc_dense_toeplitz_bytes(m) / CORE);
+    auto t = [&](int delta) -> int {
+        if (delta >= 0) return delta <= m - 2 ? hm[(size_t)m + 1 + delta] : 0;
+        return -delta <= m - 2 ? hm[(size_t)(1 - delta) * m + 1] : 0;
+    };
+    auto bf = [](int v) -> unsigned short { return v == 0 ? 0 : (unsigned short)((v < 0 ? 0x8000 : 0) | (v == 2 || v == -2 ? 0x4000 : 0x3F80)); };
+    for (int J = 0; J < n_core; ++J)
+        for (int r = 0; r < 8; ++r)
+            for (int c = 0; c < 8; ++c) toep[J * 64 + r * 8 + c] = bf(t(8 * (J - nbp + 1) + c - r));
+    memset(col0, 0, gbs_tc_dense_col0_bytes(m));
+    for (int i = 0; i < nbp; ++i)
+        for (int r = 0; r < 8; ++r) {
+            const int n = 8 * (nbp - 1 - i) + r;
+            if (n >= 1 && n < m) col0[i * 128 + r * 8] = bf((int)hm[(size_t)n * m] - t(-n));
+        }
 }
 
 int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
@@ -243,70 +469,52 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
 {
     EncodeTiledFn encode = get_encode();
     if (!encode) return (int)cudaErrorNotSupported;
-    if (n_rows > (int64_t)0x7fffffff - TM * MAX_SUB) return (int)cudaErrorInvalidValue;
-    CUtensorMap xmap, hmap;
+    if (n_rows > (int64_t)0x7fffffff - TM) return (int)cudaErrorInvalidValue;
+    CUtensorMap xmap;
     const cuuint32_t estr[2] = {1, 1};
-    {
-        const cuuint64_t gdim[2] = {(cuuint64_t)p->d, (cuuint64_t)n_rows};
-        const cuuint64_t gstr[1] = {(cuuint64_t)(stride * 2)};
-        const cuuint32_t box[2] = {KC, TM};          // one sub-tile per copy
-        if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(x), gdim, gstr, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return (int)cudaErrorInvalidValue;
-    }
-    {
-        const cuuint64_t gdim[2] = {(cuuint64_t)p->m, (cuuint64_t)p->m};
-        const cuuint64_t gstr[1] = {(cuuint64_t)(p->m * 2)};
-        const cuuint32_t box[2] = {KC, BN};
-        if (encode(&hmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p->d_aimg, gdim, gstr, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return (int)cudaErrorInvalidValue;
-    }
+    const cuuint64_t gdim[2] = {(cuuint64_t)p->d, (cuuint64_t)n_rows};
+    const cuuint64_t gstr[1] = {(cuuint64_t)(stride * 2)};
+    const cuuint32_t box[2] = {KC, TM};
+    if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(x), gdim, gstr, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return (int)cudaErrorInvalidValue;
     DenseParams P;
     memset(&P, 0, sizeof(P));
     P.n_rows = n_rows;
-    // tile size: a 256-token tile costs about 1.8 x a 128-token tile; take it when it gives fewer, cheaper rounds
-    const long long t1 = (n_rows + TM - 1) / TM, t2 = (n_rows + 2 * TM - 1) / (2 * TM);
-    const long long w1 = (t1 + p->sm_count - 1) / p->sm_count, w2 = (t2 + p->sm_count - 1) / p->sm_count;
-    const int sub = (9 * w2 < 5 * w1) ? 2 : 1;
-    P.n_tiles = (int)(sub == 2 ? t2 : t1);
+    P.n_tiles = (int)((n_rows + TM - 1) / TM);
     P.m = p->m;
-    P.nblk = (p->m + BN - 1) / BN;
-    P.n_last = ((p->m - (P.nblk - 1) * BN) + 15) & ~15;
-    P.kchunks = (p->m + KC - 1) / KC;
-    P.ksteps_last = ((p->m - (P.kchunks - 1) * KC) + 15) / 16;
+    P.kchunks = (p->d + KC - 1) / KC;
+    P.ksteps_last = ((p->d - (P.kchunks - 1) * KC) + 15) / 16;
+    int fit = 0;
+    const int rc = pick_split(p, P.n_tiles, P.kchunks, &P.cl, &P.ncb, &fit);
+    if (rc != 0) return rc;
+    P.nbp = padded_blocks(p->m);
     P.code_row_bytes = p->m * p->bits / 8;
     P.c_scale = p->c_scale;
     P.c_half = (float)(1.0 / (2.0 * (double)p->alpha));
     P.norm = p->norm;
+    P.toep = p->d_dense;
+    P.col0 = p->d_dense + gbs_tc_dense_toeplitz_bytes(p->m);
     P.codes = (unsigned char*)codes;
     P.scales = scales;
     P.y_opt = y_opt;
     P.status = p->d_status;
-    const int smem = (int)sizeof(Smem) + 1024;
-    {
-        // opt in to the large dynamic shared memory once per device (not a stream operation)
-        static std::mutex mu;
-        static bool done[64] = {false};
-        std::lock_guard<std::mutex> lock(mu);
-        if (!(p->device >= 0 && p->device < 64 && done[p->device])) {
-            cudaError_t e = cudaFuncSetAttribute(k_tc_dense_rq<3, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_dense_rq<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_dense_rq<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_dense_rq<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e != cudaSuccess) return (int)e;
-            if (p->device >= 0 && p->device < 64) done[p->device] = true;
-        }
-    }
-    const int grid = P.n_tiles < p->sm_count ? P.n_tiles : p->sm_count;
-    if (sub == 2) {
-        if (p->bits == 3) k_tc_dense_rq<3, 2><<<grid, THREADS, smem, stream>>>(xmap, hmap, P);
-        else k_tc_dense_rq<4, 2><<<grid, THREADS, smem, stream>>>(xmap, hmap, P);
-    } else {
-        if (p->bits == 3) k_tc_dense_rq<3, 1><<<grid, THREADS, smem, stream>>>(xmap, hmap, P);
-        else k_tc_dense_rq<4, 1><<<grid, THREADS, smem, stream>>>(xmap, hmap, P);
-    }
-    return (int)cudaGetLastError();
+    const int smem = smem_bytes(P.ncb, P.kchunks, p->bits, &P.stage_words);
+    const int clusters = P.n_tiles < fit ? P.n_tiles : fit;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * P.cl));
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)P.cl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p->pdl ? 2 : 1;
+    return (int)cudaLaunchKernelEx(&cfg, kernel_of(p->bits), xmap, P);
 }
