@@ -132,6 +132,11 @@ bool gbs_tc_denseinv_supported(const gbs_plan* p);
 int gbs_tc_denseinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
                                int out_dtype, cudaStream_t stream);
 
+// gbs_qgemv.cu : gbs_quantized_matmul for up to GBS_QGEMV_MAX_TOKENS tokens
+#define GBS_QGEMV_MAX_TOKENS 64
+int gbs_qgemv(const gbs_plan* px, const void* codes_x, const float* scales_x, int n_tokens, const gbs_plan* pw, const void* codes_w,
+              const float* scales_w, int64_t n_out, void* out, int out_dtype, int64_t out_row_stride, cudaStream_t stream);
+
 // gbs_tc_row.cu
 bool gbs_tc_row_supported(const gbs_plan* p);
 int gbs_tc_row_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,

@@ -30,6 +30,7 @@
 #include <mutex>
 
 #include "gbs_internal.h"
+#include "gbs_qfields.cuh"
 #include "gbs_tc_common.cuh"
 
 namespace {
@@ -86,27 +87,6 @@ __device__ __forceinline__ void umma_i8(unsigned d_tmem, unsigned long long a_de
 __device__ __forceinline__ void st_shared_v4(unsigned addr, uint4 v)
 {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
-// Eight two's-complement fields (24 or 32 bits) -> two words of four int8 each: the even fields, the odd fields.
-// No sign extension is computed: a field moved to the TOP bits of its byte is the int8 value q * 2^(8 - BITS) (the
-// field's sign bit becomes the byte's), products are then scaled by a power of two that the epilogue's scale factor
-// takes out exactly, and the int32 sums stay far below 2^31 (49 * d' * 2^10 at most).  Four-bit fields already sit in
-// nibbles: one mask for the odd ones, a shift and a mask for the even ones.  Three-bit fields are first spread to one
-// per nibble by three mask-and-shift steps.
-template <int BITS>
-__device__ __forceinline__ void fields_to_int8(unsigned f, unsigned& even, unsigned& odd)
-{
-    if (BITS == 4) {
-        odd = f & 0xf0f0f0f0u;
-        even = (f << 4) & 0xf0f0f0f0u;
-    } else {
-        f = (f & 0x00000fffu) | ((f & 0x00fff000u) << 4);       // 12 bits per half-word
-        f = (f & 0x003f003fu) | ((f & 0x0fc00fc0u) << 2);       // 6 bits per byte
-        f = (f & 0x07070707u) | ((f & 0x38383838u) << 1);       // 3 bits per nibble (bit 3 of every nibble clear)
-        odd = (f << 1) & 0xe0e0e0e0u;
-        even = (f << 5) & 0xe0e0e0e0u;
-    }
 }
 
 // NF fields of a row slice, from its packed words (3 words per 4 fields at 3 bits, 1 word per field at 4 bits).
@@ -364,6 +344,14 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     gbs_device_guard guard;
     if (guard.enter(px->device) != cudaSuccess) { cudaGetLastError(); return GBS_ERR_CUDA; }
 
+    // up to 64 tokens the call is bound by reading the weights: no 128-token tile, the whole chip on the weight rows (crossover
+    // in gbs_qgemv.cu)
+    if (n_tokens <= GBS_QGEMV_MAX_TOKENS) {
+        const int e = gbs_qgemv(px, codes_x, scales_x, (int)n_tokens, pw, codes_w, scales_w, n_out, out, out_dtype, out_row_stride,
+                                static_cast<cudaStream_t>(cuda_stream));
+        if (e != 0) cudaGetLastError();
+        return e == 0 ? GBS_OK : GBS_ERR_CUDA;
+    }
     QgemmParams P;
     memset(&P, 0, sizeof(P));
     P.n_tok = n_tokens;
