@@ -11,19 +11,20 @@
 // an INTEGER contraction over the d' codes followed by one multiplication per output.  The rotated activation never
 // exists in memory as floats: this kernel reads the packed codes of both operands.  (Up to 64 tokens: gbs_qgemv.cu.)
 //
-//   * Output channels are the rows of the MMA (TMEM lane = channel), tokens its columns.  A tile is 128 channels x N tokens
-//     on one SM, or 256 x N on a pair of SMs (cta_group::2): each SM unpacks 128 rows of weights and half of the tokens, so
-//     a code of either operand is unpacked once per 256 outputs of the other.
-//   * Packed codes arrive by TMA (128 codes of every row per step, four steps ahead).  Sixteen warps unpack, one thread per row:
-//     a field moved to the top bits of its byte IS the int8 q * 2^(8-b) (the epilogue removes the power of two).  Weights go to
-//     TENSOR MEMORY (a thread's 128 int8 are 32 columns of its lane), tokens to 128-byte-swizzled K-major rows in shared memory;
-//     both use the same order of the codes inside a word (even fields, then odd), which a dot product does not see.
-//   * One thread issues tcgen05.mma kind::i8 (int32 accumulators, exact); two accumulators in TMEM, so that four epilogue
-//     warps convert and store a tile while the next one is contracted.  Lanes of a warp hold consecutive channels, so every
-//     store instruction writes 64 or 128 contiguous bytes of one token's row.
-// What bounds it: the shared-memory port (per step and SM: packed codes in and out, token operand in and out) about level
-// with the tensor pipe for pairs.  The single-SM kernel before it fetched packed codes with global loads, kept both operands in
-// shared memory and held the L1 74 % busy: 139 us for 4096 x 4096 x 4096 at 4 bits.
+//   * Output channels are the rows of the MMA (TMEM lane = channel), tokens its columns: a tile is 128 channels x up to 256
+//     tokens on one SM.
+//   * Packed codes arrive by TMA (128 codes of every row per step, several steps ahead).  Twenty-four warps unpack, one thread
+//     per row: a field moved to the top bits of its byte IS the int8 q * 2^(8-b) (the epilogue removes the power of two).
+//     Weights go to TENSOR MEMORY (a thread's 128 int8 are 32 columns of its lane), tokens to 128-byte-swizzled K-major rows in
+//     shared memory; both use the same order of the codes inside a word (even fields, then odd), which a dot product does not see.
+//   * One thread issues tcgen05.mma kind::i8 (int32 accumulators, exact).  Consecutive tiles use accumulators that overlap by
+//     half (or not at all, up to 128 tokens); four epilogue warps drain the shared half first, so that the next tile starts
+//     early.  Lanes of a warp hold consecutive channels, so every store instruction writes 64 or 128 contiguous bytes.
+// What bounds it: narrow tiles, the latencies a warp set goes through per step (about 1200 cycles: packed codes, a free stage,
+// its stores becoming visible to the tensor cores; two or three sets take turns).  256-token tiles, the shared-memory port:
+// 24 KB of packed codes in and out and 32 KB of int8 in and out are about 900 of a step's 1016 cycles, the tensor pipe 512.
+// 4096 x 4096 x 4096, 4 bits: 139 us (one 128 x 256 tile per CTA, both operands in shared memory, packed codes by global
+// loads), 118 us (256 x 192 on SM pairs, cta_group::2: the arrivals across the pair double the step), 70 us now.
 // Every wait is bounded; an expired wait records a code in the activation plan's status word.
 #include <math.h>
 #include <string.h>
@@ -37,22 +38,29 @@
 namespace {
 
 constexpr int KB = 128;                 // codes per step and row: one 128-byte line of int8
-constexpr int ROWS = 128;               // rows of each operand one SM unpacks at most
-constexpr int STAGES = 4;               // of packed codes, and of unpacked operands; even: see `set` below
-constexpr int P_OPERAND = ROWS * 64;    // packed bytes of one operand's rows in a stage (64 or 48 per row)
-constexpr int B_STAGE = ROWS * KB;      // 16 KB of int8
-constexpr int SETS = 2;                 // warp sets that take alternate steps
-constexpr int UNPACK_WARPS = 8 * SETS;  // per set: four for the weights (one per TMEM lane quadrant), four for the tokens
+constexpr int TM = 128;                 // output channels per tile
+constexpr int UNPACK_WARPS = 24;
 constexpr int EPI_WARPS = 4;
 constexpr int THREADS = 32 * (2 + UNPACK_WARPS + EPI_WARPS);
 constexpr int TMEM_COLS = 512;
-constexpr int ACC_COLS = 192;           // columns of an accumulator: two of them, and STAGES x 32 columns of weights
-constexpr int A_COL0 = 2 * ACC_COLS;
+constexpr int MAX_STAGES = 6;
 
-struct __align__(1024) Smem {
-    unsigned char p[STAGES][2][P_OPERAND];
-    unsigned char b[STAGES][B_STAGE];
-    unsigned long long pfull[STAGES], pempty[STAGES], ofull[STAGES], oempty[STAGES], tfull[2], tempty[2];
+// TW warps of a set unpack tokens (32 rows each), four unpack weights.  Sets take alternate steps; a stage belongs to one set,
+// which therefore takes part in every phase of the barriers it waits for.
+template <int TW> struct Shape {
+    static constexpr int SETS = UNPACK_WARPS / (4 + TW);            // TW = 4: three, TW = 8: two
+    static constexpr int STAGES = TW == 8 ? 4 : 6;
+    static constexpr int TN = 32 * TW;                              // tokens per tile at most
+    static constexpr int P_STAGE = (TM + TN) * 64;                  // packed bytes of a stage (64 or 48 per row)
+    static constexpr int B_STAGE = TN * KB;                         // int8 tokens of a stage
+    static constexpr int ACC_STEP = 128;                            // second accumulator's first column
+    static constexpr int A_COL0 = TW == 8 ? 384 : 256;              // weights: 32 columns per stage
+    static constexpr int SMEM = 1024 + STAGES * (P_STAGE + B_STAGE) + 512;
+    static_assert(STAGES % SETS == 0 && A_COL0 + 32 * STAGES <= TMEM_COLS, "stages");
+};
+
+struct Ctl {
+    unsigned long long pfull[MAX_STAGES], pempty[MAX_STAGES], ofull[MAX_STAGES], oempty[MAX_STAGES], tfull[2], tempty[2], tshared;
     unsigned tmem_base;
     volatile int abort_flag;
 };
@@ -76,87 +84,11 @@ __host__ __device__ constexpr unsigned instr_desc_i8(int M, int N)
 }
 
 // A from tensor memory, B from shared memory
-template <int CG>
 __device__ __forceinline__ void umma_i8_ts(unsigned d_tmem, unsigned a_tmem, unsigned long long b_desc, unsigned idesc, unsigned accumulate)
 {
-    if (CG == 2)
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::2.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
-                     ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-    else
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
-                     ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// completion of the MMAs so far, on this barrier of every SM of the pair
-template <int CG>
-__device__ __forceinline__ void commit_all(void* bar)
-{
-    if (CG == 2)
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                     ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
-    else
-        umma_commit(bar);
-}
-template <int CG>
-__device__ __forceinline__ void tmem_alloc_cg(unsigned* slot)
-{
-    if (CG == 2) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(TMEM_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-        tmem_alloc(slot, TMEM_COLS);
-    }
-}
-template <int CG>
-__device__ __forceinline__ void tmem_dealloc_cg(unsigned addr)
-{
-    if (CG == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(TMEM_COLS) : "memory");
-    else tmem_dealloc(addr, TMEM_COLS);
-}
-// arrive on a barrier of the pair's first SM (the one that issues the MMAs)
-template <int CG>
-__device__ __forceinline__ void arrive_leader(void* bar)
-{
-    if (CG == 2) {
-        unsigned a;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(bar)), "r"(0));
-        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
-    } else {
-        mbar_arrive(bar);
-    }
-}
-__device__ __forceinline__ bool try_wait_cluster(void* bar, unsigned parity)
-{
-    unsigned ok;
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(WAIT_HINT_NS) : "memory");
-    return ok != 0;
-}
-// bounded wait for arrivals of either SM of the pair
-template <int CG>
-__device__ __forceinline__ bool wait_pair(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
-{
-    if (CG == 1) return mbar_wait(abort_flag, bar, parity, status, code);
-    if (try_wait_cluster(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (unsigned i = 1;; ++i) {
-        if (try_wait_cluster(bar, parity)) return true;
-        if ((i & 15u) == 0) {
-            if (*abort_flag) return false;
-            if (global_ns() - t0 > WAIT_LIMIT_NS) break;
-        }
-    }
-    *abort_flag = 1;
-    atomicCAS(status, 0, code);
-    return false;
-}
-template <int CG>
-__device__ __forceinline__ void pair_sync()
-{
-    if (CG == 2) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
 __device__ __forceinline__ void st_shared_v4(unsigned addr, uint4 v)
@@ -169,88 +101,89 @@ __device__ __forceinline__ uint4 ld_shared_v4(unsigned addr)
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
-// 32 registers -> 32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_st32(unsigned taddr, const unsigned r[32])
+// 8 registers -> 8 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_st8(unsigned taddr, const unsigned r[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+                 ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr) : "memory");
+}
+// 16 columns of this thread's TMEM lane -> 16 registers
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned r[16])
 {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
-        ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-          "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-          "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr) : "memory");
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
 }
 
-// The 128 codes of row r in a packed stage -> 32 words of int8: per octet of codes the even fields, then the odd ones.
-// Four-bit rows are 64 bytes with the 64-byte swizzle (eight rows side by side hit all banks), three-bit rows 48 bytes plain
-// (48-byte steps do so by themselves).
+// The packed 128 codes of row r of a stage.  Four-bit rows are 64 bytes with the 64-byte swizzle (eight rows side by side hit
+// all banks), three-bit rows 48 bytes plain (48-byte steps do so by themselves).
 template <int BITS>
-__device__ __forceinline__ void unpack_row128(unsigned rows, int r, unsigned v[32])
+__device__ __forceinline__ void load_row128(unsigned rows, int r, uint4 w[BITS])
+{
+#pragma unroll
+    for (int c = 0; c < BITS; ++c)
+        w[c] = ld_shared_v4(rows + (unsigned)r * (16u * BITS) + (unsigned)((BITS == 4 ? c ^ ((r >> 1) & 3) : c) << 4));
+}
+// Codes 32 c .. 32 c + 31 of it -> eight words of int8: per octet of codes the even fields, then the odd ones.
+template <int BITS>
+__device__ __forceinline__ void unpack32(const uint4 w[BITS], int c, unsigned v[8])
 {
     if (BITS == 4) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint4 w = ld_shared_v4(rows + (unsigned)r * 64u + (unsigned)((c ^ ((r >> 1) & 3)) << 4));
-            fields_to_int8<4>(w.x, v[8 * c], v[8 * c + 1]);
-            fields_to_int8<4>(w.y, v[8 * c + 2], v[8 * c + 3]);
-            fields_to_int8<4>(w.z, v[8 * c + 4], v[8 * c + 5]);
-            fields_to_int8<4>(w.w, v[8 * c + 6], v[8 * c + 7]);
-        }
+        fields_to_int8<4>(w[c].x, v[0], v[1]);
+        fields_to_int8<4>(w[c].y, v[2], v[3]);
+        fields_to_int8<4>(w[c].z, v[4], v[5]);
+        fields_to_int8<4>(w[c].w, v[6], v[7]);
     } else {
-        unsigned w[12];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const uint4 x = ld_shared_v4(rows + (unsigned)r * 48u + 16u * c);
-            w[4 * c] = x.x; w[4 * c + 1] = x.y; w[4 * c + 2] = x.z; w[4 * c + 3] = x.w;
-        }
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const unsigned w0 = w[3 * g], w1 = w[3 * g + 1], w2 = w[3 * g + 2];
-            fields_to_int8<3>(w0, v[8 * g], v[8 * g + 1]);                       // bits above 24 are dropped by the masks
-            fields_to_int8<3>(__funnelshift_r(w0, w1, 24), v[8 * g + 2], v[8 * g + 3]);
-            fields_to_int8<3>(__funnelshift_r(w1, w2, 16), v[8 * g + 4], v[8 * g + 5]);
-            fields_to_int8<3>(w2 >> 8, v[8 * g + 6], v[8 * g + 7]);
-        }
+        const unsigned f[12] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w, w[2].x, w[2].y, w[2].z, w[2].w};
+        const unsigned w0 = f[3 * c], w1 = f[3 * c + 1], w2 = f[3 * c + 2];
+        fields_to_int8<3>(w0, v[0], v[1]);                                   // bits above 24 are dropped by the masks
+        fields_to_int8<3>(__funnelshift_r(w0, w1, 24), v[2], v[3]);
+        fields_to_int8<3>(__funnelshift_r(w1, w2, 16), v[4], v[5]);
+        fields_to_int8<3>(w2 >> 8, v[6], v[7]);
     }
 }
 
-template <int XBITS, int WBITS, typename OutT, int CG>
+template <int XBITS, int WBITS, typename OutT, int TW>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
                                                          const __grid_constant__ QgemmParams P)
 {
+    typedef Shape<TW> SH;
+    constexpr int STAGES = SH::STAGES, SETS = SH::SETS, SET_WARPS = 4 + TW;
     extern __shared__ unsigned char smem_raw[];
-    Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* sm_b = base;
+    unsigned char* sm_p = base + STAGES * SH::B_STAGE;                            // a stage: weight rows, then token rows
+    Ctl* S = reinterpret_cast<Ctl*>(sm_p + STAGES * SH::P_STAGE);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = CG == 2 ? (int)(blockIdx.x & 1) : 0;
-    const int first = (int)blockIdx.x / CG, step = (int)gridDim.x / CG;          // tiles first, first + step, ..
-    const int nb = P.n / CG;                                                      // token rows this SM unpacks
     constexpr int WB = WBITS * 16, XB = XBITS * 16;                               // packed bytes per row and step
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&S->pfull[s], 1);
-            mbar_init(&S->pempty[s], 8);
-            mbar_init(&S->ofull[s], 8 * CG);
+            mbar_init(&S->pempty[s], SET_WARPS);
+            mbar_init(&S->ofull[s], SET_WARPS);
             mbar_init(&S->oempty[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&S->tfull[a], 1);
-            mbar_init(&S->tempty[a], EPI_WARPS * CG);
+            mbar_init(&S->tempty[a], EPI_WARPS);
         }
+        mbar_init(&S->tshared, EPI_WARPS);
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc_cg<CG>(&S->tmem_base);
+    if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
-    __syncwarp();
-    pair_sync<CG>();                                                             // the peer's barriers are ready
     tc_fence_after();
     const unsigned tmem_base = S->tmem_base;
     // programmatic dependent launch: the codes may still be being written until this returns
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int first = (int)blockIdx.x, step = (int)gridDim.x;
     const int n_mine = first < P.tiles ? (P.tiles - first + step - 1) / step : 0;
 
     if (warp == 0) {
@@ -260,152 +193,178 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
             bool ok = true;
             for (int i = 0; ok && i < n_mine; ++i) {
                 const int tile = first + i * step, mt = tile % P.m_tiles, nt = tile / P.m_tiles;
-                const int w0 = (mt * CG + rank) * ROWS, x0 = nt * P.n + rank * nb;
                 for (int kb = 0; kb < P.kblocks; ++kb, ++c) {
                     const int s = c % STAGES;
                     if (!mbar_wait(&S->abort_flag, &S->pempty[s], ((c / STAGES) & 1) ^ 1, P.status, 1)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&S->pfull[s], (unsigned)(ROWS * WB + nb * XB));
-                    tma_load_2d(S->p[s][0], &wmap, &S->pfull[s], kb * WB, w0);
-                    tma_load_2d(S->p[s][1], &xmap, &S->pfull[s], kb * XB, x0);
+                    mbar_arrive_expect_tx(&S->pfull[s], (unsigned)(TM * WB + P.n * XB));
+                    tma_load_2d(sm_p + s * SH::P_STAGE, &wmap, &S->pfull[s], kb * WB, mt * TM);
+                    tma_load_2d(sm_p + s * SH::P_STAGE + TM * 64, &xmap, &S->pfull[s], kb * XB, nt * P.n);
                 }
             }
             if (!ok) drain_copies(S->pfull, STAGES, c);
         }
     } else if (warp == 1) {
-        // ------------------------------ MMA issuer (the pair's first SM) ------------------------------
-        if (lane == 0 && rank == 0) {
-            const unsigned idesc = instr_desc_i8(ROWS * CG, P.n);
+        // ------------------------------ MMA issuer ------------------------------
+        if (lane == 0) {
+            const unsigned idesc = instr_desc_i8(TM, P.n);
             int c = 0;
             bool ok = true;
             for (int i = 0; ok && i < n_mine; ++i) {
                 const int a = i & 1;
-                if (!wait_pair<CG>(&S->abort_flag, &S->tempty[a], ((i >> 1) & 1) ^ 1, P.status, 3)) break;
+                if (!mbar_wait(&S->abort_flag, &S->tempty[a], ((i >> 1) & 1) ^ 1, P.status, 3)) break;
+                // the columns shared with the tile before are drained first
+                if (TW == 8 && !mbar_wait(&S->abort_flag, &S->tshared, (i & 1) ^ 1, P.status, 3)) break;
                 for (int kb = 0; kb < P.kblocks; ++kb, ++c) {
                     const int s = c % STAGES;
-                    if (!wait_pair<CG>(&S->abort_flag, &S->ofull[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
+                    if (!mbar_wait(&S->abort_flag, &S->ofull[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
                     // an instruction takes 32 codes: eight columns of the weights' lanes, 32 bytes of the tokens' lines
-                    const unsigned long long bd = smem_desc(smem_u32(S->b[s]), 16, 1024, 2);
+                    const unsigned long long bd = smem_desc(smem_u32(sm_b + s * SH::B_STAGE), 16, 1024, 2);
 #pragma unroll
                     for (int ks = 0; ks < KB / 32; ++ks)
-                        umma_i8_ts<CG>(tmem_base + a * ACC_COLS, tmem_base + A_COL0 + s * 32 + ks * 8, bd + (unsigned long long)(2 * ks),
-                                       idesc, (kb | ks) != 0 ? 1u : 0u);
-                    commit_all<CG>(&S->oempty[s]);
+                        umma_i8_ts(tmem_base + a * SH::ACC_STEP, tmem_base + SH::A_COL0 + s * 32 + ks * 8, bd + (unsigned long long)(2 * ks),
+                                   idesc, (kb | ks) != 0 ? 1u : 0u);
+                    umma_commit(&S->oempty[s]);
                 }
-                if (ok) commit_all<CG>(&S->tfull[a]);
+                if (ok) umma_commit(&S->tfull[a]);
             }
         }
     } else if (warp < 2 + UNPACK_WARPS) {
         // ------------------------------ unpack ------------------------------
-        // Two sets of eight warps take alternate steps, so that one set's waits (packed codes, a free stage, its own stores
-        // becoming visible) are covered by the other's work.  STAGES is even: a stage belongs to one set, which therefore takes
-        // part in every phase of the barriers it waits for.
-        const int set = (warp - 2) >> 3, role = ((warp - 2) >> 2) & 1, q = warp & 3, r = q * 32 + lane;
-        const unsigned lane_base = tmem_base + ((unsigned)(q * 32) << 16) + A_COL0;
+        // Sets take alternate steps, so that one set's waits are covered by the others' work.
+        const int set = (warp - 2) / SET_WARPS, member = (warp - 2) % SET_WARPS;
+        const bool weights = member < 4;
+        const int r = weights ? (warp & 3) * 32 + lane : (member - 4) * 32 + lane;     // weights: the warp's own lane quadrant
+        const unsigned lane_base = tmem_base + ((unsigned)((warp & 3) * 32) << 16) + SH::A_COL0;
         const int total = n_mine * P.kblocks;
-        const bool have = role == 0 || r < nb;
+        const bool have = weights || r < P.n;
         for (int c = set; c < total; c += SETS) {
             const int s = c % STAGES;
             const unsigned ph = (unsigned)(c / STAGES) & 1u;
             bool ok = mbar_wait(&S->abort_flag, &S->pfull[s], ph, P.status, 4);
             if (!__all_sync(0xffffffffu, ok)) break;                             // a warp leaves as one
-            unsigned v[32];
-            if (role == 0) unpack_row128<WBITS>(smem_u32(S->p[s][0]), r, v);
-            else if (have) unpack_row128<XBITS>(smem_u32(S->p[s][1]), r, v);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S->pempty[s]);
-            ok = mbar_wait(&S->abort_flag, &S->oempty[s], ph ^ 1u, P.status, 5);
-            if (!__all_sync(0xffffffffu, ok)) break;
-            if (role == 0) {
+            const unsigned rows = smem_u32(sm_p + s * SH::P_STAGE);
+            if (weights) {
+                uint4 w[WBITS];
+                load_row128<WBITS>(rows, r, w);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S->pempty[s]);
+                ok = mbar_wait(&S->abort_flag, &S->oempty[s], ph ^ 1u, P.status, 5);
+                if (!__all_sync(0xffffffffu, ok)) break;
                 tc_fence_after();
-                tmem_st32(lane_base + s * 32, v);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    unsigned v[8];
+                    unpack32<WBITS>(w, k, v);
+                    tmem_st8(lane_base + s * 32 + k * 8, v);
+                }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
             } else {
+                uint4 w[XBITS];
+                if (have) load_row128<XBITS>(rows + TM * 64, r, w);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S->pempty[s]);
+                ok = mbar_wait(&S->abort_flag, &S->oempty[s], ph ^ 1u, P.status, 5);
+                if (!__all_sync(0xffffffffu, ok)) break;
                 if (have) {
-                    const unsigned line = smem_u32(S->b[s]) + (unsigned)r * 128u;
+                    const unsigned line = smem_u32(sm_b + s * SH::B_STAGE) + (unsigned)r * 128u;
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        st_shared_v4(line + (unsigned)((k ^ (r & 7)) << 4), make_uint4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]));
+                    for (int k = 0; k < 4; ++k) {
+                        unsigned v[8];
+                        unpack32<XBITS>(w, k, v);
+                        st_shared_v4(line + (unsigned)(((2 * k) ^ (r & 7)) << 4), make_uint4(v[0], v[1], v[2], v[3]));
+                        st_shared_v4(line + (unsigned)(((2 * k + 1) ^ (r & 7)) << 4), make_uint4(v[4], v[5], v[6], v[7]));
+                    }
                 }
                 // make the generic-proxy writes visible to the tensor cores' (async proxy) reads, then signal
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             }
             __syncwarp();
-            if (lane == 0) arrive_leader<CG>(&S->ofull[s]);
+            if (lane == 0) mbar_arrive(&S->ofull[s]);
         }
     } else {
         // ------------------------------ epilogue: lane = output channel, column = token ------------------------------
         const int q = warp & 3;
         for (int i = 0; i < n_mine; ++i) {
             const int tile = first + i * step, mt = tile % P.m_tiles, nt = tile / P.m_tiles, a = i & 1;
-            const long long o = (long long)(mt * CG + rank) * ROWS + q * 32 + lane;
+            const long long o = (long long)mt * TM + q * 32 + lane;
             const long long t0 = (long long)nt * P.n;
             const float dw = o < P.n_out ? __ldg(P.sw + o) : 0.f;
             const bool ok = mbar_wait(&S->abort_flag, &S->tfull[a], (i >> 1) & 1, P.status, 6);
             if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after();
-            for (int c0 = 0; c0 < P.n; c0 += 32) {
-                unsigned v[32];
-                tmem_ld32_issue(tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(a * ACC_COLS + c0), v);
+            // TMEM columns [128, 256) belong to both accumulators of a wide tile: the upper half of the even ones, the lower
+            // half of the odd ones, drained first
+            const int shift = (TW == 8 && a == 0) ? 128 : 0;
+            for (int j = 0; j < SH::TN; j += 32) {
+                const int c0 = TW == 8 ? (j + shift) & 255 : j;
+                if (TW == 8 && j == 128) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&S->tshared);
+                }
+                if (c0 >= P.n) continue;
                 // the int8 operands were q * 2^(8 - bits): take the two powers of two out again (exact)
                 const float dx_l = t0 + c0 + lane < P.n_tok ? __ldg(P.sx + t0 + c0 + lane) * (1.f / (float)(1 << (16 - XBITS - WBITS))) : 0.f;
-                tmem_ld_wait(v);
-                const int cols = (int)((P.n_tok - t0 - c0) < 32 ? (P.n_tok - t0 - c0) : 32);
                 OutT* dst = reinterpret_cast<OutT*>(P.out) + (t0 + c0) * P.out_stride + o;
+                const int cols = (int)((P.n_tok - t0 - c0) < 32 ? (P.n_tok - t0 - c0) : 32);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const float dx = __shfl_sync(0xffffffffu, dx_l, e);
-                    const float f = (float)(int)v[e] * (dx * dw);
-                    if (e < cols && o < P.n_out) {
-                        if (sizeof(OutT) == 4) *reinterpret_cast<float*>(dst) = f;
-                        else *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(f);
+                for (int hf = 0; hf < 2; ++hf) {
+                    unsigned v[16];
+                    tmem_ld16(tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(a * SH::ACC_STEP + c0 + 16 * hf), v);
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const float dx = __shfl_sync(0xffffffffu, dx_l, 16 * hf + e);
+                        const float f = (float)(int)v[e] * (dx * dw);
+                        if (16 * hf + e < cols && o < P.n_out) {
+                            if (sizeof(OutT) == 4) *reinterpret_cast<float*>(dst) = f;
+                            else *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(f);
+                        }
+                        dst += P.out_stride;
                     }
-                    dst += P.out_stride;
                 }
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) arrive_leader<CG>(&S->tempty[a]);
+            if (lane == 0) mbar_arrive(&S->tempty[a]);
         }
     }
 
-    // ---- teardown: every role has left its loop (normally or after a wait expired); no SM of a pair leaves before the other
+    // ---- teardown: every role has left its loop (normally or after a wait expired); TMEM is freed
     tc_fence_before();
     __syncthreads();
-    __syncwarp();
-    pair_sync<CG>();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc_cg<CG>(tmem_base);
+        tmem_dealloc(tmem_base, TMEM_COLS);
     }
 }
 
 typedef void (*QgemmKernel)(const CUtensorMap, const CUtensorMap, const QgemmParams);
-template <int CG>
+template <int TW>
 QgemmKernel pick(int xbits, int wbits, int out_dtype)
 {
     static const QgemmKernel table[2][2][2] = {
-        {{k_tc_qgemm<3, 3, float, CG>, k_tc_qgemm<3, 3, __nv_bfloat16, CG>}, {k_tc_qgemm<3, 4, float, CG>, k_tc_qgemm<3, 4, __nv_bfloat16, CG>}},
-        {{k_tc_qgemm<4, 3, float, CG>, k_tc_qgemm<4, 3, __nv_bfloat16, CG>}, {k_tc_qgemm<4, 4, float, CG>, k_tc_qgemm<4, 4, __nv_bfloat16, CG>}}};
+        {{k_tc_qgemm<3, 3, float, TW>, k_tc_qgemm<3, 3, __nv_bfloat16, TW>}, {k_tc_qgemm<3, 4, float, TW>, k_tc_qgemm<3, 4, __nv_bfloat16, TW>}},
+        {{k_tc_qgemm<4, 3, float, TW>, k_tc_qgemm<4, 3, __nv_bfloat16, TW>}, {k_tc_qgemm<4, 4, float, TW>, k_tc_qgemm<4, 4, __nv_bfloat16, TW>}}};
     return table[xbits - 3][wbits - 3][out_dtype == GBS_DTYPE_F32 ? 0 : 1];
 }
 
-// Tile shape.  A step of 128 codes keeps the tensor pipe busy for 2 N cycles whatever the pairing, and the unpacking warps for
-// about 300 + N; tiles go in waves over the SMs (or pairs).  The shape with the least total is taken: pairs with N = 192
-// where the output fills the chip, single SMs with narrow tiles where it does not.
-void pick_tile(long long n_tok, long long n_out, int kblocks, int sm_count, int* cg_out, int* n_out_cols)
+// Tokens per tile.  A step of 128 codes was measured at 600 cycles up to 96 tokens and 2.6 more per token beyond (1016 at 256);
+// tiles go in waves over the SMs.  The width with the least total is taken: 256 where the output fills the chip, narrow tiles
+// on more SMs where it does not.
+int pick_tokens(long long n_tok, long long n_out, int kblocks, int sm_count)
 {
     double best = 0.0;
-    *cg_out = 0;
-    for (int cg = 1; cg <= 2; ++cg)
-        for (int n = 32; n <= (cg == 2 ? ACC_COLS : ROWS); n += 32) {
-            const long long tiles = ((n_out + ROWS * cg - 1) / (ROWS * cg)) * ((n_tok + n - 1) / n);
-            const long long waves = (tiles + sm_count / cg - 1) / (sm_count / cg);
-            const double unit = 2.0 * n > 300.0 + n ? 2.0 * n : 300.0 + n;
-            const double cost = (double)waves * kblocks * unit + 8.0 * n;
-            if (*cg_out == 0 || cost < best) { best = cost; *cg_out = cg; *n_out_cols = n; }
-        }
+    int n_best = 0;
+    for (int n = 32; n <= 256; n += 32) {
+        const long long tiles = ((n_out + TM - 1) / TM) * ((n_tok + n - 1) / n);
+        const long long waves = (tiles + sm_count - 1) / sm_count;
+        const double unit = n <= 96 ? 600.0 : 600.0 + 2.6 * (n - 96);
+        const double cost = (double)waves * kblocks * unit + 8.0 * n;
+        if (n_best == 0 || cost < best) { best = cost; n_best = n; }
+    }
+    return n_best;
 }
 
 bool encode_codes(EncodeTiledFn encode, CUtensorMap* map, const void* codes, int64_t rows, int row_bytes, int bits, int box_rows)
@@ -432,7 +391,7 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     // one symmetric scale per token and per output channel, so that the scales leave the contraction
     if (px->group != 0 || pw->group != 0 || px->asym || pw->asym) return GBS_ERR_UNSUPPORTED;
     if (px->d_pad % KB != 0) return GBS_ERR_UNSUPPORTED;
-    if (px->smem_optin < (int)(sizeof(Smem) + 1024)) return GBS_ERR_UNSUPPORTED;
+    if (px->smem_optin < (int)(Shape<8>::SMEM)) return GBS_ERR_UNSUPPORTED;
     if (n_tokens == 0 || n_out == 0) return GBS_OK;
     if (!codes_x || !scales_x || !codes_w || !scales_w || !out) return GBS_ERR_INVALID_ARG;
     const int esz = out_dtype == GBS_DTYPE_F32 ? 4 : 2;
@@ -464,23 +423,23 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     P.out = out;
     P.out_stride = out_row_stride;
     P.status = px->d_status;
-    int cg = 1;
-    pick_tile(n_tokens, n_out, P.kblocks, px->sm_count, &cg, &P.n);
-    P.m_tiles = (int)((n_out + ROWS * cg - 1) / (ROWS * cg));
+    P.n = pick_tokens(n_tokens, n_out, P.kblocks, px->sm_count);
+    P.m_tiles = (int)((n_out + TM - 1) / TM);
     const long long tiles = (long long)P.m_tiles * ((n_tokens + P.n - 1) / P.n);
     if (tiles > 0x7fffffff / 2) return GBS_ERR_INVALID_ARG;
     P.tiles = (int)tiles;
     CUtensorMap wmap, xmap;
-    if (!encode_codes(encode, &wmap, codes_w, n_out, pw->d_pad * pw->bits / 8, pw->bits, ROWS) ||
-        !encode_codes(encode, &xmap, codes_x, n_tokens, px->d_pad * px->bits / 8, px->bits, P.n / cg))
+    if (!encode_codes(encode, &wmap, codes_w, n_out, pw->d_pad * pw->bits / 8, pw->bits, TM) ||
+        !encode_codes(encode, &xmap, codes_x, n_tokens, px->d_pad * px->bits / 8, px->bits, P.n))
         return GBS_ERR_CUDA;
-    const int smem = (int)sizeof(Smem) + 1024;
-    QgemmKernel kernel = cg == 2 ? pick<2>(px->bits, pw->bits, out_dtype) : pick<1>(px->bits, pw->bits, out_dtype);
+    const bool wide = P.n > 128;
+    const int smem = wide ? Shape<8>::SMEM : Shape<4>::SMEM;
+    QgemmKernel kernel = wide ? pick<8>(px->bits, pw->bits, out_dtype) : pick<4>(px->bits, pw->bits, out_dtype);
     {
         // opt in to the large dynamic shared memory once per device and instantiation (not a stream operation)
         static std::mutex mu;
         static bool done[64][16] = {{false}};
-        const int ki = (cg - 1) * 8 + (px->bits - 3) * 4 + (pw->bits - 3) * 2 + (out_dtype == GBS_DTYPE_F32 ? 0 : 1);
+        const int ki = (wide ? 8 : 0) + (px->bits - 3) * 4 + (pw->bits - 3) * 2 + (out_dtype == GBS_DTYPE_F32 ? 0 : 1);
         std::lock_guard<std::mutex> lock(mu);
         if (!(px->device >= 0 && px->device < 64 && done[px->device][ki])) {
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
@@ -490,27 +449,16 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
             if (px->device >= 0 && px->device < 64) done[px->device][ki] = true;
         }
     }
-    const int slots = px->sm_count / cg;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(cg * (P.tiles < slots ? P.tiles : slots)));
+    cfg.gridDim = dim3((unsigned)(P.tiles < px->sm_count ? P.tiles : px->sm_count));
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = static_cast<cudaStream_t>(cuda_stream);
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    if (cg == 2) {
-        attr[na].id = cudaLaunchAttributeClusterDimension;
-        attr[na].val.clusterDim.x = 2;
-        attr[na].val.clusterDim.y = attr[na].val.clusterDim.z = 1;
-        ++na;
-    }
-    if (px->pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = (unsigned)na;
+    cfg.numAttrs = px->pdl ? 1 : 0;
     if (cudaLaunchKernelEx(&cfg, kernel, wmap, xmap, P) != cudaSuccess) { cudaGetLastError(); return GBS_ERR_CUDA; }
     return GBS_OK;
 }
