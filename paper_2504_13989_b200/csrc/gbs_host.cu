@@ -276,6 +276,8 @@ extern "C" int gbs_rotate_quantize(const gbs_plan_t* p, const void* x, int x_dty
         e = gbs_tc_uvm_rotate_quantize(p, x, n_rows, x_row_stride, codes, scales, y_opt, stream);
     else if (p->variant == GBS_VARIANT_TC_ROW && x_dtype == GBS_DTYPE_BF16)
         e = gbs_tc_row_rotate_quantize(p, x, n_rows, x_row_stride, codes, scales, y_opt, stream);
+    else if (x_dtype == GBS_DTYPE_F32 && gbs_tc_uvf_v(p) != 0)
+        e = gbs_tc_uvf_rotate_quantize(p, x, n_rows, x_row_stride, codes, scales, y_opt, stream);
     else
         e = gbs_generic_rotate_quantize(p, x, x_dtype, n_rows, x_row_stride, codes, scales, y_opt, stream);
     if (e != 0) cudaGetLastError();
