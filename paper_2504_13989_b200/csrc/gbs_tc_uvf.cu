@@ -12,8 +12,10 @@
 //   * Maxima: group = 32 2^g coordinates, or one scale per token.  Across the warps that share it through shared memory and a
 //     named barrier (token: 128 or 256 threads; group at V = 64: the pair of warps); then Delta, rounding, clipping, packing
 //     (Sections 2.1, 3.1) from registers.
-// What bounds it: about 500 issue slots per 32 values (220 of them the split) against 128 bytes of HBM read; the shared-memory
-// kernel that ran fp32 rows passes every value through shared memory five times.  3001 x 4096, 4 bits: 43.5 us before.
+// What bounds it: latency.  A warp issues about 700 instructions per 32 values of a lane (220 of them the split) at 8 cycles
+// each, sixteen warps cover half of that, and taking out any one part (two of three planes, the split, the epilogue) gains
+// less than a tenth.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 19.0 now; 7000 x 3584, groups of 128: 117.6 ->
+// 32.6.  Tried and slower: loads reissued piece by piece inside the split; tiles prefetched into L2 further ahead.
 // Every wait is bounded; an expired wait records a code in the plan's status word, and a warp whose wait ran out brings a
 // pattern no maximum can have to the barrier it shares, so that all who wait there leave with it.
 #include <string.h>
@@ -134,7 +136,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
     const unsigned tmem_base = S->tmem_base;
     const int n_mine = (P.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
 
-    if (warp == 1) {
+    if (warp == 0) {
+        // ------------------------------ L2 prefetch ------------------------------
+        // the registers hold one tile ahead, for part of a tile's time; DRAM wants more in flight.  Paced by the splits: one
+        // tile beyond the loads (82.8 -> 70.7 us for 7000 x 8192); further ahead queues in front of other blocks' loads.
+        if (lane < TOK) {
+            auto prefetch = [&](int n) {
+                const long long row = ((long long)blockIdx.x + (long long)n * gridDim.x) * TOK + lane;
+                if (n < n_mine && row < P.n_rows)
+                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.x + row * P.stride), "r"(P.d * 4) : "memory");
+            };
+            for (int n = 0; n + 2 < n_mine; ++n) {
+                if (!mbar_wait(&S->abort_flag, &S->full[n % STAGES], (unsigned)(n / STAGES) & 1u, P.status, 5)) break;
+                prefetch(n + 2);
+            }
+        }
+    } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0) {
             constexpr unsigned IDESC = instr_desc(UMAX, NCOLS);
@@ -185,14 +202,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
                                    ((((unsigned)b0 >> 4) ^ (V == 32 ? (unsigned)((u0 >> 1) & 3) : (unsigned)(u0 & 7))) << 4) + ((unsigned)b0 & 8u);
         // its rows are sixteen or twice sixteen, and so is Upad's granule
         const bool rows0 = wt * (1024 / V) < P.Upad, rows4 = wt * (1024 / V) + 512 / V < P.Upad;
+        const bool whole = wt * 1024 + 1024 <= P.d;
         uint4 x[8];
         auto fetch = [&](int n) {
             const long long row = row_first + (long long)n * row_step;
             const bool in = n < n_mine && row < P.n_rows;
             const float* src = P.x + row * P.stride + e0;
+            if (in && whole) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                x[j] = (in && e0 + 128 * j < P.d) ? __ldg(reinterpret_cast<const uint4*>(src + 128 * j)) : make_uint4(0u, 0u, 0u, 0u);
+                for (int j = 0; j < 8; ++j) x[j] = __ldg(reinterpret_cast<const uint4*>(src + 128 * j));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    x[j] = (in && e0 + 128 * j < P.d) ? __ldg(reinterpret_cast<const uint4*>(src + 128 * j)) : make_uint4(0u, 0u, 0u, 0u);
+            }
         };
         auto split_tile = [&](int n) -> bool {
             const int s = n % STAGES;
