@@ -334,7 +334,11 @@ extern "C" int gbs_clip_error(const gbs_plan_t* p, const void* x, int x_dtype, i
     DeviceGuard g;
     if (g.enter(p->device) != cudaSuccess) { cudaGetLastError(); return GBS_ERR_CUDA; }
     int e;
-    if (p->variant == GBS_VARIANT_TC_UV && x_dtype == GBS_DTYPE_BF16)
+    if (p->variant == GBS_VARIANT_TC_UV && x_dtype == GBS_DTYPE_BF16 && !err_rows_opt &&
+        (e = gbs_tc_uv_clip_histogram(p, x, n_rows, x_row_stride, alphas_host, K, err_sum, static_cast<cudaStream_t>(cuda_stream))) !=
+            GBS_UVCLIP_NOT_SERVED)
+        ;
+    else if (p->variant == GBS_VARIANT_TC_UV && x_dtype == GBS_DTYPE_BF16)
         e = gbs_tc_uv_clip_error(p, x, n_rows, x_row_stride, alphas_host, K, err_sum, err_rows_opt,
                                  static_cast<cudaStream_t>(cuda_stream));
     else if (p->variant == GBS_VARIANT_TC_ROW && x_dtype == GBS_DTYPE_BF16)

@@ -81,6 +81,11 @@ int gbs_generic_dequantize(const gbs_plan* p, const void* codes, const float* sc
                            void* out, int out_dtype, int inverse, cudaStream_t stream);
 size_t gbs_generic_smem_bytes(const gbs_plan* p, int* rows_per_cta);
 
+// gbs_tc_uvclip.cu : clip-ratio scoring of the UV family by histogram, where it applies
+#define GBS_UVCLIP_NOT_SERVED (-1)
+int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, const float* alphas, int K,
+                             double* err_sum, cudaStream_t stream);
+
 // gbs_tc_uvf.cu : rotate-quantize of fp32 rows on the tensor cores (three bf16 planes)
 int gbs_tc_uvf_v(const gbs_plan* p);            // the in-register factor of the path, 0 if it does not serve the plan
 int gbs_tc_uvf_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,

@@ -1,0 +1,396 @@
+// gbs_clip_error for bf16 rows of the UV family with one scale per token, by histogram instead of one pass per candidate.
+//
+// With t = |y| / M (M = the token's max|y|), candidate k quantizes |y| / M to the level l = number of its thresholds
+// (j + 1/2) alpha_k / D, j = 0 .. D-1, that t has reached (Sections 2.1, 3.1: rounding to the nearest level, clipping at D).
+// With D' = alpha_k / D the error is  M^2 (t - D' l)^2 = M^2 [t^2 - 2 D' t l + D'^2 l^2],  so all K candidates follow from how
+// many values (W0) and which sum of t (W1) lie beyond each of the K D thresholds:
+//        sum t l = sum_j W1(beyond threshold j),    sum l^2 = sum_j (2 j + 1) W0(beyond threshold j).
+// One histogram over the sorted thresholds replaces 5 K operations per value by about 15 whatever K is.
+//   * Front end as in gbs_tc_uv.cu: TMA, A X on tcgen05, H_32 in registers, the token's maximum over its four warps.
+//   * t becomes a 22-bit integer in the mantissa of one FMA.  Its high 12 bits index a table of cells; an entry holds the
+//     number of thresholds below the cell and the low 10 bits of the one threshold inside it, placed so that adding the
+//     value's low bits carries into the bin index when the threshold is reached.  (The host takes this path only where no two
+//     different thresholds share a cell.)
+//   * Two shared-memory atomics per value (count, and the FMA's bits themselves: the exponent pattern is removed with the count)
+//     into COPIES interleaved histograms per token, so that a warp's lanes rarely meet: measured 2 cycles per 32 values with 32
+//     copies and 6 with 8, against 3 - 4 for the table lookup.  Everything is an integer: exact in any order.  Values below
+//     every threshold need no bin.
+//   * After a token its 128 threads add the copies up, weigh them with M^2 in fp64 and clear them.  t's rounding (2^-23 M, without
+//     bias) is the only approximation.  The t^2 terms would cancel against the others; instead the error of candidate 0 is summed
+//     directly, as the per-candidate kernel does, and the histogram gives the differences from it.
+// What bounds it: the shared-memory port, about 1100 cycles per token (lookups, atomics, adding up) against 700 issue slots.
+// 32 768 x 4096, 3 bits, K = 32: 829 us with five fp32 operations per value and candidate.
+#include <math.h>
+#include <string.h>
+
+#include <mutex>
+
+#include "gbs_internal.h"
+#include "gbs_tc_common.cuh"
+
+namespace {
+
+constexpr int V = 32, TOK = 4, UMAX = 128;
+constexpr int STAGES = 2;                          // a tile takes far longer than its loads
+constexpr int STAGE_COLS = TOK * V;
+constexpr int STAGE_BYTES_MAX = TOK * UMAX * V * 2;
+constexpr int A_BYTES = UMAX * UMAX * 2;
+constexpr int EPI_WARPS = 4 * TOK;
+constexpr int THREADS = 32 * (2 + EPI_WARPS);
+constexpr int TMEM_COLS = 256;
+constexpr int CELL_BITS = 10, CELLS = 1 << 12;     // t is an integer of 22 bits
+constexpr int HIST_WORDS = TOK * 2 * 3584;         // [token][count, sum][bin][copy]
+constexpr int MAX_BINS = 448;                      // thresholds: K D at most
+constexpr unsigned POISON = 0xffffffffu;
+
+struct __align__(1024) Smem {
+    unsigned char a[A_BYTES];
+    unsigned char b[STAGES][STAGE_BYTES_MAX];
+    unsigned hist[HIST_WORDS];
+    unsigned lut[CELLS];
+    unsigned red[TOK][2][4];                       // maxima, by tile parity
+    double direct[EPI_WARPS];
+    unsigned long long full[STAGES], empty[STAGES], tfull[STAGES], tempty[STAGES];
+    unsigned long long abar;
+    unsigned tmem_base;
+    volatile int abort_flag;
+};
+
+struct ClipParams {
+    long long n_rows;
+    int n_groups;                 // ceil(n_rows / TOK)
+    int U, Upad, ksteps;
+    int K, levels, n_thr;
+    float scale;                  // of t as an integer
+    float norm2;                  // 1 / d'
+    float c_half0, c_delta0;      // candidate 0: 1 / (2 alpha), alpha / D
+    const unsigned char* a_img;
+    double* err_sum;
+    int* status;
+    float delta[GBS_MAX_CANDIDATES];              // alpha_k / D
+    unsigned thr[MAX_BINS];                       // sorted, different, one per cell at most
+    unsigned short idx[GBS_MAX_CANDIDATES][7];    // threshold j of candidate k
+};
+
+__device__ __forceinline__ unsigned ld_shared(unsigned a)
+{
+    unsigned v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+
+// COPIES x BINS is the same for every instantiation: as many copies as the thresholds leave room for
+template <int COPIES>
+__global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ ClipParams P)
+{
+    constexpr int BINS = HIST_WORDS / TOK / 2 / COPIES;
+    constexpr int PER = (BINS + 127) / 128;                       // bins a thread adds up
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    Smem* S = reinterpret_cast<Smem*>(smem_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned stage_bytes = (unsigned)(TOK * P.Upad * V * 2);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&S->full[s], 1);
+            mbar_init(&S->empty[s], 1);
+            mbar_init(&S->tfull[s], 1);
+            mbar_init(&S->tempty[s], EPI_WARPS);
+        }
+        mbar_init(&S->abar, 1);
+        S->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_arrive_expect_tx(&S->abar, A_BYTES);
+        bulk_load(S->a, P.a_img, A_BYTES, &S->abar);          // plan-owned, immutable: needs no ordering
+    }
+    if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
+    for (int i = threadIdx.x; i < HIST_WORDS / 4; i += THREADS) reinterpret_cast<uint4*>(S->hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (threadIdx.x < EPI_WARPS) S->direct[threadIdx.x] = 0.0;
+    // cell c: thresholds below it (binary search), and where the one inside it lies
+    for (int c = threadIdx.x; c < CELLS; c += THREADS) {
+        int lo = 0, hi = P.n_thr;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (P.thr[mid] < ((unsigned)c << CELL_BITS)) lo = mid + 1; else hi = mid;
+        }
+        const unsigned next = lo < P.n_thr ? P.thr[lo] : 0xffffffffu;
+        unsigned e = (unsigned)lo << CELL_BITS;
+        if ((next >> CELL_BITS) == (unsigned)c) e += (1u << CELL_BITS) - (next & ((1u << CELL_BITS) - 1u));
+        S->lut[c] = e;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned tmem_base = S->tmem_base;
+    const int n_mine = (P.n_groups - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+
+    double w0[PER], w1[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) w0[i] = w1[i] = 0.0;
+    if (warp == 0) {
+        // ------------------------------ TMA producer ------------------------------
+        if (lane == 0) {
+            int it = 0;
+            for (int g = blockIdx.x; g < P.n_groups; g += gridDim.x, ++it) {
+                const int s = it % STAGES;
+                if (!mbar_wait(&S->abort_flag, &S->empty[s], ((it / STAGES) & 1) ^ 1, P.status, 1)) break;
+                mbar_arrive_expect_tx(&S->full[s], stage_bytes);
+                tma_load_3d(S->b[s], &tmap, &S->full[s], 0, 0, g * TOK);
+            }
+            if (S->abort_flag) drain_copies(S->full, STAGES, it);
+        }
+    } else if (warp == 1) {
+        // ------------------------------ MMA issuer ------------------------------
+        if (lane == 0) {
+            constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS);
+            const unsigned long long ad0 = smem_desc(smem_u32(S->a), 16, 1024, 2);
+            const unsigned long long bd0 = smem_desc(smem_u32(S->b[0]), (unsigned)(P.Upad * V * 2), 512, 4);
+            const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
+            const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
+            bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
+            for (int it = 0; ok && it < n_mine; ++it) {
+                const int s = it % STAGES;
+                const unsigned ph = (it / STAGES) & 1;
+                if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
+                if (!mbar_wait(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
+                tc_fence_after();
+                unsigned a_lo = ad_lo0, b_lo = bd_lo0 + (unsigned)s * (STAGE_BYTES_MAX >> 4);
+                const unsigned d_tmem = tmem_base + s * STAGE_COLS;
+                umma_f16_words<false>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
+                for (int ks = 1; ks < P.ksteps; ++ks) {
+                    a_lo += (ks & 3) ? 2u : (unsigned)((UMAX * 128 - 96) >> 4);
+                    b_lo += 1024u >> 4;
+                    umma_f16_words<true>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
+                }
+                umma_commit(&S->empty[s]);
+                umma_commit(&S->tfull[s]);
+            }
+        }
+    } else {
+        // ------------------------------ histogram ------------------------------
+        const int t = (warp - 2) >> 2, q = warp & 3, ti = q * 32 + lane;
+        const unsigned taddr0 = tmem_base + ((unsigned)(q * 32) << 16) + t * V;
+        unsigned* hist = S->hist + t * 2 * BINS * COPIES;
+        constexpr unsigned BIN_STEP = COPIES * 4, SUM_OFF = BINS * COPIES * 4;
+        // value v in bin b > 0 (b thresholds reached) is recorded at row b - 1
+        const unsigned hb = smem_u32(hist) + (unsigned)(lane % COPIES) * 4u - BIN_STEP;
+        const unsigned lut = smem_u32(S->lut);
+        const float twoD = (float)(2 * P.levels), MAGIC = 8388608.f, mD = MAGIC + (float)P.levels;
+        double direct = 0.0;
+        for (int it = 0; it < n_mine; ++it) {
+            const int s = it % STAGES;
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull[s], (it / STAGES) & 1, P.status, 4, false));
+            unsigned r[32];
+            unsigned mb = POISON;
+            if (ok) {
+                tc_fence_after();
+                tmem_ld32_issue(taddr0 + s * STAGE_COLS, r);
+                tmem_ld_wait(r);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S->tempty[s]);
+                mb = __reduce_max_sync(0xffffffffu, __float_as_uint(fwht32_absmax(r)));
+            }
+            // the token's maximum; behind this barrier its histogram is clear as well.  A warp whose wait ran out comes too,
+            // with a pattern no maximum has, and all four leave.
+            unsigned* slot = S->red[t][it & 1];
+            if (lane == 0) slot[q] = mb;
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
+            mb = max(max(slot[0], slot[1]), max(slot[2], slot[3]));
+            if (mb == POISON) break;
+            const float M = __uint_as_float(mb);
+            const float rM = M > 0.f ? 1.f / M : 0.f;
+            const float sc = rM * P.scale, a1 = P.c_half0 * rM, dl = -P.c_delta0 * M;
+            float e0 = 0.f, e1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const float y = __uint_as_float(r[i]);
+                // candidate 0, directly
+                const float w = __saturatef(fmaf(y, a1, 0.5f));
+                const float err = fmaf(fmaf(w, twoD, MAGIC) - mD, dl, y);
+                if (i & 1) e1 = fmaf(err, err, e1); else e0 = fmaf(err, err, e0);
+                const unsigned b = __float_as_uint(fmaf(fabsf(y), sc, MAGIC));
+                const unsigned e = ld_shared(lut + ((b >> (CELL_BITS - 2)) & (unsigned)(4 * CELLS - 4)));
+                const unsigned bin = (e + (b & ((1u << CELL_BITS) - 1u))) >> CELL_BITS;
+                if (bin != 0u) {
+                    const unsigned at = hb + bin * BIN_STEP;
+                    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
+                    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at + SUM_OFF), "r"(b) : "memory");
+                }
+            }
+            direct += (double)(e0 + e1);
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
+            const double m2 = (double)M * (double)M;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const int bin = ti + 128 * i;
+                if (bin < P.n_thr) {
+                    uint4* row = reinterpret_cast<uint4*>(hist + bin * COPIES);
+                    uint4* row1 = reinterpret_cast<uint4*>(hist + (BINS + bin) * COPIES);
+                    uint4 c = make_uint4(0u, 0u, 0u, 0u), m = c;
+                    const uint4 zero = c;
+#pragma unroll
+                    for (int j = 0; j < COPIES / 4; ++j) {
+                        const int jj = (j + lane) % (COPIES / 4);          // eight lanes side by side: different banks
+                        const uint4 x = row[jj], z = row1[jj];
+                        row[jj] = zero;
+                        row1[jj] = zero;
+                        c.x += x.x; c.y += x.y; c.z += x.z; c.w += x.w;
+                        m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
+                    }
+                    // a component has at most 1024 values below 2^22: what is left without the exponent patterns fits 32 bits
+                    constexpr unsigned E = 0x4B000000u;
+                    const double sum = (double)(m.x - c.x * E) + (double)(m.y - c.y * E) + (double)(m.z - c.z * E) + (double)(m.w - c.w * E);
+                    w0[i] += m2 * (double)(c.x + c.y + c.z + c.w);
+                    w1[i] += m2 * sum;
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) direct += __shfl_xor_sync(0xffffffffu, direct, o);
+        if (lane == 0) S->direct[warp - 2] = direct;
+    }
+
+    // ---- the block's totals: [bin] over the four token slots, then from the last threshold down
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, TMEM_COLS);
+    }
+    double* tot = reinterpret_cast<double*>(S->hist);              // [slot][2][MAX_BINS]
+    if (warp >= 2) {
+        const int t = (warp - 2) >> 2, ti = (warp & 3) * 32 + lane;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (ti + 128 * i < P.n_thr) {
+                tot[(t * 2) * MAX_BINS + ti + 128 * i] = w0[i];
+                tot[(t * 2 + 1) * MAX_BINS + ti + 128 * i] = w1[i];
+            }
+    }
+    __syncthreads();
+    double* suf = tot + TOK * 2 * MAX_BINS;                        // [2][MAX_BINS]: sum over bins b, b + 1, ..
+    if (warp < 2) {
+        // warp 0 the counts, warp 1 the sums: a contiguous piece per lane, pieces joined from the right
+        const int per = (P.n_thr + 31) / 32, b0 = lane * per;
+        double s = 0.0;
+        for (int b = b0; b < b0 + per && b < P.n_thr; ++b)
+            for (int t = 0; t < TOK; ++t) s += tot[(t * 2 + warp) * MAX_BINS + b];
+        double after = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double v = __shfl_down_sync(0xffffffffu, after, o);
+            if (lane + o < 32) after += v;
+        }
+        after -= s;                                                // the pieces to the right of this one
+        for (int b = (b0 + per < P.n_thr ? b0 + per : P.n_thr) - 1; b >= b0; --b) {
+            for (int t = 0; t < TOK; ++t) after += tot[(t * 2 + warp) * MAX_BINS + b];
+            suf[warp * MAX_BINS + b] = after;
+        }
+    }
+    __syncthreads();
+    // error of candidate k without its t^2 part
+    auto part = [&](int k) -> double {
+        const double d = (double)P.delta[k];
+        double l1 = 0.0, l2 = 0.0;
+        for (int j = 0; j < P.levels; ++j) {
+            const int b = P.idx[k][j];
+            l2 += (double)(2 * j + 1) * suf[b];
+            l1 += suf[MAX_BINS + b];
+        }
+        return d * d * l2 - 2.0 * d * (l1 / (double)P.scale);
+    };
+    if (threadIdx.x < P.K) {
+        double direct = 0.0;
+        for (int i = 0; i < EPI_WARPS; ++i) direct += S->direct[i];
+        const int k = threadIdx.x;
+        atomicAdd(&P.err_sum[k], (direct + (k ? part(k) - part(0) : 0.0)) * (double)P.norm2);
+    }
+}
+
+typedef void (*ClipKernel)(const CUtensorMap, const ClipParams);
+
+}  // namespace
+
+// Scores K clip ratios, or returns GBS_UVCLIP_NOT_SERVED where this path does not apply (group scales, per-row sums, thresholds
+// too close to one another): the caller then takes the per-candidate kernel.
+int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, const float* alphas, int K,
+                             double* err_sum, cudaStream_t stream)
+{
+    EncodeTiledFn encode = get_encode();
+    if (p->group != 0 || !encode || p->smem_optin < (int)sizeof(Smem) || n_rows > (int64_t)0x7fffffff - TOK) return GBS_UVCLIP_NOT_SERVED;
+    ClipParams P;
+    memset(&P, 0, sizeof(P));
+    const int D = p->levels;
+    // t = 1 must stay below 2^22 after rounding
+    P.scale = 4194304.f - 8.f;
+    unsigned long long used[CELLS / 64] = {0};
+    unsigned at[CELLS];
+    unsigned short rank[CELLS];
+    for (int k = 0; k < K; ++k)
+        for (int j = 0; j < D; ++j) {
+            const unsigned T = (unsigned)ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale), c = T >> CELL_BITS;
+            if (c >= CELLS || ((used[c >> 6] >> (c & 63) & 1) && at[c] != T)) return GBS_UVCLIP_NOT_SERVED;
+            used[c >> 6] |= 1ull << (c & 63);
+            at[c] = T;
+        }
+    for (int w = 0; w < CELLS / 64; ++w)
+        for (unsigned long long m = used[w]; m; m &= m - 1) {
+            const int c = w * 64 + __builtin_ctzll(m);
+            rank[c] = (unsigned short)P.n_thr;
+            P.thr[P.n_thr++] = at[c];
+        }
+    for (int k = 0; k < K; ++k) {
+        P.delta[k] = (float)((double)alphas[k] / (double)D);
+        for (int j = 0; j < D; ++j)
+            P.idx[k][j] = rank[(unsigned)ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale) >> CELL_BITS];
+    }
+    CUtensorMap tmap;
+    const int U = p->d_pad / V;
+    P.Upad = (U + 15) & ~15;
+    const cuuint64_t gdim[3] = {(cuuint64_t)V, (cuuint64_t)(p->d / V), (cuuint64_t)n_rows};
+    const cuuint64_t gstr[2] = {(cuuint64_t)(V * 2), (cuuint64_t)(stride * 2)};
+    const cuuint32_t box[3] = {V, (cuuint32_t)P.Upad, TOK}, estr[3] = {1, 1, 1};
+    if (encode(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return (int)cudaErrorInvalidValue;
+    P.n_rows = n_rows;
+    P.n_groups = (int)((n_rows + TOK - 1) / TOK);
+    P.U = U;
+    P.ksteps = P.Upad / 16;
+    P.K = K;
+    P.levels = D;
+    P.norm2 = (float)(1.0 / (double)p->d_pad);
+    P.c_half0 = (float)(1.0 / (2.0 * (double)alphas[0]));
+    P.c_delta0 = P.delta[0];
+    P.a_img = p->d_aimg;
+    P.err_sum = err_sum;
+    P.status = p->d_status;
+    static const ClipKernel kernels[3] = {k_tc_uv_clip<32>, k_tc_uv_clip<16>, k_tc_uv_clip<8>};
+    {
+        // opt in to the large dynamic shared memory once per device (not a stream operation)
+        static std::mutex mu;
+        static bool done[64] = {false};
+        std::lock_guard<std::mutex> lock(mu);
+        if (!(p->device >= 0 && p->device < 64 && done[p->device])) {
+            for (ClipKernel k : kernels) {
+                const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+                if (e != cudaSuccess) return (int)e;
+            }
+            if (p->device >= 0 && p->device < 64) done[p->device] = true;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(P.n_groups < p->sm_count ? P.n_groups : p->sm_count));
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = sizeof(Smem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p->pdl ? 1 : 0;
+    return (int)cudaLaunchKernelEx(&cfg, kernels[P.n_thr <= 112 ? 0 : P.n_thr <= 224 ? 1 : 2], tmap, P);
+}
