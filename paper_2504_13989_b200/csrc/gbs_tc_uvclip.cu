@@ -13,13 +13,14 @@
 //     different thresholds share a cell.)
 //   * Two shared-memory atomics per value (count, and the FMA's bits themselves: the exponent pattern is removed with the count)
 //     into COPIES interleaved histograms per token, so that a warp's lanes rarely meet: measured 2 cycles per 32 values with 32
-//     copies and 6 with 8, against 3 - 4 for the table lookup.  Everything is an integer: exact in any order.  Values below
-//     every threshold need no bin.
+//     copies and 6 with 8, against 3 - 4 for the table lookup.  Everything is an integer: exact in any order.
 //   * After a token its 128 threads add the copies up, weigh them with M^2 in fp64 and clear them.  t's rounding (2^-23 M, without
 //     bias) is the only approximation.  The t^2 terms would cancel against the others; instead the error of candidate 0 is summed
 //     directly, as the per-candidate kernel does, and the histogram gives the differences from it.
-// What bounds it: the shared-memory port, about 1100 cycles per token (lookups, atomics, adding up) against 700 issue slots.
-// 32 768 x 4096, 3 bits, K = 32: 829 us with five fp32 operations per value and candidate.
+// What bounds it: the shared-memory port, 85 % busy: per token 1250 cycles (lookups 430, atomics 330, adding up and clearing
+// 390, the MMA's operands 130) against 820 issue slots per scheduler.
+// 32 768 x 4096, K = 32: 829 us with five fp32 operations per value and candidate; now 188 us at 3 bits (32 copies), 251 us at
+// 4 bits (16 copies); K = 8: 248 -> 165 us.  512 rows, K = 8: 19.2 -> 14.4 us.
 #include <math.h>
 #include <string.h>
 
@@ -39,7 +40,8 @@ constexpr int EPI_WARPS = 4 * TOK;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int TMEM_COLS = 256;
 constexpr int CELL_BITS = 10, CELLS = 1 << 12;     // t is an integer of 22 bits
-constexpr int HIST_WORDS = TOK * 2 * 3584;         // [token][count, sum][bin][copy]
+constexpr int HIST_ROWS = 3584;                    // words of a token's counts (and of its sums): bins x copies
+constexpr int HIST_WORDS = TOK * 2 * (HIST_ROWS + 32);   // [token][count, sum][one row nobody reads, bins][copy]
 constexpr int MAX_BINS = 448;                      // thresholds: K D at most
 constexpr unsigned POISON = 0xffffffffu;
 
@@ -75,7 +77,7 @@ struct ClipParams {
 __device__ __forceinline__ unsigned ld_shared(unsigned a)
 {
     unsigned v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));          // the table does not change once it is built
     return v;
 }
 
@@ -83,7 +85,7 @@ __device__ __forceinline__ unsigned ld_shared(unsigned a)
 template <int COPIES>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ ClipParams P)
 {
-    constexpr int BINS = HIST_WORDS / TOK / 2 / COPIES;
+    constexpr int BINS = HIST_ROWS / COPIES;
     constexpr int PER = (BINS + 127) / 128;                       // bins a thread adds up
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>(smem_raw);
@@ -106,17 +108,24 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     for (int i = threadIdx.x; i < HIST_WORDS / 4; i += THREADS) reinterpret_cast<uint4*>(S->hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x < EPI_WARPS) S->direct[threadIdx.x] = 0.0;
-    // cell c: thresholds below it (binary search), and where the one inside it lies
-    for (int c = threadIdx.x; c < CELLS; c += THREADS) {
+    unsigned* thr = reinterpret_cast<unsigned*>(S->b[0]);          // the first loads come later
+    for (int i = threadIdx.x; i < P.n_thr; i += THREADS) thr[i] = P.thr[i];
+    __syncthreads();
+    {
+        // cell c: thresholds below it, and where the one inside it lies; a run of cells per thread, found by one binary search
+        constexpr int RUN = (CELLS + THREADS - 1) / THREADS;
+        const int c0 = threadIdx.x * RUN;
         int lo = 0, hi = P.n_thr;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if (P.thr[mid] < ((unsigned)c << CELL_BITS)) lo = mid + 1; else hi = mid;
+            if (thr[mid] < ((unsigned)c0 << CELL_BITS)) lo = mid + 1; else hi = mid;
         }
-        const unsigned next = lo < P.n_thr ? P.thr[lo] : 0xffffffffu;
-        unsigned e = (unsigned)lo << CELL_BITS;
-        if ((next >> CELL_BITS) == (unsigned)c) e += (1u << CELL_BITS) - (next & ((1u << CELL_BITS) - 1u));
-        S->lut[c] = e;
+        for (int c = c0; c < c0 + RUN && c < CELLS; ++c) {
+            unsigned e = (unsigned)lo << CELL_BITS;
+            const unsigned next = lo < P.n_thr ? thr[lo] : 0xffffffffu;
+            if ((next >> CELL_BITS) == (unsigned)c) { e += (1u << CELL_BITS) - (next & ((1u << CELL_BITS) - 1u)); ++lo; }
+            S->lut[c] = e;
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -132,6 +141,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     if (warp == 0) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the thresholds read from the first stage
             int it = 0;
             for (int g = blockIdx.x; g < P.n_groups; g += gridDim.x, ++it) {
                 const int s = it % STAGES;
@@ -172,9 +182,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         // ------------------------------ histogram ------------------------------
         const int t = (warp - 2) >> 2, q = warp & 3, ti = q * 32 + lane;
         const unsigned taddr0 = tmem_base + ((unsigned)(q * 32) << 16) + t * V;
-        unsigned* hist = S->hist + t * 2 * BINS * COPIES;
-        constexpr unsigned BIN_STEP = COPIES * 4, SUM_OFF = BINS * COPIES * 4;
-        // value v in bin b > 0 (b thresholds reached) is recorded at row b - 1
+        unsigned* hist = S->hist + t * 2 * (HIST_ROWS + 32) + 32;            // behind a row for values below every threshold
+        constexpr unsigned BIN_STEP = COPIES * 4;
+        constexpr int SUM_OFF = (HIST_ROWS + 32) * 4;
+        // bin b (b thresholds reached) is row b - 1: bin 0 lands in the row before the first, which costs less than a predicate
+        // (a predicated reduction becomes a branch: 264 us instead of 250)
         const unsigned hb = smem_u32(hist) + (unsigned)(lane % COPIES) * 4u - BIN_STEP;
         const unsigned lut = smem_u32(S->lut);
         const float twoD = (float)(2 * P.levels), MAGIC = 8388608.f, mD = MAGIC + (float)P.levels;
@@ -204,20 +216,29 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
             const float rM = M > 0.f ? 1.f / M : 0.f;
             const float sc = rM * P.scale, a1 = P.c_half0 * rM, dl = -P.c_delta0 * M;
             float e0 = 0.f, e1 = 0.f;
+            // eight values at a time: their lookups are in flight together
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const float y = __uint_as_float(r[i]);
-                // candidate 0, directly
-                const float w = __saturatef(fmaf(y, a1, 0.5f));
-                const float err = fmaf(fmaf(w, twoD, MAGIC) - mD, dl, y);
-                if (i & 1) e1 = fmaf(err, err, e1); else e0 = fmaf(err, err, e0);
-                const unsigned b = __float_as_uint(fmaf(fabsf(y), sc, MAGIC));
-                const unsigned e = ld_shared(lut + ((b >> (CELL_BITS - 2)) & (unsigned)(4 * CELLS - 4)));
-                const unsigned bin = (e + (b & ((1u << CELL_BITS) - 1u))) >> CELL_BITS;
-                if (bin != 0u) {
+            for (int i0 = 0; i0 < 32; i0 += 8) {
+                unsigned b[8], e[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    b[i] = __float_as_uint(fmaf(fabsf(__uint_as_float(r[i0 + i])), sc, MAGIC));
+                    e[i] = ld_shared(lut + ((b[i] >> (CELL_BITS - 2)) & (unsigned)(4 * CELLS - 4)));
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    // candidate 0, directly
+                    const float y = __uint_as_float(r[i0 + i]);
+                    const float w = __saturatef(fmaf(y, a1, 0.5f));
+                    const float err = fmaf(fmaf(w, twoD, MAGIC) - mD, dl, y);
+                    if (i & 1) e1 = fmaf(err, err, e1); else e0 = fmaf(err, err, e0);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const unsigned bin = (e[i] + (b[i] & ((1u << CELL_BITS) - 1u))) >> CELL_BITS;
                     const unsigned at = hb + bin * BIN_STEP;
                     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
-                    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at + SUM_OFF), "r"(b) : "memory");
+                    asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(at), "r"(b[i]), "n"(SUM_OFF) : "memory");
                 }
             }
             direct += (double)(e0 + e1);
@@ -228,7 +249,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                 const int bin = ti + 128 * i;
                 if (bin < P.n_thr) {
                     uint4* row = reinterpret_cast<uint4*>(hist + bin * COPIES);
-                    uint4* row1 = reinterpret_cast<uint4*>(hist + (BINS + bin) * COPIES);
+                    uint4* row1 = reinterpret_cast<uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
                     uint4 c = make_uint4(0u, 0u, 0u, 0u), m = c;
                     const uint4 zero = c;
 #pragma unroll
@@ -271,13 +292,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
             }
     }
     __syncthreads();
+    for (int i = threadIdx.x; i < 2 * P.n_thr; i += THREADS) {
+        double* d = tot + (i < P.n_thr ? i : MAX_BINS + i - P.n_thr);
+        d[0] = (d[0] + d[2 * MAX_BINS]) + (d[4 * MAX_BINS] + d[6 * MAX_BINS]);
+    }
+    __syncthreads();
     double* suf = tot + TOK * 2 * MAX_BINS;                        // [2][MAX_BINS]: sum over bins b, b + 1, ..
     if (warp < 2) {
         // warp 0 the counts, warp 1 the sums: a contiguous piece per lane, pieces joined from the right
         const int per = (P.n_thr + 31) / 32, b0 = lane * per;
         double s = 0.0;
         for (int b = b0; b < b0 + per && b < P.n_thr; ++b)
-            for (int t = 0; t < TOK; ++t) s += tot[(t * 2 + warp) * MAX_BINS + b];
+            s += tot[warp * MAX_BINS + b];
         double after = s;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -286,7 +312,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         }
         after -= s;                                                // the pieces to the right of this one
         for (int b = (b0 + per < P.n_thr ? b0 + per : P.n_thr) - 1; b >= b0; --b) {
-            for (int t = 0; t < TOK; ++t) after += tot[(t * 2 + warp) * MAX_BINS + b];
+            after += tot[warp * MAX_BINS + b];
             suf[warp * MAX_BINS + b] = after;
         }
     }
