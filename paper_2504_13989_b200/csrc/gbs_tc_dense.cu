@@ -11,16 +11,18 @@
 //     m = 1544 instead of 4.8 MB), and with the output blocks taken in descending order the descriptor's two strides are
 //     both +128 bytes.  A CTA's share (31 KB) stays in shared memory; only the rows of X move.
 //   * Column 0 of H (constant -1) is repaired by one more MMA per tile with a 16-column operand whose column 0 holds
-//     H[n][0] - t(-n).  Row 0 (x_0 - sum of the others) is summed by the epilogue threads of the CTA that owns it, from the
-//     X stages as they pass.
+//     H[n][0] - t(-n).  Row 0 (x_0 - sum of the others) is an extra 16-row operand, the same for every k-step but the first,
+//     contracted by the last CTA of the cluster, which has the fewest coordinates; it sends the value to the first.
 //   * One sweep.  A token's m fp32 values do not fit one SM's TMEM, so a CLUSTER of CTAs takes 128 tokens and each CTA up to
 //     512 output coordinates: TMEM lane t holds the CTA's coordinates of token t, and the CTAs exchange their maxima of
 //     every token through distributed shared memory before quantizing (Sections 2.1, 3.1).
 //   * Packed rows are m b / 8 bytes (579 at m = 1544, b = 3: any alignment): a warp packs its 32 tokens' codes into shared
-//     memory and writes each row's piece as aligned words, lanes side by side.
-// What bounds it: the tensor pipe, 2 d m flops per token.  4096 x 1536, b = 4: 176 us with two sweeps over streamed chunks
-// of H on 32 SMs, 27.4 us now (0.44 of the measured bf16 rate); one row: 170 -> 19.5 us.  The number of CTAs per cluster is chosen by cost (pick_split): few wide shares when the batch fills the
-// chip, more and narrower ones when it does not.
+//     memory and writes the rows' pieces as words, sixteen lanes to a row, several rows in flight.
+// What bounds it: the tensor pipe, 2 d m flops per token, and what stands around it.  4096 x 1536, b = 4: 176 us with two sweeps
+// over streamed chunks of H on 32 SMs; 27.4 us with one sweep over the Toeplitz operand, of which 13.9 were the MMAs (a poll and
+// a commit per 64 columns cost 217 of 1050 cycles: hence 128 columns per stage), 1.6 the first CTA's waiting for its threads
+// to sum row 0 from the stages, 6.6 storing the codes row after row.  The number of CTAs per cluster is chosen by cost
+// (pick_split): few wide shares when the batch fills the chip, more and narrower ones when it does not.
 // Every wait is bounded; an expired wait records a code in the plan's status word.
 #include <math.h>
 #include <stdlib.h>
@@ -34,19 +36,22 @@
 namespace {
 
 constexpr int TM = 128;                 // tokens per tile (MMA M)
-constexpr int KC = 64;                  // input coordinates per stage (one 128-byte swizzled line of bf16)
-constexpr int STAGES = 6;
-constexpr int A_STAGE = TM * KC * 2;    // 16 KB
+constexpr int KC = 128;                 // input coordinates per stage: two boxes of one 128-byte swizzled line of bf16 per token
+constexpr int MAX_STAGES = 3;           // two where a large order's table leaves no room for three
+constexpr int A_BOX = TM * 64 * 2;      // 16 KB
+constexpr int A_STAGE = 2 * A_BOX;
 constexpr int EW = 4;                   // epilogue warps per TMEM lane quadrant: each takes a quarter of the coordinates
 constexpr int EPI_WARPS = 4 * EW;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int TMEM_COLS = 512;
 constexpr int MAX_CL = 8;               // CTAs per cluster
 constexpr int CORE = 128;               // bytes of a core matrix: 8 rows x 8 bf16
+constexpr int ROW0_BYTES = 2 * 4 * CORE;   // row 0 as a 16-row operand: the first k-step's, the others'
 
 struct Ctl {
     float tmax[2][MAX_CL * EW][TM];     // [tile parity][CTA and quarter][token]: maxima of every share of a token
-    unsigned long long full[STAGES], empty[STAGES], tfull, tempty, tbar, maxbar[2];
+    float y0[2][TM];                    // coordinate 0, from the cluster's last CTA
+    unsigned long long full[MAX_STAGES], empty[MAX_STAGES], tfull, tempty, tbar, maxbar[2];
     unsigned tmem_base;
     volatile int abort_flag;
 };
@@ -56,14 +61,16 @@ struct DenseParams {
     int n_tiles;
     int m;                        // d' = order of H_m
     int cl;                       // CTAs per cluster
-    int ncb;                      // 8-coordinate output blocks per CTA, a multiple of 4
-    int kchunks;                  // ceil(d / 64)
+    int ncb, ncb_last;            // 8-coordinate output blocks per CTA and of the last CTA, multiples of 4
+    int kchunks;                  // ceil(d / 128)
     int ksteps_last;              // MMAs (K = 16) of the last chunk
     int nbp;                      // output blocks the Toeplitz and column tables are laid out for
     int code_row_bytes;
+    int stages;
     int stage_words;              // words of a token's row in a warp's packing buffer (odd)
     float c_scale, c_half, norm;
     const unsigned char* toep;    // core matrices J = kb - nb + nbp - 1
+    const unsigned char* row0;    // ROW0_BYTES
     const unsigned char* col0;    // core matrix pairs (column repair, zeros) of block nbp - 1 - i at i
     unsigned char* codes;
     float* scales;
@@ -117,6 +124,13 @@ __device__ __forceinline__ bool cluster_wait(volatile int* abort_flag, void* bar
     return false;
 }
 
+// one column of this thread's TMEM lane
+__device__ __forceinline__ unsigned tmem_ld1(unsigned taddr)
+{
+    unsigned v;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;" : "=r"(v) : "r"(taddr) : "memory");
+    return v;
+}
 // 32 accumulator columns of four output blocks (descending) into coordinate order
 __device__ __forceinline__ void load_chunk(unsigned taddr, unsigned y[32])
 {
@@ -135,21 +149,28 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int toep_n = P.kchunks * (KC / 8) + P.ncb;               // core matrices of this CTA's share
     unsigned char* sm_x = base;
-    unsigned char* sm_t = sm_x + STAGES * A_STAGE;
-    unsigned char* sm_e = sm_t + toep_n * CORE;
-    unsigned* sm_pack = reinterpret_cast<unsigned*>(sm_e + P.ncb * 2 * CORE);
+    unsigned char* sm_t = sm_x + P.stages * A_STAGE;
+    unsigned char* sm_e = sm_t + (P.kchunks * (KC / 8) + P.ncb) * CORE;
+    unsigned char* sm_r = sm_e + P.ncb * 2 * CORE;
+    unsigned* sm_pack = reinterpret_cast<unsigned*>(sm_r + ROW0_BYTES);
     Ctl* S = reinterpret_cast<Ctl*>(sm_pack + (EPI_WARPS * 32 * P.stage_words + 3) / 4 * 4);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank();
     const int cluster = (int)blockIdx.x / P.cl, n_clusters = (int)gridDim.x / P.cl;
     const int nb0 = rank * P.ncb;                                  // first output block of this CTA
+    const bool last = rank == P.cl - 1;
+    const int ncb = last ? P.ncb_last : P.ncb;                     // its blocks, a multiple of 4
+    const int toep_n = P.kchunks * (KC / 8) + ncb;                 // core matrices of its share
+    // coordinate 0's sixteen columns: behind the last CTA's blocks, or where two blocks of padding would be (blocks descend, so
+    // padding comes first)
+    const int skip = last && nb0 + ncb - P.m / 8 >= 2 ? 2 : 0;
+    const int col_r = skip ? 0 : 8 * ncb;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < P.stages; ++s) {
             mbar_init(&S->full[s], 1);
-            mbar_init(&S->empty[s], rank == 0 ? 1 + 4 : 1);        // the MMAs, and in CTA 0 the warps that sum row 0
+            mbar_init(&S->empty[s], 1);
         }
         mbar_init(&S->tfull, 1);
         mbar_init(&S->tempty, EPI_WARPS);
@@ -159,10 +180,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // plan-owned, immutable tables: need no ordering
-        mbar_arrive_expect_tx(&S->tbar, (unsigned)(toep_n * CORE + P.ncb * 2 * CORE));
-        const int first = P.nbp - nb0 - P.ncb;
+        mbar_arrive_expect_tx(&S->tbar, (unsigned)(toep_n * CORE + ncb * 2 * CORE + ROW0_BYTES));
+        const int first = P.nbp - nb0 - ncb;
         bulk_load(sm_t, P.toep + (size_t)first * CORE, (unsigned)(toep_n * CORE), &S->tbar);
-        bulk_load(sm_e, P.col0 + (size_t)first * 2 * CORE, (unsigned)(P.ncb * 2 * CORE), &S->tbar);
+        bulk_load(sm_e, P.col0 + (size_t)first * 2 * CORE, (unsigned)(ncb * 2 * CORE), &S->tbar);
+        bulk_load(sm_r, P.row0, ROW0_BYTES, &S->tbar);
     }
     if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     tc_fence_before();
@@ -179,55 +201,61 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
     if (warp == 0) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
-            int c = 0;                                             // stage uses so far
+            int c = 0, s = 0;                                      // stage uses so far, the stage of the next
+            unsigned ph = 0;
             bool ok = true;
             for (int i = 0; ok && i < n_mine; ++i) {
                 const int row0 = (cluster + i * n_clusters) * TM;
                 for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
-                    const int s = c % STAGES;
-                    if (!mbar_wait(&S->abort_flag, &S->empty[s], ((c / STAGES) & 1) ^ 1, P.status, 1)) { ok = false; break; }
+                    if (!mbar_wait(&S->abort_flag, &S->empty[s], ph ^ 1, P.status, 1)) { ok = false; break; }
                     mbar_arrive_expect_tx(&S->full[s], A_STAGE);
                     tma_load_2d(sm_x + s * A_STAGE, &xmap, &S->full[s], kc * KC, row0);
+                    tma_load_2d(sm_x + s * A_STAGE + A_BOX, &xmap, &S->full[s], kc * KC + 64, row0);
+                    if (++s == P.stages) { s = 0; ph ^= 1; }
                 }
             }
-            if (!ok) drain_copies(S->full, STAGES, c);
+            if (!ok) drain_copies(S->full, P.stages, c);
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         if (lane == 0) {
             // the CTA's columns as one or two MMAs of at most 256, each a multiple of 32
-            const int n1 = P.ncb <= 32 ? P.ncb : (P.ncb / 2 + 3) / 4 * 4, n2 = P.ncb - n1;
+            const int n = ncb - skip, n1 = n <= 32 ? n : (n / 2 + 3) / 4 * 4, n2 = n - n1;
             const unsigned idesc1 = instr_desc(TM, 8 * n1, false), idesc2 = instr_desc(TM, 8 * n2, false);
+            constexpr unsigned IDESC_R = instr_desc(TM, 16, false);
             // unswizzled core matrices: leading offset = next 8 columns, stride offset = next 8 rows of the operand
-            const unsigned long long td0 = smem_desc(smem_u32(sm_t), CORE, CORE, 0);
-            const unsigned long long ed0 = smem_desc(smem_u32(sm_e), CORE, 2 * CORE, 0);
-            const unsigned tmem2 = tmem_base + 8 * n1;
+            const unsigned long long td0 = smem_desc(smem_u32(sm_t) + skip * CORE, CORE, CORE, 0);
+            const unsigned long long ed0 = smem_desc(smem_u32(sm_e) + skip * 2 * CORE, CORE, 2 * CORE, 0);
+            const unsigned long long rd0 = smem_desc(smem_u32(sm_r), CORE, 2 * CORE, 0);
+            const unsigned tmem1 = tmem_base + 8 * skip, tmem2 = tmem1 + 8 * n1, tmem_r = tmem_base + col_r;
             const unsigned long long step2 = (unsigned long long)(n1 * CORE / 16), estep2 = (unsigned long long)(n1 * 2 * CORE / 16);
             bool ok = mbar_wait(&S->abort_flag, &S->tbar, 0, P.status, 6);
-            int c = 0;
+            int s = 0;
+            unsigned ph = 0;
             for (int i = 0; ok && i < n_mine; ++i) {
                 // the accumulators fill the CTA's share of TMEM: the next tile waits for the epilogue
                 if (!mbar_wait(&S->abort_flag, &S->tempty, (i & 1) ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 unsigned long long td = td0;
-                for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
-                    const int s = c % STAGES;
-                    if (!mbar_wait(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
+                for (int kc = 0; kc < P.kchunks; ++kc) {
+                    if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
                     unsigned long long ad = smem_desc(smem_u32(sm_x + s * A_STAGE), 16, 1024, 2);
                     const int ks_n = (kc == P.kchunks - 1) ? P.ksteps_last : KC / 16;
                     if (kc == 0) {
                         // column 0: H[n][0] - t(-n) against x_0 (the other fifteen columns of the operand are zero)
-                        umma_f16(tmem_base, ad, ed0, idesc1, 0u);
+                        umma_f16(tmem1, ad, ed0, idesc1, 0u);
                         if (n2) umma_f16(tmem2, ad, ed0 + estep2, idesc2, 0u);
                     }
                     for (int ks = 0; ks < ks_n; ++ks) {
-                        umma_f16(tmem_base, ad, td, idesc1, 1u);
+                        umma_f16(tmem1, ad, td, idesc1, 1u);
                         if (n2) umma_f16(tmem2, ad, td + step2, idesc2, 1u);
-                        ad += 2;                                   // 32 bytes of the 128-byte line
+                        if (last) umma_f16(tmem_r, ad, (kc | ks) != 0 ? rd0 + 4 * CORE / 16 : rd0, IDESC_R, (kc | ks) != 0 ? 1u : 0u);
+                        ad += ks == 3 ? (A_BOX - 96) / 16 : 2;     // 32 bytes of the 128-byte line, then the second box
                         td += 2 * CORE / 16;                       // two core matrices on
                     }
                     umma_commit(&S->empty[s]);
+                    if (++s == P.stages) { s = 0; ph ^= 1; }
                 }
                 if (ok) umma_commit(&S->tfull);
             }
@@ -237,42 +265,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
         const int q = warp & 3;                            // TMEM lane quadrant this warp may access
         const int h = (warp - 2) >> 2;                     // which quarter of the CTA's coordinates
         const int tok = q * 32 + lane;
-        const int chunks = P.ncb / 4;                      // of 32 coordinates
+        const int chunks = ncb / 4;                        // of 32 coordinates
         const int ch0 = h * chunks / EW, ch1 = (h + 1) * chunks / EW;
         const unsigned lane_base = tmem_base + ((unsigned)(q * 32) << 16);
         const int nfirst = (nb0 + 4 * ch0) * 8;            // first coordinate of this warp
-        const bool sums_row0 = rank == 0 && ch0 == 0 && ch1 > 0;   // one warp per quadrant (a small share leaves some without)
+        const bool has0 = rank == 0 && ch0 == 0 && ch1 > 0;        // coordinate 0 is among this warp's
+        const bool sends0 = last && h == 0;
         unsigned* pack = sm_pack + (warp - 2) * 32 * P.stage_words;
-        int c = 0;
         bool ok = true;
         for (int i = 0; ok && i < n_mine; ++i) {
             const long long row0 = ((long long)cluster + (long long)i * n_clusters) * TM;
             const long long row = row0 + tok;
             const bool live = row < P.n_rows;
-            float y0 = 0.f;
-            if (sums_row0) {
-                // coordinate 0: x_0 - (x_1 + x_2 + ..), from the stages as they pass (columns beyond d are zero)
-                float s4[4] = {0.f, 0.f, 0.f, 0.f}, x0 = 0.f;
-                for (int kc = 0; ok && kc < P.kchunks; ++kc, ++c) {
-                    const int s = c % STAGES;
-                    ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 5));
-                    if (!ok) break;
-                    const uint4* line = reinterpret_cast<const uint4*>(sm_x + s * A_STAGE + tok * 128);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint4 v = line[j ^ (tok & 7)];
-                        if (kc == 0 && j == 0) x0 = __uint_as_float(v.x << 16);
-                        s4[0] += __uint_as_float(v.x << 16); s4[1] += __uint_as_float(v.x & 0xffff0000u);
-                        s4[2] += __uint_as_float(v.y << 16); s4[3] += __uint_as_float(v.y & 0xffff0000u);
-                        s4[0] += __uint_as_float(v.z << 16); s4[1] += __uint_as_float(v.z & 0xffff0000u);
-                        s4[2] += __uint_as_float(v.w << 16); s4[3] += __uint_as_float(v.w & 0xffff0000u);
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&S->empty[s]);
-                }
-                y0 = 2.f * x0 - ((s4[0] + s4[1]) + (s4[2] + s4[3]));
-            }
-            if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull, i & 1, P.status, 4));
+            ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull, i & 1, P.status, 4));
             if (!ok) break;
             tc_fence_after();
             float M = 0.f;
@@ -280,14 +285,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
                 const int n_here = P.m - (nb0 + 4 * ch) * 8;               // live coordinates from here on
                 if (n_here <= 0) break;
                 unsigned y[32];
-                load_chunk(lane_base + (unsigned)(8 * (P.ncb - 4 - 4 * ch)), y);
-                if (sums_row0 && ch == 0) y[0] = __float_as_uint(y0);
+                load_chunk(lane_base + (unsigned)(8 * (ncb - 4 - 4 * ch)), y);
+                if (has0 && ch == 0) y[0] = 0u;                            // in the maximum of the CTA that has it
                 if (n_here < 32) {
 #pragma unroll
                     for (int e = 0; e < 32; ++e)
                         if (e >= n_here) y[e] = 0u;                        // coordinates beyond m
                 }
                 M = fmaxf(M, absmax32(y));
+            }
+            if (sends0) {
+                const float y0 = __uint_as_float(tmem_ld1(lane_base + col_r));
+                M = fmaxf(M, fabsf(y0));
+                peer_store(peer_addr(smem_u32(&S->y0[i & 1][tok]), 0u), y0);
             }
             // the token's maximum over all shares of all CTAs
             const unsigned mine = smem_u32(&S->tmax[i & 1][rank * EW + h][tok]), bar = smem_u32(&S->maxbar[i & 1]);
@@ -303,8 +313,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
                 const int n0 = (nb0 + 4 * ch) * 8, n_here = P.m - n0;
                 if (n_here <= 0) break;
                 unsigned y[32];
-                load_chunk(lane_base + (unsigned)(8 * (P.ncb - 4 - 4 * ch)), y);
-                if (sums_row0 && ch == 0) y[0] = __float_as_uint(y0);
+                load_chunk(lane_base + (unsigned)(8 * (ncb - 4 - 4 * ch)), y);
+                if (has0 && ch == 0) y[0] = __float_as_uint(S->y0[i & 1][tok]);
                 unsigned out[BITS];
                 quantize_pack32<BITS>(y, a1, out);
 #pragma unroll
@@ -321,27 +331,26 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
             __syncwarp();
             if (lane == 0) mbar_arrive(&S->tempty);
             if (rank == 0 && h == 0 && live) P.scales[row] = P.c_scale * M;
-            // this warp's 32 rows, one after the other: aligned words, lanes side by side
+            // this warp's 32 rows as words, sixteen lanes to a row (a piece is at most 64 bytes; 48 where rows are unaligned)
             const int n_codes = (P.m - nfirst) < (ch1 - ch0) * 32 ? (P.m - nfirst) : (ch1 - ch0) * 32;
-            if (n_codes > 0) {
-                const int nbytes = n_codes * BITS / 8;
-                for (int r = 0; r < 32; ++r) {
-                    if (row0 + q * 32 + r >= P.n_rows) break;
-                    unsigned char* dst = P.codes + (row0 + q * 32 + r) * P.code_row_bytes + nfirst / 8 * BITS;
-                    const int off = (int)(reinterpret_cast<uintptr_t>(dst) & 3u);
-                    const unsigned* src = pack + r * P.stage_words;
-                    unsigned* words = reinterpret_cast<unsigned*>(dst - off);
-                    for (int j = lane; 4 * j < off + nbytes; j += 32) {
-                        const unsigned lo = j > 0 ? src[j - 1] : 0u, hi = src[j];
-                        const unsigned v = off ? __funnelshift_l(lo, hi, 8 * off) : hi;
-                        const int b0 = 4 * j - off;                            // first byte of the piece this word covers
-                        if (b0 >= 0 && b0 + 4 <= nbytes) {
-                            words[j] = v;
-                        } else {
+            const int nbytes = n_codes > 0 ? n_codes * BITS / 8 : 0;
+            const int j = lane & 15;
+            unsigned char* piece = P.codes + (row0 + q * 32 + (lane >> 4)) * P.code_row_bytes + nfirst / 8 * BITS;
+#pragma unroll 4
+            for (int r = lane >> 4; r < 32; r += 2, piece += 2 * P.code_row_bytes) {
+                const int off = (int)(reinterpret_cast<uintptr_t>(piece) & 3u);
+                const unsigned* src = pack + r * P.stage_words;
+                const unsigned lo = j > 0 ? src[j - 1] : 0u, hi = src[j];
+                const unsigned v = off ? __funnelshift_l(lo, hi, 8 * off) : hi;
+                const int b0 = 4 * j - off;                                    // first byte of the piece this word covers
+                unsigned char* dst = piece + b0;
+                if (row0 + q * 32 + r < P.n_rows) {
+                    if (b0 >= 0 && b0 + 4 <= nbytes) {
+                        *reinterpret_cast<unsigned*>(dst) = v;
+                    } else {
 #pragma unroll
-                            for (int b = 0; b < 4; ++b)
-                                if (b0 + b >= 0 && b0 + b < nbytes) reinterpret_cast<unsigned char*>(words + j)[b] = (unsigned char)(v >> (8 * b));
-                        }
+                        for (int b = 0; b < 4; ++b)
+                            if (b0 + b >= 0 && b0 + b < nbytes) dst[b] = (unsigned char)(v >> (8 * b));
                     }
                 }
             }
@@ -361,11 +370,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
 }
 
 // shared memory of a CTA that takes `ncb` output blocks of a contraction over `kchunks` chunks
-int smem_bytes(int ncb, int kchunks, int bits, int* stage_words)
+int smem_bytes(int ncb, int kchunks, int stages, int* stage_words)
 {
-    const int w = (((ncb / 4 + EW - 1) / EW) * bits + 1) | 1;      // one word beyond the last is read when rows are unaligned
+    const int w = 17;                                              // sixteen words are read whatever the share; odd: different banks
     if (stage_words) *stage_words = w;
-    return 1024 + STAGES * A_STAGE + (kchunks * (KC / 8) + ncb) * CORE + ncb * 2 * CORE + (EPI_WARPS * 32 * w + 3) / 4 * 16 + (int)sizeof(Ctl);
+    return 1024 + stages * A_STAGE + (kchunks * (KC / 8) + ncb) * CORE + ncb * 2 * CORE + ROW0_BYTES + (EPI_WARPS * 32 * w + 3) / 4 * 16 + (int)sizeof(Ctl);
 }
 
 typedef void (*DenseKernel)(const CUtensorMap, const DenseParams);
@@ -398,8 +407,8 @@ int clusters_at_once(const gbs_plan* p, int cl)
     return n;
 }
 
-// How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 64), a tile's
-// epilogue and exchange a few thousand, and the clusters that fit at once take the tiles in waves: the split with the
+// How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 64), a stage's poll and
+// commit 220, a tile's epilogue and exchange a few thousand, and the clusters that fit at once take the tiles in waves: the split with the
 // least total is taken.  n_tiles = 0 only asks whether a split exists.
 int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* ncb_out, int* fit_out)
 {
@@ -408,12 +417,13 @@ int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* nc
     *cl_out = 0;
     for (int want = 1; want <= MAX_CL; ++want) {
         const int ncb = ((nb + want - 1) / want + 3) / 4 * 4, cl = (nb + ncb - 1) / ncb;
-        if (ncb > 64 || smem_bytes(ncb, kchunks, p->bits, nullptr) > p->smem_optin) continue;
+        const int real = nb - (cl - 1) * ncb, last = (real + 3) / 4 * 4;      // sixteen columns for coordinate 0 must fit
+        if (ncb > 64 || (last - real < 2 && 8 * last + 16 > TMEM_COLS) || smem_bytes(ncb, kchunks, 2, nullptr) > p->smem_optin) continue;
         const int fit = n_tiles ? clusters_at_once(p, cl) : 1;
         if (fit < 1) return (int)cudaErrorInvalidConfiguration;
         const int waves = (n_tiles + fit - 1) / fit;
         const double mma = ncb <= 32 ? (ncb * 4 < 64 ? 64.0 : ncb * 4.0) : (ncb * 4 < 128 ? 128.0 : ncb * 4.0);
-        const double cost = waves * (4.0 * kchunks * mma + 2500.0 + 20.0 * ncb);
+        const double cost = waves * (kchunks * (8.0 * mma + 220.0) + 4500.0 + 20.0 * ncb);
         if (*cl_out == 0 || cost < best) { best = cost; *cl_out = cl; *ncb_out = ncb; *fit_out = fit; }
     }
     return 0;
@@ -440,10 +450,11 @@ void gbs_tc_dense_image(const int8_t* hm, int m, unsigned short* img)
 }
 
 size_t gbs_tc_dense_toeplitz_bytes(int m) { return (size_t)((m + KC - 1) / KC * (KC / 8) + padded_blocks(m)) * CORE; }
-size_t gbs_tc_dense_col0_bytes(int m) { return (size_t)padded_blocks(m) * 2 * CORE; }
+size_t gbs_tc_dense_col0_bytes(int m) { return (size_t)padded_blocks(m) * 2 * CORE + ROW0_BYTES; }
 
 // The forward path's tables: the Toeplitz core matrices (J = kb - nb + nbp - 1; row r, column c: t(8 (kb - nb) + c - r)) and
-// the repair of column 0 (block nbp - 1 - i at i).  t(k - n) = H[n][k] for n, k >= 1; zero where no such pair exists.
+// the repair of column 0 (block nbp - 1 - i at i), with row 0 behind it (core matrices: rows 0 .. 7 of columns 0 .. 7 and 8 .. 15,
+// then rows 8 .. 15, zero).  t(k - n) = H[n][k] for n, k >= 1; zero where no such pair exists.
 void gbs_tc_dense_tables(const int8_t* hm, int m, unsigned short* toep, unsigned short* col0)
 {
     const int nbp = padded_blocks(m);
@@ -462,6 +473,9 @@ void gbs_tc_dense_tables(const int8_t* hm, int m, unsigned short* toep, unsigned
             const int n = 8 * (nbp - 1 - i) + r;
             if (n >= 1 && n < m) col0[i * 128 + r * 8] = bf((int)hm[(size_t)n * m] - t(-n));
         }
+    unsigned short* row0 = col0 + (size_t)nbp * 128;
+    for (int v = 0; v < 2; ++v)
+        for (int k = 0; k < 16; ++k) row0[v * 256 + (k >> 3) * 64 + (k & 7)] = bf(v == 0 && k == 0 ? 1 : -1);
 }
 
 int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
@@ -474,7 +488,7 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
     const cuuint32_t estr[2] = {1, 1};
     const cuuint64_t gdim[2] = {(cuuint64_t)p->d, (cuuint64_t)n_rows};
     const cuuint64_t gstr[1] = {(cuuint64_t)(stride * 2)};
-    const cuuint32_t box[2] = {KC, TM};
+    const cuuint32_t box[2] = {64, TM};
     if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(x), gdim, gstr, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -489,6 +503,7 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
     int fit = 0;
     const int rc = pick_split(p, P.n_tiles, P.kchunks, &P.cl, &P.ncb, &fit);
     if (rc != 0) return rc;
+    P.ncb_last = ((p->m / 8 - (P.cl - 1) * P.ncb) + 3) / 4 * 4;
     P.nbp = padded_blocks(p->m);
     P.code_row_bytes = p->m * p->bits / 8;
     P.c_scale = p->c_scale;
@@ -496,11 +511,13 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
     P.norm = p->norm;
     P.toep = p->d_dense;
     P.col0 = p->d_dense + gbs_tc_dense_toeplitz_bytes(p->m);
+    P.row0 = P.col0 + (size_t)padded_blocks(p->m) * 2 * CORE;
     P.codes = (unsigned char*)codes;
     P.scales = scales;
     P.y_opt = y_opt;
     P.status = p->d_status;
-    const int smem = smem_bytes(P.ncb, P.kchunks, p->bits, &P.stage_words);
+    P.stages = smem_bytes(P.ncb, P.kchunks, MAX_STAGES, nullptr) <= p->smem_optin ? MAX_STAGES : 2;
+    const int smem = smem_bytes(P.ncb, P.kchunks, P.stages, &P.stage_words);
     const int clusters = P.n_tiles < fit ? P.n_tiles : fit;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * P.cl));
