@@ -72,6 +72,14 @@ __device__ __forceinline__ bool mbar_wait(volatile int* abort_flag, void* bar, u
     return mbar_wait_slow(abort_flag, bar, parity, status, code, watch_abort);
 }
 
+// The same for a whole warp: every lane waits, and the answer is one the compiler knows to be warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
+{
+    return __all_sync(0xffffffffu, mbar_wait(abort_flag, bar, parity, status, code));
+}
+// The warp's index, likewise.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // A producer that leaves its loop through the abort flag has copies on their way into the block's shared memory.  It
 // gives the stages it armed (uses it_next - 1, it_next - 2, .. of a ring of n_stages `full` barriers; use i fills stage
 // i % n_stages in phase (i / n_stages) & 1) a bounded time, two milliseconds in all, to complete before the block ends.
@@ -117,43 +125,35 @@ __device__ __forceinline__ void tmem_dealloc(unsigned addr, unsigned cols)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// MMAs and commits are issued by a whole warp that has not diverged, the one lane that executes them elected inside the asm
+// (the same lane every time, as commits need).  The operands then live in uniform registers and the loop around them is uniform
+// code: an MMA takes its nominal time (52 cycles at N = 64, 64 at 128, 104 at 208, 128 at 256).  Inside `if (lane == 0)` the
+// compiler moves every operand per MMA, which cost 68 cycles in the simplest loop, 120 - 170 with two accumulators or a
+// conditional MMA in it, and 295 with descriptors chosen at run time, whatever N.
 __device__ __forceinline__ void umma_f16(unsigned d_tmem, unsigned long long a_desc, unsigned long long b_desc,
                                          unsigned idesc, unsigned accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// The same with the descriptors as (low, high) words and the accumulate flag fixed at compile time: the
-// issuing thread shares its scheduler with busy epilogue warps, so every instruction it spends between two
-// MMAs delays the tensor cores; a k-step then costs one add on each low word and the MMA itself.
+// The same with the descriptors as (low, high) words and the accumulate flag fixed at compile time: a k-step then costs one
+// add on each low word and the MMA itself.
 template <bool ACCUMULATE>
 __device__ __forceinline__ void umma_f16_words(unsigned d_tmem, unsigned a_lo, unsigned a_hi, unsigned b_lo, unsigned b_hi,
                                                unsigned idesc)
 {
-    if (ACCUMULATE) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-            "setp.eq.b32 p, 0, 0;\n\t"
-            "mov.b64 da, {%1, %2};\n\t"
-            "mov.b64 db, {%3, %4};\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 p, 0, 0;\n\t"
-            "mov.b64 da, {%1, %2};\n\t"
-            "mov.b64 db, {%3, %4};\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
-    }
+    umma_f16(d_tmem, (unsigned long long)a_hi << 32 | a_lo, (unsigned long long)b_hi << 32 | b_lo, idesc, ACCUMULATE ? 1u : 0u);
 }
 __device__ __forceinline__ void umma_commit(void* bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane -> 32 registers.  The load is asynchronous:

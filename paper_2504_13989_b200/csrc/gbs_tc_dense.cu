@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
     unsigned char* sm_r = sm_e + P.ncb * 2 * CORE;
     unsigned* sm_pack = reinterpret_cast<unsigned*>(sm_r + ROW0_BYTES);
     Ctl* S = reinterpret_cast<Ctl*>(sm_pack + (EPI_WARPS * 32 * P.stage_words + 3) / 4 * 4);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank();
     const int cluster = (int)blockIdx.x / P.cl, n_clusters = (int)gridDim.x / P.cl;
     const int nb0 = rank * P.ncb;                                  // first output block of this CTA
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             // the CTA's columns as one or two MMAs of at most 256, each a multiple of 32
             const int n = ncb - skip, n1 = n <= 32 ? n : (n / 2 + 3) / 4 * 4, n2 = n - n1;
             const unsigned idesc1 = instr_desc(TM, 8 * n1, false), idesc2 = instr_desc(TM, 8 * n2, false);
@@ -229,16 +229,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
             const unsigned long long rd0 = smem_desc(smem_u32(sm_r), CORE, 2 * CORE, 0);
             const unsigned tmem1 = tmem_base + 8 * skip, tmem2 = tmem1 + 8 * n1, tmem_r = tmem_base + col_r;
             const unsigned long long step2 = (unsigned long long)(n1 * CORE / 16), estep2 = (unsigned long long)(n1 * 2 * CORE / 16);
-            bool ok = mbar_wait(&S->abort_flag, &S->tbar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->tbar, 0, P.status, 6);
             int s = 0;
             unsigned ph = 0;
             for (int i = 0; ok && i < n_mine; ++i) {
                 // the accumulators fill the CTA's share of TMEM: the next tile waits for the epilogue
-                if (!mbar_wait(&S->abort_flag, &S->tempty, (i & 1) ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty, (i & 1) ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 unsigned long long td = td0;
                 for (int kc = 0; kc < P.kchunks; ++kc) {
-                    if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) { ok = false; break; }
+                    if (!mbar_wait_warp(&S->abort_flag, &S->full[s], ph, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
                     unsigned long long ad = smem_desc(smem_u32(sm_x + s * A_STAGE), 16, 1024, 2);
                     const int ks_n = (kc == P.kchunks - 1) ? P.ksteps_last : KC / 16;

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_inv(const __grid_consta
 {
     extern __shared__ unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_inv(const __grid_consta
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             const unsigned idesc_full = instr_desc(TM, BN, true);
             const unsigned idesc_last = instr_desc(TM, P.n_last, true);
             int c = 0, nb_count = 0;
@@ -115,11 +115,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_inv(const __grid_consta
                 for (int nb = 0; ok && nb < P.nblk; ++nb, ++nb_count) {
                     const int buf = nb_count & 1;
                     const unsigned idesc = (nb == P.nblk - 1) ? idesc_last : idesc_full;
-                    if (!mbar_wait(&S->abort_flag, &S->tempty[buf], ((nb_count >> 1) & 1) ^ 1, P.status, 3)) { ok = false; break; }
+                    if (!mbar_wait_warp(&S->abort_flag, &S->tempty[buf], ((nb_count >> 1) & 1) ^ 1, P.status, 3)) { ok = false; break; }
                     tc_fence_after();
                     for (int kc = 0; kc < P.kchunks; ++kc, ++c) {
                         const int s = c % STAGES;
-                        if (!mbar_wait(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
+                        if (!mbar_wait_warp(&S->abort_flag, &S->full[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
                         tc_fence_after();
                         // A: K-major, one 128-byte line per token, 32 bytes per k-step.  B: N-major, atoms of 8 rotated
                         // coordinates x 64 output coordinates (1024 bytes), the next 64 output coordinates 8 KB away;

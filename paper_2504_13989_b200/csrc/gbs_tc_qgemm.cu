@@ -86,8 +86,8 @@ __host__ __device__ constexpr unsigned instr_desc_i8(int M, int N)
 // A from tensor memory, B from shared memory
 __device__ __forceinline__ void umma_i8_ts(unsigned d_tmem, unsigned a_tmem, unsigned long long b_desc, unsigned idesc, unsigned accumulate)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
     unsigned char* sm_b = base;
     unsigned char* sm_p = base + STAGES * SH::B_STAGE;                            // a stage: weight rows, then token rows
     Ctl* S = reinterpret_cast<Ctl*>(sm_p + STAGES * SH::P_STAGE);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     constexpr int WB = WBITS * 16, XB = XBITS * 16;                               // packed bytes per row and step
 
     if (threadIdx.x == 0) {
@@ -205,18 +205,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             const unsigned idesc = instr_desc_i8(TM, P.n);
             int c = 0;
             bool ok = true;
             for (int i = 0; ok && i < n_mine; ++i) {
                 const int a = i & 1;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[a], ((i >> 1) & 1) ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[a], ((i >> 1) & 1) ^ 1, P.status, 3)) break;
                 // the columns shared with the tile before are drained first
-                if (TW == 8 && !mbar_wait(&S->abort_flag, &S->tshared, (i & 1) ^ 1, P.status, 3)) break;
+                if (TW == 8 && !mbar_wait_warp(&S->abort_flag, &S->tshared, (i & 1) ^ 1, P.status, 3)) break;
                 for (int kb = 0; kb < P.kblocks; ++kb, ++c) {
                     const int s = c % STAGES;
-                    if (!mbar_wait(&S->abort_flag, &S->ofull[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
+                    if (!mbar_wait_warp(&S->abort_flag, &S->ofull[s], (c / STAGES) & 1, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
                     // an instruction takes 32 codes: eight columns of the weights' lanes, 32 bytes of the tokens' lines
                     const unsigned long long bd = smem_desc(smem_u32(sm_b + s * SH::B_STAGE), 16, 1024, 2);

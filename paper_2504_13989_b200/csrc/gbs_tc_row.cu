@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_row_rq(const __grid_constant_
 {
     extern __shared__ unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
 
     // ---- set-up: thread 0 arms the load barriers and starts the first loads at once; one thread of
     // warp 2 arms the remaining barriers; warp 1 allocates TMEM.  One block barrier joins the three.
@@ -130,20 +130,20 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_row_rq(const __grid_constant_
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             constexpr unsigned IDESC = instr_desc(TILE, DP, false);
             const unsigned h_base = smem_u32(S->h);
             const unsigned long long xd0 = smem_desc(smem_u32(S->x[0]), 16, 1024, 2);
             const unsigned long long hd0 = smem_desc(h_base, 16, 1024, 2);
             const unsigned xd_lo0 = (unsigned)xd0, xd_hi = (unsigned)(xd0 >> 32);
             const unsigned hd_lo0 = (unsigned)hd0, hd_hi = (unsigned)(hd0 >> 32);
-            bool ok = mbar_wait(&S->abort_flag, &S->hbar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->hbar, 0, P.status, 6);
             int it = 0;
             for (int t = blockIdx.x; ok && t < P.n_tiles; t += gridDim.x, ++it) {
                 const int s = it % STAGES;
                 const unsigned ph = (it / STAGES) & 1;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 // only the address fields (bytes >> 4, low words) of the two K-major descriptors change between
                 // k-steps: 32 bytes inside the 128-byte swizzled row, the second K block TILE*128 bytes further

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__
 {
     extern __shared__ unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const unsigned stage_bytes = (unsigned)(TOK * P.Upad * V * 2);
 
     // ---- set-up.  Thread 0 arms the load barriers and starts the first loads at once; one thread of
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__
     } else if (warp == 1 || warp >= 2 + EPI_WARPS) {
         // ------------------------------ MMA issuers ------------------------------
         const int issuer = warp == 1 ? 0 : warp - (2 + EPI_WARPS) + 1;        // takes tiles issuer, issuer + N_ISSUERS, ..
-        if (lane == 0) {
+        {
             constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS);
             const unsigned a_base = smem_u32(S->a);
             const unsigned tok_bytes = (unsigned)(P.Upad * V * 2);
@@ -208,13 +208,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__
             const unsigned long long bd0 = smem_desc(smem_u32(S->b[0]), tok_bytes, 512, 4);
             const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
             const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
-            bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->abar, 0, P.status, 6);
             int it = issuer;
             for (int g = blockIdx.x + issuer * (int)gridDim.x; ok && g < P.n_groups; g += N_ISSUERS * (int)gridDim.x, it += N_ISSUERS) {
                 const int s = it % STAGES;
                 const unsigned ph = (it / STAGES) & 1;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 // A: k-step ks = 32 bytes inside the 128-byte swizzled row of block ks/4 (blocks UMAX*128 B apart);
                 // 8-row groups 1024 B apart.  B: 16 u-rows of 64 bytes per k-step (1024 B); 8-row groups 512 B

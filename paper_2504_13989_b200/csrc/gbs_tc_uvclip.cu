@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     constexpr int PER = (BINS + 127) / 128;                       // bins a thread adds up
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>(smem_raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const unsigned stage_bytes = (unsigned)(TOK * P.Upad * V * 2);
 
     if (threadIdx.x == 0) {
@@ -153,18 +153,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS);
             const unsigned long long ad0 = smem_desc(smem_u32(S->a), 16, 1024, 2);
             const unsigned long long bd0 = smem_desc(smem_u32(S->b[0]), (unsigned)(P.Upad * V * 2), 512, 4);
             const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
             const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
-            bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->abar, 0, P.status, 6);
             for (int it = 0; ok && it < n_mine; ++it) {
                 const int s = it % STAGES;
                 const unsigned ph = (it / STAGES) & 1;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 unsigned a_lo = ad_lo0, b_lo = bd_lo0 + (unsigned)s * (STAGE_BYTES_MAX >> 4);
                 const unsigned d_tmem = tmem_base + s * STAGE_COLS;

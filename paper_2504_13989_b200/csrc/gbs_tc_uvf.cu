@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
     constexpr int TOK_WARPS = 4 * HALVES;                  // warps of a token
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>(smem_raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const unsigned slab_bytes = (unsigned)(P.Upad * V * 2);      // a token's rows in a plane
 
     if (threadIdx.x == 0) {
@@ -153,18 +153,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             constexpr unsigned IDESC = instr_desc(UMAX, NCOLS);
             constexpr unsigned KSTEP = (16 * V * 2) >> 4;          // sixteen u-lines of V bf16
             const unsigned long long ad0 = smem_desc(smem_u32(S->a), 16, 1024, 2);
             const unsigned long long bd0 = smem_desc(smem_u32(S->b[0]), slab_bytes, 8 * V * 2, V == 32 ? 4 : 2);
             const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
             const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
-            bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->abar, 0, P.status, 6);
             for (int it = 0; ok && it < n_mine; ++it) {
                 const int s = it % STAGES, c = it % ACCS;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], (unsigned)(it / STAGES) & 1u, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[c], ((unsigned)(it / ACCS) & 1u) ^ 1u, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], (unsigned)(it / STAGES) & 1u, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[c], ((unsigned)(it / ACCS) & 1u) ^ 1u, P.status, 3)) break;
                 tc_fence_after();
                 // only the address fields (bytes >> 4, low words) of the descriptors change between k-steps
                 const unsigned d_tmem = tmem_base + c * NCOLS;

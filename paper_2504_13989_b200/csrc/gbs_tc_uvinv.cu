@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
     unsigned char* sm_a = base;
     unsigned char* sm_b = base + A_BYTES;
     Bars* S = reinterpret_cast<Bars*>(base + A_BYTES + STAGES * STAGE_BYTES);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const unsigned slab_bytes = (unsigned)(P.Upad * V * 2);       // a token's operand rows: U lines of V halves
 
     if (threadIdx.x == 0) {
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
 
     if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             // fp16 operands: the two type fields of instr_desc (bf16) cleared
             constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS) & ~((1u << 7) | (1u << 10));
             constexpr unsigned KSTEP = (16 * V * 2) >> 4;          // sixteen u-lines of V halves
@@ -153,11 +153,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
             const unsigned long long bd0 = smem_desc(smem_u32(sm_b), slab_bytes, 8 * V * 2, V == 32 ? 4 : 2);
             const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
             const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
-            bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->abar, 0, P.status, 6);
             for (int it = 0; ok && it < n_mine; ++it) {
                 const int s = it % STAGES, c = it % ACCS;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], (unsigned)(it / STAGES) & 1u, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[c], ((unsigned)(it / ACCS) & 1u) ^ 1u, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], (unsigned)(it / STAGES) & 1u, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[c], ((unsigned)(it / ACCS) & 1u) ^ 1u, P.status, 3)) break;
                 tc_fence_after();
                 // only the address fields (bytes >> 4, low words) of the descriptors change between k-steps
                 const unsigned d_tmem = tmem_base + c * STAGE_COLS;

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(threads_for(GLOG), 1) k_tc_uvm_rq(const __grid
     constexpr int TSTAGES = (G == 8) ? 2 : 4;     // TMEM stages
     extern __shared__ unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int nst = P.n_stages;
     const int n_tok = (int)P.n_rows;
 
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(threads_for(GLOG), 1) k_tc_uvm_rq(const __grid
         constexpr int NISS = issuers_for(GLOG);
         const int issuer = warp == 1 ? 0 : warp - (2 + EPI_WARPS) + 1;      // takes tokens issuer, issuer + NISS, ..
         // ------------------------------ MMA issuer ------------------------------
-        if (lane == 0) {
+        {
             constexpr unsigned IDESC = instr_desc(UMAX, NCOLS);
             const unsigned a_base = smem_u32(S->a);
             const unsigned chunk_bytes = (unsigned)(P.Upad * V * 2);  // one chunk (N atom of 32): Upad rows of 64 bytes
@@ -242,12 +242,12 @@ __global__ void __launch_bounds__(threads_for(GLOG), 1) k_tc_uvm_rq(const __grid
             const unsigned long long bd0 = smem_desc(smem_u32(S->b), chunk_bytes, 512, 4);
             const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
             const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
-            bool ok = mbar_wait(&S->abort_flag, &S->abar, 0, P.status, 6);
+            bool ok = mbar_wait_warp(&S->abort_flag, &S->abar, 0, P.status, 6);
             int it = issuer;
             for (int tk = blockIdx.x + issuer * (int)gridDim.x; ok && tk < n_tok; tk += NISS * (int)gridDim.x, it += NISS) {
                 const int s = it % nst, ts = it % TSTAGES;
-                if (!mbar_wait(&S->abort_flag, &S->full[s], (it / nst) & 1, P.status, 2)) break;
-                if (!mbar_wait(&S->abort_flag, &S->tempty[ts], ((it / TSTAGES) & 1) ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], (it / nst) & 1, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[ts], ((it / TSTAGES) & 1) ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 // only the address fields (bytes >> 4, low words) of the descriptors change between k-steps
                 unsigned a_lo = ad_lo0, b_lo = bd_lo0 + (unsigned)s * ((unsigned)P.stage_bytes >> 4);

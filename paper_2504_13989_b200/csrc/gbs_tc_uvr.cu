@@ -152,6 +152,10 @@ __device__ __forceinline__ bool mbar_wait_inline(volatile int* abort_flag, void*
     atomicCAS(status, 0, code);
     return false;
 }
+__device__ __forceinline__ bool mbar_wait_warp_inline(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
+{
+    return __all_sync(0xffffffffu, mbar_wait_inline(abort_flag, bar, parity, status, code));
+}
 
 // Lane quadrant at which the second block's slabs of the it-th token of this CTA start.
 __device__ __forceinline__ int rot_of(int it, int nb2) { return nb2 == 3 ? (it & 1) : ((it * nb2) & 3); }
@@ -166,7 +170,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
     Ctl* S = reinterpret_cast<Ctl*>(base);
     unsigned char* a_smem = base + CTL_BYTES;
     unsigned char* ring = a_smem + P.a_bytes;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int n_tok = (int)P.n_rows;
     constexpr int tstride = TWO ? 2 * NCOLS : NCOLS;          // accumulator columns per token
     // accumulator stages: two tokens of two blocks, or four tokens of one block
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
         // instruction of its own loop), and one thread alone does not keep the epilogue fed.  U > 128: thread 0
         // contracts the first block of every token, thread 1 the second (a stage returns to the producer after both
         // commits).  U <= 128: the threads take alternate tokens.
-        if (lane == 0) {
+        {
             const int issuer = warp - 1;
             constexpr unsigned IDESC = instr_desc(128, NCOLS, true);
             // A: K-major, one 128-byte line per row and 64-column atom, 32 bytes per k-step.  B: N-major, atoms of 8
@@ -253,7 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
             const unsigned bd_lo0 = ((smem_u32(ring) >> 4) & 0x3fffu) | ((unsigned)(P.g * (SLICE_BYTES / 2) >> 4) << 16);
             // few live values: the loop must fit the 32 registers this warpgroup keeps; a spill in it costs the tensor
             // pipe more than any arithmetic
-            bool ok = mbar_wait_inline(&S->abort_flag, &S->abar, 0, P.status, 6);
+            bool ok = mbar_wait_warp_inline(&S->abort_flag, &S->abar, 0, P.status, 6);
             const int n_mine = ((int)blockIdx.x < n_tok) ? (n_tok - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
             const int chunks = (P.nslices + P.g - 1) / P.g;
             int s = 0;
@@ -265,14 +269,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
                     continue;
                 }
                 const int ts = it & (tstages - 1);
-                if (!mbar_wait_inline(&S->abort_flag, &S->tempty[ts], ((it / tstages) & 1) ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp_inline(&S->abort_flag, &S->tempty[ts], ((it / tstages) & 1) ^ 1, P.status, 3)) break;
                 tc_fence_after();
                 const unsigned d = tmem_base + ts * tstride + (TWO ? issuer * NCOLS : 0);
                 // the second block's rows come from a window of the image that starts 128 - 32 rot rows into it
                 unsigned a_lo = ad_lo0 + ((TWO && issuer) ? (unsigned)((128 - 32 * rot_of(it, P.nb2)) * 128) >> 4 : 0u);
                 int kk = 0;                           // k-step of the token
                 for (int c = 0; c < chunks; ++c) {
-                    if (!mbar_wait_inline(&S->abort_flag, &S->full[s], ph, P.status, 2)) { ok = false; break; }
+                    if (!mbar_wait_warp_inline(&S->abort_flag, &S->full[s], ph, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
                     unsigned b_lo = bd_lo0 + (unsigned)(s * P.g) * (SLICE_BYTES >> 4);
                     const int kend = kk + 2 * P.g < P.ksteps ? kk + 2 * P.g : P.ksteps;
