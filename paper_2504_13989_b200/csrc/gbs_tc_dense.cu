@@ -303,8 +303,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
             const unsigned mine = smem_u32(&S->tmax[i & 1][rank * EW + h][tok]), bar = smem_u32(&S->maxbar[i & 1]);
             for (int r = 0; r < P.cl; ++r) peer_store(peer_addr(mine, (unsigned)r), M);
             __syncwarp();
-            if (lane == 0)
-                for (int r = 0; r < P.cl; ++r) peer_arrive(peer_addr(bar, (unsigned)r));
+            if (lane < P.cl) peer_arrive(peer_addr(bar, (unsigned)lane));
             ok = __all_sync(0xffffffffu, cluster_wait(&S->abort_flag, &S->maxbar[i & 1], (unsigned)(i >> 1) & 1u, P.status, 7));
             if (!ok) break;
             for (int r = 0; r < P.cl * EW; ++r) M = fmaxf(M, S->tmax[i & 1][r][tok]);
@@ -335,22 +334,30 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
             const int n_codes = (P.m - nfirst) < (ch1 - ch0) * 32 ? (P.m - nfirst) : (ch1 - ch0) * 32;
             const int nbytes = n_codes > 0 ? n_codes * BITS / 8 : 0;
             const int j = lane & 15;
+            const unsigned* words = pack + (lane >> 4) * P.stage_words + j;
             unsigned char* piece = P.codes + (row0 + q * 32 + (lane >> 4)) * P.code_row_bytes + nfirst / 8 * BITS;
-#pragma unroll 4
-            for (int r = lane >> 4; r < 32; r += 2, piece += 2 * P.code_row_bytes) {
-                const int off = (int)(reinterpret_cast<uintptr_t>(piece) & 3u);
-                const unsigned* src = pack + r * P.stage_words;
-                const unsigned lo = j > 0 ? src[j - 1] : 0u, hi = src[j];
-                const unsigned v = off ? __funnelshift_l(lo, hi, 8 * off) : hi;
-                const int b0 = 4 * j - off;                                    // first byte of the piece this word covers
-                unsigned char* dst = piece + b0;
-                if (row0 + q * 32 + r < P.n_rows) {
-                    if (b0 >= 0 && b0 + 4 <= nbytes) {
-                        *reinterpret_cast<unsigned*>(dst) = v;
-                    } else {
 #pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            if (b0 + b >= 0 && b0 + b < nbytes) dst[b] = (unsigned char)(v >> (8 * b));
+            for (int part = 0; part < 2; ++part) {                             // eight rows' words in flight at a time
+                unsigned lo[8], hi[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    hi[e] = words[(16 * part + 2 * e) * P.stage_words];
+                    lo[e] = j > 0 ? words[(16 * part + 2 * e) * P.stage_words - 1] : 0u;
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e, piece += 2 * P.code_row_bytes) {
+                    const int off = (int)(reinterpret_cast<uintptr_t>(piece) & 3u);
+                    const unsigned v = __funnelshift_l(lo[e], hi[e], 8 * off);
+                    const int b0 = 4 * j - off;                                // first byte of the piece this word covers
+                    unsigned char* dst = piece + b0;
+                    if (row0 + q * 32 + 16 * part + 2 * e + (lane >> 4) < P.n_rows) {
+                        if (b0 >= 0 && b0 + 4 <= nbytes) {
+                            *reinterpret_cast<unsigned*>(dst) = v;
+                        } else if (b0 < nbytes) {
+#pragma unroll
+                            for (int b = 0; b < 4; ++b)
+                                if (b0 + b >= 0 && b0 + b < nbytes) dst[b] = (unsigned char)(v >> (8 * b));
+                        }
                     }
                 }
             }
@@ -415,15 +422,18 @@ int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* nc
     const int nb = p->m / 8;
     double best = 0.0;
     *cl_out = 0;
-    for (int want = 1; want <= MAX_CL; ++want) {
-        const int ncb = ((nb + want - 1) / want + 3) / 4 * 4, cl = (nb + ncb - 1) / ncb;
-        const int real = nb - (cl - 1) * ncb, last = (real + 3) / 4 * 4;      // sixteen columns for coordinate 0 must fit
-        if (ncb > 64 || (last - real < 2 && 8 * last + 16 > TMEM_COLS) || smem_bytes(ncb, kchunks, 2, nullptr) > p->smem_optin) continue;
+    for (int ncb = 4; ncb <= 64; ncb += 4) {
+        const int cl = (nb + ncb - 1) / ncb, real = nb - (cl - 1) * ncb, last = (real + 3) / 4 * 4;
+        if (cl > MAX_CL || (last - real < 2 && 8 * last + 16 > TMEM_COLS) ||      // sixteen columns for coordinate 0 must fit
+            smem_bytes(ncb, kchunks, 2, nullptr) > p->smem_optin)
+            continue;
         const int fit = n_tiles ? clusters_at_once(p, cl) : 1;
         if (fit < 1) return (int)cudaErrorInvalidConfiguration;
         const int waves = (n_tiles + fit - 1) / fit;
-        const double mma = ncb <= 32 ? (ncb * 4 < 64 ? 64.0 : ncb * 4.0) : (ncb * 4 < 128 ? 128.0 : ncb * 4.0);
-        const double cost = waves * (kchunks * (8.0 * mma + 220.0) + 4500.0 + 20.0 * ncb);
+        const auto mma = [](int blocks) { return blocks <= 32 ? (blocks * 4 < 64 ? 64.0 : blocks * 4.0) : (blocks * 4 < 128 ? 128.0 : blocks * 4.0); };
+        double step = mma(last) + 100.0;                                          // the last CTA has coordinate 0's MMA as well
+        if (cl > 1 && mma(ncb) > step) step = mma(ncb);
+        const double cost = waves * (kchunks * (8.0 * step + 220.0) + 4500.0 + 20.0 * ncb);
         if (*cl_out == 0 || cost < best) { best = cost; *cl_out = cl; *ncb_out = ncb; *fit_out = fit; }
     }
     return 0;

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     constexpr int PER = (BINS + 127) / 128;                       // bins a thread adds up
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>(smem_raw);
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned stage_bytes = (unsigned)(TOK * P.Upad * V * 2);
 
     if (threadIdx.x == 0) {
