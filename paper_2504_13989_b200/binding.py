@@ -5,12 +5,13 @@ PyTorch is used for device memory and streams.  There is no CPU fallback: if the
 library is missing or a call fails, a GbsError is raised.
 
 Plan's per-call methods go through _native.so (csrc/gbs_torch.cpp), which does the regular call's checks,
-allocations and marshalling in C and answers None for every other call; those take the functions below.
+allocations and marshalling in C; every other call takes the functions below.
 """
 from __future__ import annotations
 
 import ctypes
 import os
+import weakref
 
 import torch
 
@@ -419,9 +420,15 @@ class Plan:
         self._native = native()
         self.handle = gbs_plan_create_ex(d, d_pad, m, bits, group, alpha, GBS_PLAN_ASYMMETRIC if asymmetric else 0)
         self.info = gbs_plan_info(self.handle)
+        # the regular per-call path, without a Python frame; it passes what it does not handle to the methods below
+        self._calls = self._native.Calls(self.handle, weakref.ref(self))
+        for name in ("rotate_quantize", "dequantize", "quantized_matmul", "clip_error"):
+            if getattr(type(self), name) is getattr(Plan, name):          # a subclass's own method stays
+                self.__dict__[name] = getattr(self._calls, name)
 
     def close(self):
         if getattr(self, "handle", None):
+            self._calls.clear()
             gbs_plan_destroy(self.handle)
             self.handle = None
 

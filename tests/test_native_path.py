@@ -18,6 +18,8 @@ def test_irregular_calls_are_handed_on():
     assert nat.dequantize(0, x, x, False, torch.float32, None, None) is None
     assert nat.quantized_matmul(0, x, x, 0, x, x, torch.float32, None, None) is None
     assert nat.clip_error(0, x, [0.5], None) is None
+    with pytest.raises(ValueError):
+        nat.Calls(0, None)
 
 
 @pytest.mark.gpu
@@ -60,3 +62,43 @@ def test_native_and_python_paths_agree():
             plan.dequantize(ref[0], ref[1], dtype=torch.float16)
         with pytest.raises(binding.GbsError):
             plan.clip_error(x, [1.5])
+
+
+@pytest.mark.gpu
+def test_methods_take_arguments_as_plan_declares_them():
+    """The per-plan C methods parse like the Python methods they stand for, share their errors, and end with the plan."""
+    gbs_build.build()
+    x = synth.make_host("llama4096", 3).to(DEV)
+    big = synth.make_host("llama4096", 700).to(DEV)                       # outputs beyond the shared allocation's size
+    with Plan(4096, bits=4, alpha=0.9) as plan:
+        for rows in (x, big):
+            codes, scales, y = plan.rotate_quantize(rows, True, None, None)
+            c2, s2, y2 = plan.rotate_quantize(x=rows, want_y=True, stream=torch.cuda.current_stream())
+            c3, s3, y3 = Plan.rotate_quantize(plan, rows)                  # the class's own method
+            assert torch.equal(codes, c2) and torch.equal(scales, s2) and torch.equal(y, y2) and y3 is None
+            assert torch.equal(codes, c3) and torch.equal(scales, s3)
+            for t, shape, dtype in ((codes, (len(rows), 2048), torch.uint8), (scales, (len(rows), 1), torch.float32)):
+                assert t.shape == shape and t.dtype == dtype and t.is_contiguous() and t.data_ptr() % 16 == 0
+            a = plan.dequantize(codes, scales, True, torch.bfloat16)
+            b = plan.dequantize(scales=scales, codes=codes, dtype=torch.bfloat16, inverse=True)
+            assert torch.equal(a, b) and plan.dequantize(codes, scales).dtype == torch.float32
+            out = torch.empty_like(a)
+            assert plan.dequantize(codes, scales, inverse=True, out=out) is out and torch.equal(out, a)
+            mm = plan.quantized_matmul(codes, scales, plan, codes, scales)
+            assert torch.equal(mm, plan.quantized_matmul(codes, scales, plan_w=plan, codes_w=codes, scales_w=scales, dtype=torch.float32))
+        assert plan.clip_error(x, alphas=[0.5, 1.0]).shape == (2,)
+        err, per_row = plan.clip_error(x, [0.5, 1.0], want_rows=True)
+        assert per_row.shape == (3, 2)
+        for call in (lambda: plan.rotate_quantize(), lambda: plan.rotate_quantize(x, x=x), lambda: plan.rotate_quantize(x, wanty=1),
+                     lambda: plan.rotate_quantize(x, False, None, None, 1), lambda: plan.dequantize(codes)):
+            with pytest.raises(TypeError):
+                call()
+        kept = plan.rotate_quantize
+    with pytest.raises(binding.GbsError):
+        kept(x)
+
+    class Mine(Plan):
+        def rotate_quantize(self, x, **kw):
+            return "mine"
+    with Mine(4096) as plan:
+        assert plan.rotate_quantize(x) == "mine" and plan.dequantize(codes, scales).shape == (700, 4096)
