@@ -11,8 +11,8 @@
 //     m = 1544 instead of 4.8 MB), and with the output blocks taken in descending order the descriptor's two strides are
 //     both +128 bytes.  A CTA's share (31 KB) stays in shared memory; only the rows of X move.
 //   * Column 0 of H (constant -1) is repaired by one more MMA per tile with a 16-column operand whose column 0 holds
-//     H[n][0] - t(-n).  Row 0 (x_0 - sum of the others) is an extra 16-row operand, the same for every k-step but the first,
-//     contracted by the last CTA of the cluster, which has the fewest coordinates; it sends the value to the first.
+//     H[n][0] - t(-n).  Row 0 (2 x_0 - sum of all) is an extra 16-row operand, the same for every k-step, contracted by
+//     the last CTA of the cluster, which has the fewest coordinates; it sends the value to the first.
 //   * One sweep.  A token's m fp32 values do not fit one SM's TMEM, so a CLUSTER of CTAs takes 128 tokens and each CTA up to
 //     512 output coordinates: TMEM lane t holds the CTA's coordinates of token t, and the CTAs exchange their maxima of
 //     every token through distributed shared memory before quantizing (Sections 2.1, 3.1).
@@ -46,7 +46,7 @@ constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int TMEM_COLS = 512;
 constexpr int MAX_CL = 8;               // CTAs per cluster
 constexpr int CORE = 128;               // bytes of a core matrix: 8 rows x 8 bf16
-constexpr int ROW0_BYTES = 2 * 4 * CORE;   // row 0 as a 16-row operand: the first k-step's, the others'
+constexpr int ROW0_BYTES = 2 * 4 * CORE;   // row 0 as 16-row operands: 2 at column 0, and all -1
 
 struct Ctl {
     float tmax[2][MAX_CL * EW][TM];     // [tile parity][CTA and quarter][token]: maxima of every share of a token
@@ -122,6 +122,22 @@ __device__ __forceinline__ bool cluster_wait(volatile int* abort_flag, void* bar
     *abort_flag = 1;
     atomicCAS(status, 0, code);
     return false;
+}
+
+// n k-steps of one stage: 32 bytes of the 128-byte line each, four to a box; the operand moves on by `step`
+__device__ __forceinline__ void steps(unsigned d_tmem, unsigned long long ad, unsigned long long bd, unsigned step, unsigned idesc, int n)
+{
+    if (n == KC / 16) {
+#pragma unroll
+        for (int ks = 0; ks < KC / 16; ++ks)
+            umma_f16(d_tmem, ad + (unsigned long long)(2 * (ks & 3) + (ks >> 2) * (A_BOX / 16)), bd + (unsigned long long)(step * ks), idesc, 1u);
+    } else {
+        for (int ks = 0; ks < n; ++ks) {
+            umma_f16(d_tmem, ad, bd, idesc, 1u);
+            ad += ks == 3 ? (A_BOX - 96) / 16 : 2;
+            bd += step;
+        }
+    }
 }
 
 // one column of this thread's TMEM lane
@@ -240,20 +256,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
                 for (int kc = 0; kc < P.kchunks; ++kc) {
                     if (!mbar_wait_warp(&S->abort_flag, &S->full[s], ph, P.status, 2)) { ok = false; break; }
                     tc_fence_after();
-                    unsigned long long ad = smem_desc(smem_u32(sm_x + s * A_STAGE), 16, 1024, 2);
+                    const unsigned long long ad = smem_desc(smem_u32(sm_x + s * A_STAGE), 16, 1024, 2);
                     const int ks_n = (kc == P.kchunks - 1) ? P.ksteps_last : KC / 16;
                     if (kc == 0) {
-                        // column 0: H[n][0] - t(-n) against x_0 (the other fifteen columns of the operand are zero)
+                        // column 0: H[n][0] - t(-n) against x_0, and coordinate 0: 2 x_0 (the other columns of these are zero)
                         umma_f16(tmem1, ad, ed0, idesc1, 0u);
                         if (n2) umma_f16(tmem2, ad, ed0 + estep2, idesc2, 0u);
+                        if (last) umma_f16(tmem_r, ad, rd0, IDESC_R, 0u);
                     }
-                    for (int ks = 0; ks < ks_n; ++ks) {
-                        umma_f16(tmem1, ad, td, idesc1, 1u);
-                        if (n2) umma_f16(tmem2, ad, td + step2, idesc2, 1u);
-                        if (last) umma_f16(tmem_r, ad, (kc | ks) != 0 ? rd0 + 4 * CORE / 16 : rd0, IDESC_R, (kc | ks) != 0 ? 1u : 0u);
-                        ad += ks == 3 ? (A_BOX - 96) / 16 : 2;     // 32 bytes of the 128-byte line, then the second box
-                        td += 2 * CORE / 16;                       // two core matrices on
-                    }
+                    // one operand after the other, each in a loop of its own: a condition between two MMAs doubles their time
+                    steps(tmem1, ad, td, 2 * CORE / 16, idesc1, ks_n);
+                    if (n2) steps(tmem2, ad, td + step2, 2 * CORE / 16, idesc2, ks_n);
+                    if (last) steps(tmem_r, ad, rd0 + 4 * CORE / 16, 0, IDESC_R, ks_n);
+                    td += (unsigned long long)(2 * CORE / 16 * (KC / 16));
                     umma_commit(&S->empty[s]);
                     if (++s == P.stages) { s = 0; ph ^= 1; }
                 }
@@ -485,7 +500,7 @@ void gbs_tc_dense_tables(const int8_t* hm, int m, unsigned short* toep, unsigned
         }
     unsigned short* row0 = col0 + (size_t)nbp * 128;
     for (int v = 0; v < 2; ++v)
-        for (int k = 0; k < 16; ++k) row0[v * 256 + (k >> 3) * 64 + (k & 7)] = bf(v == 0 && k == 0 ? 1 : -1);
+        for (int k = 0; k < 16; ++k) row0[v * 256 + (k >> 3) * 64 + (k & 7)] = bf(v ? -1 : (k == 0 ? 2 : 0));
 }
 
 int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
