@@ -81,6 +81,11 @@ int gbs_generic_dequantize(const gbs_plan* p, const void* codes, const float* sc
                            void* out, int out_dtype, int inverse, cudaStream_t stream);
 size_t gbs_generic_smem_bytes(const gbs_plan* p, int* rows_per_cta);
 
+// gbs_tc_uv2.cu : rotate-quantize of bf16 rows, 4096 < d' = 64 U <= 8192
+bool gbs_tc_uv2_supported(const gbs_plan* p);
+int gbs_tc_uv2_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
+                               float* scales, float* y_opt, cudaStream_t stream);
+
 // gbs_tc_uvclip.cu : clip-ratio scoring of the UV family by histogram, where it applies
 #define GBS_UVCLIP_NOT_SERVED (-1)
 int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, const float* alphas, int K,
