@@ -11,7 +11,7 @@
 //
 // What bounds it: HBM (48 or 64 bytes read and 256 or 512 written per row).  About 7 issue slots per value without any
 // shared memory, barrier or tensor-core round trip; the tensor-core form this replaces waited on that round trip with 16
-// warps per SM.  262 144 rows, 4 bits, asymmetric -> bf16: 33.2 us before.
+// warps per SM.  262 144 rows, 4 bits, asymmetric -> bf16: 33.2 us before, 19.5 now (4.4 TB/s).
 #include <string.h>
 
 #include "gbs_internal.h"
