@@ -393,6 +393,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
                 if (slab == 0 && lane == 0) P.scales[row] = P.c_scale * M;
             }
             if (lane_live) {
+                if (P.y_opt) {                        // first: behind the codes the rows would have to stay live
+                    float* yo = P.y_opt + row * (long long)P.d_pad + (size_t)up * NCOLS;
+                    store_y(yo, r0, P.norm);
+                    store_y(yo + 32, r1, P.norm);
+                    store_y(yo + 64, r2, P.norm);
+                    store_y(yo + 96, r3, P.norm);
+                }
                 unsigned out[4 * BITS];
                 // per-group factors are formed chunk by chunk: four more live values would not fit the register budget
                 quantize_pack32<BITS>(r0, GROUPED ? ((mc[0] > 0.f) ? __fdividef(P.c_half, mc[0]) : 0.f) : a1t, out);
@@ -400,13 +407,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
                 quantize_pack32<BITS>(r2, GROUPED ? ((mc[2] > 0.f) ? __fdividef(P.c_half, mc[2]) : 0.f) : a1t, out + 2 * BITS);
                 quantize_pack32<BITS>(r3, GROUPED ? ((mc[3] > 0.f) ? __fdividef(P.c_half, mc[3]) : 0.f) : a1t, out + 3 * BITS);
                 store_codes<BITS>(P.codes + row * P.code_row_bytes + (size_t)up * (NCOLS * BITS / 8), out);
-                if (P.y_opt) {
-                    float* yo = P.y_opt + row * (long long)P.d_pad + (size_t)up * NCOLS;
-                    store_y(yo, r0, P.norm);
-                    store_y(yo + 32, r1, P.norm);
-                    store_y(yo + 64, r2, P.norm);
-                    store_y(yo + 96, r3, P.norm);
-                }
             }
         }
     }
