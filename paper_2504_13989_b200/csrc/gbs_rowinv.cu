@@ -11,7 +11,7 @@
 //
 // What bounds it: HBM (48 or 64 bytes read and 256 or 512 written per row).  About 7 issue slots per value without any
 // shared memory, barrier or tensor-core round trip; the tensor-core form this replaces waited on that round trip with 16
-// warps per SM.  262 144 rows, 4 bits, asymmetric -> bf16: 33.2 us before, 19.5 now (4.4 TB/s).
+// warps per SM.  262 144 rows, 4 bits, asymmetric -> bf16: 33.2 us before, 19.2 now (4.5 TB/s).
 #include <string.h>
 
 #include "gbs_internal.h"
@@ -20,8 +20,8 @@
 namespace {
 
 constexpr int DP = 128;
-constexpr int RI_THREADS = 128;
-constexpr int RI_BLOCKS = 5;          // per SM: 102 registers per thread, of which 64 hold the row
+constexpr int RI_THREADS = 32;        // single warps: a finished one makes room for the next at once (blocks of 128: 19.6 us, 19.15 so)
+constexpr int RI_BLOCKS = 20;         // per SM: 102 registers per thread, of which 64 hold the row
 
 struct RowInvParams {
     long long n_rows;
