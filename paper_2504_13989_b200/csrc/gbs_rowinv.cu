@@ -58,11 +58,11 @@ __global__ void __launch_bounds__(RI_THREADS, RI_BLOCKS) k_row_inv(const __grid_
     // h[4 o + i] = (coordinate 8 o + i, coordinate 8 o + 4 + i)
     unsigned h[64];
 #pragma unroll
-    for (int o = 0; o < 16; ++o) unpack_octet<BITS, ASYM, NW>(w, o, h + 4 * o);
+    for (int o = 0; o < 16; ++o) rotate_octet<BITS, ASYM, NW, false>(w, o, h + 4 * o);
 #pragma unroll
     for (int i = 0; i < 64; ++i) h[i] = hpair(h[i]);
 #pragma unroll
-    for (int s = 1; s < 64; s <<= 1)
+    for (int s = 4; s < 64; s <<= 1)
 #pragma unroll
         for (int i = 0; i < 64; ++i)
             if ((i & s) == 0) {

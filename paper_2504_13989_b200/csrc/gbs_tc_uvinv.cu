@@ -80,17 +80,17 @@ struct InvParams {
     int* status;
 };
 
-// V codes of one row u -> V/2 packed halves h[4 o + i] = (8 o + i, 8 o + 4 + i), times 2^-24, after H_V; offset removed.
-template <int BITS, int V>
+// V codes of one row u -> V/2 packed halves h[4 o + i] = (8 o + i, 8 o + 4 + i), times 2^-24 (LIFT: 2^-10), after H_V; offset removed.
+template <int BITS, int V, bool LIFT>
 __device__ __forceinline__ void unpack_rotate(const unsigned* w, unsigned h[V / 2])
 {
     constexpr int NW = V * BITS / 32;
 #pragma unroll
-    for (int o = 0; o < V / 8; ++o) unpack_octet<BITS, false, NW>(w, o, h + 4 * o);
+    for (int o = 0; o < V / 8; ++o) rotate_octet<BITS, false, NW, LIFT>(w, o, h + 4 * o);
 #pragma unroll
     for (int i = 0; i < V / 2; ++i) h[i] = hpair(h[i]);
 #pragma unroll
-    for (int s = 1; s < V / 2; s <<= 1)
+    for (int s = 4; s < V / 2; s <<= 1)
 #pragma unroll
         for (int i = 0; i < V / 2; ++i)
             if ((i & s) == 0) {
@@ -98,7 +98,9 @@ __device__ __forceinline__ void unpack_rotate(const unsigned* w, unsigned h[V / 
                 h[i] = hadd2(a, b);
                 h[i + s] = hsub2(a, b);
             }
-    h[0] = hsub2(h[0], (unsigned)(V << (BITS - 1)));        // low half: V * 2^(b-1) * 2^-24
+    // low half: V 2^(b-1) times 2^-24, a subnormal, or 2^-10
+    constexpr unsigned LOG = (V == 32 ? 5 : 6) + BITS - 1;
+    h[0] = hsub2(h[0], LIFT ? (LOG + 5) << 10 : 1u << LOG);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -233,7 +235,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
         auto unpack_tile = [&](int n, const Fetched& B, float& fac) -> bool {
             const int it = n * GROUPS + grp, s = it % STAGES;
             unsigned h[V / 2];
-            unpack_rotate<BITS, V>(B.raw, h);
+            unpack_rotate<BITS, V, SPLIT>(B.raw, h);
             unsigned sh2 = 0u, sl2 = 0u;
             if (SPLIT) {
                 // scales relative to 2^e, the power of two below the token's largest: s = Delta 2^(14-e) in (0, 2^15)
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         if (SPLIT) {
-                            const unsigned n1 = hmul2(h[4 * c + e], 0x74007400u);          // times 2^14: n * 2^-10
+                            const unsigned n1 = h[4 * c + e];                              // n * 2^-10
                             ph[e] = hmul2(n1, sh2);
                             pl[e] = hfma2(n1, sl2, hfma2(n1, sh2, ph[e] ^ 0x80008000u));
                         } else {
