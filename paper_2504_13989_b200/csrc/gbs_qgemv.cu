@@ -49,15 +49,16 @@ template <int BITS> struct Packed {
             for (int i = 0; i < BITS; ++i) w[i] = __ldg(reinterpret_cast<const unsigned*>(p) + i);
         }
     }
-    // fields 8 o .. 8 o + 7 -> even and odd ones
-    __device__ __forceinline__ void octet(int o, unsigned& even, unsigned& odd) const
-    {
-        unsigned f;
-        if (BITS == 4) f = w[o < BITS ? o : 0];
-        else f = o == 0 ? w[0] : o == 1 ? __funnelshift_r(w[0], w[1], 24) : o == 2 ? __funnelshift_r(w[1], w[2], 16) : w[2] >> 8;
-        fields_to_int8<BITS>(f, even, odd);
-    }
 };
+
+template <int BITS>
+__device__ __forceinline__ void gather_in_place(unsigned w[BITS])
+{
+    unsigned p[BITS];
+    gather_octets<BITS>(w, p);
+#pragma unroll
+    for (int i = 0; i < BITS; ++i) w[i] = p[i];
+}
 
 __device__ __forceinline__ void mma_s8(int c[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1)
 {
@@ -112,15 +113,21 @@ __global__ void __launch_bounds__(32 * WARPS) k_qgemv(const __grid_constant__ Qg
 #pragma unroll
         for (int p = 0; p < PF; ++p) {
             if (kb0 + p < kb1) {
+                if (XBITS == 3 || WBITS == 3) {
+#pragma unroll
+                    for (int i = 0; i < 2 * MT; ++i) gather_in_place<WBITS>(w[p][i].w);
+#pragma unroll
+                    for (int n = 0; n < NT; ++n) gather_in_place<XBITS>(x[p][n].w);
+                }
 #pragma unroll
                 for (int o = 0; o < 4; ++o) {
                     unsigned a[2 * MT][2];
 #pragma unroll
-                    for (int i = 0; i < 2 * MT; ++i) w[p][i].octet(o, a[i][0], a[i][1]);
+                    for (int i = 0; i < 2 * MT; ++i) field_pair<WBITS>(w[p][i].w, o, a[i][0], a[i][1]);
 #pragma unroll
                     for (int n = 0; n < NT; ++n) {
                         unsigned b0, b1;
-                        x[p][n].octet(o, b0, b1);
+                        field_pair<XBITS>(x[p][n].w, o, b0, b1);
 #pragma unroll
                         for (int m = 0; m < MT; ++m)
                             mma_s8(acc[m][n], a[2 * m][0], a[2 * m + 1][0], a[2 * m][1], a[2 * m + 1][1], b0, b1);

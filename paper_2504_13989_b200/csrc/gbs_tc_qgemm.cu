@@ -16,7 +16,7 @@
 //   * Packed codes arrive by TMA (128 codes of every row per step, several steps ahead).  Twenty-four warps unpack, one thread
 //     per row: a field moved to the top bits of its byte IS the int8 q * 2^(8-b) (the epilogue removes the power of two).
 //     Weights go to TENSOR MEMORY (a thread's 128 int8 are 32 columns of its lane), tokens to 128-byte-swizzled K-major rows in
-//     shared memory; both use the same order of the codes inside a word (even fields, then odd), which a dot product does not see.
+//     shared memory; both use the same order of the codes, which a dot product does not see.
 //   * One thread issues tcgen05.mma kind::i8 (int32 accumulators, exact).  Consecutive tiles use accumulators that overlap by
 //     half (or not at all, up to 128 tokens); four epilogue warps drain the shared half first, so that the next tile starts
 //     early.  Lanes of a warp hold consecutive channels, so every store instruction writes 64 or 128 contiguous bytes.
@@ -127,23 +127,21 @@ __device__ __forceinline__ void load_row128(unsigned rows, int r, uint4 w[BITS])
     for (int c = 0; c < BITS; ++c)
         w[c] = ld_shared_v4(rows + (unsigned)r * (16u * BITS) + (unsigned)((BITS == 4 ? c ^ ((r >> 1) & 3) : c) << 4));
 }
-// Codes 32 c .. 32 c + 31 of it -> eight words of int8: per octet of codes the even fields, then the odd ones.
-template <int BITS>
+// Codes 32 c .. 32 c + 31 of it -> eight words of int8.
+template <int BITS, bool GATHER>
 __device__ __forceinline__ void unpack32(const uint4 w[BITS], int c, unsigned v[8])
 {
-    if (BITS == 4) {
-        fields_to_int8<4>(w[c].x, v[0], v[1]);
-        fields_to_int8<4>(w[c].y, v[2], v[3]);
-        fields_to_int8<4>(w[c].z, v[4], v[5]);
-        fields_to_int8<4>(w[c].w, v[6], v[7]);
+    const unsigned f[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
+                            w[2].x, w[2].y, w[2].z, w[2].w, w[BITS - 1].x, w[BITS - 1].y, w[BITS - 1].z, w[BITS - 1].w};
+    unsigned p[BITS];
+    if (GATHER) {
+        gather_octets<BITS>(f + BITS * c, p);
     } else {
-        const unsigned f[12] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w, w[2].x, w[2].y, w[2].z, w[2].w};
-        const unsigned w0 = f[3 * c], w1 = f[3 * c + 1], w2 = f[3 * c + 2];
-        fields_to_int8<3>(w0, v[0], v[1]);                                   // bits above 24 are dropped by the masks
-        fields_to_int8<3>(__funnelshift_r(w0, w1, 24), v[2], v[3]);
-        fields_to_int8<3>(__funnelshift_r(w1, w2, 16), v[4], v[5]);
-        fields_to_int8<3>(w2 >> 8, v[6], v[7]);
+#pragma unroll
+        for (int i = 0; i < BITS; ++i) p[i] = f[BITS * c + i];
     }
+#pragma unroll
+    for (int o = 0; o < 4; ++o) field_pair<BITS>(p, o, v[2 * o], v[2 * o + 1]);
 }
 
 template <int XBITS, int WBITS, typename OutT, int TW>
@@ -255,7 +253,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     unsigned v[8];
-                    unpack32<WBITS>(w, k, v);
+                    unpack32<WBITS, XBITS == 3 || WBITS == 3>(w, k, v);
                     tmem_st8(lane_base + s * 32 + k * 8, v);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -272,7 +270,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         unsigned v[8];
-                        unpack32<XBITS>(w, k, v);
+                        unpack32<XBITS, XBITS == 3 || WBITS == 3>(w, k, v);
                         st_shared_v4(line + (unsigned)(((2 * k) ^ (r & 7)) << 4), make_uint4(v[0], v[1], v[2], v[3]));
                         st_shared_v4(line + (unsigned)(((2 * k + 1) ^ (r & 7)) << 4), make_uint4(v[4], v[5], v[6], v[7]));
                     }
