@@ -1,5 +1,5 @@
 // gbs_quantized_matmul for a few tokens (a decoding step): out[t][o] = Delta_x[t] Delta_w[o] sum_j q_x[t][j] q_w[o][j] with
-// n_tokens <= 64 (Section 4.2, Eq. (2)); the tile kernel of gbs_tc_qgemm.cu serves larger batches.
+// n_tokens <= 64 (Section 4.2, Eq. (2)); the tile kernel of gbs_tc_qgemm.cu serves larger batches, and wide outputs (the rule is there).
 //
 // With this few tokens the call reads the packed weights once and does little with them, so what bounds it is how much of
 // the chip reads at once and how many latencies follow one another, not the tensor pipe.  A 128 x 256 output tile per CTA

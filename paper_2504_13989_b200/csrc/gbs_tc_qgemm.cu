@@ -68,6 +68,7 @@ struct Ctl {
 struct QgemmParams {
     long long n_tok, n_out;
     int n;                              // tokens per tile (MMA N)
+    int xbox;                           // token rows a load brings: n, or all tokens if they are fewer
     int m_tiles, tiles;                 // channel tiles, all tiles
     int kblocks;                        // d' / 128
     const float* sx;
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
                 for (int kb = 0; kb < P.kblocks; ++kb, ++c) {
                     const int s = c % STAGES;
                     if (!mbar_wait(&S->abort_flag, &S->pempty[s], ((c / STAGES) & 1) ^ 1, P.status, 1)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&S->pfull[s], (unsigned)(TM * WB + P.n * XB));
+                    mbar_arrive_expect_tx(&S->pfull[s], (unsigned)(TM * WB + P.xbox * XB));
                     tma_load_2d(sm_p + s * SH::P_STAGE, &wmap, &S->pfull[s], kb * WB, mt * TM);
                     tma_load_2d(sm_p + s * SH::P_STAGE + TM * 64, &xmap, &S->pfull[s], kb * XB, nt * P.n);
                 }
@@ -365,6 +366,19 @@ int pick_tokens(long long n_tok, long long n_out, int kblocks, int sm_count)
     return n_best;
 }
 
+// Whether the few-token kernel (gbs_qgemv.cu) is the faster one.  Its time grows with the channels, by these cycles per channel and
+// step of 128 codes for up to 8, 16, 32 and 64 tokens (4096-wide rows, 8192 and 14336 channels; four bits, three bits on a side); a
+// wave of tiles costs 600 per step whatever it holds, with much the same start.  So 64 tokens go to the tiles beyond 5800 (4300)
+// channels, 32 beyond 10 300 (7800), 16 beyond 18 200 (8800).  48 tokens -> 14336, four bits: 28.5 us here, 12.4 in tiles; 4096: 7.9
+// and 10.8.
+bool few_tokens(long long n_tok, long long n_out, bool three, int sm_count)
+{
+    if (n_tok > GBS_QGEMV_MAX_TOKENS) return false;
+    static const double per_channel[2][4] = {{0.021, 0.033, 0.058, 0.103}, {0.035, 0.068, 0.077, 0.140}};
+    const long long tiles = (n_out + TM - 1) / TM, waves = (tiles + sm_count - 1) / sm_count;
+    return (double)n_out * per_channel[three ? 1 : 0][n_tok <= 8 ? 0 : n_tok <= 16 ? 1 : n_tok <= 32 ? 2 : 3] <= 600.0 * (double)waves;
+}
+
 bool encode_codes(EncodeTiledFn encode, CUtensorMap* map, const void* codes, int64_t rows, int row_bytes, int bits, int box_rows)
 {
     const cuuint64_t gdim[2] = {(cuuint64_t)row_bytes, (cuuint64_t)rows};
@@ -400,9 +414,8 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     gbs_device_guard guard;
     if (guard.enter(px->device) != cudaSuccess) { cudaGetLastError(); return GBS_ERR_CUDA; }
 
-    // up to 64 tokens the call is bound by reading the weights: no 128-token tile, the whole chip on the weight rows (crossover
-    // in gbs_qgemv.cu)
-    if (n_tokens <= GBS_QGEMV_MAX_TOKENS) {
+    // a few tokens are bound by latencies: no 128-channel tile, the whole chip on the weight rows
+    if (few_tokens(n_tokens, n_out, px->bits == 3 || pw->bits == 3, px->sm_count)) {
         const int e = gbs_qgemv(px, codes_x, scales_x, (int)n_tokens, pw, codes_w, scales_w, n_out, out, out_dtype, out_row_stride,
                                 static_cast<cudaStream_t>(cuda_stream));
         if (e != 0) cudaGetLastError();
@@ -422,13 +435,17 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     P.out_stride = out_row_stride;
     P.status = px->d_status;
     P.n = pick_tokens(n_tokens, n_out, P.kblocks, px->sm_count);
+    // Rows of a box beyond the tensor's end are slow to fill where no swizzle is set (16 of 32 rows of three-bit codes: 15.8 us instead
+    // of 12.2 at 14336 channels).  What shared memory holds beyond the box goes into sums that are not stored.  (A map of its own for
+    // the last of several token tiles costs other calls as much as it gains.)
+    P.xbox = n_tokens < P.n ? (int)n_tokens : P.n;
     P.m_tiles = (int)((n_out + TM - 1) / TM);
     const long long tiles = (long long)P.m_tiles * ((n_tokens + P.n - 1) / P.n);
     if (tiles > 0x7fffffff / 2) return GBS_ERR_INVALID_ARG;
     P.tiles = (int)tiles;
     CUtensorMap wmap, xmap;
     if (!encode_codes(encode, &wmap, codes_w, n_out, pw->d_pad * pw->bits / 8, pw->bits, TM) ||
-        !encode_codes(encode, &xmap, codes_x, n_tokens, px->d_pad * px->bits / 8, px->bits, P.n))
+        !encode_codes(encode, &xmap, codes_x, n_tokens, px->d_pad * px->bits / 8, px->bits, P.xbox))
         return GBS_ERR_CUDA;
     const bool wide = P.n > 128;
     const int smem = wide ? Shape<8>::SMEM : Shape<4>::SMEM;

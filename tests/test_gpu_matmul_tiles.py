@@ -24,6 +24,7 @@ def _codes(n, d, bits, seed):
 
 @pytest.mark.parametrize("d,n_tok,n_out", [
     (128, 1, 16), (128, 8, 17), (256, 9, 31), (1024, 17, 33), (1024, 33, 100), (1024, 64, 257),       # the few-token kernel
+    (128, 1, 18000), (256, 16, 9001), (128, 16, 18300), (256, 17, 11003), (256, 33, 4400), (128, 64, 6001),   # few tokens, many channels
     (128, 65, 1), (384, 65, 127), (1024, 96, 128), (640, 129, 129), (1024, 191, 1000),                # single SMs
     (512, 3000, 4090), (256, 4097, 5000), (128, 20000, 300), (384, 97, 40000),                        # enough tiles for pairs
 ])
