@@ -688,25 +688,25 @@ def extras(device, stream, args, peak, sampler=None):
             "us_per_launch": ms * 1e3, "tops": tops,
             "roofline": {"bound": "tensor", "unit": "TOP/s", "achieved": tops, "peak": i8_peak, "frac": tops / i8_peak,
                          "note": "int8 peak = 2 x the %s bf16 figure (nominal int8 : bf16 ratio); the kernel is bound by "
-                                 "unpacking the codes to int8, not by the tensor pipe" % bf16_kind}}
+                                 "the shared-memory port (packed codes in and out, int8 in and out), not by the tensor pipe" % bf16_kind}}
         del px, pw, cx, sx, cw, sw, outm
     ms = time_loop(lambda i: torch.matmul(xq, wq.t()), 8)
     out["bf16_matmul_of_the_unquantized_operands_4096x4096x4096"] = {"us_per_launch": ms * 1e3,
                                                                      "note": "library GEMM, context only"}
     del xq, wq
     torch.cuda.empty_cache()
-    # the full Paley order (width 1536 -> d' = m = 1544): the rotation is a dense contraction with H_m, forward in
-    # two sweeps (max|.|, then quantize: 2 x 2 m^2 flops per token), inverse in one (2 m d flops per token)
+    # the full Paley order (width 1536 -> d' = m = 1544): the rotation is a dense contraction with H_m, 2 m d flops per
+    # token forward as well as inverse
     pd = Plan(1536, 1544, 1544, 3, 0, 0.9)
     for n_d in (4096, 65536):
         xd = (torch.randn((n_d, 1536), generator=torch.Generator().manual_seed(11)) * 0.5).to(torch.bfloat16).to(device)
         od = pd.alloc_outputs(n_d, device)
         ms = time_loop(lambda i: pd.rotate_quantize(xd, out=od, stream=stream), 4)
-        tf = 2.0 * 2.0 * n_d * 1544.0 * 1544.0 / ms / 1e9
+        tf = 2.0 * n_d * 1544.0 * 1536.0 / ms / 1e9
         out["paley1544_b3_%d_rows" % n_d] = {
             "us_per_launch": ms * 1e3, "mrows_per_s": n_d / ms / 1e3, "kernel_family": pd.info.variant,
             "roofline": {"bound": "tensor", "unit": "TFLOP/s", "achieved": tf, "peak": bf16_tf, "frac": tf / bf16_tf,
-                         "note": "two dense sweeps with H_1544 per token; peak = the %s bf16 figure" % bf16_kind}}
+                         "note": "one dense contraction with H_1544 per token; peak = the %s bf16 figure" % bf16_kind}}
         if True:
             xh = torch.empty((n_d, 1536), dtype=torch.bfloat16, device=device)
             ms = time_loop(lambda i: pd.dequantize(od[0], od[1], inverse=True, out=xh, stream=stream), 4)
@@ -748,16 +748,15 @@ def extras(device, stream, args, peak, sampler=None):
     sm_mhz = (sampler.median_mhz_since(mark) if sampler else None) or 1965.0
     ms = statistics.median(layer_ms)
     evals = wc.n_rows * wc.d_pad * 32
-    alu_peak = 148 * 128 * sm_mhz * 1e6                   # fp32 lanes x sampled SM clock: lane-operations per second
     out["clip_error_K32"] = {"ms_per_layer_262144_tokens": ms, "ms_32_layers": sum(layer_ms),
                              "ms_per_layer_min_max": [min(layer_ms), max(layer_ms)],
                              "gevals_per_s": evals / ms / 1e6, "mtokens_per_s": wc.n_rows / ms / 1e3,
                              "hbm_gbs": wc.n_rows * wc.d * 2 / ms / 1e6,
-                             "roofline": {"bound": "alu", "unit": "Glane-op/s", "achieved": 5 * evals / ms / 1e6,
-                                          "peak": alu_peak / 1e9, "frac": 5 * evals / ms / 1e6 / (alu_peak / 1e9),
-                                          "sm_mhz_sampled": sm_mhz,
-                                          "note": "5 fp32 operations per value and candidate; peak = 148 SMs x 128 "
-                                                  "lanes x the SM clock sampled during these launches"}}
+                             "sm_mhz_sampled": sm_mhz,
+                             "roofline": {"bound": "hbm", "unit": "GB/s", "achieved": wc.n_rows * wc.d * 2 / ms / 1e6, "peak": peak,
+                                          "frac": wc.n_rows * wc.d * 2 / ms / 1e6 / peak,
+                                          "note": "one histogram per token scores all candidates; bound by the shared-memory "
+                                                  "port (table lookups and atomics)"}}
     # Algorithm 1's bracket search on the last layer's tensor (eps = 1/64): rounds of <= 31 probes, blocking
     out["search_clip_ratio_eps_1_64"] = {"alpha": res.alpha, "iterations": res.iterations, "rounds": res.rounds,
                                          "evaluations": res.evaluations, "wall_ms_per_layer_262144_tokens": dt * 1e3}
