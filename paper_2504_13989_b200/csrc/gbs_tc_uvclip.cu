@@ -14,13 +14,18 @@
 //   * Two shared-memory atomics per value (count, and the FMA's bits themselves: the exponent pattern is removed with the count)
 //     into COPIES interleaved histograms per token, so that a warp's lanes rarely meet: measured 2 cycles per 32 values with 32
 //     copies and 6 with 8, against 3 - 4 for the table lookup.  Everything is an integer: exact in any order.
-//   * After a token its 128 threads add the copies up, weigh them with M^2 in fp64 and clear them.  t's rounding (2^-23 M, without
-//     bias) is the only approximation.  The t^2 terms would cancel against the others; instead the error of candidate 0 is summed
-//     directly, as the per-candidate kernel does, and the histogram gives the differences from it.
-// What bounds it: the shared-memory port, 85 % busy: per token 1250 cycles (lookups 430, atomics 330, adding up and clearing
-// 390, the MMA's operands 130) against 820 issue slots per scheduler.
-// 32 768 x 4096, K = 32: 829 us with five fp32 operations per value and candidate; now 188 us at 3 bits (32 copies), 251 us at
-// 4 bits (16 copies); K = 8: 248 -> 165 us.  512 rows, K = 8: 19.2 -> 14.4 us.
+//   * After a token its 128 threads add the copies up, weigh them with M^2 in fp64 and clear them.  The t^2 term is the sum of the
+//     same integers' squares, in 64 bits, so the three parts of the error belong to one and the same t and may cancel down to the
+//     16 digits of fp64: a candidate that fits a batch exactly is as accurate as the others, wherever it stands in the list.
+//     t's rounding is the only approximation: at most 2^-23, so that an error E over n values moves by at most
+//     2^-22 M sqrt(n E) + n 2^-46 M^2 -- the size of Delta's rounding in the per-candidate kernel -- and, where the values differ,
+//     by the square root of n less.
+// What bounds it: the shared-memory port: per token about 430 cycles of lookups, 330 of atomics, 390 of adding up and clearing and
+// 130 of the MMA's operands.
+// 32 768 x 4096, K = 32: 829 us with five fp32 operations per value and candidate; now 171 us at 3 bits (32 copies), 250 us at
+// 4 bits (16 copies); K = 8: 249 -> 156 us, K = 1: 249 -> 155 (the per-candidate kernel takes eight at a time).  512 rows, K = 8:
+// 19.6 -> 13.3 us.  With the error of candidate 0 summed directly and the others as differences from it, which loses a
+// candidate whose error is far smaller (equal magnitudes, alpha = 1: negative sums), the first two were 189 and 252 us.
 #include <math.h>
 #include <string.h>
 
@@ -51,7 +56,7 @@ struct __align__(1024) Smem {
     unsigned hist[HIST_WORDS];
     unsigned lut[CELLS];
     unsigned red[TOK][2][4];                       // maxima, by tile parity
-    double direct[EPI_WARPS];
+    double square[EPI_WARPS];                      // sums of t^2
     unsigned long long full[STAGES], empty[STAGES], tfull[STAGES], tempty[STAGES];
     unsigned long long abar;
     unsigned tmem_base;
@@ -65,11 +70,10 @@ struct ClipParams {
     int K, levels, n_thr;
     float scale;                  // of t as an integer
     float norm2;                  // 1 / d'
-    float c_half0, c_delta0;      // candidate 0: 1 / (2 alpha), alpha / D
     const unsigned char* a_img;
     double* err_sum;
     int* status;
-    float delta[GBS_MAX_CANDIDATES];              // alpha_k / D
+    float alpha[GBS_MAX_CANDIDATES];
     unsigned thr[MAX_BINS];                       // sorted, different, one per cell at most
     unsigned short idx[GBS_MAX_CANDIDATES][7];    // threshold j of candidate k
 };
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     }
     if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     for (int i = threadIdx.x; i < HIST_WORDS / 4; i += THREADS) reinterpret_cast<uint4*>(S->hist)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (threadIdx.x < EPI_WARPS) S->direct[threadIdx.x] = 0.0;
+    if (threadIdx.x < EPI_WARPS) S->square[threadIdx.x] = 0.0;
     unsigned* thr = reinterpret_cast<unsigned*>(S->b[0]);          // the first loads come later
     for (int i = threadIdx.x; i < P.n_thr; i += THREADS) thr[i] = P.thr[i];
     __syncthreads();
@@ -189,8 +193,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         // (a predicated reduction becomes a branch: 264 us instead of 250)
         const unsigned hb = smem_u32(hist) + (unsigned)(lane % COPIES) * 4u - BIN_STEP;
         const unsigned lut = smem_u32(S->lut);
-        const float twoD = (float)(2 * P.levels), MAGIC = 8388608.f, mD = MAGIC + (float)P.levels;
-        double direct = 0.0;
+        constexpr float MAGIC = 8388608.f;
+        constexpr unsigned E = 0x4B000000u;                       // its bit pattern
+        double square = 0.0;
+        float poison = 0.f;                                       // NaN once a value was not finite
         for (int it = 0; it < n_mine; ++it) {
             const int s = it % STAGES;
             const bool ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull[s], (it / STAGES) & 1, P.status, 4, false));
@@ -213,9 +219,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
             mb = max(max(slot[0], slot[1]), max(slot[2], slot[3]));
             if (mb == POISON) break;
             const float M = __uint_as_float(mb);
-            const float rM = M > 0.f ? 1.f / M : 0.f;
-            const float sc = rM * P.scale, a1 = P.c_half0 * rM, dl = -P.c_delta0 * M;
-            float e0 = 0.f, e1 = 0.f;
+            float lift = 1.f;                                      // scale / M must not overflow
+            if (M < 0x1p-96f) {
+                lift = 0x1p64f;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * lift);
+            }
+            const float sc = M > 0.f ? P.scale / (M * lift) : 0.f;
+            // every one of the 32 values is a signed sum of all that came out of TMEM: the first shows whether one was not finite
+            poison = fmaf(__uint_as_float(r[0]), 0.f, poison);
+            unsigned long long sq = 0ull;                          // 32 squares below 2^44
             // eight values at a time: their lookups are in flight together
 #pragma unroll
             for (int i0 = 0; i0 < 32; i0 += 8) {
@@ -226,13 +239,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                     e[i] = ld_shared(lut + ((b[i] >> (CELL_BITS - 2)) & (unsigned)(4 * CELLS - 4)));
                 }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    // candidate 0, directly
-                    const float y = __uint_as_float(r[i0 + i]);
-                    const float w = __saturatef(fmaf(y, a1, 0.5f));
-                    const float err = fmaf(fmaf(w, twoD, MAGIC) - mD, dl, y);
-                    if (i & 1) e1 = fmaf(err, err, e1); else e0 = fmaf(err, err, e0);
-                }
+                for (int i = 0; i < 8; ++i) sq += (unsigned long long)(b[i] - E) * (b[i] - E);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const unsigned bin = (e[i] + (b[i] & ((1u << CELL_BITS) - 1u))) >> CELL_BITS;
@@ -241,9 +248,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                     asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(at), "r"(b[i]), "n"(SUM_OFF) : "memory");
                 }
             }
-            direct += (double)(e0 + e1);
             asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
             const double m2 = (double)M * (double)M;
+            square += m2 * (double)sq;
 #pragma unroll
             for (int i = 0; i < PER; ++i) {
                 const int bin = ti + 128 * i;
@@ -262,7 +269,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                         m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
                     }
                     // a component has at most 1024 values below 2^22: what is left without the exponent patterns fits 32 bits
-                    constexpr unsigned E = 0x4B000000u;
                     const double sum = (double)(m.x - c.x * E) + (double)(m.y - c.y * E) + (double)(m.z - c.z * E) + (double)(m.w - c.w * E);
                     w0[i] += m2 * (double)(c.x + c.y + c.z + c.w);
                     w1[i] += m2 * sum;
@@ -270,8 +276,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
             }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) direct += __shfl_xor_sync(0xffffffffu, direct, o);
-        if (lane == 0) S->direct[warp - 2] = direct;
+        for (int o = 16; o > 0; o >>= 1) square += __shfl_xor_sync(0xffffffffu, square, o);
+        if (__any_sync(0xffffffffu, poison != 0.f)) square = __longlong_as_double(0x7ff8000000000000ll);
+        if (lane == 0) S->square[warp - 2] = square;
     }
 
     // ---- the block's totals: [bin] over the four token slots, then from the last threshold down
@@ -317,22 +324,18 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         }
     }
     __syncthreads();
-    // error of candidate k without its t^2 part
-    auto part = [&](int k) -> double {
-        const double d = (double)P.delta[k];
-        double l1 = 0.0, l2 = 0.0;
+    if (threadIdx.x < P.K) {
+        const int k = threadIdx.x;
+        const double d = (double)P.alpha[k] / (double)P.levels, scale = (double)P.scale;
+        double t2 = 0.0, l1 = 0.0, l2 = 0.0;
+        for (int i = 0; i < EPI_WARPS; ++i) t2 += S->square[i];
         for (int j = 0; j < P.levels; ++j) {
             const int b = P.idx[k][j];
             l2 += (double)(2 * j + 1) * suf[b];
             l1 += suf[MAX_BINS + b];
         }
-        return d * d * l2 - 2.0 * d * (l1 / (double)P.scale);
-    };
-    if (threadIdx.x < P.K) {
-        double direct = 0.0;
-        for (int i = 0; i < EPI_WARPS; ++i) direct += S->direct[i];
-        const int k = threadIdx.x;
-        atomicAdd(&P.err_sum[k], (direct + (k ? part(k) - part(0) : 0.0)) * (double)P.norm2);
+        const double err = (t2 / scale - 2.0 * d * l1) / scale + d * d * l2;
+        atomicAdd(&P.err_sum[k], (err < 0.0 ? 0.0 : err) * (double)P.norm2);       // what fp64 leaves of an exact fit; NaN stays
     }
 }
 
@@ -369,7 +372,7 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
             P.thr[P.n_thr++] = at[c];
         }
     for (int k = 0; k < K; ++k) {
-        P.delta[k] = (float)((double)alphas[k] / (double)D);
+        P.alpha[k] = alphas[k];
         for (int j = 0; j < D; ++j)
             P.idx[k][j] = rank[(unsigned)ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale) >> CELL_BITS];
     }
@@ -389,8 +392,6 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
     P.K = K;
     P.levels = D;
     P.norm2 = (float)(1.0 / (double)p->d_pad);
-    P.c_half0 = (float)(1.0 / (2.0 * (double)alphas[0]));
-    P.c_delta0 = P.delta[0];
     P.a_img = p->d_aimg;
     P.err_sum = err_sum;
     P.status = p->d_status;
