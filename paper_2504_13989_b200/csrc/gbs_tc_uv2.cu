@@ -15,8 +15,10 @@
 //     (Sections 2.1, 3.1).
 // What bounds it: instruction issue, as for the narrower widths.  8192 rows, 4 bits, one scale per token: 8192 wide 46.8 us on
 // the three-sweep kernel, 42.5 here; 5120 wide 41.1 -> 34.8; 5120 wide, 3 bits, groups of 128: 44.1 -> 30.4.
-// Every wait is bounded; an expired wait records a code in the plan's status word, and a warp whose wait ran out brings a
-// pattern no maximum can have to the barrier it shares, so that all who wait there leave with it.
+// Every wait is bounded; an expired wait records a code in the plan's status word.  A warp whose wait ran out brings a pattern no
+// maximum can have to the barrier it shares, and all who meet it there leave their loop with it.  With one scale per token they go on
+// bringing it to the barriers of the tiles that are left: a warp that rested in this tile knows nothing of it yet and will wait for
+// them.  (The two warps of a group always have rows in the same tiles.)
 #include <string.h>
 
 #include <mutex>
@@ -176,7 +178,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv2(const __grid_constant__ C
         const int gl = 1 << P.glog;                // lanes per group
         const long long row_step = (long long)gridDim.x * TOK;
         long long row = (long long)blockIdx.x * TOK + t;
-        for (int it = 0; it < n_mine; ++it, row += row_step) {
+        int it = 0;
+        for (; it < n_mine; ++it, row += row_step) {
             const int s = it % STAGES;
             // A warp without rows in this tile has none in any tile of this stage (there are as many stages as quadrants), so it
             // takes part in every phase of the barriers it waits for.
@@ -253,6 +256,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv2(const __grid_constant__ C
                         yo[i] = make_float4(__uint_as_float(r[4 * i]) * P.norm, __uint_as_float(r[4 * i + 1]) * P.norm,
                                             __uint_as_float(r[4 * i + 2]) * P.norm, __uint_as_float(r[4 * i + 3]) * P.norm);
                 }
+            }
+        }
+        if (!GROUPED) {
+            // after an expired wait: the barriers of the tiles that are left
+            for (++it; it < n_mine; ++it) {
+                const int s = it % STAGES, slab = rotate ? (q - it) & 3 : q;
+                if (slab >= P.slabs) continue;
+                if (lane == 0) S->red.tok[s][t][slab * 2 + half] = POISON;
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + t * STAGES + s), "r"(64 * P.slabs) : "memory");
             }
         }
     }
