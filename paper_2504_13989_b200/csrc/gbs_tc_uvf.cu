@@ -14,8 +14,9 @@
 //     (Sections 2.1, 3.1) from registers.
 // What bounds it: latency.  A warp issues about 700 instructions per 32 values of a lane (220 of them the split) at 8 cycles
 // each, sixteen warps cover half of that, and taking out any one part (two of three planes, the split, the epilogue) gains
-// less than a tenth.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 19.0 now; 7000 x 3584, groups of 128: 117.6 ->
-// 32.6.  Tried and slower: loads reissued piece by piece inside the split; tiles prefetched into L2 further ahead.
+// less than a tenth.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 16.6 now; 7000 x 3584, groups of 128: 117.6 ->
+// 27.7; 7000 x 8192, 4 bits: 61.7.  Tried and slower: loads reissued piece by piece inside the split; tiles prefetched into L2
+// further ahead; the prefetches in a warp of their own that waits for the splits (18.2, 31.4 and 73.3 us).
 // Every wait is bounded; an expired wait records a code in the plan's status word, and a warp whose wait ran out brings a
 // pattern no maximum can have to the barrier it shares, so that all who wait there leave with it.
 #include <string.h>
@@ -36,7 +37,7 @@ constexpr int A_BYTES = UMAX * UMAX * 2;
 constexpr int PLANE_BYTES = UMAX * NCOLS * 2;     // one bf16 plane of a tile at U = 128
 constexpr int STAGE_BYTES = 3 * PLANE_BYTES;      // lo, mid, hi
 constexpr int EPI_WARPS = 16;
-constexpr int THREADS = 32 * (2 + EPI_WARPS);
+constexpr int THREADS = 32 * (1 + EPI_WARPS);
 constexpr unsigned POISON = 0xffffffffu;          // no maximum of absolute values has the sign bit set
 
 struct __align__(1024) Smem {
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
         mbar_arrive_expect_tx(&S->abar, A_BYTES);
         bulk_load(S->a, P.a_img, A_BYTES, &S->abar);          // plan-owned, immutable: needs no ordering
     }
-    if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
+    if (warp == 0) tmem_alloc(&S->tmem_base, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -137,21 +138,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
     const int n_mine = (P.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
 
     if (warp == 0) {
-        // ------------------------------ L2 prefetch ------------------------------
-        // the registers hold one tile ahead, for part of a tile's time; DRAM wants more in flight.  Paced by the splits: one
-        // tile beyond the loads (82.8 -> 70.7 us for 7000 x 8192); further ahead queues in front of other blocks' loads.
-        if (lane < TOK) {
-            auto prefetch = [&](int n) {
-                const long long row = ((long long)blockIdx.x + (long long)n * gridDim.x) * TOK + lane;
-                if (n < n_mine && row < P.n_rows)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.x + row * P.stride), "r"(P.d * 4) : "memory");
-            };
-            for (int n = 0; n + 2 < n_mine; ++n) {
-                if (!mbar_wait(&S->abort_flag, &S->full[n % STAGES], (unsigned)(n / STAGES) & 1u, P.status, 5)) break;
-                prefetch(n + 2);
-            }
-        }
-    } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         {
             constexpr unsigned IDESC = instr_desc(UMAX, NCOLS);
@@ -183,10 +169,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
                 umma_commit(&S->tfull[c]);
             }
         }
-    } else if (warp >= 2) {
+    } else {
         // ------------------------------ split + epilogue ------------------------------
         const int q = warp & 3;                                    // TMEM lane quadrant this warp may access
-        const int w = (warp - 2) >> 2;
+        const int w = (warp - 1) >> 2;
         const int t = w / HALVES, half = w % HALVES;               // token slot of its tiles, half of the V outputs
         const int up = q * 32 + lane;                              // output row u' it reads
         const int wt = q * HALVES + half;                          // its place among the token's warps
@@ -216,6 +202,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
                 for (int j = 0; j < 8; ++j)
                     x[j] = (in && e0 + 128 * j < P.d) ? __ldg(reinterpret_cast<const uint4*>(src + 128 * j)) : make_uint4(0u, 0u, 0u, 0u);
             }
+        };
+        // The registers hold one tile ahead, for part of a tile's time; DRAM wants more in flight.  Paced by the splits, one tile
+        // beyond the loads, by a token's first warp (82.8 -> 70.7 us for 7000 x 8192); further ahead queues in front of other
+        // blocks' loads.
+        const bool prefetches = wt == 0 && lane == 0;
+        auto prefetch = [&](int n) {
+            const long long row = row_first + (long long)n * row_step;
+            if (prefetches && n < n_mine && row < P.n_rows)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.x + row * P.stride), "r"(P.d * 4) : "memory");
         };
         auto split_tile = [&](int n) -> bool {
             const int s = n % STAGES;
@@ -247,11 +242,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
         fetch(0);
         bool alive = split_tile(0);
         fetch(1);
+        prefetch(2);
         long long row = row_first;
         for (int n = 0; n < n_mine; ++n, row += row_step) {
             if (alive && n + 1 < n_mine) {
                 alive = split_tile(n + 1);
                 fetch(n + 2);
+                prefetch(n + 3);
             }
             const int c = n % ACCS;
             if (alive) alive = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull[c], (unsigned)(n / ACCS) & 1u, P.status, 4));
@@ -330,7 +327,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
     // ---- teardown: every role leaves its loop (normally or after a wait expired), then TMEM is freed
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);
     }
