@@ -5,13 +5,13 @@ PyTorch is used for device memory and streams.  There is no CPU fallback: if the
 library is missing or a call fails, a GbsError is raised.
 
 Plan's per-call methods go through _native.so (csrc/gbs_torch.cpp), which does the regular call's checks,
-allocations and marshalling in C; every other call takes the functions below.
+allocations and marshalling in C; every other call takes the functions below.  When it is loaded, with the first
+plan of a process, its method objects take the place of those methods in the class.
 """
 from __future__ import annotations
 
 import ctypes
 import os
-import weakref
 
 import torch
 
@@ -142,6 +142,9 @@ def native():
             from . import _native
         except ImportError as e:
             raise GbsErrorMissing("_native.so does not load (%s) -- run `python -m paper_2504_13989_b200.build`" % e) from e
+        for name, f in _PYTHON_METHODS.items():
+            if Plan.__dict__.get(name) is f:                      # a method that was replaced stays
+                setattr(Plan, name, _native.method(name, f, Plan.alloc_outputs if name == "rotate_quantize" else None))
         _native_module = _native
     return _native_module
 
@@ -417,14 +420,10 @@ class Plan:
     def __init__(self, d: int, d_pad: int | None = None, m: int = 1, bits: int = 4, group: int = 0,
                  alpha: float = 1.0, asymmetric: bool = False):
         d_pad = d if d_pad is None else d_pad
-        self._native = native()
+        calls = native().Calls
         self.handle = gbs_plan_create_ex(d, d_pad, m, bits, group, alpha, GBS_PLAN_ASYMMETRIC if asymmetric else 0)
         self.info = gbs_plan_info(self.handle)
-        # the regular per-call path, without a Python frame; it passes what it does not handle to the methods below
-        self._calls = self._native.Calls(self.handle, weakref.ref(self))
-        for name in ("rotate_quantize", "dequantize", "quantized_matmul", "clip_error"):
-            if getattr(type(self), name) is getattr(Plan, name):          # a subclass's own method stays
-                self.__dict__[name] = getattr(self._calls, name)
+        self._calls = calls(self.handle)                           # what the native methods know of this plan
 
     def close(self):
         if getattr(self, "handle", None):
@@ -454,9 +453,6 @@ class Plan:
         return codes, scales, y
 
     def rotate_quantize(self, x: torch.Tensor, want_y: bool = False, out=None, stream=None):
-        done = self._native.rotate_quantize(self.handle, x, want_y, out, stream)
-        if done is not None:
-            return done
         n_rows = x.numel() // self.info.d
         codes, scales, y = out if out is not None else self.alloc_outputs(n_rows, x.device, want_y)
         gbs_rotate_quantize(self.handle, x, codes, scales, y, stream)
@@ -464,9 +460,6 @@ class Plan:
 
     def dequantize(self, codes: torch.Tensor, scales: torch.Tensor, inverse: bool = False,
                    dtype=torch.float32, out=None, stream=None) -> torch.Tensor:
-        done = self._native.dequantize(self.handle, codes, scales, inverse, dtype, out, stream)
-        if done is not None:
-            return done
         n_rows = codes.shape[0]
         width = self.info.d if inverse else self.info.d_pad
         if out is None:
@@ -475,10 +468,6 @@ class Plan:
         return out
 
     def clip_error(self, x: torch.Tensor, alphas, want_rows: bool = False, err_sum=None, stream=None):
-        if err_sum is None and not want_rows:
-            done = self._native.clip_error(self.handle, x, alphas, stream)
-            if done is not None:
-                return done
         n_rows = x.numel() // self.info.d
         K = len(alphas)
         if err_sum is None:
@@ -497,9 +486,6 @@ class Plan:
     def quantized_matmul(self, codes_x, scales_x, plan_w: "Plan", codes_w, scales_w, dtype=torch.float32, out=None,
                          stream=None) -> torch.Tensor:
         """The layer's output from the packed codes of activations (this plan) and weights (plan_w)."""
-        done = self._native.quantized_matmul(self.handle, codes_x, scales_x, plan_w.handle, codes_w, scales_w, dtype, out, stream)
-        if done is not None:
-            return done
         if out is None:
             out = torch.empty((codes_x.shape[0], codes_w.shape[0]), dtype=dtype, device=codes_x.device)
         gbs_quantized_matmul(self.handle, codes_x, scales_x, plan_w.handle, codes_w, scales_w, out, stream)
@@ -523,6 +509,10 @@ class Plan:
             scales_host.copy_(scales, non_blocking=True)
         s.synchronize()
         return codes_host, scales_host
+
+
+# the methods that _native.so has a regular call for
+_PYTHON_METHODS = {name: Plan.__dict__[name] for name in ("rotate_quantize", "dequantize", "quantized_matmul", "clip_error")}
 
 
 class HostPipeline:

@@ -9,9 +9,11 @@
 // device, a shape or stride that needs a view, an output that is too small, a non-zero status): that call then takes
 // the Python path, which raises the error or makes the view.  Nothing is enqueued before the checks have passed.
 //
-// Two ways in: the module's functions, which take the plan's handle, and a Calls object per plan, whose methods stand in the
-// plan's instance dictionary under the names of Plan's methods.  The second saves the Python frame around each call (0.9 of
-// 5.3 us for 16 rows); what it does not handle it passes to the method of the class.
+// Two ways in: the module's functions, for a caller that has the plan's handle alone, and method objects that stand in the class
+// under the names of Plan's methods, over the Python functions they were.  A method object binds like a function, so that a
+// bound method keeps its plan, a subclass may override it and a class attribute may be replaced; it finds the plan's handle in the
+// Calls object of the instance.  It saves the Python frame around each call (0.9 of 5.3 us for 16 rows); what it does not handle it
+// passes to the function it wraps.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -19,6 +21,8 @@
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
 #include <cuda_runtime_api.h>
+#include <stddef.h>
+#include <string.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -299,30 +303,28 @@ PyObject* with_handle(PyObject*, PyObject* const* a, Py_ssize_t n)
     return F(ref, a);
 }
 
-// ---- Calls(handle, weak reference to the plan object)
+// ---- Calls(handle): the plan's handle and sizes for the methods below, until clear()
 struct Calls {
     PyObject_HEAD
     PlanRef ref;              // ref.plan is null once the plan is closed
-    PyObject* owner;
 };
+PyTypeObject* calls_type = nullptr;
 
 int calls_init(PyObject* self, PyObject* args, PyObject*)
 {
     Calls* c = reinterpret_cast<Calls*>(self);
-    PyObject *handle, *owner;
-    if (!PyArg_ParseTuple(args, "OO", &handle, &owner)) return -1;
+    PyObject *handle, *unused;
+    if (!PyArg_ParseTuple(args, "O|O", &handle, &unused)) return -1;
     if (!plan_of(handle, &c->ref.plan, &c->ref.info)) {
         c->ref.plan = nullptr;
         PyErr_SetString(PyExc_ValueError, "gbs: not a plan handle");
         return -1;
     }
-    Py_XSETREF(c->owner, Py_NewRef(owner));
     return 0;
 }
 void calls_dealloc(PyObject* self)
 {
     PyTypeObject* type = Py_TYPE(self);
-    Py_XDECREF(reinterpret_cast<Calls*>(self)->owner);
     type->tp_free(self);
     Py_DECREF(type);
 }
@@ -339,54 +341,6 @@ struct Method {
     const char* args[8];
     PyObject* (*call)(const PlanRef&, PyObject* const* given);
 };
-
-// the plan object's own method, for what the C function does not handle
-PyObject* by_class(Calls* c, const Method& m, PyObject* const* args, Py_ssize_t n, PyObject* kwnames)
-{
-    PyObject* owner = PyObject_CallNoArgs(c->owner);
-    if (!owner) return nullptr;
-    PyObject* f = PyObject_GetAttrString(reinterpret_cast<PyObject*>(Py_TYPE(owner)), m.name);
-    PyObject* out = nullptr;
-    if (f) {
-        const Py_ssize_t all = n + (kwnames ? PyTuple_GET_SIZE(kwnames) : 0);
-        PyObject** v = static_cast<PyObject**>(PyMem_Malloc(sizeof(PyObject*) * (all + 1)));
-        if (v) {
-            v[0] = owner;
-            for (Py_ssize_t i = 0; i < all; ++i) v[i + 1] = args[i];
-            out = PyObject_Vectorcall(f, v, n + 1, kwnames);
-            PyMem_Free(v);
-        } else {
-            PyErr_NoMemory();
-        }
-        Py_DECREF(f);
-    }
-    Py_DECREF(owner);
-    return out;
-}
-
-template <const Method& M>
-PyObject* method(PyObject* self, PyObject* const* args, Py_ssize_t n, PyObject* kwnames)
-{
-    Calls* c = reinterpret_cast<Calls*>(self);
-    PyObject* given[8] = {nullptr};
-    bool regular = c->ref.plan && n <= M.count;
-    for (Py_ssize_t i = 0; regular && i < n; ++i) given[i] = args[i];
-    const Py_ssize_t nk = kwnames ? PyTuple_GET_SIZE(kwnames) : 0;
-    for (Py_ssize_t k = 0; regular && k < nk; ++k) {
-        int at = -1;
-        for (int i = 0; i < M.count && at < 0; ++i)
-            if (PyUnicode_CompareWithASCIIString(PyTuple_GET_ITEM(kwnames, k), M.args[i]) == 0) at = i;
-        regular = at >= 0 && !given[at];
-        if (regular) given[at] = args[n + k];
-    }
-    for (int i = 0; regular && i < M.required; ++i) regular = given[i] != nullptr;
-    if (regular) {
-        PyObject* out = M.call(c->ref, given);
-        if (out != Py_None) return out;
-        Py_DECREF(out);
-    }
-    return by_class(c, M, args, n, kwnames);
-}
 
 PyObject* or_none(PyObject* o) { return o ? o : Py_None; }
 
@@ -413,22 +367,132 @@ constexpr Method CLIP = {"clip_error", 5, 2, {"x", "alphas", "want_rows", "err_s
     return do_clip_error(r, a);
 }};
 
+// ---- method(name, function, alloc_outputs): a function of Plan with the regular call in front of it
+struct MethodObject {
+    PyObject_HEAD
+    vectorcallfunc vectorcall;
+    const Method* method;
+    PyObject* wrapped;
+    PyObject* alloc;          // Plan.alloc_outputs, or null where the call allocates without it
+};
+PyObject *name_calls = nullptr, *name_alloc = nullptr;
+
+// whether the plan's outputs come from Plan's own alloc_outputs (a subclass or an instance may have another)
+bool own_alloc(PyObject* plan, PyObject* alloc)
+{
+    PyObject* f = PyObject_GetAttr(plan, name_alloc);
+    if (!f) { PyErr_Clear(); return false; }
+    const bool own = PyMethod_Check(f) && PyMethod_GET_FUNCTION(f) == alloc;
+    Py_DECREF(f);
+    return own;
+}
+
+PyObject* method_call(PyObject* self, PyObject* const* args, size_t nargsf, PyObject* kwnames)
+{
+    const MethodObject* o = reinterpret_cast<MethodObject*>(self);
+    const Method& M = *o->method;
+    const Py_ssize_t n = PyVectorcall_NARGS(nargsf) - 1, nk = kwnames ? PyTuple_GET_SIZE(kwnames) : 0;
+    PyObject* calls = n >= 0 ? PyObject_GetAttr(args[0], name_calls) : nullptr;
+    if (!calls) PyErr_Clear();
+    PyObject* given[8] = {nullptr};
+    bool regular = calls && Py_TYPE(calls) == calls_type && reinterpret_cast<Calls*>(calls)->ref.plan && n <= M.count;
+    for (Py_ssize_t i = 0; regular && i < n; ++i) given[i] = args[1 + i];
+    for (Py_ssize_t k = 0; regular && k < nk; ++k) {
+        int at = -1;
+        for (int i = 0; i < M.count && at < 0; ++i)
+            if (PyUnicode_CompareWithASCIIString(PyTuple_GET_ITEM(kwnames, k), M.args[i]) == 0) at = i;
+        regular = at >= 0 && !given[at];
+        if (regular) given[at] = args[1 + n + k];
+    }
+    for (int i = 0; regular && i < M.required; ++i) regular = given[i] != nullptr;
+    if (regular && o->alloc) regular = own_alloc(args[0], o->alloc);
+    PyObject* out = nullptr;
+    if (regular) {
+        const PlanRef ref = reinterpret_cast<Calls*>(calls)->ref;      // the caller's argument keeps the plan
+        out = M.call(ref, given);
+        if (out == Py_None) { Py_DECREF(out); regular = false; }
+    }
+    Py_XDECREF(calls);
+    return regular ? out : PyObject_Vectorcall(o->wrapped, args, nargsf, kwnames);
+}
+
+
+PyObject* method_get(PyObject* self, PyObject* obj, PyObject*) { return obj ? PyMethod_New(self, obj) : Py_NewRef(self); }
+// name, documentation, signature, module: the wrapped function's
+PyObject* method_getattro(PyObject* self, PyObject* name)
+{
+    PyObject* wrapped = reinterpret_cast<MethodObject*>(self)->wrapped;
+    if (PyUnicode_CompareWithASCIIString(name, "__wrapped__") == 0) return Py_NewRef(wrapped);
+    if (PyUnicode_CompareWithASCIIString(name, "__class__") == 0 || PyUnicode_CompareWithASCIIString(name, "__call__") == 0)
+        return PyObject_GenericGetAttr(self, name);
+    return PyObject_GetAttr(wrapped, name);
+}
+int method_traverse(PyObject* self, visitproc visit, void* arg)
+{
+    MethodObject* o = reinterpret_cast<MethodObject*>(self);
+    Py_VISIT(Py_TYPE(self));
+    Py_VISIT(o->wrapped);
+    Py_VISIT(o->alloc);
+    return 0;
+}
+int method_clear(PyObject* self)
+{
+    MethodObject* o = reinterpret_cast<MethodObject*>(self);
+    Py_CLEAR(o->wrapped);
+    Py_CLEAR(o->alloc);
+    return 0;
+}
+void method_dealloc(PyObject* self)
+{
+    PyTypeObject* type = Py_TYPE(self);
+    PyObject_GC_UnTrack(self);
+    method_clear(self);
+    type->tp_free(self);
+    Py_DECREF(type);
+}
+PyTypeObject* method_type = nullptr;
+const Method* const METHODS[] = {&ROTATE, &DEQUANTIZE, &MATMUL, &CLIP};
+
+PyObject* make_method(PyObject*, PyObject* args)
+{
+    const char* name;
+    PyObject *wrapped, *alloc;
+    if (!PyArg_ParseTuple(args, "sOO", &name, &wrapped, &alloc)) return nullptr;
+    const Method* m = nullptr;
+    for (const Method* c : METHODS)
+        if (strcmp(name, c->name) == 0) m = c;
+    if (!m) { PyErr_Format(PyExc_ValueError, "gbs: no native method '%s'", name); return nullptr; }
+    MethodObject* o = reinterpret_cast<MethodObject*>(method_type->tp_alloc(method_type, 0));
+    if (!o) return nullptr;
+    o->vectorcall = method_call;
+    o->method = m;
+    o->wrapped = Py_NewRef(wrapped);
+    o->alloc = alloc == Py_None ? nullptr : Py_NewRef(alloc);
+    return reinterpret_cast<PyObject*>(o);
+}
+
 template <class F> PyCFunction cfunc(F f) { return reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(f)); }
 
-PyMethodDef calls_methods[] = {{ROTATE.name, cfunc(method<ROTATE>), METH_FASTCALL | METH_KEYWORDS, nullptr},
-                               {DEQUANTIZE.name, cfunc(method<DEQUANTIZE>), METH_FASTCALL | METH_KEYWORDS, nullptr},
-                               {MATMUL.name, cfunc(method<MATMUL>), METH_FASTCALL | METH_KEYWORDS, nullptr},
-                               {CLIP.name, cfunc(method<CLIP>), METH_FASTCALL | METH_KEYWORDS, nullptr},
-                               {"clear", calls_clear, METH_NOARGS, nullptr},
-                               {nullptr, nullptr, 0, nullptr}};
+PyMethodDef calls_methods[] = {{"clear", calls_clear, METH_NOARGS, nullptr}, {nullptr, nullptr, 0, nullptr}};
 PyType_Slot calls_slots[] = {{Py_tp_init, reinterpret_cast<void*>(calls_init)}, {Py_tp_dealloc, reinterpret_cast<void*>(calls_dealloc)},
                              {Py_tp_new, reinterpret_cast<void*>(PyType_GenericNew)}, {Py_tp_methods, calls_methods}, {0, nullptr}};
 PyType_Spec calls_spec = {"paper_2504_13989_b200._native.Calls", sizeof(Calls), 0, Py_TPFLAGS_DEFAULT, calls_slots};
+
+PyMemberDef method_members[] = {{"__vectorcalloffset__", Py_T_PYSSIZET, offsetof(MethodObject, vectorcall), Py_READONLY, nullptr},
+                                {nullptr, 0, 0, 0, nullptr}};
+PyType_Slot method_slots[] = {{Py_tp_dealloc, reinterpret_cast<void*>(method_dealloc)}, {Py_tp_traverse, reinterpret_cast<void*>(method_traverse)},
+                              {Py_tp_clear, reinterpret_cast<void*>(method_clear)}, {Py_tp_call, reinterpret_cast<void*>(PyVectorcall_Call)},
+                              {Py_tp_descr_get, reinterpret_cast<void*>(method_get)}, {Py_tp_getattro, reinterpret_cast<void*>(method_getattro)},
+                              {Py_tp_members, method_members}, {0, nullptr}};
+PyType_Spec method_spec = {"paper_2504_13989_b200._native.Method", sizeof(MethodObject), 0,
+                           Py_TPFLAGS_DEFAULT | Py_TPFLAGS_HAVE_GC | Py_TPFLAGS_HAVE_VECTORCALL | Py_TPFLAGS_METHOD_DESCRIPTOR |
+                               Py_TPFLAGS_DISALLOW_INSTANTIATION, method_slots};
 
 PyMethodDef methods[] = {{ROTATE.name, cfunc(with_handle<do_rotate_quantize, 5>), METH_FASTCALL, nullptr},
                          {DEQUANTIZE.name, cfunc(with_handle<do_dequantize, 7>), METH_FASTCALL, nullptr},
                          {MATMUL.name, cfunc(with_handle<do_quantized_matmul, 9>), METH_FASTCALL, nullptr},
                          {CLIP.name, cfunc(with_handle<do_clip_error, 4>), METH_FASTCALL, nullptr},
+                         {"method", make_method, METH_VARARGS, nullptr},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
@@ -436,13 +500,15 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 PyMODINIT_FUNC PyInit__native(void)
 {
+    name_calls = PyUnicode_InternFromString("_calls");
+    name_alloc = PyUnicode_InternFromString("alloc_outputs");
+    calls_type = reinterpret_cast<PyTypeObject*>(PyType_FromSpec(&calls_spec));
+    method_type = reinterpret_cast<PyTypeObject*>(PyType_FromSpec(&method_spec));
     PyObject* m = PyModule_Create(&module);
-    PyObject* type = m ? PyType_FromSpec(&calls_spec) : nullptr;
-    if (!type || PyModule_AddObjectRef(m, "Calls", type) < 0) {
-        Py_XDECREF(type);
+    if (!name_calls || !name_alloc || !calls_type || !method_type || !m ||
+        PyModule_AddObjectRef(m, "Calls", reinterpret_cast<PyObject*>(calls_type)) < 0) {
         Py_XDECREF(m);
         return nullptr;
     }
-    Py_DECREF(type);
     return m;
 }

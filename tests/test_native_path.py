@@ -102,3 +102,85 @@ def test_methods_take_arguments_as_plan_declares_them():
             return "mine"
     with Mine(4096) as plan:
         assert plan.rotate_quantize(x) == "mine" and plan.dequantize(codes, scales).shape == (700, 4096)
+
+
+def test_native_methods_bind_like_functions():
+    """The method objects over Plan's functions: they bind to whatever object they are looked up on, keep it alive, show the
+    function's name and signature, and hand on what is not a regular call -- here on a stand-in without a plan."""
+    import functools
+    import gc
+    import inspect
+    import weakref
+    gbs_build.build()
+    nat = binding.native()
+    for name, f in binding._PYTHON_METHODS.items():
+        m = Plan.__dict__[name]
+        assert type(m).__name__ == "Method" and m.__wrapped__ is f and m.__name__ == name
+        assert inspect.signature(getattr(Plan, name)) == inspect.signature(f) and m.__doc__ == f.__doc__
+
+    class Other:
+        clip_error = nat.method("clip_error", lambda self, x, alphas, want_rows=False: (self, x, alphas, want_rows), None)
+
+    class Derived(Other):
+        def clip_error(self, x, alphas):
+            return super().clip_error(x, alphas=alphas, want_rows=True)
+
+    o, d = Other(), Derived()
+    assert o.clip_error(1, 2) == (o, 1, 2, False) and d.clip_error(1, 2) == (d, 1, 2, True) and Other.clip_error(o, 1, 2)[0] is o
+    with pytest.raises(TypeError):
+        o.clip_error(1)
+    kept, ref = functools.partial(o.clip_error, 1), weakref.ref(o)
+    del o
+    gc.collect()
+    assert ref() is not None and kept(2)[0] is ref()                          # a bound method owns its object
+    del kept
+    gc.collect()
+    assert ref() is None
+    with pytest.raises(ValueError):
+        nat.method("close", None, None)
+
+
+@pytest.mark.gpu
+def test_a_method_outlives_the_name_of_its_plan():
+    import functools
+    import gc
+    gbs_build.build()
+    x = synth.make_host("llama4096", 3).to(DEV)
+    with Plan(4096, bits=4, alpha=0.9) as plan:
+        codes, scales, _ = plan.rotate_quantize(x)
+        rows = plan.dequantize(codes, scales, inverse=True)
+        mm = plan.quantized_matmul(codes, scales, plan, codes, scales)
+        err = plan.clip_error(x, [0.5, 1.0])
+    assert torch.equal(Plan(4096, bits=4, alpha=0.9).rotate_quantize(x)[0], codes)
+    quantize, restore = Plan(4096, bits=4, alpha=0.9).rotate_quantize, functools.partial(Plan(4096, bits=4).dequantize, inverse=True)
+    multiply, score = Plan(4096, bits=4).quantized_matmul, Plan(4096, bits=4).clip_error
+    gc.collect()
+    assert torch.equal(quantize(x)[0], codes) and torch.equal(restore(codes, scales), rows)
+    assert torch.equal(multiply(codes, scales, Plan(4096, bits=4), codes, scales), mm)
+    assert torch.allclose(score(x, [0.5, 1.0]), err, rtol=1e-12)
+
+
+@pytest.mark.gpu
+def test_a_method_replaced_on_the_class_reaches_plans_that_exist(monkeypatch):
+    gbs_build.build()
+    x = synth.make_host("llama4096", 3).to(DEV)
+    with Plan(4096) as plan:
+        original = Plan.rotate_quantize
+        calls = []
+        monkeypatch.setattr(Plan, "rotate_quantize", lambda self, *a, **k: calls.append(self) or original(self, *a, **k))
+        codes, scales, _ = plan.rotate_quantize(x)
+        assert calls == [plan] and codes.shape == (3, 2048)
+        monkeypatch.undo()
+        plan.rotate_quantize(x)
+        assert calls == [plan]
+        # outputs come from the plan's alloc_outputs, whoever replaced it
+        pool = plan.alloc_outputs(3, DEV)
+        plan.alloc_outputs = lambda n_rows, device, want_y=False: pool
+        got = plan.rotate_quantize(x)
+        assert got[0] is pool[0] and got[1] is pool[1] and torch.equal(got[0], codes)
+
+    class Pooled(Plan):
+        def alloc_outputs(self, n_rows, device, want_y=False):
+            return pool
+    with Pooled(4096) as plan:
+        assert plan.rotate_quantize(x)[0] is pool[0]
