@@ -117,6 +117,8 @@ void empty_pair(int64_t r, int64_t cb, int64_t cs, const at::Device& device, at:
     codes->unsafeGetTensorImpl()->set_sizes_contiguous({r, cb});
 }
 
+// A C++ exception (an allocation that fails, a tensor without memory of its own) makes the call an irregular one.  Whatever can throw
+// stands before the GIL is released: a tensor's pointer, in particular, is asked for before.
 #define GBS_BEGIN try {
 #define GBS_END } catch (...) { PyErr_Clear(); } Py_RETURN_NONE;
 
@@ -142,10 +144,10 @@ PyObject* do_rotate_quantize(const PlanRef& ref, PyObject* const* a)
             !buffer_ok(scales, device, rows * info.scale_floats_per_row) || scales->scalar_type() != at::kFloat ||
             (oy != Py_None && (!buffer_ok(y, device, rows * info.d_pad) || y->scalar_type() != at::kFloat)))
             Py_RETURN_NONE;
+        void *xp = x->data_ptr(), *cp = codes->data_ptr(), *sp = scales->data_ptr(), *yp = y ? y->data_ptr() : nullptr;
         int rc;
         Py_BEGIN_ALLOW_THREADS
-        rc = gbs_rotate_quantize(plan, x->data_ptr(), dt, rows, stride, codes->data_ptr(), static_cast<float*>(scales->data_ptr()),
-                                 y ? static_cast<float*>(y->data_ptr()) : nullptr, stream);
+        rc = gbs_rotate_quantize(plan, xp, dt, rows, stride, cp, static_cast<float*>(sp), static_cast<float*>(yp), stream);
         Py_END_ALLOW_THREADS
         if (rc != GBS_OK) Py_RETURN_NONE;
         Py_INCREF(a[3]);
@@ -156,10 +158,10 @@ PyObject* do_rotate_quantize(const PlanRef& ref, PyObject* const* a)
     at::Tensor codes, scales, y;
     empty_pair(rows, info.code_bytes_per_row, info.scale_floats_per_row, device, &codes, &scales);
     if (want_y) y = empty2(rows, info.d_pad, at::kFloat, device);
+    void *xp = x->data_ptr(), *cp = codes.data_ptr(), *sp = scales.data_ptr(), *yp = want_y ? y.data_ptr() : nullptr;
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = gbs_rotate_quantize(plan, x->data_ptr(), dt, rows, stride, codes.data_ptr(), static_cast<float*>(scales.data_ptr()),
-                             want_y ? static_cast<float*>(y.data_ptr()) : nullptr, stream);
+    rc = gbs_rotate_quantize(plan, xp, dt, rows, stride, cp, static_cast<float*>(sp), static_cast<float*>(yp), stream);
     Py_END_ALLOW_THREADS
     if (rc != GBS_OK) Py_RETURN_NONE;
     PyObject* out = PyTuple_New(3);
@@ -209,10 +211,10 @@ PyObject* do_dequantize(const PlanRef& ref, PyObject* const* a)
     at::Tensor out;
     int dt;
     if (!output_of(a[5], a[4], rows, inverse ? info.d : info.d_pad, device, &out, &dt)) Py_RETURN_NONE;
+    void *cp = codes->data_ptr(), *sp = scales->data_ptr(), *op = out.data_ptr();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = gbs_dequantize(plan, codes->data_ptr(), static_cast<const float*>(scales->data_ptr()), rows, out.data_ptr(), dt,
-                        inverse ? GBS_INVERSE_ROTATE : 0, stream);
+    rc = gbs_dequantize(plan, cp, static_cast<const float*>(sp), rows, op, dt, inverse ? GBS_INVERSE_ROTATE : 0, stream);
     Py_END_ALLOW_THREADS
     if (rc != GBS_OK) Py_RETURN_NONE;
     if (a[5] != Py_None) return Py_NewRef(a[5]);
@@ -246,10 +248,11 @@ PyObject* do_quantized_matmul(const PlanRef& ref, PyObject* const* a)
         if (!t || t->dim() != 2 || t->size(0) != n_tok || t->size(1) != n_out) Py_RETURN_NONE;
     }
     if (!output_of(a[7], a[6], n_tok, n_out, device, &out, &dt)) Py_RETURN_NONE;
+    void *cxp = cx->data_ptr(), *sxp = sx->data_ptr(), *cwp = cw->data_ptr(), *swp = sw->data_ptr(), *op = out.data_ptr();
     int rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = gbs_quantized_matmul(px, cx->data_ptr(), static_cast<const float*>(sx->data_ptr()), n_tok, pw, cw->data_ptr(),
-                              static_cast<const float*>(sw->data_ptr()), n_out, out.data_ptr(), dt, n_out, stream);
+    rc = gbs_quantized_matmul(px, cxp, static_cast<const float*>(sxp), n_tok, pw, cwp, static_cast<const float*>(swp), n_out, op, dt, n_out,
+                              stream);
     Py_END_ALLOW_THREADS
     if (rc != GBS_OK) Py_RETURN_NONE;
     if (a[7] != Py_None) return Py_NewRef(a[7]);
@@ -283,11 +286,13 @@ PyObject* do_clip_error(const PlanRef& ref, PyObject* const* a)
     }
     // the sums are zeroed on the stream that adds to them
     at::Tensor err = at::detail::empty_cuda({static_cast<int64_t>(K)}, at::kDouble, x->device(), std::nullopt);
+    void *xp = x->data_ptr(), *ep = err.data_ptr();
     int rc = GBS_ERR_CUDA;
     Py_BEGIN_ALLOW_THREADS
-    if (cudaMemsetAsync(err.data_ptr(), 0, sizeof(double) * static_cast<size_t>(K), static_cast<cudaStream_t>(stream)) == cudaSuccess)
-        rc = gbs_clip_error(plan, x->data_ptr(), dt, rows, stride, alphas, static_cast<int>(K), static_cast<double*>(err.data_ptr()),
-                            nullptr, stream);
+    if (cudaMemsetAsync(ep, 0, sizeof(double) * static_cast<size_t>(K), static_cast<cudaStream_t>(stream)) == cudaSuccess)
+        rc = gbs_clip_error(plan, xp, dt, rows, stride, alphas, static_cast<int>(K), static_cast<double*>(ep), nullptr, stream);
+    else
+        cudaGetLastError();                               // the Python path reports it; later launches of others must not
     Py_END_ALLOW_THREADS
     if (rc != GBS_OK) Py_RETURN_NONE;
     return THPVariable_Wrap(std::move(err));

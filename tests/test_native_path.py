@@ -184,3 +184,27 @@ def test_a_method_replaced_on_the_class_reaches_plans_that_exist(monkeypatch):
             return pool
     with Pooled(4096) as plan:
         assert plan.rotate_quantize(x)[0] is pool[0]
+
+
+@pytest.mark.gpu
+def test_tensors_without_memory_are_refused():
+    """A batched tensor's data pointer throws in C++, a fake tensor's is null: the call is handed to the Python path, which raises,
+    and the process lives."""
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    gbs_build.build()
+    x = synth.make_host("llama4096", 2).to(DEV)
+    with Plan(4096) as plan:
+        codes, scales, _ = plan.rotate_quantize(x)
+        out, rows, mm = plan.alloc_outputs(1, DEV), torch.empty(1, 4096, device=DEV), torch.empty(1, 1, device=DEV)
+        for call in (lambda r, c, s: plan.rotate_quantize(r)[0], lambda r, c, s: plan.rotate_quantize(r, out=out)[0],
+                     lambda r, c, s: plan.clip_error(r, [0.5]), lambda r, c, s: plan.dequantize(c[None], s[None]),
+                     lambda r, c, s: plan.quantized_matmul(c[None], s[None], plan, c[None], s[None], out=mm)):
+            with pytest.raises(RuntimeError):
+                torch.vmap(call)(x, codes, scales)
+        mode = FakeTensorMode()
+        fx, fc, fs = (mode.from_tensor(t) for t in (x, codes, scales))
+        for call in (lambda: plan.rotate_quantize(fx, out=plan.alloc_outputs(2, DEV)), lambda: plan.dequantize(fc, fs)):
+            with pytest.raises(Exception):
+                call()
+        torch.cuda.synchronize()
+        assert torch.equal(plan.rotate_quantize(x)[0], codes)
