@@ -69,7 +69,7 @@ def test_methods_take_arguments_as_plan_declares_them():
     """The per-plan C methods parse like the Python methods they stand for, share their errors, and end with the plan."""
     gbs_build.build()
     x = synth.make_host("llama4096", 3).to(DEV)
-    big = synth.make_host("llama4096", 700).to(DEV)                       # outputs beyond the shared allocation's size
+    big = synth.make_host("llama4096", 700).to(DEV)
     with Plan(4096, bits=4, alpha=0.9) as plan:
         for rows in (x, big):
             codes, scales, y = plan.rotate_quantize(rows, True, None, None)
@@ -208,3 +208,20 @@ def test_tensors_without_memory_are_refused():
                 call()
         torch.cuda.synchronize()
         assert torch.equal(plan.rotate_quantize(x)[0], codes)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows", [1, 3, 700])
+def test_outputs_have_storages_of_their_own(rows):
+    """Codes and scales are saved, kept, resized and freed each by itself."""
+    gbs_build.build()
+    x = synth.make_host("llama4096", rows).to(DEV)
+    with Plan(4096, bits=4) as plan:
+        codes, scales, y = plan.rotate_quantize(x, want_y=True)
+        outs = (codes, scales, y, plan.dequantize(codes, scales), plan.quantized_matmul(codes, scales, plan, codes, scales))
+        assert len({t.untyped_storage().data_ptr() for t in outs}) == len(outs)
+        for t in outs:
+            assert t.storage_offset() == 0 and t.untyped_storage().nbytes() == t.numel() * t.element_size()
+        want = scales.clone()
+        codes.untyped_storage().resize_(0)
+        assert torch.equal(scales, want)
