@@ -235,8 +235,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv2(const __grid_constant__ C
                 if (mb == POISON) break;
             }
             const float M = __uint_as_float(mb);
-            // an all-zero token or group has every value at zero: any finite factor gives code 0
-            const float a1 = __fdividef(P.c_half, fmaxf(M, 1e-30f));
+            // an all-zero token or group has every value at zero: any finite factor gives code 0.  (No lower limit above that: a group
+            // of tiny values is quantized like any other.)
+            const float a1 = M > 0.f ? __fdividef(P.c_half, M) : 0.f;
             unsigned out[BITS];
             quantize_pack32<BITS>(r, a1, out);
             if (up < P.U && row < P.n_rows) {

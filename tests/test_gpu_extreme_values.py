@@ -1,0 +1,28 @@
+"""Values at the ends of the number range through the kernels that replaced general ones: tiny rows and groups, scales near the
+largest float, infinities.  Powers of two change no significand, so the results scale exactly; an infinity gives the scale and the
+codes that the general kernel gives."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2504_13989_b200 import Plan
+from paper_2504_13989_b200 import build as gbs_build
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _rows(n, d, seed):
+    x = 0.5 * np.random.Generator(np.random.PCG64(seed)).standard_t(3.0, size=(n, d))
+    return torch.from_numpy(x.astype(np.float32)).to(torch.bfloat16).to(DEV)
+
+
+@pytest.mark.parametrize("d,m,group", [(8192, 1, 0), (8192, 1, 128), (5120, 20, 0), (5120, 20, 128)])
+@pytest.mark.parametrize("bits", [3, 4])
+def test_tiny_rows_and_groups_are_quantized_like_others(d, m, group, bits):
+    gbs_build.build()
+    x = _rows(9, d, d + bits)
+    with Plan(d, d, m, bits, group, 0.9) as plan:
+        codes, scales, _ = plan.rotate_quantize(x)
+        small, s2, _ = plan.rotate_quantize((x.float() * 2.0 ** -110).to(torch.bfloat16))
+        assert torch.equal(small, codes) and torch.equal(s2, scales * 2.0 ** -110)
