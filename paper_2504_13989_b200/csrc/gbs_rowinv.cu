@@ -70,9 +70,17 @@ __global__ void __launch_bounds__(RI_THREADS, RI_BLOCKS) k_row_inv(const __grid_
                 h[i] = hadd2(a, b);
                 h[i + s] = hsub2(a, b);
             }
-    const float sc = delta * P.norm * 16777216.f;            // the halves are integers times 2^-24
+    float sc = delta * P.norm * 16777216.f;                  // the halves are integers times 2^-24
     const float add0 = ASYM ? 128.f * lo * P.norm : 0.f;
     constexpr float OFF0 = (ASYM ? 0.f : 128.f * (float)(1 << (BITS - 1))) / 16777216.f;
+    float off0 = OFF0;
+    if (!(fabsf(sc) <= 3.4028234e38f)) {
+        // a scale beyond 2^107: the halves as the integers they stand for (below 2048), exactly
+#pragma unroll
+        for (int i = 0; i < 64; ++i) h[i] = hmul2(hmul2(h[i], 0x6c006c00u), 0x6c006c00u);                      // 2^12 twice
+        sc = delta * P.norm;
+        off0 = OFF0 * 16777216.f;
+    }
     OutT* dst = reinterpret_cast<OutT*>(P.out) + row * (long long)P.d;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {                            // sixteen coordinates each
@@ -86,7 +94,7 @@ __global__ void __launch_bounds__(RI_THREADS, RI_BLOCKS) k_row_inv(const __grid_
                 f[8 * o + i] = v.x;
                 f[8 * o + 4 + i] = v.y;
             }
-        if (c == 0) f[0] -= OFF0;
+        if (c == 0) f[0] -= off0;
 #pragma unroll
         for (int e = 0; e < 16; ++e) f[e] = (c == 0 && e == 0) ? fmaf(f[0], sc, add0) : f[e] * sc;
         store_values<16>(dst + 16 * c, f, P.wide != 0);

@@ -304,6 +304,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
             const bool store = row < P.n_rows && up * V < P.d;
             OutT* dst = reinterpret_cast<OutT*>(P.out) + row * (long long)P.d + up * V;
             tc_fence_after();
+            float lift = 1.f;
+            if (!SPLIT && !(fabsf(fac[0]) <= 3.4028234e38f)) {
+                // a scale beyond 2^104 sqrt(d') (or not finite): the power of two on its own
+                fac[0] = row < P.n_rows ? __ldg(P.scales + row) * P.norm : 0.f;
+                lift = 16777216.f;
+            }
 #pragma unroll
             for (int half = 0; half < V / 32; ++half) {
                 unsigned r[32];
@@ -321,6 +327,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
                     for (int o = 0; o < 4; ++o)
 #pragma unroll
                         for (int e = 0; e < 8; ++e) f[8 * o + (e >> 1) + 4 * (e & 1)] = __uint_as_float(r[8 * o + e]) * fac[0];
+                    if (!SPLIT && lift != 1.f) {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) f[i] *= lift;
+                    }
                     store_values<32>(dst + half * 32, f, P.wide != 0);
                 }
             }

@@ -26,3 +26,18 @@ def test_tiny_rows_and_groups_are_quantized_like_others(d, m, group, bits):
         codes, scales, _ = plan.rotate_quantize(x)
         small, s2, _ = plan.rotate_quantize((x.float() * 2.0 ** -110).to(torch.bfloat16))
         assert torch.equal(small, codes) and torch.equal(s2, scales * 2.0 ** -110)
+
+
+@pytest.mark.parametrize("d,m,group,asym", [(4096, 1, 0, False), (3584, 28, 0, False), (8192, 1, 0, False), (4096, 1, 128, False),
+                                            (128, 1, 0, False), (128, 1, 128, True)])
+@pytest.mark.parametrize("bits", [3, 4])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_large_scales_are_restored(d, m, group, asym, bits, dtype):
+    gbs_build.build()
+    x = _rows(70, d, d + bits)
+    with Plan(d, d, m, bits, group, 0.9, asymmetric=asym) as plan:
+        codes, scales, _ = plan.rotate_quantize(x)
+        up = 2.0 ** 112
+        want = plan.dequantize(codes, scales, inverse=True, dtype=dtype)
+        got = plan.dequantize(codes, scales * up, inverse=True, dtype=dtype)
+        assert bool(torch.isfinite(got).all()) and torch.equal(got, want * up)
