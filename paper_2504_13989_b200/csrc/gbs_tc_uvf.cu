@@ -100,6 +100,9 @@ __device__ __forceinline__ unsigned below(unsigned x)
 {
     return __float_as_uint(__uint_as_float(x) - __uint_as_float(x & 0xffff0000u));
 }
+// The same for any x: infinities leave a finite number instead of inf - inf, so that their sums stay infinite.  (What a finite x
+// leaves is below 2^121; the minimum passes over a NaN.)
+__device__ __forceinline__ unsigned below_any(unsigned x) { return __float_as_uint(fminf(__uint_as_float(below(x)), 0x1p121f)); }
 
 template <int BITS, int V, bool GROUPED, bool WANT_Y>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ UvfParams P)
@@ -220,7 +223,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const unsigned x0 = x[j].x, x1 = x[j].y, x2 = x[j].z, x3 = x[j].w;
-                const unsigned m0 = below(x0), m1 = below(x1), m2 = below(x2), m3 = below(x3);
+                const unsigned m0 = below_any(x0), m1 = below_any(x1), m2 = below_any(x2), m3 = below_any(x3);
                 const unsigned l0 = below(m0), l1 = below(m1), l2 = below(m2), l3 = below(m3);
                 // 128 elements on is 256 bytes on, and two (V = 64) or four rows: that much of the swizzle is a constant
                 const unsigned dst = (dst0 ^ (32u * (unsigned)(j & (HALVES == 1 ? 1 : 3)))) + 256u * j;

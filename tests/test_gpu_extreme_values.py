@@ -41,3 +41,21 @@ def test_large_scales_are_restored(d, m, group, asym, bits, dtype):
         want = plan.dequantize(codes, scales, inverse=True, dtype=dtype)
         got = plan.dequantize(codes, scales * up, inverse=True, dtype=dtype)
         assert bool(torch.isfinite(got).all()) and torch.equal(got, want * up)
+
+
+@pytest.mark.parametrize("d,m,group,at", [(4096, 1, 0, 0), (4096, 1, 128, 4095), (3584, 28, 0, 1000), (8192, 1, 0, 77), (5120, 20, 128, 5000)])
+@pytest.mark.parametrize("value", [float("inf"), float("-inf")])
+def test_an_infinity_in_an_fp32_row(d, m, group, at, value, monkeypatch):
+    gbs_build.build()
+    x = _rows(6, d, d).float() * 1.001
+    want_rest = x.clone()
+    x[3, at] = value
+    with Plan(d, d, m, 4, group, 0.9) as plan:
+        codes, scales, y = plan.rotate_quantize(x, want_y=True)
+        rest = plan.rotate_quantize(want_rest)
+    monkeypatch.setenv("GBS_FORCE_GENERIC", "1")
+    with Plan(d, d, m, 4, group, 0.9) as plan:
+        c2, s2, y2 = plan.rotate_quantize(x, want_y=True)
+    assert bool(torch.isinf(scales[3]).all()) and torch.equal(scales[3], s2[3]) and torch.equal(codes[3], c2[3]) and torch.equal(y[3], y2[3])
+    others = [0, 1, 2, 4, 5]
+    assert torch.equal(codes[others], rest[0][others]) and torch.equal(scales[others], rest[1][others])
