@@ -69,6 +69,9 @@ struct DenseParams {
     int stages;
     int stage_words;              // words of a token's row in a warp's packing buffer (odd)
     float c_scale, c_half, norm;
+    const unsigned short* x;      // the rows (bf16), for what the tensor map does not show
+    long long stride;
+    int d;
     const unsigned char* toep;    // core matrices J = kb - nb + nbp - 1
     const unsigned char* row0;    // ROW0_BYTES
     const unsigned char* col0;    // core matrix pairs (column repair, zeros) of block nbp - 1 - i at i
@@ -344,7 +347,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&S->tempty);
-            if (rank == 0 && h == 0 && live) P.scales[row] = P.c_scale * M;
+            if (rank == 0 && h == 0 && live) {
+                // An infinity among the sixteen elements that meet column 0's repair is multiplied by its zeros there: every rotated
+                // value is NaN, which a maximum passes over.  Its scale is infinite, as for an infinity anywhere else.
+                if (M == 0.f) {
+                    const unsigned short* x = P.x + row * P.stride;
+                    for (int j = 0; j < 16 && j < P.d; ++j)
+                        if ((__ldg(x + j) & 0x7fffu) == 0x7f80u) M = __uint_as_float(0x7f800000u);
+                }
+                P.scales[row] = P.c_scale * M;
+            }
             // this warp's 32 rows as words, sixteen lanes to a row (a piece is at most 64 bytes; 48 where rows are unaligned)
             const int n_codes = (P.m - nfirst) < (ch1 - ch0) * 32 ? (P.m - nfirst) : (ch1 - ch0) * 32;
             const int nbytes = n_codes > 0 ? n_codes * BITS / 8 : 0;
@@ -523,6 +535,9 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
     P.n_rows = n_rows;
     P.n_tiles = (int)((n_rows + TM - 1) / TM);
     P.m = p->m;
+    P.d = p->d;
+    P.x = (const unsigned short*)x;
+    P.stride = stride;
     P.kchunks = (p->d + KC - 1) / KC;
     P.ksteps_last = ((p->d - (P.kchunks - 1) * KC) + 15) / 16;
     int fit = 0;

@@ -59,3 +59,20 @@ def test_an_infinity_in_an_fp32_row(d, m, group, at, value, monkeypatch):
     assert bool(torch.isinf(scales[3]).all()) and torch.equal(scales[3], s2[3]) and torch.equal(codes[3], c2[3]) and torch.equal(y[3], y2[3])
     others = [0, 1, 2, 4, 5]
     assert torch.equal(codes[others], rest[0][others]) and torch.equal(scales[others], rest[1][others])
+
+
+@pytest.mark.parametrize("d,m", [(1536, 1544), (480, 480), (8, 128)])
+@pytest.mark.parametrize("at", [0, 1, 7, 15, 16, 300])
+def test_an_infinity_in_a_row_of_a_full_order(d, m, at):
+    gbs_build.build()
+    x = _rows(133, d, d)
+    with Plan(d, m, m, 4, 0, 0.9) as plan:
+        want = plan.rotate_quantize(x)
+        bad = x.clone()
+        bad[130, at % d] = float("inf")
+        codes, scales, _ = plan.rotate_quantize(bad)
+    assert bool(torch.isinf(scales[130]).all())
+    # every value times a factor of zero: NaN, which clips to the lowest code, -D
+    assert bool((codes[130] == 0x99).all())
+    others = [i for i in range(133) if i != 130]
+    assert torch.equal(codes[others], want[0][others]) and torch.equal(scales[others], want[1][others])
