@@ -10,7 +10,8 @@
 //   * t becomes a 22-bit integer in the mantissa of one FMA.  Its high 12 bits index a table of cells; an entry holds the
 //     number of thresholds below the cell and the low 10 bits of the one threshold inside it, placed so that adding the
 //     value's low bits carries into the bin index when the threshold is reached.  (The host takes this path only where no two
-//     different thresholds share a cell.)
+//     different thresholds share a cell.  Thresholds that are one and the same number, such as 1.5 x 0.5 and 0.5 x 1.5 over D, may come
+//     out one unit of t apart when the ratios are rounded to floats; they count as one, the lower.)
 //   * Two shared-memory atomics per value (count, and the FMA's bits themselves: the exponent pattern is removed with the count)
 //     into COPIES interleaved histograms per token, so that a warp's lanes rarely meet: measured 2 cycles per 32 values with 32
 //     copies and 6 with 8, against 3 - 4 for the table lookup.  Everything is an integer: exact in any order.
@@ -356,14 +357,18 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
     // t = 1 must stay below 2^22 after rounding
     P.scale = 4194304.f - 8.f;
     unsigned long long used[CELLS / 64] = {0};
-    unsigned at[CELLS];
+    unsigned at[CELLS], last[CELLS];               // the lowest and the highest threshold of a cell
     unsigned short rank[CELLS];
+    constexpr unsigned SAME = 1;                   // alpha rounds to 2^-25, an eighth of a unit; ceil makes one of it
     for (int k = 0; k < K; ++k)
         for (int j = 0; j < D; ++j) {
             const unsigned T = (unsigned)ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale), c = T >> CELL_BITS;
-            if (c >= CELLS || ((used[c >> 6] >> (c & 63) & 1) && at[c] != T)) return GBS_UVCLIP_NOT_SERVED;
+            if (c >= CELLS) return GBS_UVCLIP_NOT_SERVED;
+            const bool seen = used[c >> 6] >> (c & 63) & 1;
+            at[c] = seen && at[c] < T ? at[c] : T;
+            last[c] = seen && last[c] > T ? last[c] : T;
+            if (last[c] - at[c] > SAME) return GBS_UVCLIP_NOT_SERVED;
             used[c >> 6] |= 1ull << (c & 63);
-            at[c] = T;
         }
     for (int w = 0; w < CELLS / 64; ++w)
         for (unsigned long long m = used[w]; m; m &= m - 1) {
