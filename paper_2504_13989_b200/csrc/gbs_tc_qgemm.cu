@@ -405,6 +405,7 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     if (px->d_pad % KB != 0) return GBS_ERR_UNSUPPORTED;
     if (px->smem_optin < (int)(Shape<8>::SMEM)) return GBS_ERR_UNSUPPORTED;
     if (n_tokens == 0 || n_out == 0) return GBS_OK;
+    if (n_tokens > (int64_t)0x7fffffff - 256 || n_out > (int64_t)0x7fffffff - 256) return GBS_ERR_INVALID_ARG;   // TMA coordinates are 32-bit
     if (!codes_x || !scales_x || !codes_w || !scales_w || !out) return GBS_ERR_INVALID_ARG;
     const int esz = out_dtype == GBS_DTYPE_F32 ? 4 : 2;
     if ((reinterpret_cast<uintptr_t>(codes_x) & 15u) || (reinterpret_cast<uintptr_t>(codes_w) & 15u) ||
@@ -423,7 +424,6 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     }
     EncodeTiledFn encode = get_encode();
     if (!encode) return GBS_ERR_CUDA;
-    if (n_tokens > (int64_t)0x7fffffff - 256 || n_out > (int64_t)0x7fffffff - 256) return GBS_ERR_INVALID_ARG;   // TMA coordinates are 32-bit
     QgemmParams P;
     memset(&P, 0, sizeof(P));
     P.n_tok = n_tokens;
