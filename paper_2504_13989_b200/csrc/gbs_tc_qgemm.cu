@@ -366,17 +366,19 @@ int pick_tokens(long long n_tok, long long n_out, int kblocks, int sm_count)
     return n_best;
 }
 
-// Whether the few-token kernel (gbs_qgemv.cu) is the faster one.  Its time grows with the channels, by these cycles per channel and
-// step of 128 codes for up to 8, 16, 32 and 64 tokens (4096-wide rows, 8192 and 14336 channels; four bits, three bits on a side); a
-// wave of tiles costs 600 per step whatever it holds, with much the same start.  So 64 tokens go to the tiles beyond 5800 (4300)
-// channels, 32 beyond 10 300 (7800), 16 beyond 18 200 (8800).  48 tokens -> 14336, four bits: 28.5 us here, 12.4 in tiles; 4096: 7.9
-// and 10.8.
+// Whether the few-token kernel (gbs_qgemv.cu) is the faster one.  Its time grows with the channels of an SM: these cycles per channel and
+// step of 128 codes on 148 SMs for up to 8, 16, 32 and 64 tokens (measured with 4096-wide rows, 8192 and 14336 channels; four bits,
+// three bits on a side).  Tiles of 128 channels come in waves over the SMs, 600 cycles a step whatever they hold, with much the same
+// start.  So within the first wave (18 944 channels) 64 tokens go to the tiles beyond 5800 (4300) channels, 32 beyond 10 300 (7800), 16
+// beyond 18 200 (8800), and where a new wave begins the few-token kernel is the faster one again for a while.  48 tokens -> 14336, four
+// bits: 28.5 us here, 12.4 in tiles; 4096: 7.9 and 10.8.
 bool few_tokens(long long n_tok, long long n_out, bool three, int sm_count)
 {
     if (n_tok > GBS_QGEMV_MAX_TOKENS) return false;
     static const double per_channel[2][4] = {{0.021, 0.033, 0.058, 0.103}, {0.035, 0.068, 0.077, 0.140}};
     const long long tiles = (n_out + TM - 1) / TM, waves = (tiles + sm_count - 1) / sm_count;
-    return (double)n_out * per_channel[three ? 1 : 0][n_tok <= 8 ? 0 : n_tok <= 16 ? 1 : n_tok <= 32 ? 2 : 3] <= 600.0 * (double)waves;
+    const double cycles = per_channel[three ? 1 : 0][n_tok <= 8 ? 0 : n_tok <= 16 ? 1 : n_tok <= 32 ? 2 : 3] * 148.0 / sm_count;
+    return (double)n_out * cycles <= 600.0 * (double)waves;
 }
 
 bool encode_codes(EncodeTiledFn encode, CUtensorMap* map, const void* codes, int64_t rows, int row_bytes, int bits, int box_rows)
