@@ -45,10 +45,9 @@ constexpr int UMAX = 128;              // largest tensor-core factor
 constexpr int STAGE_BYTES_MAX = TOK * UMAX * V * 2;   // 32 KB of bf16
 constexpr int A_BYTES = UMAX * UMAX * 2;              // 32 KB: A as bf16, two K blocks of 64
 constexpr int EPI_WARPS = 4 * TOK;
-// Two threads issue the MMAs, on alternate tiles: in the running kernel a tcgen05.mma takes about three times
-// as long as alone on the SM and one issuing thread is busy for most of a tile's period; the second one (on
-// another scheduler) takes 1 - 3 % off the steady state.  Every stage must belong to one issuer, so that the
-// phase parities it waits for cannot alias: the count divides STAGES.
+// Two warps issue the MMAs, on alternate tiles, so that one's polls and commits (a couple of hundred cycles beside the MMAs' own) are
+// covered by the other's: 65 536 x 4096, 4 bits: 112.8 us with two, 113.5 with one; 65 536 x 3584, 3 bits, groups of 128: 105.1 and
+// 105.7.  Every stage must belong to one issuer, so that the phase parities it waits for cannot alias: the count divides STAGES.
 constexpr int N_ISSUERS = 2;
 static_assert(STAGES % N_ISSUERS == 0, "a stage is served by one MMA issuer");
 constexpr int THREADS = 32 * (1 + N_ISSUERS + EPI_WARPS);   // producer, issuers (warp 1 and the last ones), epilogue

@@ -294,7 +294,7 @@ Uv2Kernel kernel_of(int bits, bool grouped, bool want_y)
 // at most a warp's).
 bool gbs_tc_uv2_supported(const gbs_plan* p)
 {
-    return p->variant == GBS_VARIANT_TC_UVM && p->uvm_glog == 1 && !p->asym && p->d % V == 0 &&
+    return p->variant == GBS_VARIANT_TC_UVM && p->uvm_glog == 1 && !p->asym &&
            (p->group == 0 || (p->group >= 2 * V && p->group <= 32 * V)) && p->smem_optin >= (int)sizeof(Smem) + 1024;
 }
 

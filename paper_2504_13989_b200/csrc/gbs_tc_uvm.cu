@@ -32,9 +32,10 @@ constexpr int A_BYTES = UMAX * UMAX * 2;
 constexpr int B_BYTES = 160 * 1024;               // shared memory for the row stages
 constexpr int MAX_STAGES = 4;
 constexpr int EPI_WARPS = 16;
-// With G = 2 a token is one 128 x 64 x K contraction and the epilogue per token is short: the thread that issues
-// the MMAs (about 200 cycles each in the running kernel) is then the bottleneck, and a second issuing thread on
-// another scheduler takes every other token (55 -> 42 us for 8192 x 8192).  With G = 4 or 8 it does not pay.
+// With G = 2 a token is one 128 x 64 x K contraction and the epilogue per token is short: what an issuing warp does around its MMAs
+// (two polls and two commits per token) is then the bottleneck, and a second one on another scheduler takes every other token
+// (65 536 x 8192, 4 bits, groups of 32: 376 -> 312 us; 65 536 x 5120, 3 bits, groups of 64: 348 -> 308).  With G = 4 or 8, and in
+// clip scoring, it does not pay.
 // Every shared-memory and TMEM stage stays with one issuer (both stage counts are even), so the phase
 // parities an issuer waits for cannot alias.
 __host__ __device__ constexpr int issuers_for(int glog) { return glog == 1 ? 2 : 1; }
@@ -602,15 +603,17 @@ int gbs_tc_uvm_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows,
     const int grid = (int)(n_rows < p->sm_count ? n_rows : p->sm_count);
     const bool pdl = p->pdl != 0;
     cudaError_t e;
+    // d' = 64 U with one scale per token is gbs_tc_uv2.cu's, and so are its groups of 128 to 2048; those of 32 and 64 come here
+    if (glog == 1 && p->group == 0) return (int)cudaErrorNotSupported;
 #define GBS_UVM_LAUNCH(B, GL)                                                                   \
     (p->group ? launch(k_tc_uvm_rq<B, GL, true, false>, threads_for(GL), grid, smem, stream, pdl, tmap, P)        \
               : launch(k_tc_uvm_rq<B, GL, false, false>, threads_for(GL), grid, smem, stream, pdl, tmap, P))
     if (p->bits == 3) {
-        if (glog == 1) e = GBS_UVM_LAUNCH(3, 1);
+        if (glog == 1) e = launch(k_tc_uvm_rq<3, 1, true, false>, threads_for(1), grid, smem, stream, pdl, tmap, P);
         else if (glog == 2) e = GBS_UVM_LAUNCH(3, 2);
         else e = GBS_UVM_LAUNCH(3, 3);
     } else {
-        if (glog == 1) e = GBS_UVM_LAUNCH(4, 1);
+        if (glog == 1) e = launch(k_tc_uvm_rq<4, 1, true, false>, threads_for(1), grid, smem, stream, pdl, tmap, P);
         else if (glog == 2) e = GBS_UVM_LAUNCH(4, 2);
         else e = GBS_UVM_LAUNCH(4, 3);
     }

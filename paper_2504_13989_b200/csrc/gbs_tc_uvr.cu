@@ -239,11 +239,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvr_rq(const __grid_constant_
         }
       } else if (warp <= 2) {
         // ------------------------------ MMA issuers ------------------------------
-        // Two issuing threads on two schedulers: what costs an issuing thread time is not the MMAs (64 cycles each on the
-        // tensor pipe) but what stands between them (the poll of a stage's barrier, the commit that returns it, every
-        // instruction of its own loop), and one thread alone does not keep the epilogue fed.  U > 128: thread 0
-        // contracts the first block of every token, thread 1 the second (a stage returns to the producer after both
-        // commits).  U <= 128: the threads take alternate tokens.
+        // Two issuing warps on two schedulers: what costs an issuer time is not the MMAs (64 cycles each on the tensor pipe) but
+        // what stands between them (the poll of a stage's barrier, the commit that returns it).  U > 128: warp 1 contracts
+        // the first block of every token, warp 2 the second (a stage returns to the producer after both commits).  U <= 128:
+        // they take alternate tokens.  (One issuer was measured on the narrower kernels only: gbs_tc_uv.cu, gbs_tc_uvm.cu.)
         {
             const int issuer = warp - 1;
             constexpr unsigned IDESC = instr_desc(128, NCOLS, true);
