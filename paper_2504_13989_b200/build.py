@@ -14,6 +14,7 @@ LIB = os.path.join(PKG, "libgbs.so")
 NATIVE = os.path.join(PKG, "_native.so")
 NATIVE_SRC = os.path.join(CSRC, "gbs_torch.cpp")
 
+NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")        # its toolkit's headers serve _native.so as well
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
     "-O3", "-std=c++17", "-lineinfo",
@@ -41,14 +42,13 @@ def native_command(obj: str) -> list:
     return ["g++", "-O3", "-std=c++20", "-fPIC", "-Wall", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
             "-I", os.path.join(ROOT, "include"), "-isystem", inc,
             "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", sysconfig.get_paths()["include"],
-            "-isystem", "/usr/local/cuda/include", "-c", NATIVE_SRC, "-o", obj]
+            "-isystem", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"), "-c", NATIVE_SRC, "-o", obj]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu under csrc/ into libgbs.so; returns its path."""
     if not force and not is_stale():
         return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     objs = []
     build_dir = os.path.join(PKG, "_build")
     os.makedirs(build_dir, exist_ok=True)
@@ -64,7 +64,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objs.append(obj)
         if fresh(obj, src):
             continue
-        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
+        cmd = [NVCC] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd)))
     native_obj = os.path.join(build_dir, "gbs_torch.o")
     if not fresh(native_obj, NATIVE_SRC):
@@ -72,9 +72,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         procs.append((cmd, subprocess.Popen(cmd)))
     for cmd, pr in procs:
         if pr.wait() != 0:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+            raise RuntimeError("compilation failed: " + " ".join(cmd))
     tmp = LIB + ".tmp.%d" % os.getpid()
-    subprocess.check_call([nvcc, "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])
+    subprocess.check_call([NVCC, "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)
     # libgbs.so is found beside _native.so; torch's libraries are already loaded when the package is imported
     import torch
