@@ -52,11 +52,6 @@ struct DenseInvParams {
     int* status;
 };
 
-__device__ __forceinline__ void st_shared_v4(unsigned addr, uint4 v)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
 // bf16 bit pattern of a small integer (exact for |q| <= 256)
 __device__ __forceinline__ unsigned bf16_of_int(int q) { return __float_as_uint((float)q) >> 16; }
 

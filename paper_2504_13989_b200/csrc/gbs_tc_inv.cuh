@@ -71,11 +71,6 @@ __device__ __forceinline__ void rotate_octet(const unsigned* w, int o, unsigned 
     }
 }
 
-__device__ __forceinline__ void st_shared_v4(unsigned addr, uint4 v)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
 // 32 bytes: one store where the address allows (a full DRAM sector per thread), else two
 __device__ __forceinline__ void store32(void* p, const unsigned w[8], bool wide)
 {

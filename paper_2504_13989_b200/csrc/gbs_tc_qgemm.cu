@@ -92,10 +92,6 @@ __device__ __forceinline__ void umma_i8_ts(unsigned d_tmem, unsigned a_tmem, uns
                  ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
-__device__ __forceinline__ void st_shared_v4(unsigned addr, uint4 v)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
 __device__ __forceinline__ uint4 ld_shared_v4(unsigned addr)
 {
     uint4 v;
