@@ -278,7 +278,7 @@ extern "C" int gbs_rotate_quantize(const gbs_plan_t* p, const void* x, int x_dty
         e = gbs_tc_uvm_rotate_quantize(p, x, n_rows, x_row_stride, codes, scales, y_opt, stream);
     else if (p->variant == GBS_VARIANT_TC_ROW && x_dtype == GBS_DTYPE_BF16)
         e = gbs_tc_row_rotate_quantize(p, x, n_rows, x_row_stride, codes, scales, y_opt, stream);
-    else if (x_dtype == GBS_DTYPE_F32 && gbs_tc_uvf_v(p) != 0)
+    else if (x_dtype == GBS_DTYPE_F32 && gbs_tc_uvf_serves(p, n_rows))
         e = gbs_tc_uvf_rotate_quantize(p, x, n_rows, x_row_stride, codes, scales, y_opt, stream);
     else
         e = gbs_generic_rotate_quantize(p, x, x_dtype, n_rows, x_row_stride, codes, scales, y_opt, stream);
@@ -303,7 +303,7 @@ extern "C" int gbs_dequantize(const gbs_plan_t* p, const void* codes, const floa
     int e;
     if ((flags & GBS_INVERSE_ROTATE) && p->variant == GBS_VARIANT_TC_DENSE)
         e = gbs_tc_denseinv_dequantize(p, codes, scales, n_rows, out, out_dtype, static_cast<cudaStream_t>(cuda_stream));
-    else if ((flags & GBS_INVERSE_ROTATE) && gbs_tc_uvinv_supported(p))
+    else if ((flags & GBS_INVERSE_ROTATE) && gbs_tc_uvinv_serves(p, n_rows, out_dtype))
         e = gbs_tc_uvinv_dequantize(p, codes, scales, n_rows, out, out_dtype, static_cast<cudaStream_t>(cuda_stream));
     else if ((flags & GBS_INVERSE_ROTATE) && gbs_rowinv_supported(p, scales))
         e = gbs_rowinv_dequantize(p, codes, scales, n_rows, out, out_dtype, static_cast<cudaStream_t>(cuda_stream));

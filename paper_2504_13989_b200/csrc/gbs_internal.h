@@ -93,12 +93,13 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
 
 // gbs_tc_uvf.cu : rotate-quantize of fp32 rows on the tensor cores (three bf16 planes)
 int gbs_tc_uvf_v(const gbs_plan* p);            // the in-register factor of the path, 0 if it does not serve the plan
+bool gbs_tc_uvf_serves(const gbs_plan* p, int64_t n_rows);
 int gbs_tc_uvf_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
                                float* scales, float* y_opt, cudaStream_t stream);
 
 // gbs_tc_uvinv.cu : gbs_dequantize with inverse rotation on the tensor cores
 int gbs_tc_uvinv_v(const gbs_plan* p);          // the factor V of the path, 0 if it does not serve the shape
-bool gbs_tc_uvinv_supported(const gbs_plan* p);
+bool gbs_tc_uvinv_serves(const gbs_plan* p, int64_t n_rows, int out_dtype);
 int gbs_tc_uvinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
                             int out_dtype, cudaStream_t stream);
 

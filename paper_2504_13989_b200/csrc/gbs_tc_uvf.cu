@@ -341,6 +341,19 @@ int gbs_tc_uvf_v(const gbs_plan* p)
     return 0;
 }
 
+// The calls it takes: all of those plans' but the ones that the shared-memory kernel does faster.  That kernel's time goes with the rows,
+// the width and the order m; here a tile of 128 / V tokens takes much the same whatever the width.  So with m = 1 a width of 512 stays
+// there, 1024 up to 28 rows per SM (64 with group scales), 2048 up to one and a half.  (4 bits, shared memory and here: 5000 x 512:
+// 10.9 and 16.7 us; 1200 x 1024: 6.6 and 7.3, 5000: 19.8 and 19.1, with groups of 128: 20.3 and 21.0; 150 x 2048: 3.8 and 4.0, 300:
+// 4.5 and 4.2; 16 x 4096: 4.9 and 4.6.)
+bool gbs_tc_uvf_serves(const gbs_plan* p, int64_t n_rows)
+{
+    if (gbs_tc_uvf_v(p) == 0) return false;
+    if (p->m != 1 || p->d_pad > 2048) return true;
+    if (p->d_pad > 1024) return 2 * n_rows > 3 * (int64_t)p->sm_count;
+    return p->d_pad > 512 && n_rows > (p->group ? 64 : 28) * (int64_t)p->sm_count;
+}
+
 int gbs_tc_uvf_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes, float* scales,
                                float* y_opt, cudaStream_t stream)
 {

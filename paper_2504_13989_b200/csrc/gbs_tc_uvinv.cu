@@ -410,8 +410,21 @@ int gbs_tc_uvinv_v(const gbs_plan* p)
     return 0;
 }
 
-// The plans this path serves: those that got an image of A^T.
-bool gbs_tc_uvinv_supported(const gbs_plan* p) { return p->inv_v != 0 && p->d_aimg_t != nullptr; }
+// The calls this path takes: of the plans that got an image of A^T, all but those the shared-memory kernel does faster.  That kernel's time
+// goes with the rows, the width and the order m; here a tile of 128 / V tokens takes much the same whatever the width, and a
+// quarter of the lanes or less have rows below d' = 2048.  So with m = 1 and group scales (their operand is two planes) widths up to
+// 2048 stay there while the rows are few, in rows per SM: 1024 wide: 6 (bf16) and 24 (fp32), 2048 wide: 2 and 5; 512 wide: always.
+// (4 bits, groups of 128, shared memory and here: 5000 x 512 -> bf16: 9.1 and 13.5 us; 600 x 1024 -> bf16: 3.9 and 4.4, 1800: 7.3 and
+// 7.0; 2400 x 1024 -> fp32: 9.4 and 9.9, 5000: 17.1 and 16.0; 220 x 2048 -> bf16: 3.3 and 3.5, 400: 3.9 and 3.7; 600 x 2048 -> fp32: 5.5
+// and 6.0, 900: 7.0 and 6.3.)  One scale per token and m = 1 is faster here at every width: 100 x 512 -> bf16: 3.6 and 2.7.
+bool gbs_tc_uvinv_serves(const gbs_plan* p, int64_t n_rows, int out_dtype)
+{
+    if (p->inv_v == 0 || p->d_aimg_t == nullptr) return false;
+    if (p->group == 0 || p->m != 1 || p->d_pad > 2048) return true;
+    const bool f32 = out_dtype == GBS_DTYPE_F32;
+    const int per_sm = p->d_pad > 1024 ? (f32 ? 5 : 2) : (f32 ? 24 : 6);
+    return p->d_pad > 512 && n_rows > (int64_t)per_sm * p->sm_count;
+}
 
 int gbs_tc_uvinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
                             int out_dtype, cudaStream_t stream)

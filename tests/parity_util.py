@@ -2,6 +2,8 @@
 rotated fp32 values within 1e-5 relative L2 per row, scales within 1e-6 relative, integer codes
 identical except at rounding ties (mismatch fraction <= 1e-4, never more than one level),
 clip-error sums within 1e-5 relative."""
+import warnings
+
 import numpy as np
 import torch
 
@@ -80,3 +82,17 @@ def oracle_rq(x: torch.Tensor, w_or_plan, bits: int, dense: bool = False, alpha:
     else:
         d, d_pad, m = w_or_plan
     return oracle.rotate_quantize_rows(synth.to_oracle_array(x), d, d_pad, m, bits, group, alpha, dense=dense)
+
+
+def kernels_of(call, path):
+    """Names of the kernels that a call launches, from the graph it is captured into (written to `path`)."""
+    call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        call()
+    g.enable_debug_mode()
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")
+        g.debug_dump(str(path))
+    return path.read_text()

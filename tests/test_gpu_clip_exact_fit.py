@@ -4,8 +4,6 @@ either order, and rows too small or not finite.
 
 Tolerance: a value's t = |y| / M is rounded to 2^-22 M, so each residual is off by at most 2^-23 M and an error E over n values by
 2^-22 M sqrt(n E) + n 2^-46 M^2; 1e-6 of E more for the fp32 rotation and M."""
-import warnings
-
 import numpy as np
 import pytest
 import torch
@@ -13,6 +11,7 @@ import torch
 import oracle
 from paper_2504_13989_b200 import Plan, synth
 from paper_2504_13989_b200 import build as gbs_build
+from parity_util import kernels_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -66,20 +65,6 @@ def test_a_value_that_is_not_finite_shows_in_every_sum(bad):
         assert not bool(torch.isfinite(plan.clip_error(x.to(DEV), [0.5, 0.75, 1.0])).any())
 
 
-def _kernels_of(call, path):
-    """Names of the kernels that a call launches, from the graph it is captured into."""
-    call()
-    torch.cuda.synchronize()
-    g = torch.cuda.CUDAGraph(keep_graph=True)
-    with torch.cuda.graph(g):
-        call()
-    g.enable_debug_mode()
-    with warnings.catch_warnings():
-        warnings.simplefilter("ignore")
-        g.debug_dump(str(path))
-    return path.read_text()
-
-
 @pytest.mark.parametrize("bits,K", [(3, 5), (3, 10), (3, 20), (3, 31), (3, 50), (4, 9), (4, 18), (4, 27), (4, 32), (4, 64)])
 def test_evenly_spaced_candidates_take_the_histogram(bits, K, tmp_path):
     """Many thresholds (j + 1/2) alpha_k / D coincide but for a rounding of alpha to float; the call must not fall back for it."""
@@ -89,10 +74,10 @@ def test_evenly_spaced_candidates_take_the_histogram(bits, K, tmp_path):
     ref = oracle.clip_error_rows(synth.to_oracle_array(x), 4096, 4096, 1, bits, 0, alphas)
     with Plan(4096, 4096, 1, bits, 0, 0.9) as plan:
         xd = x.to(DEV)
-        names = _kernels_of(lambda: plan.clip_error(xd, alphas), tmp_path / "clip.dot")
+        names = kernels_of(lambda: plan.clip_error(xd, alphas), tmp_path / "clip.dot")
         assert "k_tc_uv_clip" in names and "k_tc_uv_rq" not in names
         got = plan.clip_error(xd, alphas).cpu().numpy()
         assert np.all(np.abs(got - ref) <= 1e-5 * ref)
         # thresholds that are close but not the same still go to the per-candidate kernel
-        names = _kernels_of(lambda: plan.clip_error(xd, [0.6, 0.60001]), tmp_path / "other.dot")
+        names = kernels_of(lambda: plan.clip_error(xd, [0.6, 0.60001]), tmp_path / "other.dot")
         assert "k_tc_uv_rq" in names and "k_tc_uv_clip" not in names
