@@ -345,11 +345,14 @@ typedef void (*ClipKernel)(const CUtensorMap, const ClipParams);
 }  // namespace
 
 // Scores K clip ratios, or returns GBS_UVCLIP_NOT_SERVED where this path does not apply (group scales, per-row sums, thresholds
-// too close to one another): the caller then takes the per-candidate kernel.
+// too close to one another): the caller then takes the per-candidate kernel.  So it does where that is the faster one: a tile per block at
+// most and candidates for one of its passes (eight), where building the table is what counts (64 x 4096, K = 8: 6.8 us there, 7.0 here at
+// 3 bits, 7.4 at 4; 600 rows, 4 bits: 11.2 and 10.1).
 int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, const float* alphas, int K,
                              double* err_sum, cudaStream_t stream)
 {
     EncodeTiledFn encode = get_encode();
+    if (K <= 8 && n_rows <= (int64_t)TOK * p->sm_count) return GBS_UVCLIP_NOT_SERVED;
     if (p->group != 0 || !encode || p->smem_optin < (int)sizeof(Smem) || n_rows > (int64_t)0x7fffffff - TOK) return GBS_UVCLIP_NOT_SERVED;
     ClipParams P;
     memset(&P, 0, sizeof(P));
