@@ -77,11 +77,12 @@ typedef struct gbs_plan_info {
     int asymmetric;                /* 1 for a GBS_PLAN_ASYMMETRIC plan                */
     int scale_floats_per_row;      /* scales_per_row, or 2 * scales_per_row when asymmetric */
     int variant;                   /* kernel family chosen for bf16 rows: 0 = generic shared-memory path,
-                                      1 = tensor-core path for d' = 32 * U with U = m * 2^j <= 128, U % 16 == 0,
+                                      1 = tensor-core path for d' = 32 * U with 16 <= U = m * 2^j <= 128,
                                       d % 32 == 0 and group in {0, 32 .. 1024}, 2 = tensor-core path for
                                       d' = 128 rows (m = 1, group in {0, 32, 64, 128}), 3 = tensor-core path for
-                                      4096 < d' = 32 * G * U <= 32768 (G in {2, 4, 8}, U as above, per-token
-                                      scales, d a multiple of 32 * G), 4 = dense tensor-core contraction with the full
+                                      4096 < d' = 32 * G * U <= 32768 (G in {2, 4, 8}, U as above, d a multiple of
+                                      32 * G, group 0 or 32 .. 1024 * G; two kernels: one sweep for G = 2 with
+                                      group 0 or 128 .. 2048, three otherwise), 4 = dense tensor-core contraction with the full
                                       Paley matrix (d' = m), 5 = as 3 where also d' = 128 * U with 80 <= U <= 256,
                                       d % 128 == 0 and group <= 4096: rotate-quantize keeps the rest of the transform
                                       in registers, clip scoring runs as in 3 (GBS_NO_UVR=1 forces 3) (set GBS_FORCE_GENERIC=1 in the
@@ -224,10 +225,13 @@ int gbs_static_device_status(int* out);
  *   codes, scales  device, layouts as written by gbs_rotate_quantize
  *   out            device, n_rows * (d' or d) elements of out_dtype, rows contiguous,
  *                  16-byte aligned
- * The inverse rotation of plans with one symmetric scale per token in the tensor-core family
- * (widths d' = 32 U, 16 <= U <= 128, d a multiple of 32), and of d' = 128 rows with one scale or
- * (Delta, lo) pair per row, runs on the tensor cores: the integer codes are rotated exactly and
- * multiplied by Delta / sqrt(d') once at the end.
+ * The inverse rotation of symmetric plans with d' = 32 U (d a multiple of 32) or, beyond 4096, d' = 64 U (d a multiple of
+ * 64), 16 <= U <= 128, and one scale per token or per group of at least 32 or 64 runs on the tensor cores; with one scale
+ * the integer codes are rotated exactly and multiplied by Delta / sqrt(d') once at the end, with groups the operand
+ * q * Delta is held to 22 bits below the token's largest scale.  Where m = 1, d' <= 2048 and the plan has groups, a
+ * general kernel takes widths and numbers of rows at which it is faster; a row's result may then differ in the last fp32
+ * bits with the number of rows.  d' = 128 rows with one scale or (Delta, lo) pair per row are rotated exactly in
+ * registers.
  */
 int gbs_dequantize(const gbs_plan_t* plan, const void* codes, const float* scales, int64_t n_rows,
                    void* out, int out_dtype, int flags, void* cuda_stream);
@@ -241,6 +245,10 @@ int gbs_dequantize(const gbs_plan_t* plan, const void* codes, const float* scale
  *   K             1 .. GBS_MAX_CANDIDATES
  *   err_sum       device, K doubles, ACCUMULATED into (the caller zeroes them)
  *   err_rows_opt  NULL, or device n_rows * K floats receiving the per-row sums
+ * Which kernel scores a call depends on its shape, its list and whether per-row sums are asked for: one histogram for all
+ * candidates (d' <= 4096, group 0, bf16) or a pass per eight.  Both round each residual to about 2^-23 max|y|, so one alpha's
+ * sum from two calls agrees to about 1e-7 of the sum where the rows are ordinary, and to 2^-22 max|y| sqrt(n err) where the
+ * candidate fits n values almost exactly; a search that compares sums from different calls decides closer ties by chance.
  */
 int gbs_clip_error(const gbs_plan_t* plan, const void* x, int x_dtype, int64_t n_rows,
                    int64_t x_row_stride, const float* alphas_host, int K, double* err_sum,
@@ -297,8 +305,8 @@ int gbs_weight_rotate_quantize(const gbs_plan_t* plan, const void* w, int w_dtyp
  * tensor cores (exact); the rotated activation is never materialised as floats.
  *   plan_x, codes_x, scales_x, n_tokens   activations as written by gbs_rotate_quantize
  *   plan_w, codes_w, scales_w, n_out      weights as written by gbs_weight_rotate_quantize
- *   out, out_dtype, out_row_stride        device, [n_tokens, n_out] fp32 or bf16, row stride in elements (>= n_out);
- *                                         rows that start on 16-byte boundaries get vector stores
+ *   out, out_dtype, out_row_stride        device, [n_tokens, n_out] fp32 or bf16, row stride in elements (>= n_out),
+ *                                         any alignment of its type
  * Limits: both plans on one device with the same d, d' and m, symmetric, group 0 (one scale per token and per
  * output channel, so the scales leave the sum), d' a multiple of 128; bits may differ (3 or 4 each).  Other plans
  * return GBS_ERR_UNSUPPORTED.

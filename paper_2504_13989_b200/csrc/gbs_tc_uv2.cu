@@ -13,8 +13,9 @@
 //   * Maxima: one scale per token over the warps of the token (named barrier), or one per group of 64 * 2^g coordinates over
 //     2^g lanes and the two halves (shuffles and a barrier of the pair).  Delta, rounding, clipping, packing as everywhere
 //     (Sections 2.1, 3.1).
-// What bounds it: instruction issue, as for the narrower widths.  8192 rows, 4 bits, one scale per token: 8192 wide 46.8 us on
-// the three-sweep kernel, 42.5 here; 5120 wide 41.1 -> 34.8; 5120 wide, 3 bits, groups of 128: 44.1 -> 30.4.
+// What bounds it: instruction issue, as for the narrower widths.  8192 rows, 4 bits, one scale per token, called back to back for
+// seconds: 8192 wide 46.8 us on the three-sweep kernel, 42.5 here; 5120 wide 41.1 -> 34.8; 5120 wide, 3 bits, groups of 128: 44.1 -> 30.4.
+// In bursts, on a cool GPU: 35.0, 32.1 and 27.6.
 // Every wait is bounded; an expired wait records a code in the plan's status word.  A warp whose wait ran out brings a pattern no
 // maximum can have to the barrier it shares, and all who meet it there leave their loop with it.  With one scale per token they go on
 // bringing it to the barriers of the tiles that are left: a warp that rested in this tile knows nothing of it yet and will wait for

@@ -14,8 +14,8 @@
 //     (Sections 2.1, 3.1) from registers.
 // What bounds it: latency.  A warp issues about 700 instructions per 32 values of a lane (220 of them the split) at 8 cycles
 // each, sixteen warps cover half of that, and taking out any one part (two of three planes, the split, the epilogue) gains
-// less than a tenth.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 16.6 now; 7000 x 3584, groups of 128: 117.6 ->
-// 27.7; 7000 x 8192, 4 bits: 61.7.  Tried and slower: loads reissued piece by piece inside the split; tiles prefetched into L2
+// less than a tenth.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 16.95 now; 7000 x 3584, groups of 128: 117.6
+// -> 28.3; 7000 x 8192, 4 bits: 63.3.  Tried and slower: loads reissued piece by piece inside the split; tiles prefetched into L2
 // further ahead; the prefetches in a warp of their own that waits for the splits (18.2, 31.4 and 73.3 us).
 // Every wait is bounded; an expired wait records a code in the plan's status word, and a warp whose wait ran out brings a
 // pattern no maximum can have to the barrier it shares, so that all who wait there leave with it.

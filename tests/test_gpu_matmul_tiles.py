@@ -1,5 +1,5 @@
-"""gbs_quantized_matmul at the edges of its kernels: the few-token kernel and the tile kernel on either side of 64 tokens, single
-SMs and SM pairs, ragged channels and tokens, every pair of bit widths.  Codes are drawn directly; the expected value is the
+"""gbs_quantized_matmul at the edges of its kernels: the few-token kernel and the tile kernel on either side of the rule between
+them, narrow and wide tiles, ragged channels and tokens, every pair of bit widths.  Codes are drawn directly; the expected value is the
 float64 product of the unpacked codes (exact: |sum| <= 49 d' < 2^53) times the two scales."""
 import numpy as np
 import pytest
@@ -25,8 +25,8 @@ def _codes(n, d, bits, seed):
 @pytest.mark.parametrize("d,n_tok,n_out", [
     (128, 1, 16), (128, 8, 17), (256, 9, 31), (1024, 17, 33), (1024, 33, 100), (1024, 64, 257),       # the few-token kernel
     (128, 1, 18000), (256, 16, 9001), (128, 16, 18300), (256, 17, 11003), (256, 33, 4400), (128, 64, 6001),   # few tokens, many channels
-    (128, 65, 1), (384, 65, 127), (1024, 96, 128), (640, 129, 129), (1024, 191, 1000),                # single SMs
-    (512, 3000, 4090), (256, 4097, 5000), (128, 20000, 300), (384, 97, 40000),                        # enough tiles for pairs
+    (128, 65, 1), (384, 65, 127), (1024, 96, 128), (640, 129, 129), (1024, 191, 1000),                # tiles, few
+    (512, 3000, 4090), (256, 4097, 5000), (128, 20000, 300), (384, 97, 40000),                        # several waves of tiles
 ])
 @pytest.mark.parametrize("bx,bw,dtype", [(4, 4, torch.bfloat16), (3, 3, torch.float32), (3, 4, torch.float32), (4, 3, torch.bfloat16)])
 def test_against_the_exact_integer_product(d, n_tok, n_out, bx, bw, dtype):
