@@ -5,7 +5,7 @@
 // With D' = alpha_k / D the error is  M^2 (t - D' l)^2 = M^2 [t^2 - 2 D' t l + D'^2 l^2],  so all K candidates follow from how
 // many values (W0) and which sum of t (W1) lie beyond each of the K D thresholds:
 //        sum t l = sum_j W1(beyond threshold j),    sum l^2 = sum_j (2 j + 1) W0(beyond threshold j).
-// One histogram over the sorted thresholds replaces 5 K operations per value by about 15 whatever K is.
+// One histogram over the sorted thresholds replaces 5 K operations per value by about 12 whatever K is.
 //   * Front end as in gbs_tc_uv.cu: TMA, A X on tcgen05, H_32 in registers, the token's maximum over its four warps.
 //   * t becomes a 22-bit integer in the mantissa of one FMA.  Its high 12 bits index a table of cells; an entry holds the
 //     number of thresholds below the cell and the low 10 bits of the one threshold inside it, placed so that adding the
