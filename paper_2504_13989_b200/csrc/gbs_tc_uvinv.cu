@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
         const unsigned swz = V == 32 ? (unsigned)((up >> 1) & 3) : (unsigned)(up & 7);
         const int n_grp = (n_mine - grp + GROUPS - 1) / GROUPS;    // tiles of this group
         const long long row_first = t < P.tok ? ((long long)blockIdx.x + (long long)grp * gridDim.x) * P.tok + t : P.n_rows;
-        const long long row_step = (long long)GROUPS * gridDim.x * P.tok;
+        const long long row_step = (long long)GROUPS * gridDim.x * TOK;            // fewer than TOK to a tile: one tile per block
         const bool live_u = up < P.U;
 
         // Packed codes and scales of one tile, fetched two tiles ahead of their unpacking (one tile is less than the latency
