@@ -148,6 +148,16 @@ __device__ __forceinline__ void umma_f16_words(unsigned d_tmem, unsigned a_lo, u
 {
     umma_f16(d_tmem, (unsigned long long)a_hi << 32 | a_lo, (unsigned long long)b_hi << 32 | b_lo, idesc, ACCUMULATE ? 1u : 0u);
 }
+// A from tensor memory (a row per lane, two bf16 per column), B from shared memory
+__device__ __forceinline__ void umma_f16_ts(unsigned d_tmem, unsigned a_tmem, unsigned long long b_desc, unsigned idesc, unsigned accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void umma_commit(void* bar)
 {
     asm volatile(
@@ -185,6 +195,14 @@ __device__ __forceinline__ void tmem_ld_wait(unsigned r[32])
         :: "memory");
 }
 
+// 16 registers -> 16 columns of this thread's TMEM lane (asynchronous)
+__device__ __forceinline__ void tmem_st16(unsigned taddr, const uint4 w[4])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};"
+        ::"r"(w[0].x), "r"(w[0].y), "r"(w[0].z), "r"(w[0].w), "r"(w[1].x), "r"(w[1].y), "r"(w[1].z), "r"(w[1].w),
+          "r"(w[2].x), "r"(w[2].y), "r"(w[2].z), "r"(w[2].w), "r"(w[3].x), "r"(w[3].y), "r"(w[3].z), "r"(w[3].w), "r"(taddr) : "memory");
+}
 // 16 columns of this thread's TMEM lane (asynchronous)
 __device__ __forceinline__ void tmem_ld16_issue(unsigned taddr, unsigned r[16])
 {

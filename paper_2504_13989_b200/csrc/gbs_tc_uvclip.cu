@@ -7,26 +7,29 @@
 //        sum t l = sum_j W1(beyond threshold j),    sum l^2 = sum_j (2 j + 1) W0(beyond threshold j).
 // One histogram over the sorted thresholds replaces 5 K operations per value by about 12 whatever K is.
 //   * Front end as in gbs_tc_uv.cu: TMA, A X on tcgen05, H_32 in registers, the token's maximum over its four warps.
-//   * t becomes a 22-bit integer in the mantissa of one FMA.  Its high 12 bits index a table of cells; an entry holds the
-//     number of thresholds below the cell and the low 10 bits of the one threshold inside it, placed so that adding the
-//     value's low bits carries into the bin index when the threshold is reached.  (The host takes this path only where no two
-//     different thresholds share a cell.  Thresholds that are one and the same number, such as 1.5 x 0.5 and 0.5 x 1.5 over D, may come
+//   * t becomes a 22-bit integer in the mantissa of one FMA.  Its high bits index a table of cells; an entry holds the
+//     number of thresholds below the cell and the low bits of the one threshold inside it, placed so that adding the
+//     value's low bits carries into the bin index when the threshold is reached.  Cells are as wide as they can be without two
+//     different thresholds in one (512 of them do for ratios k / 64 and 3 bits), and the room that leaves in the table's 64 KB holds copies
+//     of an entry side by side, one per lane at 512 cells: lanes then meet in a bank as rarely as the copies allow (one copy of
+//     4096 cells: 3.4 cycles per lookup of a warp).  (Below 4096 cells' width the call goes to the per-candidate kernel.
+//     Thresholds that are one and the same number, such as 1.5 x 0.5 and 0.5 x 1.5 over D, may come
 //     out one unit of t apart when the ratios are rounded to floats; they count as one, the lower.)
-//   * Two shared-memory atomics per value (count, and the FMA's bits themselves: the exponent pattern is removed with the count)
+//   * Two shared-memory atomics per value (count and t)
 //     into COPIES interleaved histograms per token, so that a warp's lanes rarely meet: measured 2 cycles per 32 values with 32
-//     copies and 6 with 8, against 3 - 4 for the table lookup.  Everything is an integer: exact in any order.
-//   * After a token its 128 threads add the copies up, weigh them with M^2 in fp64 and clear them.  The t^2 term is the sum of the
+//     copies and 6 with 8.  Everything is an integer: exact in any order.
+//   * After a token its 128 threads add the copies up and weigh them with M^2 in fp64.  Nothing is cleared: the words grow modulo 2^32
+//     and a token's part is the difference from the total before it, which its thread keeps.  The t^2 term is the sum of the
 //     same integers' squares, in 64 bits, so the three parts of the error belong to one and the same t and may cancel down to the
 //     16 digits of fp64: a candidate that fits a batch exactly is as accurate as the others, wherever it stands in the list.
 //     t's rounding is the only approximation: at most 2^-23, so that an error E over n values moves by at most
 //     2^-22 M sqrt(n E) + n 2^-46 M^2 -- the size of Delta's rounding in the per-candidate kernel -- and, where the values differ,
 //     by the square root of n less.
-// What bounds it: the shared-memory port: per token about 430 cycles of lookups, 330 of atomics, 390 of adding up and clearing and
-// 130 of the MMA's operands.
-// 32 768 x 4096, K = 32: 829 us with five fp32 operations per value and candidate; now 171 us at 3 bits (32 copies), 250 us at
-// 4 bits (16 copies); K = 8: 249 -> 156 us, K = 1: 249 -> 155 (the per-candidate kernel takes eight at a time).  512 rows, K = 8:
-// 19.6 -> 13.3 us.  With the error of candidate 0 summed directly and the others as differences from it, which loses a
-// candidate whose error is far smaller (equal magnitudes, alpha = 1: negative sums), the first two were 189 and 252 us.
+//   * A stands in tensor memory, so that an MMA reads one operand from shared memory and the table has the other's room.
+// What bounds it: the shared-memory port (per token about 130 cycles of lookups, 330 of atomics, 200 of adding up, 65 of the MMA's operand)
+// and instruction issue (about 700 slots of each scheduler).
+// 32 768 x 4096, K = 32, 3 bits: 829 us with five fp32 operations per value and candidate; 171.4 with one copy of the table, histograms
+// that were cleared for every token (390 cycles with the adding up) and A in shared memory; 135.2 now.
 #include <math.h>
 #include <string.h>
 
@@ -38,28 +41,28 @@
 namespace {
 
 constexpr int V = 32, TOK = 4, UMAX = 128;
-constexpr int STAGES = 2;                          // a tile takes far longer than its loads
+constexpr int STAGES = 2;                          // accumulators; one set of rows in shared memory: a tile takes far longer than its load
 constexpr int STAGE_COLS = TOK * V;
 constexpr int STAGE_BYTES_MAX = TOK * UMAX * V * 2;
-constexpr int A_BYTES = UMAX * UMAX * 2;
+constexpr int A_COL0 = STAGES * STAGE_COLS;        // A in tensor memory: a row per lane, two entries per column
 constexpr int EPI_WARPS = 4 * TOK;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
-constexpr int TMEM_COLS = 256;
-constexpr int CELL_BITS = 10, CELLS = 1 << 12;     // t is an integer of 22 bits
+constexpr int TMEM_COLS = 512;
+constexpr int T_BITS = 22;                         // t is an integer of 22 bits
+constexpr int TABLE_LOG = 14;                      // words of the table of cells: cells x copies
+constexpr int MIN_CELL_BITS = 10, MAX_CELL_BITS = 13;          // bits of t inside a cell: 4096 cells x 4 copies .. 512 x 32
 constexpr int HIST_ROWS = 3584;                    // words of a token's counts (and of its sums): bins x copies
 constexpr int HIST_WORDS = TOK * 2 * (HIST_ROWS + 32);   // [token][count, sum][one row nobody reads, bins][copy]
 constexpr int MAX_BINS = 448;                      // thresholds: K D at most
 constexpr unsigned POISON = 0xffffffffu;
 
 struct __align__(1024) Smem {
-    unsigned char a[A_BYTES];
-    unsigned char b[STAGES][STAGE_BYTES_MAX];
+    unsigned char b[STAGE_BYTES_MAX];
     unsigned hist[HIST_WORDS];
-    unsigned lut[CELLS];
+    unsigned lut[1 << TABLE_LOG];
     unsigned red[TOK][2][4];                       // maxima, by tile parity
     double square[EPI_WARPS];                      // sums of t^2
-    unsigned long long full[STAGES], empty[STAGES], tfull[STAGES], tempty[STAGES];
-    unsigned long long abar;
+    unsigned long long full, empty, tfull[STAGES], tempty[STAGES];
     unsigned tmem_base;
     volatile int abort_flag;
 };
@@ -69,6 +72,7 @@ struct ClipParams {
     int n_groups;                 // ceil(n_rows / TOK)
     int U, Upad, ksteps;
     int K, levels, n_thr;
+    int cell_bits;                // the largest number for which no cell holds two different thresholds
     float scale;                  // of t as an integer
     float norm2;                  // 1 / d'
     const unsigned char* a_img;
@@ -98,46 +102,62 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     const unsigned stage_bytes = (unsigned)(TOK * P.Upad * V * 2);
 
     if (threadIdx.x == 0) {
+        mbar_init(&S->full, 1);
+        mbar_init(&S->empty, 1);
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&S->full[s], 1);
-            mbar_init(&S->empty[s], 1);
             mbar_init(&S->tfull[s], 1);
             mbar_init(&S->tempty[s], EPI_WARPS);
         }
-        mbar_init(&S->abar, 1);
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mbar_arrive_expect_tx(&S->abar, A_BYTES);
-        bulk_load(S->a, P.a_img, A_BYTES, &S->abar);          // plan-owned, immutable: needs no ordering
     }
     if (warp == 1) tmem_alloc(&S->tmem_base, TMEM_COLS);
     for (int i = threadIdx.x; i < HIST_WORDS / 4; i += THREADS) reinterpret_cast<uint4*>(S->hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x < EPI_WARPS) S->square[threadIdx.x] = 0.0;
-    unsigned* thr = reinterpret_cast<unsigned*>(S->b[0]);          // the first loads come later
+    unsigned* thr = reinterpret_cast<unsigned*>(S->b);             // the first load comes later
     for (int i = threadIdx.x; i < P.n_thr; i += THREADS) thr[i] = P.thr[i];
+    tc_fence_before();
     __syncthreads();
-    {
+    tc_fence_after();
+    const unsigned tmem_base = S->tmem_base;
+    const int copies_log = P.cell_bits + TABLE_LOG - T_BITS;       // of an entry: 4 .. 32, side by side
+    if (threadIdx.x < (1 << (T_BITS - MAX_CELL_BITS))) {
         // cell c: thresholds below it, and where the one inside it lies; a run of cells per thread, found by one binary search
-        constexpr int RUN = (CELLS + THREADS - 1) / THREADS;
-        const int c0 = threadIdx.x * RUN;
+        const int run = 1 << (MAX_CELL_BITS - P.cell_bits), c0 = threadIdx.x * run;
+        const unsigned in_cell = 1u << P.cell_bits;
         int lo = 0, hi = P.n_thr;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if (thr[mid] < ((unsigned)c0 << CELL_BITS)) lo = mid + 1; else hi = mid;
+            if (thr[mid] < ((unsigned)c0 << P.cell_bits)) lo = mid + 1; else hi = mid;
         }
-        for (int c = c0; c < c0 + RUN && c < CELLS; ++c) {
-            unsigned e = (unsigned)lo << CELL_BITS;
+        for (int c = c0; c < c0 + run; ++c) {
+            unsigned e = (unsigned)lo << P.cell_bits;
             const unsigned next = lo < P.n_thr ? thr[lo] : 0xffffffffu;
-            if ((next >> CELL_BITS) == (unsigned)c) { e += (1u << CELL_BITS) - (next & ((1u << CELL_BITS) - 1u)); ++lo; }
-            S->lut[c] = e;
+            if ((next >> P.cell_bits) == (unsigned)c) { e += in_cell - (next & (in_cell - 1u)); ++lo; }
+            uint4* entry = reinterpret_cast<uint4*>(S->lut + (c << copies_log));
+            const int quads = 1 << (copies_log - 2);
+            for (int j = 0; j < quads; ++j) entry[(j + lane) & (quads - 1)] = make_uint4(e, e, e, e);   // lanes side by side: different banks
         }
+    }
+    if (warp >= 2 && warp < 6) {
+        // A (plan-owned, immutable: needs no ordering) from its image, two blocks of 64 columns, 128-byte swizzled rows, to tensor memory
+        const int r = (warp & 3) * 32 + lane;
+        const unsigned at = tmem_base + ((unsigned)((warp & 3) * 32) << 16) + A_COL0;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            uint4 w[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                w[c] = __ldg(reinterpret_cast<const uint4*>(P.a_img + (h >> 1) * (UMAX * 128) + r * 128 + (((4 * (h & 1) + c) ^ (r & 7)) << 4)));
+            tmem_st16(at + h * 16, w);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const unsigned tmem_base = S->tmem_base;
     const int n_mine = (P.n_groups - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
 
     double w0[PER], w1[PER];
@@ -146,40 +166,30 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     if (warp == 0) {
         // ------------------------------ TMA producer ------------------------------
         if (lane == 0) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the thresholds read from the first stage
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the thresholds were read from where the rows go
             int it = 0;
             for (int g = blockIdx.x; g < P.n_groups; g += gridDim.x, ++it) {
-                const int s = it % STAGES;
-                if (!mbar_wait(&S->abort_flag, &S->empty[s], ((it / STAGES) & 1) ^ 1, P.status, 1)) break;
-                mbar_arrive_expect_tx(&S->full[s], stage_bytes);
-                tma_load_3d(S->b[s], &tmap, &S->full[s], 0, 0, g * TOK);
+                if (!mbar_wait(&S->abort_flag, &S->empty, (it & 1) ^ 1, P.status, 1)) break;
+                mbar_arrive_expect_tx(&S->full, stage_bytes);
+                tma_load_3d(S->b, &tmap, &S->full, 0, 0, g * TOK);
             }
-            if (S->abort_flag) drain_copies(S->full, STAGES, it);
+            if (S->abort_flag) drain_copies(&S->full, 1, it);
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ------------------------------
         {
             constexpr unsigned IDESC = instr_desc(UMAX, STAGE_COLS);
-            const unsigned long long ad0 = smem_desc(smem_u32(S->a), 16, 1024, 2);
-            const unsigned long long bd0 = smem_desc(smem_u32(S->b[0]), (unsigned)(P.Upad * V * 2), 512, 4);
-            const unsigned ad_lo0 = (unsigned)ad0, ad_hi = (unsigned)(ad0 >> 32);
-            const unsigned bd_lo0 = (unsigned)bd0, bd_hi = (unsigned)(bd0 >> 32);
-            bool ok = mbar_wait_warp(&S->abort_flag, &S->abar, 0, P.status, 6);
-            for (int it = 0; ok && it < n_mine; ++it) {
+            const unsigned long long bd0 = smem_desc(smem_u32(S->b), (unsigned)(P.Upad * V * 2), 512, 4);
+            for (int it = 0; it < n_mine; ++it) {
                 const int s = it % STAGES;
-                const unsigned ph = (it / STAGES) & 1;
-                if (!mbar_wait_warp(&S->abort_flag, &S->full[s], ph, P.status, 2)) break;
-                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[s], ph ^ 1, P.status, 3)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->full, it & 1, P.status, 2)) break;
+                if (!mbar_wait_warp(&S->abort_flag, &S->tempty[s], ((it / STAGES) & 1) ^ 1, P.status, 3)) break;
                 tc_fence_after();
-                unsigned a_lo = ad_lo0, b_lo = bd_lo0 + (unsigned)s * (STAGE_BYTES_MAX >> 4);
+                // a k-step: eight columns of A's lanes, 1024 bytes of the rows
                 const unsigned d_tmem = tmem_base + s * STAGE_COLS;
-                umma_f16_words<false>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
-                for (int ks = 1; ks < P.ksteps; ++ks) {
-                    a_lo += (ks & 3) ? 2u : (unsigned)((UMAX * 128 - 96) >> 4);
-                    b_lo += 1024u >> 4;
-                    umma_f16_words<true>(d_tmem, a_lo, ad_hi, b_lo, bd_hi, IDESC);
-                }
-                umma_commit(&S->empty[s]);
+                for (int ks = 0; ks < P.ksteps; ++ks)
+                    umma_f16_ts(d_tmem, tmem_base + A_COL0 + ks * 8, bd0 + (unsigned long long)(ks * (1024 >> 4)), IDESC, ks != 0 ? 1u : 0u);
+                umma_commit(&S->empty);
                 umma_commit(&S->tfull[s]);
             }
         }
@@ -193,7 +203,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         // bin b (b thresholds reached) is row b - 1: bin 0 lands in the row before the first, which costs less than a predicate
         // (a predicated reduction becomes a branch: 264 us instead of 250)
         const unsigned hb = smem_u32(hist) + (unsigned)(lane % COPIES) * 4u - BIN_STEP;
-        const unsigned lut = smem_u32(S->lut);
+        const unsigned lut = smem_u32(S->lut) + ((unsigned)(lane & ((1 << copies_log) - 1)) << 2);
+        const unsigned cell_mask = (4u << TABLE_LOG) - (4u << copies_log);        // a cell's first byte in the table
+        const unsigned low_mask = (1u << P.cell_bits) - 1u;
+        const int cell_bits = P.cell_bits;
+        // the histograms only ever grow, modulo 2^32: a token's own counts and sums are what a bin has gained since the token before
+        unsigned was0[PER], was[PER][4];
+#pragma unroll
+        for (int i = 0; i < PER; ++i) was0[i] = was[i][0] = was[i][1] = was[i][2] = was[i][3] = 0u;
         constexpr float MAGIC = 8388608.f;
         constexpr unsigned E = 0x4B000000u;                       // its bit pattern
         double square = 0.0;
@@ -237,13 +254,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     b[i] = __float_as_uint(fmaf(fabsf(__uint_as_float(r[i0 + i])), sc, MAGIC));
-                    e[i] = ld_shared(lut + ((b[i] >> (CELL_BITS - 2)) & (unsigned)(4 * CELLS - 4)));
+                    e[i] = ld_shared(lut + ((b[i] >> (T_BITS - TABLE_LOG - 2)) & cell_mask));
                 }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) sq += (unsigned long long)(b[i] - E) * (b[i] - E);
+                for (int i = 0; i < 8; ++i) {
+                    b[i] -= E;
+                    sq += (unsigned long long)b[i] * b[i];
+                }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const unsigned bin = (e[i] + (b[i] & ((1u << CELL_BITS) - 1u))) >> CELL_BITS;
+                    const unsigned bin = (e[i] + (b[i] & low_mask)) >> cell_bits;
                     const unsigned at = hb + bin * BIN_STEP;
                     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at) : "memory");
                     asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(at), "r"(b[i]), "n"(SUM_OFF) : "memory");
@@ -256,23 +276,24 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
             for (int i = 0; i < PER; ++i) {
                 const int bin = ti + 128 * i;
                 if (bin < P.n_thr) {
-                    uint4* row = reinterpret_cast<uint4*>(hist + bin * COPIES);
-                    uint4* row1 = reinterpret_cast<uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
-                    uint4 c = make_uint4(0u, 0u, 0u, 0u), m = c;
-                    const uint4 zero = c;
+                    const uint4* row = reinterpret_cast<const uint4*>(hist + bin * COPIES);
+                    const uint4* row1 = reinterpret_cast<const uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
+                    unsigned c = 0u;
+                    uint4 m = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                     for (int j = 0; j < COPIES / 4; ++j) {
                         const int jj = (j + lane) % (COPIES / 4);          // eight lanes side by side: different banks
                         const uint4 x = row[jj], z = row1[jj];
-                        row[jj] = zero;
-                        row1[jj] = zero;
-                        c.x += x.x; c.y += x.y; c.z += x.z; c.w += x.w;
+                        c += (x.x + x.y) + (x.z + x.w);
                         m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
                     }
-                    // a component has at most 1024 values below 2^22: what is left without the exponent patterns fits 32 bits
-                    const double sum = (double)(m.x - c.x * E) + (double)(m.y - c.y * E) + (double)(m.z - c.z * E) + (double)(m.w - c.w * E);
-                    w0[i] += m2 * (double)(c.x + c.y + c.z + c.w);
-                    w1[i] += m2 * sum;
+                    // a component gains at most 1024 values below 2^22: less than 2^32
+                    const unsigned long long sum = ((unsigned long long)(m.x - was[i][0]) + (m.y - was[i][1])) +
+                                                   ((unsigned long long)(m.z - was[i][2]) + (m.w - was[i][3]));
+                    w0[i] += m2 * (double)(c - was0[i]);
+                    w1[i] += m2 * (double)sum;
+                    was0[i] = c;
+                    was[i][0] = m.x; was[i][1] = m.y; was[i][2] = m.z; was[i][3] = m.w;
                 }
             }
         }
@@ -359,20 +380,34 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
     const int D = p->levels;
     // t = 1 must stay below 2^22 after rounding
     P.scale = 4194304.f - 8.f;
-    unsigned long long used[CELLS / 64] = {0};
-    unsigned at[CELLS], last[CELLS];               // the lowest and the highest threshold of a cell
-    unsigned short rank[CELLS];
+    // the widest cells that no two different thresholds share
+    constexpr int CELLS = 1 << (T_BITS - MIN_CELL_BITS);
     constexpr unsigned SAME = 1;                   // alpha rounds to 2^-25, an eighth of a unit; ceil makes one of it
+    unsigned T[GBS_MAX_CANDIDATES * 7];
     for (int k = 0; k < K; ++k)
         for (int j = 0; j < D; ++j) {
-            const unsigned T = (unsigned)ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale), c = T >> CELL_BITS;
-            if (c >= CELLS) return GBS_UVCLIP_NOT_SERVED;
+            const double t = ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale);
+            if (!(t < (double)(1 << T_BITS))) return GBS_UVCLIP_NOT_SERVED;
+            T[k * D + j] = (unsigned)t;
+        }
+    unsigned long long used[CELLS / 64];
+    unsigned at[CELLS], last[CELLS];               // the lowest and the highest threshold of a cell
+    unsigned short rank[CELLS];
+    bool apart = false;
+    for (P.cell_bits = MAX_CELL_BITS; P.cell_bits >= MIN_CELL_BITS; --P.cell_bits) {
+        memset(used, 0, sizeof(used));
+        apart = true;
+        for (int i = 0; apart && i < K * D; ++i) {
+            const unsigned c = T[i] >> P.cell_bits;
             const bool seen = used[c >> 6] >> (c & 63) & 1;
-            at[c] = seen && at[c] < T ? at[c] : T;
-            last[c] = seen && last[c] > T ? last[c] : T;
-            if (last[c] - at[c] > SAME) return GBS_UVCLIP_NOT_SERVED;
+            at[c] = seen && at[c] < T[i] ? at[c] : T[i];
+            last[c] = seen && last[c] > T[i] ? last[c] : T[i];
+            apart = last[c] - at[c] <= SAME;
             used[c >> 6] |= 1ull << (c & 63);
         }
+        if (apart) break;
+    }
+    if (!apart) return GBS_UVCLIP_NOT_SERVED;
     for (int w = 0; w < CELLS / 64; ++w)
         for (unsigned long long m = used[w]; m; m &= m - 1) {
             const int c = w * 64 + __builtin_ctzll(m);
@@ -381,8 +416,7 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
         }
     for (int k = 0; k < K; ++k) {
         P.alpha[k] = alphas[k];
-        for (int j = 0; j < D; ++j)
-            P.idx[k][j] = rank[(unsigned)ceil((j + 0.5) / D * (double)alphas[k] * (double)P.scale) >> CELL_BITS];
+        for (int j = 0; j < D; ++j) P.idx[k][j] = rank[T[k * D + j] >> P.cell_bits];
     }
     CUtensorMap tmap;
     const int U = p->d_pad / V;
