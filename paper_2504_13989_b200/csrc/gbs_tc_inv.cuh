@@ -71,6 +71,21 @@ __device__ __forceinline__ void rotate_octet(const unsigned* w, int o, unsigned 
     }
 }
 
+// sixteen values as the output type's words
+__device__ __forceinline__ void pack_values(const float f[16], unsigned w[16], float)
+{
+#pragma unroll
+    for (int e = 0; e < 16; ++e) w[e] = __float_as_uint(f[e]);
+}
+__device__ __forceinline__ void pack_values(const float f[16], unsigned w[16], __nv_bfloat16)
+{
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const __nv_bfloat162 b2 = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+        w[e] = *reinterpret_cast<const unsigned*>(&b2);
+    }
+}
+
 // 32 bytes: one store where the address allows (a full DRAM sector per thread), else two
 __device__ __forceinline__ void store32(void* p, const unsigned w[8], bool wide)
 {

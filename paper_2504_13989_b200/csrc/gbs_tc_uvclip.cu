@@ -12,12 +12,11 @@
 //     value's low bits carries into the bin index when the threshold is reached.  Cells are as wide as they can be without two
 //     different thresholds in one (512 of them do for ratios k / 64 and 3 bits), and the room that leaves in the table's 64 KB holds copies
 //     of an entry side by side, one per lane at 512 cells: lanes then meet in a bank as rarely as the copies allow (one copy of
-//     4096 cells: 3.4 cycles per lookup of a warp).  (Below 4096 cells' width the call goes to the per-candidate kernel.
+//     4096 cells: 3.4 cycles per lookup of a warp).  (Where 4096 cells do not part them the call goes to the per-candidate kernel.
 //     Thresholds that are one and the same number, such as 1.5 x 0.5 and 0.5 x 1.5 over D, may come
 //     out one unit of t apart when the ratios are rounded to floats; they count as one, the lower.)
-//   * Two shared-memory atomics per value (count and t)
-//     into COPIES interleaved histograms per token, so that a warp's lanes rarely meet: measured 2 cycles per 32 values with 32
-//     copies and 6 with 8.  Everything is an integer: exact in any order.
+//   * Two shared-memory atomics per value (count and t) into COPIES interleaved histograms per token, so that a warp's lanes
+//     rarely meet: measured 2 cycles per 32 values with 32 copies and 6 with 8.  Everything is an integer: exact in any order.
 //   * After a token its 128 threads add the copies up and weigh them with M^2 in fp64.  Nothing is cleared: the words grow modulo 2^32
 //     and a token's part is the difference from the total before it, which its thread keeps.  The t^2 term is the sum of the
 //     same integers' squares, in 64 bits, so the three parts of the error belong to one and the same t and may cancel down to the

@@ -1,0 +1,34 @@
+"""KV rows restored (gbs_dequantize with inverse rotation, d' = 128): ragged last blocks and every output width, whose stores leave shared
+memory in pieces of 128 bytes; against the float64 transform of the dequantized codes, and nothing written behind the last row."""
+import numpy as np
+import pytest
+import scipy.linalg
+import torch
+
+from paper_2504_13989_b200 import Plan
+from paper_2504_13989_b200 import build as gbs_build
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("d", [32, 64, 96, 128])
+@pytest.mark.parametrize("rows", [1, 31, 32, 33, 5000])
+@pytest.mark.parametrize("bits,asym,dtype", [(4, True, torch.bfloat16), (3, False, torch.bfloat16), (3, True, torch.float32), (4, False, torch.float32)])
+def test_rows_and_widths(d, rows, bits, asym, dtype):
+    gbs_build.build()
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(rows + d)
+    x = torch.randn((rows, d), generator=gen, device=DEV).pow(3).to(torch.bfloat16)
+    h = torch.from_numpy(scipy.linalg.hadamard(128).astype(np.float64)).to(DEV)
+    with Plan(d, 128, 1, bits, 128, 1.0, asymmetric=asym) as plan:
+        codes, scales, _ = plan.rotate_quantize(x)
+        y = plan.dequantize(codes, scales, inverse=False, dtype=torch.float32).double()
+        out = torch.full((rows + 1, d), 7.0, dtype=dtype, device=DEV)
+        plan.dequantize(codes, scales, inverse=True, out=out[:rows])
+        torch.cuda.synchronize()
+        assert plan.device_status() == 0 and bool((out[rows] == 7.0).all())
+    want = (y @ h / np.sqrt(128.0))[:, :d]
+    # y is rounded to 2^-24 of its largest, 128 terms; the result once more, to its own type
+    bound = 2.0 ** -24 * 128 / np.sqrt(128.0) * y.abs().amax(dim=1, keepdim=True) + (2.0 ** -8 if dtype == torch.bfloat16 else 2.0 ** -22) * want.abs()
+    assert bool(((out[:rows].double() - want).abs() <= bound).all())
