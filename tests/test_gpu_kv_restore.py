@@ -29,6 +29,8 @@ def test_rows_and_widths(d, rows, bits, asym, dtype):
         torch.cuda.synchronize()
         assert plan.device_status() == 0 and bool((out[rows] == 7.0).all())
     want = (y @ h / np.sqrt(128.0))[:, :d]
-    # y is rounded to 2^-24 of its largest, 128 terms; the result once more, to its own type
-    bound = 2.0 ** -24 * 128 / np.sqrt(128.0) * y.abs().amax(dim=1, keepdim=True) + (2.0 ** -8 if dtype == torch.bfloat16 else 2.0 ** -22) * want.abs()
+    # y = q Delta + lo comes with two roundings of numbers up to 2 max|y|, and 128 of them add up here; the kernel multiplies the exact sum
+    # (up to 2 * 128 max|y| / Delta) by Delta / sqrt(128), three roundings, and adds 128 lo / sqrt(128), three more
+    bound = 2.0 ** -24 * (2 * 2 + 6 * 2) * 128 / np.sqrt(128.0) * y.abs().amax(dim=1, keepdim=True)
+    bound = bound + (2.0 ** -8 if dtype == torch.bfloat16 else 2.0 ** -23) * want.abs()
     assert bool(((out[:rows].double() - want).abs() <= bound).all())
