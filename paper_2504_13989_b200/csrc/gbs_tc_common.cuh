@@ -106,6 +106,12 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int c0, 
                  ::"l"(map), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 
+// The same of plain memory: 16-byte aligned, a multiple of 16 bytes.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, void* bar)
 {
     asm volatile(

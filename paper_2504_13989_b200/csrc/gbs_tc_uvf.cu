@@ -110,6 +110,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         mbar_arrive_expect_tx(&S->abar, A_BYTES);
         bulk_load(S->a, P.a_img, A_BYTES, &S->abar);          // plan-owned, immutable: needs no ordering
+        // the first tile's rows on their way to L2 (and no further) while an earlier kernel may still be writing them (3001 x 4096, 4
+        // bits: 17.8 -> 17.4 us)
+        for (int t = 0; t < TOK; ++t) {
+            const long long row = (long long)blockIdx.x * TOK + t;
+            if (row < P.n_rows) prefetch_l2(P.x + row * P.stride, P.d * 4);
+        }
     }
     if (warp == 0) tmem_alloc(&S->tmem_base, TMEM_COLS);
     tc_fence_before();
@@ -194,7 +200,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uvf(const __grid_constant__ U
         auto prefetch = [&](int n) {
             const long long row = row_first + (long long)n * row_step;
             if (prefetches && n < n_mine && row < P.n_rows)
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.x + row * P.stride), "r"(P.d * 4) : "memory");
+                prefetch_l2(P.x + row * P.stride, P.d * 4);
         };
         auto split_tile = [&](int n) -> bool {
             const int s = n % STAGES;
