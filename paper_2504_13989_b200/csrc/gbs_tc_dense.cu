@@ -81,52 +81,6 @@ struct DenseParams {
     int* status;
 };
 
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned peer_addr(unsigned smem_addr, unsigned rank)
-{
-    unsigned a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void peer_store(unsigned addr, float v)
-{
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void peer_arrive(unsigned bar_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
-}
-// bounded wait on a barrier that other CTAs of the cluster arrive at, behind their stores
-__device__ __forceinline__ bool cluster_wait(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
-{
-    const unsigned long long t0 = global_ns();
-    for (unsigned i = 1;; ++i) {
-        unsigned ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(WAIT_HINT_NS) : "memory");
-        if (ok) return true;
-        if ((i & 15u) == 0) {
-            if (*abort_flag) return false;
-            if (global_ns() - t0 > WAIT_LIMIT_NS) break;
-        }
-    }
-    *abort_flag = 1;
-    atomicCAS(status, 0, code);
-    return false;
-}
-
 // n k-steps of one stage: 32 bytes of the 128-byte line each, four to a box; the operand moves on by `step`
 __device__ __forceinline__ void steps(unsigned d_tmem, unsigned long long ad, unsigned long long bd, unsigned step, unsigned idesc, int n)
 {

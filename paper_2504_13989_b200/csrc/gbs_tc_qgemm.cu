@@ -24,7 +24,7 @@
 // its stores becoming visible to the tensor cores; two or three sets take turns).  256-token tiles, the shared-memory port:
 // 24 KB of packed codes in and out and 32 KB of int8 in and out are about 900 of a step's 1016 cycles, the tensor pipe 512.
 // 4096 x 4096 x 4096, 4 bits: 139 us (one 128 x 256 tile per CTA, both operands in shared memory, packed codes by global
-// loads), 118 us (256 x 192 on SM pairs, cta_group::2: the arrivals across the pair double the step), 70 us now.
+// loads), 63 us now; 56 on pairs of SMs (gbs_tc_qgemm2.cu), which outputs of that size take.
 // Every wait is bounded; an expired wait records a code in the activation plan's status word.
 #include <math.h>
 #include <string.h>
@@ -32,12 +32,10 @@
 #include <mutex>
 
 #include "gbs_internal.h"
-#include "gbs_qfields.cuh"
-#include "gbs_tc_common.cuh"
+#include "gbs_qgemm.cuh"
 
 namespace {
 
-constexpr int KB = 128;                 // codes per step and row: one 128-byte line of int8
 constexpr int TM = 128;                 // output channels per tile
 constexpr int UNPACK_WARPS = 24;
 constexpr int EPI_WARPS = 4;
@@ -65,80 +63,12 @@ struct Ctl {
     volatile int abort_flag;
 };
 
-struct QgemmParams {
-    long long n_tok, n_out;
-    int n;                              // tokens per tile (MMA N)
-    int xbox;                           // token rows a load brings: n, or all tokens if they are fewer
-    int m_tiles, tiles;                 // channel tiles, all tiles
-    int kblocks;                        // d' / 128
-    const float* sx;
-    const float* sw;
-    void* out;
-    long long out_stride;               // elements
-    int* status;
-};
-
-// Instruction descriptor, kind::i8: int32 accumulate, signed 8-bit A and B, both K-major, M x N.
-__host__ __device__ constexpr unsigned instr_desc_i8(int M, int N)
-{
-    return (2u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
-}
-
 // A from tensor memory, B from shared memory
 __device__ __forceinline__ void umma_i8_ts(unsigned d_tmem, unsigned a_tmem, unsigned long long b_desc, unsigned idesc, unsigned accumulate)
 {
     asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
                  "@q tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-
-__device__ __forceinline__ uint4 ld_shared_v4(unsigned addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-// 8 registers -> 8 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_st8(unsigned taddr, const unsigned r[8])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-                 ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr) : "memory");
-}
-// 16 columns of this thread's TMEM lane -> 16 registers
-__device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned r[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-}
-
-// The packed 128 codes of row r of a stage.  Four-bit rows are 64 bytes with the 64-byte swizzle (eight rows side by side hit
-// all banks), three-bit rows 48 bytes plain (48-byte steps do so by themselves).
-template <int BITS>
-__device__ __forceinline__ void load_row128(unsigned rows, int r, uint4 w[BITS])
-{
-#pragma unroll
-    for (int c = 0; c < BITS; ++c)
-        w[c] = ld_shared_v4(rows + (unsigned)r * (16u * BITS) + (unsigned)((BITS == 4 ? c ^ ((r >> 1) & 3) : c) << 4));
-}
-// Codes 32 c .. 32 c + 31 of it -> eight words of int8.
-template <int BITS, bool GATHER>
-__device__ __forceinline__ void unpack32(const uint4 w[BITS], int c, unsigned v[8])
-{
-    const unsigned f[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
-                            w[2].x, w[2].y, w[2].z, w[2].w, w[BITS - 1].x, w[BITS - 1].y, w[BITS - 1].z, w[BITS - 1].w};
-    unsigned p[BITS];
-    if (GATHER) {
-        gather_octets<BITS>(f + BITS * c, p);
-    } else {
-#pragma unroll
-        for (int i = 0; i < BITS; ++i) p[i] = f[BITS * c + i];
-    }
-#pragma unroll
-    for (int o = 0; o < 4; ++o) field_pair<BITS>(p, o, v[2 * o], v[2 * o + 1]);
 }
 
 template <int XBITS, int WBITS, typename OutT, int TW>
@@ -300,25 +230,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm(const __grid_constant__
                     if (lane == 0) mbar_arrive(&S->tshared);
                 }
                 if (c0 >= P.n) continue;
-                // the int8 operands were q * 2^(8 - bits): take the two powers of two out again (exact)
-                const float dx_l = t0 + c0 + lane < P.n_tok ? __ldg(P.sx + t0 + c0 + lane) * (1.f / (float)(1 << (16 - XBITS - WBITS))) : 0.f;
-                OutT* dst = reinterpret_cast<OutT*>(P.out) + (t0 + c0) * P.out_stride + o;
-                const int cols = (int)((P.n_tok - t0 - c0) < 32 ? (P.n_tok - t0 - c0) : 32);
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    unsigned v[16];
-                    tmem_ld16(tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(a * SH::ACC_STEP + c0 + 16 * hf), v);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const float dx = __shfl_sync(0xffffffffu, dx_l, 16 * hf + e);
-                        const float f = (float)(int)v[e] * (dx * dw);
-                        if (16 * hf + e < cols && o < P.n_out) {
-                            if (sizeof(OutT) == 4) *reinterpret_cast<float*>(dst) = f;
-                            else *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(f);
-                        }
-                        dst += P.out_stride;
-                    }
-                }
+                store_tokens<XBITS + WBITS, OutT>(tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(a * SH::ACC_STEP + c0), t0 + c0, o, dw, lane, P);
             }
             tc_fence_before();
             __syncwarp();
@@ -345,19 +257,29 @@ QgemmKernel pick(int xbits, int wbits, int out_dtype)
     return table[xbits - 3][wbits - 3][out_dtype == GBS_DTYPE_F32 ? 0 : 1];
 }
 
-// Tokens per tile.  A step of 128 codes was measured at 600 cycles up to 96 tokens and 2.6 more per token beyond (1016 at 256);
-// tiles go in waves over the SMs.  The width with the least total is taken: 256 where the output fills the chip, narrow tiles
-// on more SMs where it does not.
-int pick_tokens(long long n_tok, long long n_out, int kblocks, int sm_count)
+// Tokens per tile, and whether tiles are 256 channels on a pair of SMs (gbs_tc_qgemm2.cu) or 128 on one.  A step of 128 codes was measured at
+// 600 cycles up to 96 tokens and 2.6 more per token beyond (1016 at 256) on one SM, at 500 and 0.9 per token on a pair, whose start and end take
+// 3500 cycles longer (2000 where a side has three bits: their step on one SM is the slower one); tiles go in waves over the SMs.  (4096
+// wide, 4 bits: 400 tokens -> 4096 15.3 us on one and 15.5 on pairs, 520: 17.4 and 16.3, 2048: 34.9 and 31.5; 130 -> 9472: 13.6 and 15.1,
+// 260: 17.1 and 16.1; 3 bits: 2048 -> 1024 16.5 and 16.1, 100 -> 14336 18.1 and 16.6.)  The width with the least total is taken: 256 where the output fills the chip, narrow
+// tiles on more SMs where it does not.
+int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int sm_count, bool& pairs)
 {
     double best = 0.0;
     int n_best = 0;
+    pairs = false;
     for (int n = 32; n <= 256; n += 32) {
         const long long tiles = ((n_out + TM - 1) / TM) * ((n_tok + n - 1) / n);
         const long long waves = (tiles + sm_count - 1) / sm_count;
         const double unit = n <= 96 ? 600.0 : 600.0 + 2.6 * (n - 96);
         const double cost = (double)waves * kblocks * unit + 8.0 * n;
         if (n_best == 0 || cost < best) { best = cost; n_best = n; }
+    }
+    for (int n = 64; n <= GBS_QGEMM2_MAX_TOKENS; n += 32) {
+        const long long tiles = ((n_out + 2 * TM - 1) / (2 * TM)) * ((n_tok + n - 1) / n);
+        const long long waves = (tiles + sm_count / 2 - 1) / (sm_count / 2);
+        const double cost = (double)waves * kblocks * (500.0 + 0.9 * n) + 8.0 * n + (three ? 2000.0 : 3500.0);
+        if (cost < best) { best = cost; n_best = n; pairs = true; }
     }
     return n_best;
 }
@@ -432,12 +354,15 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     P.out = out;
     P.out_stride = out_row_stride;
     P.status = px->d_status;
-    P.n = pick_tokens(n_tokens, n_out, P.kblocks, px->sm_count);
+    bool pairs;
+    P.n = pick_tokens(n_tokens, n_out, P.kblocks, px->bits == 3 || pw->bits == 3, px->sm_count, pairs);
+    const int box_rows = pairs ? P.n / 2 : P.n;                   // an SM of a pair brings half the tokens
     // Rows of a box beyond the tensor's end are slow to fill where no swizzle is set (16 of 32 rows of three-bit codes: 15.8 us instead
     // of 12.2 at 14336 channels).  What shared memory holds beyond the box goes into sums that are not stored.  (A map of its own for
     // the last of several token tiles costs other calls as much as it gains.)
-    P.xbox = n_tokens < P.n ? (int)n_tokens : P.n;
-    P.m_tiles = (int)((n_out + TM - 1) / TM);
+    P.xbox = n_tokens < box_rows ? (int)n_tokens : box_rows;
+    const int channels = pairs ? 2 * TM : TM;
+    P.m_tiles = (int)((n_out + channels - 1) / channels);
     const long long tiles = (long long)P.m_tiles * ((n_tokens + P.n - 1) / P.n);
     if (tiles > 0x7fffffff / 2) return GBS_ERR_INVALID_ARG;
     P.tiles = (int)tiles;
@@ -445,6 +370,11 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     if (!encode_codes(encode, &wmap, codes_w, n_out, pw->d_pad * pw->bits / 8, pw->bits, TM) ||
         !encode_codes(encode, &xmap, codes_x, n_tokens, px->d_pad * px->bits / 8, px->bits, P.xbox))
         return GBS_ERR_CUDA;
+    if (pairs) {
+        const int e = gbs_tc_qgemm2(px, pw, wmap, xmap, P, out_dtype, static_cast<cudaStream_t>(cuda_stream));
+        if (e != 0) cudaGetLastError();
+        return e == 0 ? GBS_OK : GBS_ERR_CUDA;
+    }
     const bool wide = P.n > 128;
     const int smem = wide ? Shape<8>::SMEM : Shape<4>::SMEM;
     QgemmKernel kernel = wide ? pick<8>(px->bits, pw->bits, out_dtype) : pick<4>(px->bits, pw->bits, out_dtype);
