@@ -66,6 +66,8 @@ struct __align__(1024) Smem {
     volatile int abort_flag;
 };
 
+enum { ONE = 0, GROUPS = 1, GROUPS_OF_128 = 2 };      // scales: see the kernel
+
 struct UvParams {
     long long n_rows;
     int n_groups;                 // ceil(n_rows / TOK)
@@ -134,13 +136,15 @@ __device__ __forceinline__ void clip_score32(const unsigned r[32], float M, cons
 // ---------------------------------------------------------------------------------------------
 // kernel
 // ---------------------------------------------------------------------------------------------
-// GROUPED = false: one scale per token.  GROUPED = true: one scale per 2^glog adjacent lanes (32 * 2^glog
-// consecutive coordinates), 2^glog <= 32.  CLIP = true: instead of quantizing, score K clip ratios.
+// MODE = ONE: one scale per token.  MODE = GROUPS: one scale per 2^glog adjacent lanes (32 * 2^glog consecutive coordinates),
+// 2^glog <= 32; GROUPS_OF_128: glog = 2, fixed (no branch on it per tile: 8192 x 3584, 3 bits: 17.75 -> 17.54 us).  CLIP = true: instead of quantizing, score K clip ratios.
 // WANT_Y = true: also write the rotated normalised values (the parity output of gbs_rotate_quantize).
-template <int BITS, bool GROUPED, bool CLIP, bool WANT_Y>
+template <int BITS, int MODE, bool CLIP, bool WANT_Y>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__ CUtensorMap tmap,
                                                          const __grid_constant__ UvParams P)
 {
+    constexpr bool GROUPED = MODE != ONE;
+    const int glog = MODE == GROUPS_OF_128 ? 2 : P.glog;
     extern __shared__ unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = warp_index(), lane = threadIdx.x & 31;
@@ -249,11 +253,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__
             if (up < P.U && row0 < P.n_rows) n_store = (int)((P.n_rows - row0 + row_step - 1) / row_step);
             unsigned char* cptr = P.codes + row0 * P.code_row_bytes + up * (V * BITS / 8);
             const long long cstep = row_step * P.code_row_bytes;
-            float* sptr = P.scales + row0 * P.spr + (GROUPED ? (up >> P.glog) : 0);
+            float* sptr = P.scales + row0 * P.spr + (GROUPED ? (up >> glog) : 0);
             const long long sstep = row_step * P.spr;
             float* yptr = WANT_Y ? P.y_opt + row0 * (long long)P.d_pad + up * V : nullptr;
             const long long ystep = row_step * P.d_pad;
-            const unsigned gl = 1u << P.glog;     // lanes per quantization group (GROUPED)
+            const unsigned gl = 1u << glog;     // lanes per quantization group (GROUPED)
             const bool scale_writer = GROUPED ? ((lane & (gl - 1u)) == 0) : (up == 0);
             const bool arriver = lane == 0;
             // one iteration on pipeline stage s (a compile-time constant: the loop below is unrolled over the
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__
                 if (GROUPED) {
                     // fold over the 2^glog lanes of this thread's group (a redux with one mask per group would be
                     // issued once per distinct mask, which is slower for small groups)
-                    switch (P.glog) {
+                    switch (glog) {
                         case 5: M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));   // fall through
                         case 4: M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8));    // fall through
                         case 3: M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 4));    // fall through
@@ -364,7 +368,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_rq(const __grid_constant__
                 }
                 const unsigned gp = it & 1;
                 if (GROUPED) {
-                    for (int o = (1 << P.glog) >> 1; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+                    for (int o = (1 << glog) >> 1; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
                 } else {
                     // per-token max: warp-wide integer max, then the token's four quadrant warps meet at a named
                     // barrier; a warp whose wait expired still comes and raises the slot's flag first
@@ -517,18 +521,20 @@ int uv_prepare(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride,
     return 0;
 }
 
-// every instantiation, indexed [bits - 3][grouped][want_y] and [grouped] for the scoring form
+// every instantiation, indexed [bits - 3][mode][want_y] and [grouped] for the scoring form
 typedef void (*UvKernel)(const CUtensorMap, const UvParams);
-UvKernel uv_rq_kernel(int bits, bool grouped, bool want_y)
+UvKernel uv_rq_kernel(int bits, int mode, bool want_y)
 {
-    static const UvKernel table[2][2][2] = {
-        {{k_tc_uv_rq<3, false, false, false>, k_tc_uv_rq<3, false, false, true>},
-         {k_tc_uv_rq<3, true, false, false>, k_tc_uv_rq<3, true, false, true>}},
-        {{k_tc_uv_rq<4, false, false, false>, k_tc_uv_rq<4, false, false, true>},
-         {k_tc_uv_rq<4, true, false, false>, k_tc_uv_rq<4, true, false, true>}}};
-    return table[bits - 3][grouped ? 1 : 0][want_y ? 1 : 0];
+    static const UvKernel table[2][3][2] = {
+        {{k_tc_uv_rq<3, ONE, false, false>, k_tc_uv_rq<3, ONE, false, true>},
+         {k_tc_uv_rq<3, GROUPS, false, false>, k_tc_uv_rq<3, GROUPS, false, true>},
+         {k_tc_uv_rq<3, GROUPS_OF_128, false, false>, k_tc_uv_rq<3, GROUPS, false, true>}},
+        {{k_tc_uv_rq<4, ONE, false, false>, k_tc_uv_rq<4, ONE, false, true>},
+         {k_tc_uv_rq<4, GROUPS, false, false>, k_tc_uv_rq<4, GROUPS, false, true>},
+         {k_tc_uv_rq<4, GROUPS_OF_128, false, false>, k_tc_uv_rq<4, GROUPS, false, true>}}};
+    return table[bits - 3][mode][want_y ? 1 : 0];
 }
-UvKernel uv_clip_kernel(bool grouped) { return grouped ? k_tc_uv_rq<4, true, true, false> : k_tc_uv_rq<4, false, true, false>; }
+UvKernel uv_clip_kernel(bool grouped) { return grouped ? k_tc_uv_rq<4, GROUPS, true, false> : k_tc_uv_rq<4, ONE, true, false>; }
 
 // opt in to the large dynamic shared memory once per device (not a stream operation); callable from several
 // host threads at once
@@ -540,9 +546,9 @@ cudaError_t uv_opt_in(const gbs_plan* p, int smem)
     if (p->device >= 0 && p->device < 64 && attr_done[p->device]) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     for (int bits = 3; bits <= 4 && e == cudaSuccess; ++bits)
-        for (int g = 0; g < 2 && e == cudaSuccess; ++g)
+        for (int g = 0; g < 3 && e == cudaSuccess; ++g)
             for (int y = 0; y < 2 && e == cudaSuccess; ++y)
-                e = cudaFuncSetAttribute(uv_rq_kernel(bits, g != 0, y != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                e = cudaFuncSetAttribute(uv_rq_kernel(bits, g, y != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     for (int g = 0; g < 2 && e == cudaSuccess; ++g)
         e = cudaFuncSetAttribute(uv_clip_kernel(g != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess && p->device >= 0 && p->device < 64) attr_done[p->device] = true;
@@ -566,7 +572,7 @@ int gbs_tc_uv_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, 
     cudaError_t e = uv_opt_in(p, smem);
     if (e != cudaSuccess) return (int)e;
     const bool pdl = p->pdl != 0;
-    e = launch(uv_rq_kernel(p->bits, p->group != 0, y_opt != nullptr), grid, smem, stream, pdl, tmap, P);
+    e = launch(uv_rq_kernel(p->bits, p->group == 0 ? ONE : p->group == 128 ? GROUPS_OF_128 : GROUPS, y_opt != nullptr), grid, smem, stream, pdl, tmap, P);
     return (int)e;
 }
 
