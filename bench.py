@@ -687,8 +687,8 @@ def extras(device, stream, args, peak, sampler=None):
         out["quantized_matmul_x%d_w%d_4096x4096x4096" % (bx, bw)] = {
             "us_per_launch": ms * 1e3, "tops": tops,
             "roofline": {"bound": "tensor", "unit": "TOP/s", "achieved": tops, "peak": i8_peak, "frac": tops / i8_peak,
-                         "note": "int8 peak = 2 x the %s bf16 figure (nominal int8 : bf16 ratio); the kernel is bound by "
-                                 "the shared-memory port (packed codes in and out, int8 in and out), not by the tensor pipe" % bf16_kind}}
+                         "note": "int8 peak = 2 x the %s bf16 figure (nominal int8 : bf16 ratio); 512 of a "
+                                 "step's 730 cycles are the tensor pipe's, and 256 tiles count as four waves over 74 pairs" % bf16_kind}}
         del px, pw, cx, sx, cw, sw, outm
     ms = time_loop(lambda i: torch.matmul(xq, wq.t()), 8)
     out["bf16_matmul_of_the_unquantized_operands_4096x4096x4096"] = {"us_per_launch": ms * 1e3,
@@ -755,8 +755,8 @@ def extras(device, stream, args, peak, sampler=None):
                              "sm_mhz_sampled": sm_mhz,
                              "roofline": {"bound": "hbm", "unit": "GB/s", "achieved": wc.n_rows * wc.d * 2 / ms / 1e6, "peak": peak,
                                           "frac": wc.n_rows * wc.d * 2 / ms / 1e6 / peak,
-                                          "note": "one histogram per token scores all candidates; bound by the shared-memory "
-                                                  "port (table lookups and atomics)"}}
+                                          "note": "one histogram per token scores all candidates; bound by instruction issue, "
+                                                  "the shared-memory port and a token's barriers"}}
     # Algorithm 1's bracket search on the last layer's tensor (eps = 1/64): rounds of <= 31 probes, blocking
     out["search_clip_ratio_eps_1_64"] = {"alpha": res.alpha, "iterations": res.iterations, "rounds": res.rounds,
                                          "evaluations": res.evaluations, "wall_ms_per_layer_262144_tokens": dt * 1e3}
