@@ -12,11 +12,12 @@
 //   * Maxima: group = 32 2^g coordinates, or one scale per token.  Across the warps that share it through shared memory and a
 //     named barrier (token: 128 or 256 threads; group at V = 64: the pair of warps); then Delta, rounding, clipping, packing
 //     (Sections 2.1, 3.1) from registers.
-// What bounds it: latency.  A warp issues about 700 instructions per 32 values of a lane (220 of them the split) at 8 cycles
-// each, sixteen warps cover half of that, and taking out any one part (two of three planes, the split, the epilogue) gains
-// less than a tenth.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 16.95 now; 7000 x 3584, groups of 128: 117.6
-// -> 28.3; 7000 x 8192, 4 bits: 63.3.  Tried and slower: loads reissued piece by piece inside the split; tiles prefetched into L2
-// further ahead; the prefetches in a warp of their own that waits for the splits (18.2, 31.4 and 73.3 us).
+// What bounds it: 2.07 us per tile of 64 KB in a long batch (5 TB/s), of which 1.6 is one warp's chain of split and epilogue (a tile of one
+// token takes 1.75), and about 4.4 us of fill in a short one.  3001 x 4096, 4 bits: 43.7 us on the shared-memory kernel, 17.4 now; 7000 x
+// 3584, groups of 128: 117.6 -> 28.3; 7000 x 8192, 4 bits: 63.3.  Tried and slower: loads reissued piece by piece inside the split; tiles
+// prefetched into L2 further ahead; the prefetches in a warp of their own that waits for the splits (18.2, 31.4 and 73.3 us); eight warps
+// that only split beside sixteen of the epilogue (18.5); fewer tokens per tile (17.3 with three).  No change: twelve such warps, with
+// registers moved to the epilogue's; A in tensor memory.
 // Every wait is bounded; an expired wait records a code in the plan's status word, and a warp whose wait ran out brings a
 // pattern no maximum can have to the barrier it shares, so that all who wait there leave with it.
 #include <string.h>

@@ -20,7 +20,8 @@
 // against 48 - 100 bytes of HBM traffic per 32 values.  Doing H_V before the contraction in packed halves takes 80
 // instructions per 32 values where the fp32 form after the contraction took 124 packed (248 slots).
 // 8192 x 3584, 3 bits, groups of 128 -> bf16: 118.5 us on the shared-memory kernel this replaces for group scales, 27 now.
-// V = 32 takes four tokens per tile with all sixteen warps on it (two tokens and two groups of warps: 30 us).
+// V = 32 takes four tokens per tile with all sixteen warps on it (two tokens and two groups of warps: 30 us; roles apart, twelve
+// warps that unpack and sixteen for the epilogue: 14.2 -> 17.8 us for 4096 rows; sixteen and eight: no change).
 // Roles: warp 0 loads the image, warp 1 issues the MMAs, warps 2..17 unpack (ahead) and run the epilogue; warp (q, t) owns
 // TMEM lane quadrant q and token t; with V = 64 two groups of eight warps take alternate tiles.  Every wait is bounded.
 #include <math.h>
