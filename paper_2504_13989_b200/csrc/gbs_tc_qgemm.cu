@@ -285,15 +285,16 @@ int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int s
 }
 
 // Whether the few-token kernel (gbs_qgemv.cu) is the faster one.  Its time grows with the channels of an SM: these cycles per channel and
-// step of 128 codes on 148 SMs for up to 8, 16, 32 and 64 tokens (measured with 4096-wide rows, 8192 and 14336 channels; four bits,
-// three bits on a side).  Tiles of 128 channels come in waves over the SMs, 600 cycles a step whatever they hold, with much the same
-// start.  So within the first wave (18 944 channels) 64 tokens go to the tiles beyond 5800 (4300) channels, 32 beyond 10 300 (7800), 16
-// beyond 18 200 (8800), and where a new wave begins the few-token kernel is the faster one again for a while.  48 tokens -> 14336, four
-// bits: 28.5 us here, 12.4 in tiles; 4096: 7.9 and 10.8.
+// step of 128 codes on 148 SMs for up to 8, 16, 32 and 64 tokens (four bits, three bits on a side).  Beyond 16 tokens it grows in waves of 32
+// channels per SM (4736): so 32 tokens go to the tiles beyond two waves (three bits: 7800 channels) and 64 beyond one; 16 beyond 18 200
+// (8800).  Tiles of 128 channels come in waves too, 600 cycles a step whatever they hold, with much the same start; where a new one begins
+// (18 944 channels) the few-token kernel is the faster one again for a while.  Four bits, few-token kernel and tiles: 32 tokens -> 8704: 11.3
+// and 12.0 us, 10 240: 15.0 and 12.4; 64 tokens -> 4096: 8.4 and 11.4, 5760: 15.1 and 11.9; three bits: 32 -> 7168: 12.7 and 11.9, 20 ->
+// 7168: 11.6 and 12.0, 64 -> 4096: 11.0 and 12.0, 5760: 20.0 and 12.7.
 bool few_tokens(long long n_tok, long long n_out, bool three, int sm_count)
 {
     if (n_tok > GBS_QGEMV_MAX_TOKENS) return false;
-    static const double per_channel[2][4] = {{0.021, 0.033, 0.058, 0.103}, {0.035, 0.068, 0.077, 0.140}};
+    static const double per_channel[2][4] = {{0.021, 0.033, 0.0633, 0.1266}, {0.035, 0.068, 0.077, 0.1266}};
     const long long tiles = (n_out + TM - 1) / TM, waves = (tiles + sm_count - 1) / sm_count;
     const double cycles = per_channel[three ? 1 : 0][n_tok <= 8 ? 0 : n_tok <= 16 ? 1 : n_tok <= 32 ? 2 : 3] * 148.0 / sm_count;
     return (double)n_out * cycles <= 600.0 * (double)waves;
