@@ -703,7 +703,6 @@ __global__ void __launch_bounds__(NT) k_dequantize_staged(int d_pad, int glog, i
 
     // programmatic dependent launch: the codes may still be being written until this returns
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     long long tile = blockIdx.x;
     const long long tstride = gridDim.x;
 #pragma unroll
@@ -764,6 +763,8 @@ __global__ void __launch_bounds__(NT) k_dequantize_staged(int d_pad, int glog, i
             for (int h = 0; h < NST; ++h) { dl[u][h] = dl_n[u][h]; zr[u][h] = zr_n[u][h]; }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // only now, as in the direct form (16 384 x 4096, 3 bits -> bf16: 41.2 us in stream order, 40.2 with this at the start, 38.8 here)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // xhat = (H^T yhat / sqrt(d'))[0:d]: same shared-memory machinery with the transposed H_m.
