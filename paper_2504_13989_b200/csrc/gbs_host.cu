@@ -310,6 +310,7 @@ extern "C" int gbs_dequantize(const gbs_plan_t* p, const void* codes, const floa
     else
         e = gbs_generic_dequantize(p, codes, scales, n_rows, out, out_dtype, (flags & GBS_INVERSE_ROTATE) != 0,
                                    static_cast<cudaStream_t>(cuda_stream));
+    if (e != 0) cudaGetLastError();        // a failed launch is reported once, here
     return e == 0 ? GBS_OK : GBS_ERR_CUDA;
 }
 
