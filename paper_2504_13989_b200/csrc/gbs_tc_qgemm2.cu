@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
                 for (int ks = 0; ks < KB / 32; ++ks)
                     pair_mma(tmem_base + a * ACC_STEP, tmem_base + A_COL0 + s * 32 + ks * 8, bd + (unsigned long long)(2 * ks), idesc,
                              (kb | ks) != 0 ? 1u : 0u);
-                pair_commit(&S->oempty[b]);
+                // the last stages are not used again: an arrival that nobody waits for could come after the other SM's block has ended
+                if (c + STAGES < total) pair_commit(&S->oempty[b]);
             }
             if (ok) pair_commit(&S->tfull[a]);
         }
