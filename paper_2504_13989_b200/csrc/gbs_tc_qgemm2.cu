@@ -130,6 +130,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
                 }
             }
             if (!ok) drain_copies(S->pfull, BARS, c);
+            // The last stages are not used again, but the commits that free them arrive here too: not after this block has ended.  (Leaving
+            // those commits out costs a branch per step: 4096^3, 4 bits: 59.1 us instead of 56.1.)
+            for (int l = c < STAGES ? 0 : c - STAGES; ok && l < c; ++l)
+                ok = mbar_wait(&S->abort_flag, &S->oempty[l % BARS], (unsigned)(l / BARS) & 1u, P.status, 5);
         }
     } else if (warp == 1 && rank == 0) {
         // ------------------------------ MMA issuer ------------------------------
@@ -155,8 +159,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
                 for (int ks = 0; ks < KB / 32; ++ks)
                     pair_mma(tmem_base + a * ACC_STEP, tmem_base + A_COL0 + s * 32 + ks * 8, bd + (unsigned long long)(2 * ks), idesc,
                              (kb | ks) != 0 ? 1u : 0u);
-                // the last stages are not used again: an arrival that nobody waits for could come after the other SM's block has ended
-                if (c + STAGES < total) pair_commit(&S->oempty[b]);
+                pair_commit(&S->oempty[b]);
             }
             if (ok) pair_commit(&S->tfull[a]);
         }
