@@ -6,7 +6,7 @@
 // for both.  16 KB in, out, in and out again are 512 cycles.
 //   * Roles per SM: a producer, twenty-four unpacking warps in three sets that take every third step (four warps for channels, four
 //     for tokens), four epilogue warps; the pair's first SM issues all MMAs.  Accumulators overlap by half as there.
-//   * Both SMs' unpacking warps arrive at the issuer's barriers; commits are multicast to both.
+//   * Both SMs' unpacking warps arrive at the issuer's barriers (cluster scope, see pair_arrive); commits are multicast to both.
 //   * A set serves every third step and a stage of operands every fourth, so barriers are indexed by the step modulo twelve: each
 //     waiter then takes part in every phase of the barriers it waits for.
 // What bounds it: with 256 tokens a step takes about 730 cycles at 1.9 GHz, 512 of them the tensor pipe's, at the 1 kW limit (with a quarter of
@@ -61,13 +61,61 @@ __device__ __forceinline__ void pair_commit(void* bar)
                  ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
 }
 
-// Arrival at a barrier of either SM.  Of this thread's own writes nothing goes with it: what the operands need (the proxy's fence, the
-// tcgen05 fences) stands before it.  With .release.cluster it also waited for a fence of the whole GPU's scope: a step took 1250 cycles
-// instead of 730.
+// Arrivals at the issuer's barriers and waits on barriers that the other SM's threads or commits arrive at.  Between threads of two CTAs the
+// scope has to be the cluster's; what is ordered is named by the fences around them, as PTX's patterns for tcgen05 have it:
+//   * tensor memory (channels written by tcgen05.st, accumulators read by tcgen05.ld): tcgen05.wait, tcgen05.fence::before_thread_sync and a
+//     relaxed arrival; a relaxed wait and tcgen05.fence::after_thread_sync.  The same wait and fence stand behind a commit.
+//   * tokens written to shared memory: fence.proxy.async by each lane, then one release per warp; the issuer acquires before it lets the
+//     tensor cores (async proxy) read both SMs' shared memory.  Before a stage is written again the warps acquire behind the commit's wait.
+// The fences are the ones restricted to shared memory: with them 4096^3 takes 55.9 us at 4 bits and 60.5 at 3 (56.2 and 60.1 with
+// arrivals and waits of CTA scope).  An arrival with .release.cluster orders the writer's global accesses as well: 98.9 us.
 __device__ __forceinline__ void pair_arrive(unsigned bar_addr)
 {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
 }
+__device__ __forceinline__ void release_tokens()
+{
+    asm volatile("fence.proxy.async::generic.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void acquire_tokens()
+{
+    asm volatile("fence.proxy.async::generic.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void acquire_stage()
+{
+    asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory");
+}
+__device__ __forceinline__ bool pair_try_wait(void* bar, unsigned parity)
+{
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(WAIT_HINT_NS) : "memory");
+    return ok != 0;
+}
+// bounded, like mbar_wait
+__device__ __noinline__ bool pair_wait_slow(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
+{
+    const unsigned long long t0 = global_ns();
+    for (unsigned i = 1;; ++i) {
+        if (pair_try_wait(bar, parity)) return true;
+        if ((i & 15u) == 0) {
+            if (*abort_flag) return false;
+            if (global_ns() - t0 > WAIT_LIMIT_NS) break;
+        }
+    }
+    *abort_flag = 1;
+    atomicCAS(status, 0, code);
+    return false;
+}
+__device__ __forceinline__ bool pair_wait(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
+{
+    if (pair_try_wait(bar, parity)) return true;
+    return pair_wait_slow(abort_flag, bar, parity, status, code);
+}
+
 template <int XBITS, int WBITS, typename OutT>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
                                                           const __grid_constant__ QgemmParams P)
@@ -133,7 +181,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
             // The last stages are not used again, but the commits that free them arrive here too: not after this block has ended.  (Leaving
             // those commits out costs a branch per step: 4096^3, 4 bits: 59.1 us instead of 56.1.)
             for (int l = c < STAGES ? 0 : c - STAGES; ok && l < c; ++l)
-                ok = mbar_wait(&S->abort_flag, &S->oempty[l % BARS], (unsigned)(l / BARS) & 1u, P.status, 5);
+                ok = pair_wait(&S->abort_flag, &S->oempty[l % BARS], (unsigned)(l / BARS) & 1u, P.status, 5);
         }
     } else if (warp == 1 && rank == 0) {
         // ------------------------------ MMA issuer ------------------------------
@@ -142,16 +190,17 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
         bool ok = true;
         for (int i = 0; ok && i < n_mine; ++i) {
             const int a = i & 1;
-            ok = mbar_wait(&S->abort_flag, &S->tempty[a], (unsigned)((i >> 1) & 1) ^ 1u, P.status, 3);
+            ok = pair_wait(&S->abort_flag, &S->tempty[a], (unsigned)((i >> 1) & 1) ^ 1u, P.status, 3);
             // the columns shared with the tile before are drained first
-            ok = ok && mbar_wait(&S->abort_flag, &S->tshared, (unsigned)(i & 1) ^ 1u, P.status, 3);
+            ok = ok && pair_wait(&S->abort_flag, &S->tshared, (unsigned)(i & 1) ^ 1u, P.status, 3);
             if (!__all_sync(0xffffffffu, ok)) break;
             for (int kb = 0; kb < P.kblocks; ++kb, ++c) {
                 const int s = c % STAGES, b = c % BARS;
                 const unsigned ph = (unsigned)(c / BARS) & 1u;
-                ok = mbar_wait(&S->abort_flag, &S->ofull[b], ph, P.status, 2);
+                ok = pair_wait(&S->abort_flag, &S->ofull[b], ph, P.status, 2);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
+                acquire_tokens();
                 tc_fence_after();
                 // an instruction takes 32 codes: eight columns of the channels' lanes, 32 bytes of the tokens' lines
                 const unsigned long long bd = smem_desc(smem_u32(sm_b + s * B_STAGE), 16, 1024, 2);
@@ -182,7 +231,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
                 load_row128<WBITS>(rows, r, w);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S->pempty[b]);
-                ok = before < 0 || mbar_wait(&S->abort_flag, &S->oempty[before % BARS], (unsigned)(before / BARS) & 1u, P.status, 5);
+                ok = before < 0 || pair_wait(&S->abort_flag, &S->oempty[before % BARS], (unsigned)(before / BARS) & 1u, P.status, 5);
                 if (!__all_sync(0xffffffffu, ok)) break;
                 tc_fence_after();
 #pragma unroll
@@ -198,8 +247,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
                 if (have) load_row128<XBITS>(rows + TM * 64, r, w);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S->pempty[b]);
-                ok = before < 0 || mbar_wait(&S->abort_flag, &S->oempty[before % BARS], (unsigned)(before / BARS) & 1u, P.status, 5);
+                ok = before < 0 || pair_wait(&S->abort_flag, &S->oempty[before % BARS], (unsigned)(before / BARS) & 1u, P.status, 5);
                 if (!__all_sync(0xffffffffu, ok)) break;
+                acquire_stage();
                 if (have) {
                     const unsigned line = smem_u32(sm_b + (c % STAGES) * B_STAGE) + (unsigned)r * 128u;
 #pragma unroll
@@ -214,7 +264,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             }
             __syncwarp();
-            if (lane == 0) pair_arrive(ofull0 + 8u * (unsigned)b);
+            if (lane == 0) {
+                if (!channels) release_tokens();
+                pair_arrive(ofull0 + 8u * (unsigned)b);
+            }
         }
     } else if (warp >= 2) {
         // ------------------------------ epilogue: lane = output channel, column = token ------------------------------
@@ -225,7 +278,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
             const long long o = (long long)(2 * mt + rank) * TM + q * 32 + lane;
             const long long t0 = (long long)nt * P.n;
             const float dw = o < P.n_out ? __ldg(P.sw + o) : 0.f;
-            const bool ok = mbar_wait(&S->abort_flag, &S->tfull[a], (unsigned)(i >> 1) & 1u, P.status, 6);
+            const bool ok = pair_wait(&S->abort_flag, &S->tfull[a], (unsigned)(i >> 1) & 1u, P.status, 6);
             if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after();
             // columns [128, 256) belong to both accumulators: the upper half of the even tiles', the lower half of the odd ones',
