@@ -148,6 +148,11 @@ bool gbs_tc_denseinv_supported(const gbs_plan* p);
 int gbs_tc_denseinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
                                int out_dtype, cudaStream_t stream);
 
+// gbs_tc_qgemm.cu : the kernel that gbs_quantized_matmul takes on sm_count SMs of which `pairs` pairs can run the pairs' kernel, and the tokens
+// of its tiles (host arithmetic only; `three`: a side has three-bit codes)
+enum gbs_matmul_kernel { GBS_MATMUL_FEW_TOKENS = 0, GBS_MATMUL_TILES = 1, GBS_MATMUL_PAIRS = 2 };
+extern "C" int gbs_matmul_rule(int64_t n_tokens, int64_t n_out, int kblocks, int three, int sm_count, int pairs, int* tile_tokens);
+
 // gbs_qgemv.cu : gbs_quantized_matmul for up to GBS_QGEMV_MAX_TOKENS tokens
 #define GBS_QGEMV_MAX_TOKENS 64
 int gbs_qgemv(const gbs_plan* px, const void* codes_x, const float* scales_x, int n_tokens, const gbs_plan* pw, const void* codes_w,

@@ -20,9 +20,11 @@ struct QgemmParams {
 };
 
 constexpr int GBS_QGEMM2_MAX_TOKENS = 256;      // tokens per tile of the pairs' kernel
-// The pairs' kernel (gbs_tc_qgemm2.cu).  P: tokens per tile (a multiple of 32, 64 at least), tiles of 256 channels; xmap's boxes hold P.xbox <= P.n / 2 rows.
-int gbs_tc_qgemm2(const gbs_plan* px, const gbs_plan* pw, const CUtensorMap& wmap, const CUtensorMap& xmap, const QgemmParams& P, int out_dtype,
-                  cudaStream_t stream);
+// How many pairs of the device's SMs can run the pairs' kernel (gbs_tc_qgemm2.cu) at once; 0 where a cluster of two cannot be launched.
+int gbs_tc_qgemm2_pairs(const gbs_plan* px);
+// That kernel, on `pairs` of them at most.  P: tokens per tile (a multiple of 32, 64 at least), tiles of 256 channels; xmap's boxes hold P.xbox <= P.n / 2 rows.
+int gbs_tc_qgemm2(const gbs_plan* px, const gbs_plan* pw, const CUtensorMap& wmap, const CUtensorMap& xmap, const QgemmParams& P, int pairs,
+                  int out_dtype, cudaStream_t stream);
 
 namespace {
 

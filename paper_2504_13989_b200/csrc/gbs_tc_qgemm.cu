@@ -262,12 +262,12 @@ QgemmKernel pick(int xbits, int wbits, int out_dtype)
 // 3500 cycles longer (2000 where a side has three bits: their step on one SM is the slower one); tiles go in waves over the SMs.  (4096
 // wide, 4 bits: 400 tokens -> 4096 15.3 us on one and 15.5 on pairs, 520: 17.4 and 16.3, 2048: 34.9 and 31.5; 130 -> 9472: 13.6 and 15.1,
 // 260: 17.1 and 16.1; 3 bits: 2048 -> 1024 16.5 and 16.1, 100 -> 14336 18.1 and 16.6.)  The width with the least total is taken: 256 where the output fills the chip, narrow
-// tiles on more SMs where it does not.
-int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int sm_count, bool& pairs)
+// tiles on more SMs where it does not.  `pairs`: how many there are; where clusters of two cannot be launched, none.
+int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int sm_count, int pairs, bool& on_pairs)
 {
     double best = 0.0;
     int n_best = 0;
-    pairs = false;
+    on_pairs = false;
     for (int n = 32; n <= 256; n += 32) {
         const long long tiles = ((n_out + TM - 1) / TM) * ((n_tok + n - 1) / n);
         const long long waves = (tiles + sm_count - 1) / sm_count;
@@ -275,11 +275,11 @@ int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int s
         const double cost = (double)waves * kblocks * unit + 8.0 * n;
         if (n_best == 0 || cost < best) { best = cost; n_best = n; }
     }
-    for (int n = 64; n <= GBS_QGEMM2_MAX_TOKENS; n += 32) {
+    for (int n = 64; pairs > 0 && n <= GBS_QGEMM2_MAX_TOKENS; n += 32) {
         const long long tiles = ((n_out + 2 * TM - 1) / (2 * TM)) * ((n_tok + n - 1) / n);
-        const long long waves = (tiles + sm_count / 2 - 1) / (sm_count / 2);
+        const long long waves = (tiles + pairs - 1) / pairs;
         const double cost = (double)waves * kblocks * (500.0 + 0.9 * n) + 8.0 * n + (three ? 2000.0 : 3500.0);
-        if (cost < best) { best = cost; n_best = n; pairs = true; }
+        if (cost < best) { best = cost; n_best = n; on_pairs = true; }
     }
     return n_best;
 }
@@ -311,6 +311,15 @@ bool encode_codes(EncodeTiledFn encode, CUtensorMap* map, const void* codes, int
 }
 
 }  // namespace
+
+extern "C" int gbs_matmul_rule(int64_t n_tokens, int64_t n_out, int kblocks, int three, int sm_count, int pairs, int* tile_tokens)
+{
+    *tile_tokens = (int)n_tokens;
+    if (few_tokens(n_tokens, n_out, three != 0, sm_count)) return GBS_MATMUL_FEW_TOKENS;
+    bool on_pairs;
+    *tile_tokens = pick_tokens(n_tokens, n_out, kblocks, three != 0, sm_count, pairs, on_pairs);
+    return on_pairs ? GBS_MATMUL_PAIRS : GBS_MATMUL_TILES;
+}
 
 extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, const float* scales_x, int64_t n_tokens,
                                     const gbs_plan_t* pw, const void* codes_w, const float* scales_w, int64_t n_out,
@@ -355,14 +364,15 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     P.out = out;
     P.out_stride = out_row_stride;
     P.status = px->d_status;
-    bool pairs;
-    P.n = pick_tokens(n_tokens, n_out, P.kblocks, px->bits == 3 || pw->bits == 3, px->sm_count, pairs);
-    const int box_rows = pairs ? P.n / 2 : P.n;                   // an SM of a pair brings half the tokens
+    const int pairs = gbs_tc_qgemm2_pairs(px);
+    bool on_pairs;
+    P.n = pick_tokens(n_tokens, n_out, P.kblocks, px->bits == 3 || pw->bits == 3, px->sm_count, pairs, on_pairs);
+    const int box_rows = on_pairs ? P.n / 2 : P.n;                   // an SM of a pair brings half the tokens
     // Rows of a box beyond the tensor's end are slow to fill where no swizzle is set (16 of 32 rows of three-bit codes: 15.8 us instead
     // of 12.2 at 14336 channels).  What shared memory holds beyond the box goes into sums that are not stored.  (A map of its own for
     // the last of several token tiles costs other calls as much as it gains.)
     P.xbox = n_tokens < box_rows ? (int)n_tokens : box_rows;
-    const int channels = pairs ? 2 * TM : TM;
+    const int channels = on_pairs ? 2 * TM : TM;
     P.m_tiles = (int)((n_out + channels - 1) / channels);
     const long long tiles = (long long)P.m_tiles * ((n_tokens + P.n - 1) / P.n);
     if (tiles > 0x7fffffff / 2) return GBS_ERR_INVALID_ARG;
@@ -371,8 +381,8 @@ extern "C" int gbs_quantized_matmul(const gbs_plan_t* px, const void* codes_x, c
     if (!encode_codes(encode, &wmap, codes_w, n_out, pw->d_pad * pw->bits / 8, pw->bits, TM) ||
         !encode_codes(encode, &xmap, codes_x, n_tokens, px->d_pad * px->bits / 8, px->bits, P.xbox))
         return GBS_ERR_CUDA;
-    if (pairs) {
-        const int e = gbs_tc_qgemm2(px, pw, wmap, xmap, P, out_dtype, static_cast<cudaStream_t>(cuda_stream));
+    if (on_pairs) {
+        const int e = gbs_tc_qgemm2(px, pw, wmap, xmap, P, pairs, out_dtype, static_cast<cudaStream_t>(cuda_stream));
         if (e != 0) cudaGetLastError();
         return e == 0 ? GBS_OK : GBS_ERR_CUDA;
     }

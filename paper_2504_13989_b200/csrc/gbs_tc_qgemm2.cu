@@ -313,40 +313,60 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_qgemm2(const __grid_constant_
 
 typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const QgemmParams);
 
-}  // namespace
-
-int gbs_tc_qgemm2(const gbs_plan* px, const gbs_plan* pw, const CUtensorMap& wmap, const CUtensorMap& xmap, const QgemmParams& P, int out_dtype,
-                  cudaStream_t stream)
+PairKernel pick(int xbits, int wbits, int out_dtype)
 {
     static const PairKernel table[2][2][2] = {
         {{k_tc_qgemm2<3, 3, float>, k_tc_qgemm2<3, 3, __nv_bfloat16>}, {k_tc_qgemm2<3, 4, float>, k_tc_qgemm2<3, 4, __nv_bfloat16>}},
         {{k_tc_qgemm2<4, 3, float>, k_tc_qgemm2<4, 3, __nv_bfloat16>}, {k_tc_qgemm2<4, 4, float>, k_tc_qgemm2<4, 4, __nv_bfloat16>}}};
-    {
-        // opt in to the large dynamic shared memory once per device (not a stream operation)
-        static std::mutex mu;
-        static bool done[64] = {false};
-        std::lock_guard<std::mutex> lock(mu);
-        if (!(px->device >= 0 && px->device < 64 && done[px->device])) {
-            for (int i = 0; i < 8; ++i) {
-                const cudaError_t e = cudaFuncSetAttribute(table[i >> 2][i >> 1 & 1][i & 1], cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-                if (e != cudaSuccess) return (int)e;
-            }
-            if (px->device >= 0 && px->device < 64) done[px->device] = true;
-        }
-    }
-    const int pairs = px->sm_count / 2;
+    return table[xbits - 3][wbits - 3][out_dtype == GBS_DTYPE_F32 ? 0 : 1];
+}
+
+// attr[0]: clusters of two
+cudaLaunchConfig_t pair_config(cudaLaunchAttribute attr[2], int pairs)
+{
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * (P.tiles < pairs ? P.tiles : pairs)));
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = SMEM;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+}  // namespace
+
+int gbs_tc_qgemm2_pairs(const gbs_plan* px)
+{
+    // once per device (not a stream operation): the large dynamic shared memory, and how many clusters there is room for
+    static std::mutex mu;
+    static int known[64] = {0};                     // pairs + 1
+    std::lock_guard<std::mutex> lock(mu);
+    const bool keep = px->device >= 0 && px->device < 64;
+    if (keep && known[px->device] != 0) return known[px->device] - 1;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 8 && e == cudaSuccess; ++i)
+        e = cudaFuncSetAttribute(pick(3 + (i >> 2), 3 + (i >> 1 & 1), i & 1 ? GBS_DTYPE_BF16 : GBS_DTYPE_F32), cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    int pairs = 0;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = pair_config(attr, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&pairs, pick(4, 4, GBS_DTYPE_BF16), &cfg);
+    if (e != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (pairs > px->sm_count / 2) pairs = px->sm_count / 2;
+    if (keep) known[px->device] = pairs + 1;
+    return pairs;
+}
+
+int gbs_tc_qgemm2(const gbs_plan* px, const gbs_plan* pw, const CUtensorMap& wmap, const CUtensorMap& xmap, const QgemmParams& P, int pairs,
+                  int out_dtype, cudaStream_t stream)
+{
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = pair_config(attr, P.tiles < pairs ? P.tiles : pairs);
+    cfg.stream = stream;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
     cfg.numAttrs = px->pdl ? 2 : 1;
-    return (int)cudaLaunchKernelEx(&cfg, table[px->bits - 3][pw->bits - 3][out_dtype == GBS_DTYPE_F32 ? 0 : 1], wmap, xmap, P);
+    return (int)cudaLaunchKernelEx(&cfg, pick(px->bits, pw->bits, out_dtype), wmap, xmap, P);
 }
