@@ -284,20 +284,26 @@ int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int s
     return n_best;
 }
 
-// Whether the few-token kernel (gbs_qgemv.cu) is the faster one.  Its time grows with the channels of an SM: these cycles per channel and
-// step of 128 codes on 148 SMs for up to 8, 16, 32 and 64 tokens (four bits, three bits on a side).  Beyond 16 tokens it grows in waves of 32
-// channels per SM (4736): so 32 tokens go to the tiles beyond two waves (three bits: 7800 channels) and 64 beyond one; 16 beyond 18 200
-// (8800).  Tiles of 128 channels come in waves too, 600 cycles a step whatever they hold, with much the same start; where a new one begins
-// (18 944 channels) the few-token kernel is the faster one again for a while.  Four bits, few-token kernel and tiles: 32 tokens -> 8704: 11.3
-// and 12.0 us, 10 240: 15.0 and 12.4; 64 tokens -> 4096: 8.4 and 11.4, 5760: 15.1 and 11.9; three bits: 32 -> 7168: 12.7 and 11.9, 20 ->
-// 7168: 11.6 and 12.0, 64 -> 4096: 11.0 and 12.0, 5760: 20.0 and 12.7.
+// Whether the few-token kernel (gbs_qgemv.cu) is the faster one, by cycles per step of 128 codes.  Tiles of 128 channels come in waves over
+// the SMs, 600 cycles each whatever they hold, with much the same start.  The few-token kernel's 17 - 64 tokens come in waves of 32 channels
+// per SM (4736 on 148): 300 cycles each up to 32 tokens, 600 up to 64.  So 32 tokens go to the tiles beyond two such waves and 64 beyond one.
+// Up to 16 tokens, and up to 32 with three bits on a side, the time was measured to grow with the channels of an SM.  Four bits: up to 8
+// tokens never go to the tiles, up to 16 beyond 18 200 channels until the tiles' second wave begins (18 944), and so on in every wave.
+// Three bits: up to 8 tokens likewise beyond 17 100, 16 beyond 8800, 32 beyond 7800.  4096 wide, few-token kernel and tiles, four bits: 32 tokens ->
+// 8704: 11.3 and 12.0 us, 10 240: 15.0 and 12.4; 64 tokens -> 4096: 8.4 and 11.4, 5760: 15.1 and 11.9; three bits: 32 -> 7168: 12.7 and
+// 11.9, 20 -> 7168: 11.6 and 12.0, 64 -> 4096: 11.0 and 12.0, 5760: 20.0 and 12.7.
 bool few_tokens(long long n_tok, long long n_out, bool three, int sm_count)
 {
     if (n_tok > GBS_QGEMV_MAX_TOKENS) return false;
-    static const double per_channel[2][4] = {{0.021, 0.033, 0.0633, 0.1266}, {0.035, 0.068, 0.077, 0.1266}};
-    const long long tiles = (n_out + TM - 1) / TM, waves = (tiles + sm_count - 1) / sm_count;
-    const double cycles = per_channel[three ? 1 : 0][n_tok <= 8 ? 0 : n_tok <= 16 ? 1 : n_tok <= 32 ? 2 : 3] * 148.0 / sm_count;
-    return (double)n_out * cycles <= 600.0 * (double)waves;
+    const long long tiles = (n_out + TM - 1) / TM, tile_waves = (tiles + sm_count - 1) / sm_count;
+    if (n_tok > 32 || (n_tok > 16 && !three)) {
+        const long long waves = (n_out + 32ll * sm_count - 1) / (32ll * sm_count);
+        return waves * (n_tok > 32 ? 600 : 300) <= 600 * tile_waves;
+    }
+    // per channel of the whole chip, on 148 SMs
+    static const double per_channel[2][3] = {{0.021, 0.033, 0.0}, {0.035, 0.068, 0.077}};
+    const double cycles = per_channel[three ? 1 : 0][n_tok <= 8 ? 0 : n_tok <= 16 ? 1 : 2] * 148.0 / sm_count;
+    return (double)n_out * cycles <= 600.0 * (double)tile_waves;
 }
 
 bool encode_codes(EncodeTiledFn encode, CUtensorMap* map, const void* codes, int64_t rows, int row_bytes, int bits, int box_rows)

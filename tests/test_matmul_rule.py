@@ -35,3 +35,13 @@ def test_a_part_of_the_chip_is_served(n_tok, n_out, d_pad, three, sms, pairs):
 def test_large_outputs_take_pairs():
     assert rule(4096, 4096, 4096) == (PAIRS, 256)
     assert rule(4096, 4096, 4096, pairs=0) == (TILES, 256)
+
+
+@pytest.mark.parametrize("sms", [148, 100])
+def test_few_tokens_beyond_sixteen_are_counted_in_waves_of_32_channels_per_sm(sms):
+    wave = 32 * sms
+    for n_tok, three, waves in ((17, False, 2), (32, False, 2), (33, False, 1), (64, False, 1), (33, True, 1), (64, True, 1)):
+        assert rule(n_tok, waves * wave, 4096, three, sms)[0] == FEW_TOKENS
+        assert rule(n_tok, waves * wave + 1, 4096, three, sms)[0] != FEW_TOKENS
+        assert rule(n_tok, 128 * sms + 1, 4096, three, sms)[0] != FEW_TOKENS          # the tiles' second wave
+    assert rule(65, 16, 4096, False, sms)[0] != FEW_TOKENS
