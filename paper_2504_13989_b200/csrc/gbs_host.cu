@@ -305,7 +305,7 @@ extern "C" int gbs_dequantize(const gbs_plan_t* p, const void* codes, const floa
         e = gbs_tc_denseinv_dequantize(p, codes, scales, n_rows, out, out_dtype, static_cast<cudaStream_t>(cuda_stream));
     else if ((flags & GBS_INVERSE_ROTATE) && gbs_tc_uvinv_serves(p, n_rows, out_dtype))
         e = gbs_tc_uvinv_dequantize(p, codes, scales, n_rows, out, out_dtype, static_cast<cudaStream_t>(cuda_stream));
-    else if ((flags & GBS_INVERSE_ROTATE) && gbs_rowinv_supported(p, scales))
+    else if ((flags & GBS_INVERSE_ROTATE) && gbs_rowinv_serves(p, scales, n_rows))
         e = gbs_rowinv_dequantize(p, codes, scales, n_rows, out, out_dtype, static_cast<cudaStream_t>(cuda_stream));
     else
         e = gbs_generic_dequantize(p, codes, scales, n_rows, out, out_dtype, (flags & GBS_INVERSE_ROTATE) != 0,

@@ -104,7 +104,7 @@ int gbs_tc_uvinv_dequantize(const gbs_plan* p, const void* codes, const float* s
                             int out_dtype, cudaStream_t stream);
 
 // gbs_rowinv.cu : the same for d' = 128 rows with one scale (pair) per row
-bool gbs_rowinv_supported(const gbs_plan* p, const float* scales);
+bool gbs_rowinv_serves(const gbs_plan* p, const float* scales, int64_t n_rows);
 int gbs_rowinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,
                              int out_dtype, cudaStream_t stream);
 

@@ -138,10 +138,12 @@ typedef void (*RowInvKernel)(const CUtensorMap, const RowInvParams);
 
 }  // namespace
 
-// The plans this path serves: d' = 128 (the ROW family) with one scale (pair) per row and whole 32-value output chunks.
-bool gbs_rowinv_supported(const gbs_plan* p, const float* scales)
+// What this path serves: d' = 128 (the ROW family) with one scale (pair) per row and whole 32-value output chunks, as many rows as the
+// stores' 32-bit coordinates count.
+bool gbs_rowinv_serves(const gbs_plan* p, const float* scales, int64_t n_rows)
 {
-    if (p->variant != GBS_VARIANT_TC_ROW || !(p->group == 0 || p->group == DP) || p->d % 32 != 0 || !get_encode()) return false;
+    if (p->variant != GBS_VARIANT_TC_ROW || !(p->group == 0 || p->group == DP) || p->d % 32 != 0 || n_rows > 0x7fffffff || !get_encode())
+        return false;
     return !(p->asym && (reinterpret_cast<uintptr_t>(scales) & 7u));        // (Delta, lo) pairs are read as one 8-byte word
 }
 
@@ -152,7 +154,6 @@ int gbs_rowinv_dequantize(const gbs_plan* p, const void* codes, const float* sca
         {{k_row_inv<3, false, float>, k_row_inv<3, false, __nv_bfloat16>}, {k_row_inv<3, true, float>, k_row_inv<3, true, __nv_bfloat16>}},
         {{k_row_inv<4, false, float>, k_row_inv<4, false, __nv_bfloat16>}, {k_row_inv<4, true, float>, k_row_inv<4, true, __nv_bfloat16>}}};
     const long long blocks = (n_rows + RI_THREADS - 1) / RI_THREADS;
-    if (n_rows > 0x7fffffff) return (int)cudaErrorInvalidValue;            // rows are counted in 32 bits by the stores
     RowInvParams P;
     memset(&P, 0, sizeof(P));
     P.n_rows = n_rows;
