@@ -31,6 +31,13 @@ __device__ __forceinline__ unsigned hfma2(unsigned a, unsigned b, unsigned c)
     asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
+// -a, which an addition or FMA takes as a modifier of its operand
+__device__ __forceinline__ unsigned hneg2(unsigned a)
+{
+    unsigned d;
+    asm("neg.f16x2 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
+}
 // (lo, hi) -> (lo + hi, lo - hi)
 __device__ __forceinline__ unsigned hpair(unsigned v)
 {

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_inv(const __grid_constant_
                         if (SPLIT) {
                             const unsigned n1 = h[4 * c + e];                              // n * 2^-10
                             ph[e] = hmul2(n1, sh2);
-                            pl[e] = hfma2(n1, sl2, hfma2(n1, sh2, ph[e] ^ 0x80008000u));
+                            pl[e] = hfma2(n1, sl2, hfma2(n1, sh2, hneg2(ph[e])));
                         } else {
                             ph[e] = h[4 * c + e];
                         }
