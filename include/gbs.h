@@ -86,8 +86,9 @@ typedef struct gbs_plan_info {
                                       Paley matrix (d' = m), 5 = as 3 where also d' = 128 * U with 80 <= U <= 256,
                                       d % 128 == 0 and group <= 4096: rotate-quantize keeps the rest of the transform
                                       in registers, clip scoring runs as in 3 (GBS_NO_UVR=1 forces 3) (set GBS_FORCE_GENERIC=1 in the
-                                      environment before gbs_plan_create to force 0; GBS_NO_PDL=1 launches it
-                                      without programmatic stream serialization) */
+                                      environment before gbs_plan_create to force 0; GBS_NO_PDL=1: its launches,
+                                      plain dequantize and KV restore among them, without programmatic
+                                      stream serialization) */
 } gbs_plan_info_t;
 
 /*

@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(NT) k_dequantize_stream(int d_pad, int glog, i
         if (col >= d_pad) { col -= d_pad; ++row; }
     }
     // only now: blocks of the next launch that move in as the first ones of this end crowd on some of the SMs, and with four blocks to an SM
-    // the even spread counts (4096 x 4096, 4 bits -> bf16: 10.4 us in stream order, 12.2 with this at the start, 9.4 here)
+    // the even spread counts (4096 x 4096, 4 bits -> bf16, one output buffer: 10.4 us in stream order, 12.2 with this at the start, 9.4 here)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
@@ -967,7 +967,7 @@ int gbs_generic_dequantize(const gbs_plan* p, const void* codes, const float* sc
         // (and always for 4-byte outputs, where the direct form holds too few bytes in flight); measured crossover
         const bool staged = out_dtype == GBS_DTYPE_F32 || 2 * tiles >= 5 * cap2;
         // The launch overlaps the end of the one before it, as in the tensor-core families: 2000 x 4096, 4 bits, groups of 128 -> bf16 8.3 ->
-        // 5.5 us, -> fp32 12.5 -> 10.2; 4096 x 3584, 3 bits -> bf16 12.3 -> 9.8; 300 x 4096 -> fp32 6.3 -> 4.3.
+        // 6.1 us, -> fp32 12.5 -> 10.9; 4096 x 4096, 3 bits -> bf16 16.6 -> 14.2; 100 x 4096, 4 bits -> fp32 6.3 -> 4.5 (outputs in turn, more than L2).
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(staged ? grid2 : grid));
         cfg.blockDim = dim3(NT);

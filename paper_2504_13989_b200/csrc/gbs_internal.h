@@ -33,7 +33,7 @@ struct gbs_plan {
     int smem_optin;        // largest dynamic shared memory a block may opt in to
     int variant;
     float* d_hm;           // device: H_m as floats, m*m row-major, followed by H_m^T (m*m)
-    int pdl;               // tensor-core families launch with programmatic stream serialization
+    int pdl;               // launches carry programmatic stream serialization: all but the general family's rotation and the DENSE inverse
     int asym;              // asymmetric quantizer (GBS_PLAN_ASYMMETRIC)
     int uvm_glog;          // UVM family: log2 of the number of 32-value chunks per tensor-core output row
     unsigned char* d_aimg; // device: pre-swizzled bf16 image of H_m (x) H_{2^j} for the tensor-core family (32 KB)

@@ -10,10 +10,10 @@
 //   * A set serves every third step and a stage of operands every fourth, so barriers are indexed by the step modulo twelve: each
 //     waiter then takes part in every phase of the barriers it waits for.
 // What bounds it: with 256 tokens a step takes about 730 cycles at 1.9 GHz, 512 of them the tensor pipe's, at the 1 kW limit (with a quarter of
-// the MMAs 4096^3 takes 52.6 instead of 56.1 us; more stages of either kind, running indices and unpacking before the wait for a free
+// the MMAs 4096^3 takes 52.6 instead of 56 us; more stages of either kind, running indices and unpacking before the wait for a free
 // stage change nothing or cost time); 256 tiles are 3.5 waves over 74 pairs and count as four.
-// 4096 x 4096 x 4096: 4 bits 63.0 -> 56.1 us (2.45 POP/s, 0.74 of twice the measured bf16 rate), 3 bits 72.0 -> 60.6.  300 tokens -> 14336:
-// 33.3 -> 25.8 and 39.5 -> 27.3.  1000 -> 4096: 20.0 -> 18.7.
+// 4096 x 4096 x 4096: 4 bits 63.5 -> 55.9 us (2.46 POP/s, 0.74 of twice the measured bf16 rate), 3 bits 71.9 -> 60.3.  300 tokens -> 14336:
+// 29.3 -> 26.2 and 33.6 -> 28.1.  1000 -> 4096: 19.7 -> 18.3 and 22.0 -> 19.4.
 // Every wait is bounded; an expired wait records a code in the activation plan's status word, and both SMs come to the last barrier.
 #include <string.h>
 
@@ -67,8 +67,8 @@ __device__ __forceinline__ void pair_commit(void* bar)
 //     relaxed arrival; a relaxed wait and tcgen05.fence::after_thread_sync.  The same wait and fence stand behind a commit.
 //   * tokens written to shared memory: fence.proxy.async by each lane, then one release per warp; the issuer acquires before it lets the
 //     tensor cores (async proxy) read both SMs' shared memory.  Before a stage is written again the warps acquire behind the commit's wait.
-// The fences are the ones restricted to shared memory: with them 4096^3 takes 55.9 us at 4 bits and 60.5 at 3 (56.2 and 60.1 with
-// arrivals and waits of CTA scope).  An arrival with .release.cluster orders the writer's global accesses as well: 98.9 us.
+// The fences are the ones restricted to shared memory: with them 4096^3 takes 55.9 us at 4 bits and 60.3 at 3 (56.1 and 59.8 with
+// arrivals and waits of CTA scope; 700 tokens -> 9088 at 3 bits: 28.8 and 28.1).  An arrival with .release.cluster orders the writer's global accesses as well: 98.9 us.
 __device__ __forceinline__ void pair_arrive(unsigned bar_addr)
 {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");

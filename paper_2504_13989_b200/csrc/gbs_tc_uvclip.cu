@@ -228,8 +228,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                 if (lane == 0) mbar_arrive(&S->tempty[s]);
                 mb = __reduce_max_sync(0xffffffffu, __float_as_uint(fwht32_absmax(r)));
             }
-            // the token's maximum; behind this barrier its histogram is clear as well.  A warp whose wait ran out comes too,
-            // with a pattern no maximum has, and all four leave.
+            // the token's maximum.  The barrier also keeps this token's atomics behind the reads of the running totals at the token before:
+            // all four warps have them in registers when they come here.  A warp whose wait ran out comes too, with a pattern no
+            // maximum has, and all four leave.
             unsigned* slot = S->red[t][it & 1];
             if (lane == 0) slot[q] = mb;
             asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
