@@ -412,18 +412,15 @@ __device__ __forceinline__ float absmax32(const unsigned r[32])
 // ---------------------------------------------------------------------------------------------
 // epilogue arithmetic
 // ---------------------------------------------------------------------------------------------
-// H_32 on 32 registers (in place, natural order) and max|.| of the result.  The four upper stages act on
-// register pairs as they come out of TMEM (packed add/sub); the lowest stage pairs the two halves of a
-// pair and is scalar, which leaves the results as the scalars the quantizer consumes.
-__device__ __forceinline__ float fwht32_absmax(unsigned r[32])
+// H_{2 N} on N register pairs and max|.| of the result.  The upper stages act on pairs (packed add/sub); the lowest one pairs the two
+// halves of a pair and is scalar, which leaves the results as the scalars the quantizer consumes.
+template <int N>
+__device__ __forceinline__ float fwht_pairs_absmax(f32x2 p[N], unsigned* r)
 {
-    f32x2 p[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) p[i] = pk(r[2 * i], r[2 * i + 1]);
+    for (int h = 1; h < N; h <<= 1)
 #pragma unroll
-    for (int h = 1; h < 16; h <<= 1)
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
+        for (int i = 0; i < N; ++i)
             if ((i & h) == 0) {
                 const f32x2 a = p[i], b = p[i + h];
                 p[i] = add2(a, b);
@@ -431,7 +428,7 @@ __device__ __forceinline__ float fwht32_absmax(unsigned r[32])
             }
     float m = 0.f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
+    for (int i = 0; i < N; ++i) {
         unsigned ua, ub;
         unpk(p[i], ua, ub);
         const float a = __uint_as_float(ua), b = __uint_as_float(ub);
@@ -441,6 +438,23 @@ __device__ __forceinline__ float fwht32_absmax(unsigned r[32])
         m = max3(fabsf(y0), fabsf(y1), m);
     }
     return m;
+}
+// H_32 on 32 registers (in place, natural order) and max|.| of the result.
+__device__ __forceinline__ float fwht32_absmax(unsigned r[32])
+{
+    f32x2 p[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) p[i] = pk(r[2 * i], r[2 * i + 1]);
+    return fwht_pairs_absmax<16>(p, r);
+}
+// Half of H_32's outputs, in r[0 .. 15]: the first sixteen (sign = 1) or the others (sign = -1).
+__device__ __forceinline__ float fwht32_half_absmax(unsigned r[32], float sign)
+{
+    f32x2 p[8];
+    const f32x2 s = pk(__float_as_uint(sign), __float_as_uint(sign));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = fma2(pk(r[2 * i + 16], r[2 * i + 17]), s, pk(r[2 * i], r[2 * i + 1]));
+    return fwht_pairs_absmax<8>(p, r);
 }
 
 // 32 consecutive values -> codes -> packed little-endian bit stream (BITS * 4 bytes).

@@ -1,12 +1,12 @@
-// gbs_clip_error for bf16 rows of the UV family with one scale per token, by histogram instead of one pass per candidate.
+// gbs_clip_error for bf16 rows of the UV family by histogram instead of one pass per candidate.
 //
-// With t = |y| / M (M = the token's max|y|), candidate k quantizes |y| / M to the level l = number of its thresholds
+// With t = |y| / M (M = the max|y| of the token or group), candidate k quantizes |y| / M to the level l = number of its thresholds
 // (j + 1/2) alpha_k / D, j = 0 .. D-1, that t has reached (Sections 2.1, 3.1: rounding to the nearest level, clipping at D).
 // With D' = alpha_k / D the error is  M^2 (t - D' l)^2 = M^2 [t^2 - 2 D' t l + D'^2 l^2],  so all K candidates follow from how
 // many values (W0) and which sum of t (W1) lie beyond each of the K D thresholds:
 //        sum t l = sum_j W1(beyond threshold j),    sum l^2 = sum_j (2 j + 1) W0(beyond threshold j).
 // One histogram over the sorted thresholds replaces 5 K operations per value by about 12 whatever K is.
-//   * Front end as in gbs_tc_uv.cu: TMA, A X on tcgen05, H_32 in registers, the token's maximum over its four warps.
+//   * Front end as in gbs_tc_uv.cu: TMA, A X on tcgen05, H_32 in registers, the maximum over a token's four warps.
 //   * t becomes a 22-bit integer in the mantissa of one FMA.  Its high bits index a table of cells; an entry holds the
 //     number of thresholds below the cell and the low bits of the one threshold inside it, placed so that adding the
 //     value's low bits carries into the bin index when the threshold is reached.  Cells are as wide as they can be without two
@@ -17,18 +17,27 @@
 //     out one unit of t apart when the ratios are rounded to floats; they count as one, the lower.)
 //   * Two shared-memory atomics per value (count and t) into COPIES interleaved histograms per token, so that a warp's lanes
 //     rarely meet: measured 2 cycles per 32 values with 32 copies and 6 with 8.  Everything is an integer: exact in any order.
-//   * After a token its 128 threads add the copies up and weigh them with M^2 in fp64.  Nothing is cleared: the words grow modulo 2^32
-//     and a token's part is the difference from the total before it, which its thread keeps.  The t^2 term is the sum of the
-//     same integers' squares, in 64 bits, so the three parts of the error belong to one and the same t and may cancel down to the
-//     16 digits of fp64: a candidate that fits a batch exactly is as accurate as the others, wherever it stands in the list.
+//   * One scale per token: after a token its 128 threads add the copies up and weigh them with M^2 in fp64.  Nothing is cleared: the words
+//     grow modulo 2^32 and a token's part is the difference from the total before it, which its thread keeps.
+//   * One scale per group of 128 coordinates or more: the four rows of A X that make up 128 coordinates go to the same lane of the four
+//     quadrants, so a warp's lanes belong to different groups and the copy of a lane IS a group's histogram.  The copies are then weighed one by
+//     one with their groups' M^2 and cleared; every warp takes a share of the copies of every bin, so that its weights stay in
+//     registers.  (A thread per bin instead reads all 32 weights for each of them and leaves a warp idle: 32 768 x 4096, K = 32: 219 us at 3 bits
+//     and 321 at 4, against 196 and 277.)  More than 112 thresholds leave room for the histograms of two tokens, not four: two warps then share a
+//     lane, each taking half of H_32's outputs.
+//   * The t^2 term is the sum of the same integers' squares, in 64 bits, so the three parts of the error belong to one and the same t and
+//     may cancel down to the 16 digits of fp64: a candidate that fits a batch exactly is as accurate as the others, wherever it stands in the list.
 //     t's rounding is the only approximation: at most 2^-23, so that an error E over n values moves by at most
 //     2^-22 M sqrt(n E) + n 2^-46 M^2 -- the size of Delta's rounding in the per-candidate kernel -- and, where the values differ,
 //     by the square root of n less.
 //   * A stands in tensor memory, so that an MMA reads one operand from shared memory and the table has the other's room.
-// What bounds it: the shared-memory port (per token about 130 cycles of lookups, 330 of atomics, 200 of adding up, 65 of the MMA's operand)
-// and instruction issue (about 700 slots of each scheduler).
+// What bounds it: the chain of a token's four warps, with the shared-memory port 62 - 66 % busy (per token about 130 cycles of lookups, 330 of
+// atomics, 200 of adding up, 450 with groups, 65 of the MMA's operand) and 50 - 66 % of the issue slots taken.  Neither count and sum in one
+// atomic (2^24 + t, taken apart again when added up; two histograms in turn and one barrier per token: 148 us where this takes 135)
+// nor barriers that warps arrive at early and wait for late (154) nor fewer instructions per value (no change) make it faster.
 // 32 768 x 4096, K = 32, 3 bits: 829 us with five fp32 operations per value and candidate; 171.4 with one copy of the table, histograms
-// that were cleared for every token (390 cycles with the adding up) and A in shared memory; 135.2 now.
+// that were cleared for every token (390 cycles with the adding up) and A in shared memory; 135.2 now.  Groups of 128: 839 -> 196 us at 3
+// bits, 839 -> 277 at 4; K = 8: 253 -> 162 and 179.
 #include <math.h>
 #include <string.h>
 
@@ -39,19 +48,18 @@
 
 namespace {
 
-constexpr int V = 32, TOK = 4, UMAX = 128;
+constexpr int V = 32, TOK_MAX = 4, UMAX = 128;    // a tile is 4 tokens, or 2
 constexpr int STAGES = 2;                          // accumulators; one set of rows in shared memory: a tile takes far longer than its load
-constexpr int STAGE_COLS = TOK * V;
-constexpr int STAGE_BYTES_MAX = TOK * UMAX * V * 2;
-constexpr int A_COL0 = STAGES * STAGE_COLS;        // A in tensor memory: a row per lane, two entries per column
-constexpr int EPI_WARPS = 4 * TOK;
+constexpr int STAGE_BYTES_MAX = TOK_MAX * UMAX * V * 2;
+constexpr int A_COL0 = STAGES * TOK_MAX * V;       // A in tensor memory: a row per lane, two entries per column
+constexpr int EPI_WARPS = 16;                      // 16 / TOK of them to a token
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int TMEM_COLS = 512;
 constexpr int T_BITS = 22;                         // t is an integer of 22 bits
 constexpr int TABLE_LOG = 14;                      // words of the table of cells: cells x copies
 constexpr int MIN_CELL_BITS = 10, MAX_CELL_BITS = 13;          // bits of t inside a cell: 4096 cells x 4 copies .. 512 x 32
-constexpr int HIST_ROWS = 3584;                    // words of a token's counts (and of its sums): bins x copies
-constexpr int HIST_WORDS = TOK * 2 * (HIST_ROWS + 32);   // [token][count, sum][one row nobody reads, bins][copy]
+constexpr int HIST_TILE = 14336;                   // words of a tile's counts (and of its sums): tokens x bins x copies
+constexpr int HIST_WORDS = 2 * (HIST_TILE + TOK_MAX * 32);     // [token][count, sum][one row nobody reads, bins][copy]
 constexpr int MAX_BINS = 448;                      // thresholds: K D at most
 constexpr unsigned POISON = 0xffffffffu;
 
@@ -59,7 +67,8 @@ struct __align__(1024) Smem {
     unsigned char b[STAGE_BYTES_MAX];
     unsigned hist[HIST_WORDS];
     unsigned lut[1 << TABLE_LOG];
-    unsigned red[TOK][2][4];                       // maxima, by tile parity
+    unsigned red[TOK_MAX][2][256];                 // maxima, by tile parity: a word per warp, or one per lane (groups)
+    double2 weight[2][TOK_MAX][16];                // groups: M^2 of every copy, by tile parity
     double square[EPI_WARPS];                      // sums of t^2
     unsigned long long full, empty, tfull[STAGES], tempty[STAGES];
     unsigned tmem_base;
@@ -67,11 +76,11 @@ struct __align__(1024) Smem {
 };
 
 struct ClipParams {
-    long long n_rows;
-    int n_groups;                 // ceil(n_rows / TOK)
-    int U, Upad, ksteps;
+    int n_groups;                 // tiles: ceil(n_rows / TOK)
+    int Upad, ksteps;
     int K, levels, n_thr;
     int cell_bits;                // the largest number for which no cell holds two different thresholds
+    int glog;                     // groups: log2(lanes per group), a lane of four warps having four rows of A X
     float scale;                  // of t as an integer
     float norm2;                  // 1 / d'
     const unsigned char* a_img;
@@ -89,12 +98,28 @@ __device__ __forceinline__ unsigned ld_shared(unsigned a)
     return v;
 }
 
-// COPIES x BINS is the same for every instantiation: as many copies as the thresholds leave room for
-template <int COPIES>
+// an integer as a double, by its place in the mantissa of 2^52
+__device__ __forceinline__ double exact(unsigned v) { return __hiloint2double(0x43300000, (int)v) - 4503599627370496.0; }
+
+// Tokens of a tile, copies of a histogram (TOK x COPIES x bins is the same for every instantiation: as many copies as the thresholds leave
+// room for), one scale per token or per group
+template <int TOK, int COPIES, bool GROUPED>
 __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ ClipParams P)
 {
+    constexpr int HALVES = 4 / TOK;                               // warps that share a TMEM lane of a token
+    constexpr int NV = V / HALVES;                                // values of a thread
+    constexpr int TOKEN_WARPS = 4 * HALVES;
+    constexpr int STAGE_COLS = TOK * V;
+    constexpr int HIST_ROWS = HIST_TILE / TOK;                    // words of a token's counts (and of its sums)
     constexpr int BINS = HIST_ROWS / COPIES;
-    constexpr int PER = (BINS + 127) / 128;                       // bins a thread adds up
+    // Adding up: a thread takes all copies of a bin, or, with groups, every warp of a token a share (CHUNKS times four) of the copies
+    // of every bin, 32 bins at a time.
+    constexpr int CHUNKS = GROUPED ? 8 / TOKEN_WARPS : COPIES / 4;
+    constexpr int BIN_LANES = GROUPED ? 32 : 32 * TOKEN_WARPS;
+    constexpr int PER = (BINS + BIN_LANES - 1) / BIN_LANES;       // bins of a thread
+    constexpr int PARTS = GROUPED ? EPI_WARPS : TOK;               // of a bin's total
+    static_assert(TOK == 4 || GROUPED, "two warps share a lane only where groups leave no room for four tokens");
+    static_assert(!GROUPED || COPIES == 32, "a copy per lane");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem* S = reinterpret_cast<Smem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -140,7 +165,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     }
     if (warp >= 2 && warp < 6) {
         // A (plan-owned, immutable: needs no ordering) from its image, two blocks of 64 columns, 128-byte swizzled rows, to tensor memory
-        const int r = (warp & 3) * 32 + lane;
+        // groups: four neighbouring rows go to the same lane of the four quadrants, so that a warp's lanes belong to 32 different groups
+        const int r = GROUPED ? 4 * lane + (warp & 3) : (warp & 3) * 32 + lane;
         const unsigned at = tmem_base + ((unsigned)((warp & 3) * 32) << 16) + A_COL0;
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
@@ -194,7 +220,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         }
     } else {
         // ------------------------------ histogram ------------------------------
-        const int t = (warp - 2) >> 2, q = warp & 3, ti = q * 32 + lane;
+        const int w = warp - 2, t = w / TOKEN_WARPS, half = (w >> 2) % HALVES, q = warp & 3;
+        const int wt = half * 4 + q;                              // of the token's warps
+        const int bin0 = GROUPED ? lane : q * 32 + lane;
+        const int chunk0 = GROUPED ? lane + wt * CHUNKS : lane;   // eight lanes side by side: different banks
         const unsigned taddr0 = tmem_base + ((unsigned)(q * 32) << 16) + t * V;
         unsigned* hist = S->hist + t * 2 * (HIST_ROWS + 32) + 32;            // behind a row for values below every threshold
         constexpr unsigned BIN_STEP = COPIES * 4;
@@ -206,18 +235,70 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         const unsigned cell_mask = (4u << TABLE_LOG) - (4u << copies_log);        // a cell's first byte in the table
         const unsigned low_mask = (1u << P.cell_bits) - 1u;
         const int cell_bits = P.cell_bits;
-        // the histograms only ever grow, modulo 2^32: a token's own counts and sums are what a bin has gained since the token before
+        // one scale per token: the histograms only ever grow, modulo 2^32, and a token's own counts and sums are what a bin has gained
+        // since the token before
         unsigned was0[PER], was[PER][4];
 #pragma unroll
         for (int i = 0; i < PER; ++i) was0[i] = was[i][0] = was[i][1] = was[i][2] = was[i][3] = 0u;
         constexpr float MAGIC = 8388608.f;
         constexpr unsigned E = 0x4B000000u;                       // its bit pattern
-        double square = 0.0;
+        double square = 0.0, m2 = 0.0;
         float poison = 0.f;                                       // NaN once a value was not finite
+        // what the token of tile `it` left in this thread's bins
+        auto add_up = [&](int it) {
+            double2 weight[GROUPED ? CHUNKS : 1][2];               // groups: every copy is another one's
+            if (GROUPED) {
+#pragma unroll
+                for (int j = 0; j < CHUNKS; ++j) {
+                    const int jj = (chunk0 + j) % (COPIES / 4);
+                    weight[j][0] = S->weight[it & 1][t][2 * jj];
+                    weight[j][1] = S->weight[it & 1][t][2 * jj + 1];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const int bin = bin0 + BIN_LANES * i;
+                if (bin < P.n_thr) {
+                    uint4* row = reinterpret_cast<uint4*>(hist + bin * COPIES);
+                    uint4* row1 = reinterpret_cast<uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
+                    if (GROUPED) {
+                        // weighed one by one, and cleared
+#pragma unroll
+                        for (int j = 0; j < CHUNKS; ++j) {
+                            const int jj = (chunk0 + j) % (COPIES / 4);
+                            const uint4 x = row[jj], z = row1[jj];
+                            row[jj] = row1[jj] = make_uint4(0u, 0u, 0u, 0u);
+                            w0[i] = fma(weight[j][0].x, exact(x.x), w0[i]); w1[i] = fma(weight[j][0].x, exact(z.x), w1[i]);
+                            w0[i] = fma(weight[j][0].y, exact(x.y), w0[i]); w1[i] = fma(weight[j][0].y, exact(z.y), w1[i]);
+                            w0[i] = fma(weight[j][1].x, exact(x.z), w0[i]); w1[i] = fma(weight[j][1].x, exact(z.z), w1[i]);
+                            w0[i] = fma(weight[j][1].y, exact(x.w), w0[i]); w1[i] = fma(weight[j][1].y, exact(z.w), w1[i]);
+                        }
+                    } else {
+                        unsigned c = 0u;
+                        uint4 m = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                        for (int j = 0; j < CHUNKS; ++j) {
+                            const int jj = (chunk0 + j) % (COPIES / 4);
+                            const uint4 x = row[jj], z = row1[jj];
+                            c += (x.x + x.y) + (x.z + x.w);
+                            m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
+                        }
+                        // a component gains at most 1024 values below 2^22: less than 2^32
+                        const unsigned long long sum = ((unsigned long long)(m.x - was[i][0]) + (m.y - was[i][1])) +
+                                                       ((unsigned long long)(m.z - was[i][2]) + (m.w - was[i][3]));
+                        w0[i] += m2 * (double)(c - was0[i]);
+                        w1[i] += m2 * (double)sum;
+                        was0[i] = c;
+                        was[i][0] = m.x; was[i][1] = m.y; was[i][2] = m.z; was[i][3] = m.w;
+                    }
+                }
+            }
+        };
+
         for (int it = 0; it < n_mine; ++it) {
             const int s = it % STAGES;
             const bool ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull[s], (it / STAGES) & 1, P.status, 4, false));
-            unsigned r[32];
+            unsigned r[V];
             unsigned mb = POISON;
             if (ok) {
                 tc_fence_after();
@@ -226,30 +307,38 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S->tempty[s]);
-                mb = __reduce_max_sync(0xffffffffu, __float_as_uint(fwht32_absmax(r)));
+                mb = __float_as_uint(HALVES == 1 ? fwht32_absmax(r) : fwht32_half_absmax(r, half ? -1.f : 1.f));
+                if (!GROUPED) mb = __reduce_max_sync(0xffffffffu, mb);
             }
-            // the token's maximum.  The barrier also keeps this token's atomics behind the reads of the running totals at the token before:
-            // all four warps have them in registers when they come here.  A warp whose wait ran out comes too, with a pattern no
-            // maximum has, and all four leave.
             unsigned* slot = S->red[t][it & 1];
-            if (lane == 0) slot[q] = mb;
-            asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
-            mb = max(max(slot[0], slot[1]), max(slot[2], slot[3]));
-            if (mb == POISON) break;
+            if (GROUPED) slot[wt * 32 + lane] = mb;
+            else if (lane == 0) slot[q] = mb;
+            // The barrier also keeps this token's atomics behind the adding up of the token before.
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + t), "n"(32 * TOKEN_WARPS) : "memory");
+            if (GROUPED) {
+#pragma unroll
+                for (int i = 0; i < TOKEN_WARPS; ++i) mb = max(mb, slot[i * 32 + lane]);
+            } else {
+                mb = max(max(slot[0], slot[1]), max(slot[2], slot[3]));
+            }
+            if (mb == POISON) break;                               // in every lane
+            if (GROUPED)
+                for (int o = (1 << P.glog) >> 1; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
             const float M = __uint_as_float(mb);
+            if (GROUPED && wt == 0) reinterpret_cast<double*>(S->weight[it & 1][t])[lane] = (double)M * (double)M;
             float lift = 1.f;                                      // scale / M must not overflow
             if (M < 0x1p-96f) {
                 lift = 0x1p64f;
 #pragma unroll
-                for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * lift);
+                for (int i = 0; i < NV; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * lift);
             }
             const float sc = M > 0.f ? P.scale / (M * lift) : 0.f;
-            // every one of the 32 values is a signed sum of all that came out of TMEM: the first shows whether one was not finite
+            // every value is a signed sum of all that came out of TMEM: the first shows whether one was not finite
             poison = fmaf(__uint_as_float(r[0]), 0.f, poison);
-            unsigned long long sq = 0ull;                          // 32 squares below 2^44
+            unsigned long long sq = 0ull;                          // squares below 2^44
             // eight values at a time: their lookups are in flight together
 #pragma unroll
-            for (int i0 = 0; i0 < 32; i0 += 8) {
+            for (int i0 = 0; i0 < NV; i0 += 8) {
                 unsigned b[8], e[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -269,70 +358,51 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                     asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(at), "r"(b[i]), "n"(SUM_OFF) : "memory");
                 }
             }
-            asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
-            const double m2 = (double)M * (double)M;
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + t), "n"(32 * TOKEN_WARPS) : "memory");
+            m2 = (double)M * (double)M;
             square += m2 * (double)sq;
-#pragma unroll
-            for (int i = 0; i < PER; ++i) {
-                const int bin = ti + 128 * i;
-                if (bin < P.n_thr) {
-                    const uint4* row = reinterpret_cast<const uint4*>(hist + bin * COPIES);
-                    const uint4* row1 = reinterpret_cast<const uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
-                    unsigned c = 0u;
-                    uint4 m = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                    for (int j = 0; j < COPIES / 4; ++j) {
-                        const int jj = (j + lane) % (COPIES / 4);          // eight lanes side by side: different banks
-                        const uint4 x = row[jj], z = row1[jj];
-                        c += (x.x + x.y) + (x.z + x.w);
-                        m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
-                    }
-                    // a component gains at most 1024 values below 2^22: less than 2^32
-                    const unsigned long long sum = ((unsigned long long)(m.x - was[i][0]) + (m.y - was[i][1])) +
-                                                   ((unsigned long long)(m.z - was[i][2]) + (m.w - was[i][3]));
-                    w0[i] += m2 * (double)(c - was0[i]);
-                    w1[i] += m2 * (double)sum;
-                    was0[i] = c;
-                    was[i][0] = m.x; was[i][1] = m.y; was[i][2] = m.z; was[i][3] = m.w;
-                }
-            }
+            add_up(it);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) square += __shfl_xor_sync(0xffffffffu, square, o);
         if (__any_sync(0xffffffffu, poison != 0.f)) square = __longlong_as_double(0x7ff8000000000000ll);
-        if (lane == 0) S->square[warp - 2] = square;
+        if (lane == 0) S->square[w] = square;
     }
 
-    // ---- the block's totals: [bin] over the four token slots, then from the last threshold down
+    // ---- the block's totals: [bin] over the parts, then from the last threshold down
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);
     }
-    double* tot = reinterpret_cast<double*>(S->hist);              // [slot][2][MAX_BINS]
+    double* tot = reinterpret_cast<double*>(S->hist);              // [part][2][BINS]
     if (warp >= 2) {
-        const int t = (warp - 2) >> 2, ti = (warp & 3) * 32 + lane;
+        const int part = GROUPED ? warp - 2 : (warp - 2) / TOKEN_WARPS;
 #pragma unroll
-        for (int i = 0; i < PER; ++i)
-            if (ti + 128 * i < P.n_thr) {
-                tot[(t * 2) * MAX_BINS + ti + 128 * i] = w0[i];
-                tot[(t * 2 + 1) * MAX_BINS + ti + 128 * i] = w1[i];
+        for (int i = 0; i < PER; ++i) {
+            const int bin = (GROUPED ? lane : (warp & 3) * 32 + lane) + BIN_LANES * i;
+            if (bin < P.n_thr) {
+                tot[(part * 2) * BINS + bin] = w0[i];
+                tot[(part * 2 + 1) * BINS + bin] = w1[i];
             }
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 2 * P.n_thr; i += THREADS) {
-        double* d = tot + (i < P.n_thr ? i : MAX_BINS + i - P.n_thr);
-        d[0] = (d[0] + d[2 * MAX_BINS]) + (d[4 * MAX_BINS] + d[6 * MAX_BINS]);
+        double* d = tot + (i < P.n_thr ? i : BINS + i - P.n_thr);
+        double sum = d[0];
+        for (int part = 1; part < PARTS; ++part) sum += d[part * 2 * BINS];
+        d[0] = sum;
     }
     __syncthreads();
-    double* suf = tot + TOK * 2 * MAX_BINS;                        // [2][MAX_BINS]: sum over bins b, b + 1, ..
+    double* suf = tot + PARTS * 2 * BINS;                          // [2][BINS]: sum over bins b, b + 1, ..
     if (warp < 2) {
         // warp 0 the counts, warp 1 the sums: a contiguous piece per lane, pieces joined from the right
         const int per = (P.n_thr + 31) / 32, b0 = lane * per;
         double s = 0.0;
         for (int b = b0; b < b0 + per && b < P.n_thr; ++b)
-            s += tot[warp * MAX_BINS + b];
+            s += tot[warp * BINS + b];
         double after = s;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -341,8 +411,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         }
         after -= s;                                                // the pieces to the right of this one
         for (int b = (b0 + per < P.n_thr ? b0 + per : P.n_thr) - 1; b >= b0; --b) {
-            after += tot[warp * MAX_BINS + b];
-            suf[warp * MAX_BINS + b] = after;
+            after += tot[warp * BINS + b];
+            suf[warp * BINS + b] = after;
         }
     }
     __syncthreads();
@@ -354,7 +424,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         for (int j = 0; j < P.levels; ++j) {
             const int b = P.idx[k][j];
             l2 += (double)(2 * j + 1) * suf[b];
-            l1 += suf[MAX_BINS + b];
+            l1 += suf[BINS + b];
         }
         const double err = (t2 / scale - 2.0 * d * l1) / scale + d * d * l2;
         atomicAdd(&P.err_sum[k], (err < 0.0 ? 0.0 : err) * (double)P.norm2);       // what fp64 leaves of an exact fit; NaN stays
@@ -365,16 +435,19 @@ typedef void (*ClipKernel)(const CUtensorMap, const ClipParams);
 
 }  // namespace
 
-// Scores K clip ratios, or returns GBS_UVCLIP_NOT_SERVED where this path does not apply (group scales, per-row sums, thresholds
-// too close to one another): the caller then takes the per-candidate kernel.  So it does where that is the faster one: a tile per block at
-// most and candidates for one of its passes (eight), where building the table is what counts (64 x 4096, K = 8: 6.8 us there, 7.0 here at
-// 3 bits, 7.4 at 4; 600 rows, 4 bits: 11.2 and 10.1).
+// Scores K clip ratios, or returns GBS_UVCLIP_NOT_SERVED where this path does not apply (groups of 32 or 64, per-row sums, thresholds
+// too close to one another): the caller then takes the per-candidate kernel.  So it does where that is the faster one, with candidates for
+// one of its passes (eight) and few tiles per block, where building the table is what counts.  One scale per token: up to one (64 x 4096, K = 8:
+// 6.8 us there, 7.0 here at 3 bits, 7.4 at 4; 600 rows, 4 bits: 11.2 and 10.1).  Groups: up to three (700 rows: 16.5 and 16.7 at 3 bits,
+// 18.5 at 4; 2000: 24.9 and 22.8, 24.7).
 int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, const float* alphas, int K,
                              double* err_sum, cudaStream_t stream)
 {
     EncodeTiledFn encode = get_encode();
-    if (K <= 8 && n_rows <= (int64_t)TOK * p->sm_count) return GBS_UVCLIP_NOT_SERVED;
-    if (p->group != 0 || !encode || p->smem_optin < (int)sizeof(Smem) || n_rows > (int64_t)0x7fffffff - TOK) return GBS_UVCLIP_NOT_SERVED;
+    const bool grouped = p->group != 0;
+    if (K <= 8 && n_rows <= (int64_t)TOK_MAX * p->sm_count * (grouped ? 3 : 1)) return GBS_UVCLIP_NOT_SERVED;
+    if ((grouped && p->group < 4 * V) || !encode || p->smem_optin < (int)sizeof(Smem) || n_rows > (int64_t)0x7fffffff - TOK_MAX)
+        return GBS_UVCLIP_NOT_SERVED;
     ClipParams P;
     memset(&P, 0, sizeof(P));
     const int D = p->levels;
@@ -418,18 +491,26 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
         P.alpha[k] = alphas[k];
         for (int j = 0; j < D; ++j) P.idx[k][j] = rank[T[k * D + j] >> P.cell_bits];
     }
+    struct Form {
+        ClipKernel kernel;
+        int tok, bins;
+    };
+    static const Form forms[5] = {{k_tc_uv_clip<4, 32, false>, 4, 112}, {k_tc_uv_clip<4, 16, false>, 4, 224}, {k_tc_uv_clip<4, 8, false>, 4, 448},
+                                  {k_tc_uv_clip<4, 32, true>, 4, 112}, {k_tc_uv_clip<2, 32, true>, 2, 224}};
+    const Form* form = forms + (grouped ? 3 : 0);
+    while (form < forms + (grouped ? 5 : 3) && P.n_thr > form->bins) ++form;
+    if (form == forms + 5) return GBS_UVCLIP_NOT_SERVED;           // groups: a copy per lane leaves room for 224 thresholds
     CUtensorMap tmap;
     const int U = p->d_pad / V;
     P.Upad = (U + 15) & ~15;
     const cuuint64_t gdim[3] = {(cuuint64_t)V, (cuuint64_t)(p->d / V), (cuuint64_t)n_rows};
     const cuuint64_t gstr[2] = {(cuuint64_t)(V * 2), (cuuint64_t)(stride * 2)};
-    const cuuint32_t box[3] = {V, (cuuint32_t)P.Upad, TOK}, estr[3] = {1, 1, 1};
+    const cuuint32_t box[3] = {V, (cuuint32_t)P.Upad, (cuuint32_t)form->tok}, estr[3] = {1, 1, 1};
     if (encode(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return (int)cudaErrorInvalidValue;
-    P.n_rows = n_rows;
-    P.n_groups = (int)((n_rows + TOK - 1) / TOK);
-    P.U = U;
+    P.n_groups = (int)((n_rows + form->tok - 1) / form->tok);
+    for (int g = p->group / (4 * V); g > 1; g >>= 1) ++P.glog;
     P.ksteps = P.Upad / 16;
     P.K = K;
     P.levels = D;
@@ -437,15 +518,14 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
     P.a_img = p->d_aimg;
     P.err_sum = err_sum;
     P.status = p->d_status;
-    static const ClipKernel kernels[3] = {k_tc_uv_clip<32>, k_tc_uv_clip<16>, k_tc_uv_clip<8>};
     {
         // opt in to the large dynamic shared memory once per device (not a stream operation)
         static std::mutex mu;
         static bool done[64] = {false};
         std::lock_guard<std::mutex> lock(mu);
         if (!(p->device >= 0 && p->device < 64 && done[p->device])) {
-            for (ClipKernel k : kernels) {
-                const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+            for (const Form& f : forms) {
+                const cudaError_t e = cudaFuncSetAttribute(f.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
                 if (e != cudaSuccess) return (int)e;
             }
             if (p->device >= 0 && p->device < 64) done[p->device] = true;
@@ -461,5 +541,5 @@ int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, i
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p->pdl ? 1 : 0;
-    return (int)cudaLaunchKernelEx(&cfg, kernels[P.n_thr <= 112 ? 0 : P.n_thr <= 224 ? 1 : 2], tmap, P);
+    return (int)cudaLaunchKernelEx(&cfg, form->kernel, tmap, P);
 }
