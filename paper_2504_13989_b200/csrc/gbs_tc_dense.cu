@@ -15,14 +15,18 @@
 //     the last CTA of the cluster, which has the fewest coordinates; it sends the value to the first.
 //   * One sweep.  A token's m fp32 values do not fit one SM's TMEM, so a CLUSTER of CTAs takes 128 tokens and each CTA up to
 //     512 output coordinates: TMEM lane t holds the CTA's coordinates of token t, and the CTAs exchange their maxima of
-//     every token through distributed shared memory before quantizing (Sections 2.1, 3.1).
-//   * Packed rows are m b / 8 bytes (579 at m = 1544, b = 3: any alignment): a warp packs its 32 tokens' codes into shared
-//     memory and writes the rows' pieces as words, sixteen lanes to a row, several rows in flight.
+//     every token through distributed shared memory before quantizing (Sections 2.1, 3.1): one float per token and pair of CTAs, by st.async, so that
+//     the receiver's barrier counts the bytes and no fence stands in between (1.7 us with stores and releasing arrivals, 0.45 now).
+//     What a CTA's epilogue has waited for is all that is ever written to it, so it leaves without meeting the others again (0.5 - 0.8 us).
+//   * Two warps issue the MMAs, each for half of the columns: one's polls and commits are covered by the other's MMAs.
+//   * Packed rows are m b / 8 bytes (579 at m = 1544, b = 3: any alignment): the four warps of a lane quadrant pack its 32 tokens' codes into
+//     shared memory, and each writes the CTA's piece of eight rows as words, what is left at either end by bytes.
 // What bounds it: the tensor pipe, 2 d m flops per token, and what stands around it.  4096 x 1536, b = 4: 176 us with two sweeps
 // over streamed chunks of H on 32 SMs; 27.4 us with one sweep over the Toeplitz operand, of which 13.9 were the MMAs (a poll and
-// a commit per 64 columns cost 217 of 1050 cycles: hence 128 columns per stage), 1.6 the first CTA's waiting for its threads
-// to sum row 0 from the stages, 6.6 storing the codes row after row.  The number of CTAs per cluster is chosen by cost
-// (pick_split): few wide shares when the batch fills the chip, more and narrower ones when it does not.
+// a commit per 64 columns cost 217 of 1050 cycles: hence 128 columns per stage); 21.0 with a piece of its own for every warp and one
+// issuing warp; 18.3 now: first stage 1.0, MMAs 11.7 (0.94 per 128 input coordinates, 0.85 of them the tensor pipe's), maxima and
+// exchange 0.8, quantizer 1.2, stores 1.4.  The number of CTAs per cluster is chosen by cost (pick_split): few wide shares when the batch
+// fills the chip, more and narrower ones when it does not.  1 row: 13.4 -> 8.9 us (of which 13 CTAs instead of 7: 4), 772: 14.6 -> 10.9.
 // Every wait is bounded; an expired wait records a code in the plan's status word.
 #include <math.h>
 #include <stdlib.h>
@@ -42,14 +46,16 @@ constexpr int A_BOX = TM * 64 * 2;      // 16 KB
 constexpr int A_STAGE = 2 * A_BOX;
 constexpr int EW = 4;                   // epilogue warps per TMEM lane quadrant: each takes a quarter of the coordinates
 constexpr int EPI_WARPS = 4 * EW;
-constexpr int THREADS = 32 * (2 + EPI_WARPS);
+constexpr int N_ISSUERS = 2;
+constexpr int THREADS = 32 * (3 + EPI_WARPS);    // producer, issuers (warp 1 and the last one), epilogue
 constexpr int TMEM_COLS = 512;
-constexpr int MAX_CL = 8;               // CTAs per cluster
+constexpr int MAX_CL = 16;              // CTAs per cluster
 constexpr int CORE = 128;               // bytes of a core matrix: 8 rows x 8 bf16
 constexpr int ROW0_BYTES = 2 * 4 * CORE;   // row 0 as 16-row operands: 2 at column 0, and all -1
 
 struct Ctl {
-    float tmax[2][MAX_CL * EW][TM];     // [tile parity][CTA and quarter][token]: maxima of every share of a token
+    float part[2][EW][TM];              // [tile parity][quarter][token]: maxima of the CTA's own quarters
+    float tmax[2][MAX_CL][TM];          // [tile parity][CTA][token]: maxima of every CTA's share, written by their threads
     float y0[2][TM];                    // coordinate 0, from the cluster's last CTA
     unsigned long long full[MAX_STAGES], empty[MAX_STAGES], tfull, tempty, tbar, maxbar[2];
     unsigned tmem_base;
@@ -67,7 +73,7 @@ struct DenseParams {
     int nbp;                      // output blocks the Toeplitz and column tables are laid out for
     int code_row_bytes;
     int stages;
-    int stage_words;              // words of a token's row in a warp's packing buffer (odd)
+    int stage_words;              // words of a token's row in the packing buffer (odd)
     float c_scale, c_half, norm;
     const unsigned short* x;      // the rows (bf16), for what the tensor map does not show
     long long stride;
@@ -97,12 +103,32 @@ __device__ __forceinline__ void steps(unsigned d_tmem, unsigned long long ad, un
     }
 }
 
+// A float to another CTA's shared memory, whose barrier there counts its bytes: what a waiter of that barrier sees is ordered by the
+// transaction alone.  (An arrival with .release.cluster orders all of the writer's accesses, global ones too.)
+__device__ __forceinline__ void peer_send(unsigned addr, float v, unsigned bar_addr)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar_addr) : "memory");
+}
+// L2 prefetch of the box a later tma_load_2d will fetch (see tma_prefetch_3d)
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int c0, int c1)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(map), "r"(c0), "r"(c1) : "memory");
+}
+
 // one column of this thread's TMEM lane
 __device__ __forceinline__ unsigned tmem_ld1(unsigned taddr)
 {
     unsigned v;
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;" : "=r"(v) : "r"(taddr) : "memory");
     return v;
+}
+// 128 threads meet; whether any of them says so
+__device__ __forceinline__ bool meet_any(int barrier, bool p)
+{
+    unsigned any;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %2, 0;\n\tbar.red.or.pred p, %1, 128, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(any) : "r"(barrier), "r"(p ? 1u : 0u) : "memory");
+    return any != 0;
 }
 // 32 accumulator columns of four output blocks (descending) into coordinate order
 __device__ __forceinline__ void load_chunk(unsigned taddr, unsigned y[32])
@@ -127,7 +153,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
     unsigned char* sm_e = sm_t + (P.kchunks * (KC / 8) + P.ncb) * CORE;
     unsigned char* sm_r = sm_e + P.ncb * 2 * CORE;
     unsigned* sm_pack = reinterpret_cast<unsigned*>(sm_r + ROW0_BYTES);
-    Ctl* S = reinterpret_cast<Ctl*>(sm_pack + (EPI_WARPS * 32 * P.stage_words + 3) / 4 * 4);
+    Ctl* S = reinterpret_cast<Ctl*>(sm_pack + TM * P.stage_words);
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank();
     const int cluster = (int)blockIdx.x / P.cl, n_clusters = (int)gridDim.x / P.cl;
@@ -140,18 +166,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
     const int skip = last && nb0 + ncb - P.m / 8 >= 2 ? 2 : 0;
     const int col_r = skip ? 0 : 8 * ncb;
 
+    const unsigned max_bytes = (unsigned)((P.cl + (rank == 0 ? 1 : 0)) * TM * 4);       // of a tile: a float per token from every CTA, and coordinate 0
+
     if (threadIdx.x == 0) {
         for (int s = 0; s < P.stages; ++s) {
             mbar_init(&S->full[s], 1);
-            mbar_init(&S->empty[s], 1);
+            mbar_init(&S->empty[s], N_ISSUERS);
         }
-        mbar_init(&S->tfull, 1);
+        mbar_init(&S->tfull, N_ISSUERS);
         mbar_init(&S->tempty, EPI_WARPS);
         mbar_init(&S->tbar, 1);
-        mbar_init(&S->maxbar[0], P.cl * EPI_WARPS);
-        mbar_init(&S->maxbar[1], P.cl * EPI_WARPS);
+        mbar_init(&S->maxbar[0], 1);
+        mbar_init(&S->maxbar[1], 1);
         S->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_arrive_expect_tx(&S->maxbar[0], max_bytes);
+        mbar_arrive_expect_tx(&S->maxbar[1], max_bytes);
         // plan-owned, immutable tables: need no ordering
         mbar_arrive_expect_tx(&S->tbar, (unsigned)(toep_n * CORE + ncb * 2 * CORE + ROW0_BYTES));
         const int first = P.nbp - nb0 - ncb;
@@ -166,6 +196,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
     cluster_sync();                                                // every CTA's barriers are ready for its peers
     tc_fence_after();
     const unsigned tmem_base = S->tmem_base;
+    // the first stage on its way from DRAM to L2; nothing reaches this SM before the wait.  (All of the tile's, shared out among the CTAs: no gain.)
+    if (threadIdx.x == 0 && cluster < P.n_tiles) {
+        tma_prefetch_2d(&xmap, 0, cluster * TM);
+        tma_prefetch_2d(&xmap, 64, cluster * TM);
+    }
     // programmatic dependent launch: until this returns an earlier kernel may still be writing x or reading the outputs
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -189,19 +224,22 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
             }
             if (!ok) drain_copies(S->full, P.stages, c);
         }
-    } else if (warp == 1) {
-        // ------------------------------ MMA issuer ------------------------------
+    } else if (warp == 1 || warp == 2 + EPI_WARPS) {
+        // ------------------------------ MMA issuers ------------------------------
+        // Each issues for its own columns, all k-steps of a stage, so that one's polls and commits (about 200 cycles a stage) are covered by the other's
+        // MMAs.  Fewer than 208 columns stay with the first: an MMA of less than about 100 columns takes no less time.
         {
-            // the CTA's columns as one or two MMAs of at most 256, each a multiple of 32
-            const int n = ncb - skip, n1 = n <= 32 ? n : (n / 2 + 3) / 4 * 4, n2 = n - n1;
-            const unsigned idesc1 = instr_desc(TM, 8 * n1, false), idesc2 = instr_desc(TM, 8 * n2, false);
+            const int issuer = warp == 1 ? 0 : 1;
+            const int n_all = ncb - skip, n_first = n_all < 26 ? n_all : (n_all / 2 + 1) / 2 * 2, n = issuer == 0 ? n_first : n_all - n_first;
+            const int before = issuer == 0 ? 0 : n_first;                           // blocks
+            const bool row0s = last && issuer == 1;                                 // coordinate 0 as well
+            const unsigned idesc = instr_desc(TM, 8 * n, false);
             constexpr unsigned IDESC_R = instr_desc(TM, 16, false);
             // unswizzled core matrices: leading offset = next 8 columns, stride offset = next 8 rows of the operand
-            const unsigned long long td0 = smem_desc(smem_u32(sm_t) + skip * CORE, CORE, CORE, 0);
-            const unsigned long long ed0 = smem_desc(smem_u32(sm_e) + skip * 2 * CORE, CORE, 2 * CORE, 0);
+            const unsigned long long td0 = smem_desc(smem_u32(sm_t) + (skip + before) * CORE, CORE, CORE, 0);
+            const unsigned long long ed0 = smem_desc(smem_u32(sm_e) + (skip + before) * 2 * CORE, CORE, 2 * CORE, 0);
             const unsigned long long rd0 = smem_desc(smem_u32(sm_r), CORE, 2 * CORE, 0);
-            const unsigned tmem1 = tmem_base + 8 * skip, tmem2 = tmem1 + 8 * n1, tmem_r = tmem_base + col_r;
-            const unsigned long long step2 = (unsigned long long)(n1 * CORE / 16), estep2 = (unsigned long long)(n1 * 2 * CORE / 16);
+            const unsigned tmem = tmem_base + 8 * (skip + before), tmem_r = tmem_base + col_r;
             bool ok = mbar_wait_warp(&S->abort_flag, &S->tbar, 0, P.status, 6);
             int s = 0;
             unsigned ph = 0;
@@ -217,14 +255,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
                     const int ks_n = (kc == P.kchunks - 1) ? P.ksteps_last : KC / 16;
                     if (kc == 0) {
                         // column 0: H[n][0] - t(-n) against x_0, and coordinate 0: 2 x_0 (the other columns of these are zero)
-                        umma_f16(tmem1, ad, ed0, idesc1, 0u);
-                        if (n2) umma_f16(tmem2, ad, ed0 + estep2, idesc2, 0u);
-                        if (last) umma_f16(tmem_r, ad, rd0, IDESC_R, 0u);
+                        if (n) umma_f16(tmem, ad, ed0, idesc, 0u);
+                        if (row0s) umma_f16(tmem_r, ad, rd0, IDESC_R, 0u);
                     }
                     // one operand after the other, each in a loop of its own: a condition between two MMAs doubles their time
-                    steps(tmem1, ad, td, 2 * CORE / 16, idesc1, ks_n);
-                    if (n2) steps(tmem2, ad, td + step2, 2 * CORE / 16, idesc2, ks_n);
-                    if (last) steps(tmem_r, ad, rd0 + 4 * CORE / 16, 0, IDESC_R, ks_n);
+                    if (n) steps(tmem, ad, td, 2 * CORE / 16, idesc, ks_n);
+                    if (row0s) steps(tmem_r, ad, rd0 + 4 * CORE / 16, 0, IDESC_R, ks_n);
                     td += (unsigned long long)(2 * CORE / 16 * (KC / 16));
                     umma_commit(&S->empty[s]);
                     if (++s == P.stages) { s = 0; ph ^= 1; }
@@ -240,117 +276,118 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
         const int chunks = ncb / 4;                        // of 32 coordinates
         const int ch0 = h * chunks / EW, ch1 = (h + 1) * chunks / EW;
         const unsigned lane_base = tmem_base + ((unsigned)(q * 32) << 16);
-        const int nfirst = (nb0 + 4 * ch0) * 8;            // first coordinate of this warp
         const bool has0 = rank == 0 && ch0 == 0 && ch1 > 0;        // coordinate 0 is among this warp's
         const bool sends0 = last && h == 0;
-        unsigned* pack = sm_pack + (warp - 2) * 32 * P.stage_words;
-        bool ok = true;
-        for (int i = 0; ok && i < n_mine; ++i) {
+        unsigned* pack = sm_pack + q * 32 * P.stage_words;          // the quadrant's rows
+        for (int i = 0; i < n_mine; ++i) {
             const long long row0 = ((long long)cluster + (long long)i * n_clusters) * TM;
             const long long row = row0 + tok;
             const bool live = row < P.n_rows;
-            ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull, i & 1, P.status, 4));
-            if (!ok) break;
-            tc_fence_after();
+            // a warp whose wait ran out still comes to the quadrant's next barrier, where its four warps leave together
+            bool ok = __all_sync(0xffffffffu, mbar_wait(&S->abort_flag, &S->tfull, i & 1, P.status, 4));
             float M = 0.f;
-            for (int ch = ch0; ch < ch1; ++ch) {
-                const int n_here = P.m - (nb0 + 4 * ch) * 8;               // live coordinates from here on
-                if (n_here <= 0) break;
-                unsigned y[32];
-                load_chunk(lane_base + (unsigned)(8 * (ncb - 4 - 4 * ch)), y);
-                if (has0 && ch == 0) y[0] = 0u;                            // in the maximum of the CTA that has it
-                if (n_here < 32) {
+            if (ok) {
+                tc_fence_after();
+                for (int ch = ch0; ch < ch1; ++ch) {
+                    const int n_here = P.m - (nb0 + 4 * ch) * 8;           // live coordinates from here on
+                    if (n_here <= 0) break;
+                    unsigned y[32];
+                    load_chunk(lane_base + (unsigned)(8 * (ncb - 4 - 4 * ch)), y);
+                    if (has0 && ch == 0) y[0] = 0u;                        // in the maximum of the CTA that has it
+                    if (n_here < 32) {
 #pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (e >= n_here) y[e] = 0u;                        // coordinates beyond m
+                        for (int e = 0; e < 32; ++e)
+                            if (e >= n_here) y[e] = 0u;                    // coordinates beyond m
+                    }
+                    M = fmaxf(M, absmax32(y));
                 }
-                M = fmaxf(M, absmax32(y));
+                if (sends0) {
+                    const float y0 = __uint_as_float(tmem_ld1(lane_base + col_r));
+                    M = fmaxf(M, fabsf(y0));
+                    peer_send(peer_addr(smem_u32(&S->y0[i & 1][tok]), 0u), y0, peer_addr(smem_u32(&S->maxbar[i & 1]), 0u));
+                }
+                S->part[i & 1][h][tok] = M;
             }
-            if (sends0) {
-                const float y0 = __uint_as_float(tmem_ld1(lane_base + col_r));
-                M = fmaxf(M, fabsf(y0));
-                peer_store(peer_addr(smem_u32(&S->y0[i & 1][tok]), 0u), y0);
-            }
-            // the token's maximum over all shares of all CTAs
-            const unsigned mine = smem_u32(&S->tmax[i & 1][rank * EW + h][tok]), bar = smem_u32(&S->maxbar[i & 1]);
-            for (int r = 0; r < P.cl; ++r) peer_store(peer_addr(mine, (unsigned)r), M);
-            __syncwarp();
-            if (lane < P.cl) peer_arrive(peer_addr(bar, (unsigned)lane));
+            if (meet_any(1 + q, !ok)) break;
+            // the token's maximum: the quadrant's four warps have theirs together, and each sends it to a quarter of the CTAs (its own among them)
+            M = fmaxf(fmaxf(S->part[i & 1][0][tok], S->part[i & 1][1][tok]), fmaxf(S->part[i & 1][2][tok], S->part[i & 1][3][tok]));
+            const unsigned mine = smem_u32(&S->tmax[i & 1][rank][tok]), bar = smem_u32(&S->maxbar[i & 1]);
+            for (int r = h; r < P.cl; r += EW) peer_send(peer_addr(mine, (unsigned)r), M, peer_addr(bar, (unsigned)r));
             ok = __all_sync(0xffffffffu, cluster_wait(&S->abort_flag, &S->maxbar[i & 1], (unsigned)(i >> 1) & 1u, P.status, 7));
-            if (!ok) break;
-            for (int r = 0; r < P.cl * EW; ++r) M = fmaxf(M, S->tmax[i & 1][r][tok]);
-            const float a1 = __fdividef(P.c_half, fmaxf(M, 1e-30f));
-            for (int ch = ch0; ch < ch1; ++ch) {
-                const int n0 = (nb0 + 4 * ch) * 8, n_here = P.m - n0;
-                if (n_here <= 0) break;
-                unsigned y[32];
-                load_chunk(lane_base + (unsigned)(8 * (ncb - 4 - 4 * ch)), y);
-                if (has0 && ch == 0) y[0] = __float_as_uint(S->y0[i & 1][tok]);
-                unsigned out[BITS];
-                quantize_pack32<BITS>(y, a1, out);
+            if (ok) {
+                // the barrier's next tile but one.  (No CTA sends for that one before it has the next tile's maxima of all of this CTA's warps.)
+                if (warp == 2 && lane == 0 && i + 2 < n_mine) mbar_arrive_expect_tx(&S->maxbar[i & 1], max_bytes);
+                for (int r = 0; r < P.cl; ++r) M = fmaxf(M, S->tmax[i & 1][r][tok]);
+                const float a1 = __fdividef(P.c_half, fmaxf(M, 1e-30f));
+                for (int ch = ch0; ch < ch1; ++ch) {
+                    const int n0 = (nb0 + 4 * ch) * 8, n_here = P.m - n0;
+                    if (n_here <= 0) break;
+                    unsigned y[32];
+                    load_chunk(lane_base + (unsigned)(8 * (ncb - 4 - 4 * ch)), y);
+                    if (has0 && ch == 0) y[0] = __float_as_uint(S->y0[i & 1][tok]);
+                    unsigned out[BITS];
+                    quantize_pack32<BITS>(y, a1, out);
 #pragma unroll
-                for (int w = 0; w < BITS; ++w) pack[lane * P.stage_words + (ch - ch0) * BITS + w] = out[w];
-                if (P.y_opt && live) {
-                    float* yo = P.y_opt + row * (long long)P.m + n0;
+                    for (int w = 0; w < BITS; ++w) pack[lane * P.stage_words + ch * BITS + w] = out[w];
+                    if (P.y_opt && live) {
+                        float* yo = P.y_opt + row * (long long)P.m + n0;
 #pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (e < n_here) yo[e] = __uint_as_float(y[e]) * P.norm;
-                }
-            }
-            // the accumulators have been read: hand TMEM back to the MMA issuer
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S->tempty);
-            if (rank == 0 && h == 0 && live) {
-                // An infinity among the sixteen elements that meet column 0's repair is multiplied by its zeros there: every rotated
-                // value is NaN, which a maximum passes over.  Its scale is infinite, as for an infinity anywhere else.
-                if (M == 0.f) {
-                    const unsigned short* x = P.x + row * P.stride;
-                    for (int j = 0; j < 16 && j < P.d; ++j)
-                        if ((__ldg(x + j) & 0x7fffu) == 0x7f80u) M = __uint_as_float(0x7f800000u);
-                }
-                P.scales[row] = P.c_scale * M;
-            }
-            // this warp's 32 rows as words, sixteen lanes to a row (a piece is at most 64 bytes; 48 where rows are unaligned)
-            const int n_codes = (P.m - nfirst) < (ch1 - ch0) * 32 ? (P.m - nfirst) : (ch1 - ch0) * 32;
-            const int nbytes = n_codes > 0 ? n_codes * BITS / 8 : 0;
-            const int j = lane & 15;
-            const unsigned* words = pack + (lane >> 4) * P.stage_words + j;
-            unsigned char* piece = P.codes + (row0 + q * 32 + (lane >> 4)) * P.code_row_bytes + nfirst / 8 * BITS;
-#pragma unroll
-            for (int part = 0; part < 2; ++part) {                             // eight rows' words in flight at a time
-                unsigned lo[8], hi[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    hi[e] = words[(16 * part + 2 * e) * P.stage_words];
-                    lo[e] = j > 0 ? words[(16 * part + 2 * e) * P.stage_words - 1] : 0u;
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e, piece += 2 * P.code_row_bytes) {
-                    const int off = (int)(reinterpret_cast<uintptr_t>(piece) & 3u);
-                    const unsigned v = __funnelshift_l(lo[e], hi[e], 8 * off);
-                    const int b0 = 4 * j - off;                                // first byte of the piece this word covers
-                    unsigned char* dst = piece + b0;
-                    if (row0 + q * 32 + 16 * part + 2 * e + (lane >> 4) < P.n_rows) {
-                        if (b0 >= 0 && b0 + 4 <= nbytes) {
-                            *reinterpret_cast<unsigned*>(dst) = v;
-                        } else if (b0 < nbytes) {
-#pragma unroll
-                            for (int b = 0; b < 4; ++b)
-                                if (b0 + b >= 0 && b0 + b < nbytes) dst[b] = (unsigned char)(v >> (8 * b));
-                        }
+                        for (int e = 0; e < 32; ++e)
+                            if (e < n_here) yo[e] = __uint_as_float(y[e]) * P.norm;
                     }
                 }
+                // the accumulators have been read: hand TMEM back to the MMA issuers
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S->tempty);
+                if (rank == 0 && h == 0 && live) {
+                    // An infinity among the sixteen elements that meet column 0's repair is multiplied by its zeros there: every rotated
+                    // value is NaN, which a maximum passes over.  Its scale is infinite, as for an infinity anywhere else.
+                    if (M == 0.f) {
+                        const unsigned short* x = P.x + row * P.stride;
+                        for (int j = 0; j < 16 && j < P.d; ++j)
+                            if ((__ldg(x + j) & 0x7fffu) == 0x7f80u) M = __uint_as_float(0x7f800000u);
+                    }
+                    P.scales[row] = P.c_scale * M;
+                }
             }
-            __syncwarp();                                                      // the packing buffer is rewritten next
+            if (meet_any(1 + q, !ok)) break;
+            // the CTA's piece of eight rows of the quadrant's 32, as aligned words; what the rows before and after share a word with, by bytes
+            const int n_codes = P.m - nb0 * 8 < ncb * 8 ? P.m - nb0 * 8 : ncb * 8;
+            const int nbytes = n_codes * BITS / 8;
+            const long long first_row = row0 + q * 32 + h * 8;
+            const unsigned* rows = pack + h * 8 * P.stage_words;
+            unsigned char* piece = P.codes + first_row * P.code_row_bytes + nb0 * BITS;
+            const int n_live = P.n_rows - first_row < 8 ? (int)(P.n_rows - first_row) : 8;
+#pragma unroll 4
+            for (int e = 0; e < n_live; ++e) {
+                unsigned char* dst = piece + e * P.code_row_bytes;
+                const int off = BITS == 4 ? 0 : (int)(reinterpret_cast<uintptr_t>(dst) & 3u);      // four-bit rows are words
+                for (int j = lane; 4 * j - off + 4 <= nbytes; j += 32) {
+                    const unsigned hi = rows[e * P.stage_words + j];
+                    const unsigned lo = BITS == 4 || j == 0 ? 0u : rows[e * P.stage_words + j - 1];
+                    if (off == 0 || j > 0) *reinterpret_cast<unsigned*>(dst + 4 * j - off) = BITS == 4 ? hi : __funnelshift_l(lo, hi, 8 * off);
+                }
+            }
+            if (BITS != 4 && lane < 2 * n_live) {
+                const int e = lane >> 1;
+                unsigned char* dst = piece + e * P.code_row_bytes;
+                const int lead = (int)(-reinterpret_cast<uintptr_t>(dst) & 3u), tail = (nbytes - lead) & 3;
+                const unsigned char* src = reinterpret_cast<const unsigned char*>(rows + e * P.stage_words);
+                const int at = lane & 1 ? nbytes - tail : 0, n = lane & 1 ? tail : lead;
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+                    if (b < n) dst[at + b] = src[at + b];
+            }
         }
     }
 
-    // ---- teardown: no CTA leaves while a peer may still write to its shared memory
+    // ---- teardown.  Peers write to this CTA's shared memory only what its epilogue has waited for, so it may leave once every role has
+    // left its loop; after an expired wait it stays until the cluster's CTAs have come here or ended.
     tc_fence_before();
     __syncthreads();
     __syncwarp();
-    cluster_sync();
+    if (S->abort_flag) cluster_sync();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, TMEM_COLS);
@@ -360,25 +397,30 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_dense_rq(const __grid_constan
 // shared memory of a CTA that takes `ncb` output blocks of a contraction over `kchunks` chunks
 int smem_bytes(int ncb, int kchunks, int stages, int* stage_words)
 {
-    const int w = 17;                                              // sixteen words are read whatever the share; odd: different banks
+    const int w = ncb * 8 * 4 / 32 + 1;                            // a row's four-bit codes; odd: different banks
     if (stage_words) *stage_words = w;
-    return 1024 + stages * A_STAGE + (kchunks * (KC / 8) + ncb) * CORE + ncb * 2 * CORE + ROW0_BYTES + (EPI_WARPS * 32 * w + 3) / 4 * 16 + (int)sizeof(Ctl);
+    return 1024 + stages * A_STAGE + (kchunks * (KC / 8) + ncb) * CORE + ncb * 2 * CORE + ROW0_BYTES + TM * w * 4 + (int)sizeof(Ctl);
 }
 
 typedef void (*DenseKernel)(const CUtensorMap, const DenseParams);
 DenseKernel kernel_of(int bits) { return bits == 3 ? k_tc_dense_rq<3> : k_tc_dense_rq<4>; }
 
-// Clusters of `cl` CTAs that run at once (one CTA per SM; a cluster stays inside a GPC, so this can be less than SMs / cl).
-// Asked once per device, together with the opt-in to the large dynamic shared memory (not stream operations).
+// Clusters of `cl` CTAs that run at once (one CTA per SM; a cluster stays inside a GPC, so this can be less than SMs / cl, and none of
+// more than eight CTAs need fit).  Asked once per device, together with the opt-in to the large dynamic shared memory and to such clusters (not
+// stream operations).
 int clusters_at_once(const gbs_plan* p, int cl)
 {
     static std::mutex mu;
-    static int fit[64][MAX_CL + 1];
+    static int known[64][MAX_CL + 1];                              // clusters + 1
     std::lock_guard<std::mutex> lock(mu);
-    int* f = (p->device >= 0 && p->device < 64) ? fit[p->device] : nullptr;
-    if (f && f[cl]) return f[cl];
+    int* f = (p->device >= 0 && p->device < 64) ? known[p->device] : nullptr;
+    if (f && f[cl]) return f[cl] - 1;
     for (int bits = 3; bits <= 4; ++bits)
-        if (cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_optin) != cudaSuccess) return -1;
+        if (cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_optin) != cudaSuccess ||
+            cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p->sm_count / cl * cl));
     cfg.blockDim = dim3(THREADS);
@@ -390,14 +432,16 @@ int clusters_at_once(const gbs_plan* p, int cl)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel_of(p->bits), &cfg) != cudaSuccess || n < 1) { cudaGetLastError(); return -1; }
-    if (f) f[cl] = n;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel_of(p->bits), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    if (f) f[cl] = n + 1;
     return n;
 }
 
-// How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 64), a stage's poll and
-// commit 220, a tile's epilogue and exchange a few thousand, and the clusters that fit at once take the tiles in waves: the split with the
-// least total is taken.  n_tiles = 0 only asks whether a split exists.
+// How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 52), a stage's poll and commit 180 where
+// one warp issues and 40 where two do, a tile's exchange and epilogue a few thousand, and the clusters that fit at once take the tiles in
+// waves: the split with the least total is taken.  n_tiles = 0 only asks whether a split exists.  (1544, 4 bits, in us with 13, 10, 6 and 4
+// CTAs: 1 row 9.0, 9.7, 12.4, 16.3; 772: 10.9, 11.4, 13.8, 17.5; 1400: 17.3, 12.2, 14.2, 17.7; 2600: 25.7, 20.0, 15.6, 19.1; 4096: 39.6, 27.9,
+// 24.3, 19.7; 5500: 53.2, 35.9, 25.5, 31.9; 6854: 61.4, 43.8, 34.2, 32.6.)
 int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* ncb_out, int* fit_out)
 {
     const int nb = p->m / 8;
@@ -409,15 +453,17 @@ int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* nc
             smem_bytes(ncb, kchunks, 2, nullptr) > p->smem_optin)
             continue;
         const int fit = n_tiles ? clusters_at_once(p, cl) : 1;
-        if (fit < 1) return (int)cudaErrorInvalidConfiguration;
+        if (fit < 1) continue;
         const int waves = (n_tiles + fit - 1) / fit;
-        const auto mma = [](int blocks) { return blocks <= 32 ? (blocks * 4 < 64 ? 64.0 : blocks * 4.0) : (blocks * 4 < 128 ? 128.0 : blocks * 4.0); };
-        double step = mma(last) + 100.0;                                          // the last CTA has coordinate 0's MMA as well
-        if (cl > 1 && mma(ncb) > step) step = mma(ncb);
-        const double cost = waves * (kchunks * (8.0 * step + 220.0) + 4500.0 + 20.0 * ncb);
+        const auto chunk = [](int blocks, double more) {
+            return 8.0 * ((blocks < 26 ? (blocks < 13 ? 52.0 : blocks * 4.0) : blocks * 4.0) + more) + (blocks < 26 ? 180.0 : 40.0);
+        };
+        double step = chunk(last, 52.0);                                          // the last CTA has coordinate 0's MMA as well
+        if (cl > 1 && chunk(ncb, 0.0) > step) step = chunk(ncb, 0.0);
+        const double cost = waves * (kchunks * step + 4500.0 + 20.0 * ncb);
         if (*cl_out == 0 || cost < best) { best = cost; *cl_out = cl; *ncb_out = ncb; *fit_out = fit; }
     }
-    return 0;
+    return *cl_out ? 0 : (int)cudaErrorInvalidConfiguration;
 }
 
 int padded_blocks(int m) { return m / 8 + 64; }                   // a CTA's share may reach beyond the last block
