@@ -143,6 +143,11 @@ void gbs_tc_dense_tables(const int8_t* hm, int m, unsigned short* toep, unsigned
 int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, void* codes,
                                  float* scales, float* y_opt, cudaStream_t stream);
 
+// Its choice of a split, on host arithmetic: CTAs that share a token's coordinates (0: none) and the output blocks of each.  `query` says how many
+// clusters of `ctas` CTAs of the kernel for `bits` run at once, -1 where that cannot be said; `known` holds 2 x 17 of its answers, zero at first.
+typedef int (*gbs_cluster_query)(void* ctx, int bits, int ctas);
+extern "C" int gbs_dense_rule(int m, int d, int64_t n_rows, int bits, int smem_optin, int* known, gbs_cluster_query query, void* ctx, int* blocks);
+
 // gbs_tc_denseinv.cu : gbs_dequantize with inverse rotation for the full order
 bool gbs_tc_denseinv_supported(const gbs_plan* p);
 int gbs_tc_denseinv_dequantize(const gbs_plan* p, const void* codes, const float* scales, int64_t n_rows, void* out,

@@ -406,21 +406,11 @@ typedef void (*DenseKernel)(const CUtensorMap, const DenseParams);
 DenseKernel kernel_of(int bits) { return bits == 3 ? k_tc_dense_rq<3> : k_tc_dense_rq<4>; }
 
 // Clusters of `cl` CTAs that run at once (one CTA per SM; a cluster stays inside a GPC, so this can be less than SMs / cl, and none of
-// more than eight CTAs need fit).  Asked once per device, together with the opt-in to the large dynamic shared memory and to such clusters (not
-// stream operations).
-int clusters_at_once(const gbs_plan* p, int cl)
+// more than eight CTAs need fit), asked of the device together with the opt-in to the large dynamic shared memory and, beyond eight CTAs, to such
+// clusters (not stream operations).  -1: the question failed.
+int ask_clusters(void* plan, int bits, int cl)
 {
-    static std::mutex mu;
-    static int known[64][MAX_CL + 1];                              // clusters + 1
-    std::lock_guard<std::mutex> lock(mu);
-    int* f = (p->device >= 0 && p->device < 64) ? known[p->device] : nullptr;
-    if (f && f[cl]) return f[cl] - 1;
-    for (int bits = 3; bits <= 4; ++bits)
-        if (cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_optin) != cudaSuccess ||
-            cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
+    const gbs_plan* p = static_cast<const gbs_plan*>(plan);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p->sm_count / cl * cl));
     cfg.blockDim = dim3(THREADS);
@@ -432,38 +422,59 @@ int clusters_at_once(const gbs_plan* p, int cl)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel_of(p->bits), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-    if (f) f[cl] = n + 1;
+    if (cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_optin) != cudaSuccess ||
+        (cl > 8 && cudaFuncSetAttribute(kernel_of(bits), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+        cudaOccupancyMaxActiveClusters(&n, kernel_of(bits), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
+    }
     return n;
 }
 
+// The answer for one kernel and cluster size, or -1.  Only answers are kept: a question that failed is asked again by the next call.
+int clusters_at_once(int* known, int bits, int cl, gbs_cluster_query query, void* ctx)
+{
+    int* k = known ? known + (bits - 3) * (MAX_CL + 1) + cl : nullptr;               // clusters + 1
+    if (k && *k) return *k - 1;
+    const int n = query(ctx, bits, cl);
+    if (k && n >= 0) *k = n + 1;
+    return n;
+}
+
+struct Split {
+    int ctas, blocks, at_once;    // CTAs that share a token's coordinates, output blocks of each but the last, clusters at once
+};
+
 // How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 52), a stage's poll and commit 180 where
 // one warp issues and 40 where two do, a tile's exchange and epilogue a few thousand, and the clusters that fit at once take the tiles in
-// waves: the split with the least total is taken.  n_tiles = 0 only asks whether a split exists.  (1544, 4 bits, in us with 13, 10, 6 and 4
-// CTAs: 1 row 9.0, 9.7, 12.4, 16.3; 772: 10.9, 11.4, 13.8, 17.5; 1400: 17.3, 12.2, 14.2, 17.7; 2600: 25.7, 20.0, 15.6, 19.1; 4096: 39.6, 27.9,
-// 24.3, 19.7; 5500: 53.2, 35.9, 25.5, 31.9; 6854: 61.4, 43.8, 34.2, 32.6.)
-int pick_split(const gbs_plan* p, int n_tiles, int kchunks, int* cl_out, int* ncb_out, int* fit_out)
+// waves: the split with the least total is taken.  n_rows = 0 only asks whether a split exists.  1544, in us per launch of a graph of ten, with
+// 13, 10, 6 and 4 CTAs, 4 bits and, in brackets, 3: 1 row 8.8, 9.4, 12.1, 16.0 (9.0, 9.6, 12.2, 16.3); 772: 10.9, 11.0, 13.5, 17.3 (11.7, 11.9, 14.3,
+// 18.4); 1400: 16.7, 12.0, 13.7, 17.3 (17.7, 12.8, 14.4, 18.4), with the nine taken 11.4 (12.3); 2600: 24.3, 19.2, 15.0, 18.3 (25.5, 20.2, 15.6, 19.4);
+// 4096: 36.4, 26.7, 24.0, 19.4 (37.9, 28.0, 24.5, 20.5); 5500: 48.3, 34.1, 25.2, 31.7 (50.2, 35.6, 25.8, 32.8); 6854: 56.1, 41.3, 34.1, 32.1 (58.1,
+// 43.2, 34.8, 33.2).
+Split pick_split(int m, int d, int64_t n_rows, int bits, int smem_optin, int* known, gbs_cluster_query query, void* ctx)
 {
-    const int nb = p->m / 8;
+    const int nb = m / 8, kchunks = (d + KC - 1) / KC;
+    const int64_t n_tiles = (n_rows + TM - 1) / TM;
     double best = 0.0;
-    *cl_out = 0;
+    Split split = {0, 0, 0};
     for (int ncb = 4; ncb <= 64; ncb += 4) {
         const int cl = (nb + ncb - 1) / ncb, real = nb - (cl - 1) * ncb, last = (real + 3) / 4 * 4;
         if (cl > MAX_CL || (last - real < 2 && 8 * last + 16 > TMEM_COLS) ||      // sixteen columns for coordinate 0 must fit
-            smem_bytes(ncb, kchunks, 2, nullptr) > p->smem_optin)
+            smem_bytes(ncb, kchunks, 2, nullptr) > smem_optin)
             continue;
-        const int fit = n_tiles ? clusters_at_once(p, cl) : 1;
+        const int fit = n_rows ? clusters_at_once(known, bits, cl, query, ctx) : 1;
         if (fit < 1) continue;
-        const int waves = (n_tiles + fit - 1) / fit;
+        const int64_t waves = (n_tiles + fit - 1) / fit;
         const auto chunk = [](int blocks, double more) {
-            return 8.0 * ((blocks < 26 ? (blocks < 13 ? 52.0 : blocks * 4.0) : blocks * 4.0) + more) + (blocks < 26 ? 180.0 : 40.0);
+            return 8.0 * ((blocks < 13 ? 52.0 : blocks * 4.0) + more) + (blocks < 26 ? 180.0 : 40.0);
         };
         double step = chunk(last, 52.0);                                          // the last CTA has coordinate 0's MMA as well
         if (cl > 1 && chunk(ncb, 0.0) > step) step = chunk(ncb, 0.0);
-        const double cost = waves * (kchunks * step + 4500.0 + 20.0 * ncb);
-        if (*cl_out == 0 || cost < best) { best = cost; *cl_out = cl; *ncb_out = ncb; *fit_out = fit; }
+        const double cost = (double)waves * (kchunks * step + 4500.0 + 20.0 * ncb);
+        if (split.ctas == 0 || cost < best) { best = cost; split = {cl, ncb, fit}; }
     }
-    return *cl_out ? 0 : (int)cudaErrorInvalidConfiguration;
+    return split;
 }
 
 int padded_blocks(int m) { return m / 8 + 64; }                   // a CTA's share may reach beyond the last block
@@ -474,9 +485,14 @@ int padded_blocks(int m) { return m / 8 + 64; }                   // a CTA's sha
 bool gbs_tc_dense_supported(const gbs_plan* p)
 {
     if (!(p->k == 0 && p->m >= 128 && p->m % 8 == 0 && p->d % 8 == 0 && p->group == 0 && !p->asym && get_encode() != nullptr)) return false;
-    int cl = 0, ncb = 0, fit = 0;
-    pick_split(p, 0, (p->d + KC - 1) / KC, &cl, &ncb, &fit);
-    return cl != 0;
+    return pick_split(p->m, p->d, 0, p->bits, p->smem_optin, nullptr, nullptr, nullptr).ctas != 0;
+}
+
+extern "C" int gbs_dense_rule(int m, int d, int64_t n_rows, int bits, int smem_optin, int* known, gbs_cluster_query query, void* ctx, int* blocks)
+{
+    const Split s = pick_split(m, d, n_rows, bits, smem_optin, known, query, ctx);
+    *blocks = s.blocks;
+    return s.ctas;
 }
 
 // bf16 image of H_m, row-major (row = output coordinate, column = input coordinate): m * m * 2 bytes (the inverse path's
@@ -540,9 +556,17 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
     P.stride = stride;
     P.kchunks = (p->d + KC - 1) / KC;
     P.ksteps_last = ((p->d - (P.kchunks - 1) * KC) + 15) / 16;
-    int fit = 0;
-    const int rc = pick_split(p, P.n_tiles, P.kchunks, &P.cl, &P.ncb, &fit);
-    if (rc != 0) return rc;
+    Split split;
+    {
+        static std::mutex mu;
+        static int known[64][2 * (MAX_CL + 1)];
+        std::lock_guard<std::mutex> lock(mu);
+        split = pick_split(p->m, p->d, n_rows, p->bits, p->smem_optin, p->device >= 0 && p->device < 64 ? known[p->device] : nullptr, ask_clusters,
+                           const_cast<gbs_plan*>(p));
+    }
+    if (split.ctas == 0) return (int)cudaErrorInvalidConfiguration;
+    P.cl = split.ctas;
+    P.ncb = split.blocks;
     P.ncb_last = ((p->m / 8 - (P.cl - 1) * P.ncb) + 3) / 4 * 4;
     P.nbp = padded_blocks(p->m);
     P.code_row_bytes = p->m * p->bits / 8;
@@ -558,7 +582,7 @@ int gbs_tc_dense_rotate_quantize(const gbs_plan* p, const void* x, int64_t n_row
     P.status = p->d_status;
     P.stages = smem_bytes(P.ncb, P.kchunks, MAX_STAGES, nullptr) <= p->smem_optin ? MAX_STAGES : 2;
     const int smem = smem_bytes(P.ncb, P.kchunks, P.stages, &P.stage_words);
-    const int clusters = P.n_tiles < fit ? P.n_tiles : fit;
+    const int clusters = P.n_tiles < split.at_once ? P.n_tiles : split.at_once;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(clusters * P.cl));
     cfg.blockDim = dim3(THREADS);
