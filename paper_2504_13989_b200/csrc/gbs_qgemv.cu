@@ -81,12 +81,12 @@ __global__ void __launch_bounds__(32 * WARPS) k_qgemv(const __grid_constant__ Qg
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the int8 operands are q * 2^(8 - bits): the token's scale takes the two powers of two out again (exact)
-    const auto dx = [&](int t) { return __ldg(P.sx + t) * (1.f / (float)(1 << (16 - XBITS - WBITS))); };
-    if (SCALES_FIRST)
+    constexpr float OUT = 1.f / (float)(1 << (16 - XBITS - WBITS));
+    if constexpr (SCALES_FIRST)
         for (int i = threadIdx.x; i < 16 * MT + 8 * NT; i += 32 * WARPS) {
             const int t = i - 16 * MT;
             if (t < 0) scale_w[i] = o0 + i < P.n_out ? __ldg(P.sw + o0 + i) : 0.f;
-            else scale_x[t] = t < P.n_tok ? dx(t) : 0.f;
+            else scale_x[t] = t < P.n_tok ? __ldg(P.sx + t) * OUT : 0.f;
         }
 
     // rows beyond the last are read as the last one; their sums are not stored
@@ -160,7 +160,13 @@ __global__ void __launch_bounds__(32 * WARPS) k_qgemv(const __grid_constant__ Qg
         const int oi = i % (16 * MT), t = i / (16 * MT);
         const long long o = o0 + oi;
         if (o >= P.n_out) continue;
-        const float v = (float)sums[oi][t] * (SCALES_FIRST ? scale_x[t] * scale_w[oi] : dx(t) * __ldg(P.sw + o));
+        float v;                                                          // (both forms in one expression: 8 tokens -> 512 2.41 us instead of 2.24)
+        if constexpr (SCALES_FIRST) {
+            v = (float)sums[oi][t] * (scale_x[t] * scale_w[oi]);
+        } else {
+            const float dx = __ldg(P.sx + t) * OUT;
+            v = (float)sums[oi][t] * (dx * __ldg(P.sw + o));
+        }
         OutT* dst = reinterpret_cast<OutT*>(P.out) + (long long)t * P.out_stride + o;
         if (sizeof(OutT) == 4) *reinterpret_cast<float*>(dst) = v;
         else *reinterpret_cast<__nv_bfloat16*>(dst) = __float2bfloat16_rn(v);
