@@ -183,8 +183,14 @@ cudaError_t launch(const QgemvParams& P, bool pdl, cudaStream_t stream)
     if (P.n_tok <= 8) kernel = k_qgemv<XB, WB, OutT, 1, 1, 4>;
     else if (P.n_tok <= 16) kernel = k_qgemv<XB, WB, OutT, 1, 2, 4>;
     else if (P.n_tok <= 32) { kernel = k_qgemv<XB, WB, OutT, 2, 4, 2>; ch = 32; }
-    // (two steps of four-bit rows in flight: 64 tokens -> 4096 10.35 -> 10.05 us with the layer's other launch; of three-bit ones 11.8 -> 12.7)
-    else { kernel = k_qgemv<XB, WB, OutT, 2, 8, (XB == 4 && WB == 4 ? 2 : 1)>; ch = 32; }
+    else {
+        // Two steps of four-bit rows in flight where a warp has more than two (64 tokens -> 4096 channels, 5120 wide: 9.60 us with one and 8.90 with two;
+        // 4096: 8.12, 7.90; 2560: 6.96, 6.59; 2048: 5.31, 5.42; 1024: 3.71, 4.38).  Three bits: one (4096 wide, with the layer's other launch: 11.8, 12.7).
+        kernel = k_qgemv<XB, WB, OutT, 2, 8, 1>;
+        if constexpr (XB == 4 && WB == 4)
+            if (P.kblocks > 2 * WARPS) kernel = k_qgemv<XB, WB, OutT, 2, 8, 2>;
+        ch = 32;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((P.n_out + ch - 1) / ch));
     cfg.blockDim = dim3(32 * WARPS);
