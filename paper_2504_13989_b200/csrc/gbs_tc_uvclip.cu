@@ -67,12 +67,13 @@ struct __align__(1024) Smem {
     unsigned char b[STAGE_BYTES_MAX];
     unsigned hist[HIST_WORDS];
     unsigned lut[1 << TABLE_LOG];
-    unsigned red[TOK_MAX][2][256];                 // maxima, by tile parity: a word per warp, or one per lane (groups)
-    double2 weight[2][TOK_MAX][16];                // groups: M^2 of every copy, by tile parity
+    unsigned red[TOK_MAX][2][4];                   // maxima, by tile parity: a word per warp
     double square[EPI_WARPS];                      // sums of t^2
     unsigned long long full, empty, tfull[STAGES], tempty[STAGES];
     unsigned tmem_base;
     volatile int abort_flag;
+    double2 weight[2][TOK_MAX][16];                // groups: M^2 of every copy, by tile parity
+    unsigned lane_red[TOK_MAX][2][256];            // groups: maxima, a word per lane
 };
 
 struct ClipParams {
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         }
     } else {
         // ------------------------------ histogram ------------------------------
-        const int w = warp - 2, t = w / TOKEN_WARPS, half = (w >> 2) % HALVES, q = warp & 3;
+        const int w = warp - 2, t = GROUPED ? w / TOKEN_WARPS : w >> 2, half = (w >> 2) % HALVES, q = warp & 3;
         const int wt = half * 4 + q;                              // of the token's warps
         const int bin0 = GROUPED ? lane : q * 32 + lane;
         const int chunk0 = GROUPED ? lane + wt * CHUNKS : lane;   // eight lanes side by side: different banks
@@ -242,18 +243,17 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
         for (int i = 0; i < PER; ++i) was0[i] = was[i][0] = was[i][1] = was[i][2] = was[i][3] = 0u;
         constexpr float MAGIC = 8388608.f;
         constexpr unsigned E = 0x4B000000u;                       // its bit pattern
-        double square = 0.0, m2 = 0.0;
+        double square = 0.0;
         float poison = 0.f;                                       // NaN once a value was not finite
-        // what the token of tile `it` left in this thread's bins
-        auto add_up = [&](int it) {
-            double2 weight[GROUPED ? CHUNKS : 1][2];               // groups: every copy is another one's
-            if (GROUPED) {
+        // What the token of tile `it` left in this thread's bins.  Groups: every copy is another one's; weighed one by one, and cleared.  (The two
+        // forms share no code here: written as one they cost tokens 0.8 % and, inlined like the other, groups 1.5 %.)
+        auto add_up_groups = [&](int it) {
+            double2 weight[CHUNKS][2];
 #pragma unroll
-                for (int j = 0; j < CHUNKS; ++j) {
-                    const int jj = (chunk0 + j) % (COPIES / 4);
-                    weight[j][0] = S->weight[it & 1][t][2 * jj];
-                    weight[j][1] = S->weight[it & 1][t][2 * jj + 1];
-                }
+            for (int j = 0; j < CHUNKS; ++j) {
+                const int jj = (chunk0 + j) % (COPIES / 4);
+                weight[j][0] = S->weight[it & 1][t][2 * jj];
+                weight[j][1] = S->weight[it & 1][t][2 * jj + 1];
             }
 #pragma unroll
             for (int i = 0; i < PER; ++i) {
@@ -261,35 +261,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                 if (bin < P.n_thr) {
                     uint4* row = reinterpret_cast<uint4*>(hist + bin * COPIES);
                     uint4* row1 = reinterpret_cast<uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
-                    if (GROUPED) {
-                        // weighed one by one, and cleared
 #pragma unroll
-                        for (int j = 0; j < CHUNKS; ++j) {
-                            const int jj = (chunk0 + j) % (COPIES / 4);
-                            const uint4 x = row[jj], z = row1[jj];
-                            row[jj] = row1[jj] = make_uint4(0u, 0u, 0u, 0u);
-                            w0[i] = fma(weight[j][0].x, exact(x.x), w0[i]); w1[i] = fma(weight[j][0].x, exact(z.x), w1[i]);
-                            w0[i] = fma(weight[j][0].y, exact(x.y), w0[i]); w1[i] = fma(weight[j][0].y, exact(z.y), w1[i]);
-                            w0[i] = fma(weight[j][1].x, exact(x.z), w0[i]); w1[i] = fma(weight[j][1].x, exact(z.z), w1[i]);
-                            w0[i] = fma(weight[j][1].y, exact(x.w), w0[i]); w1[i] = fma(weight[j][1].y, exact(z.w), w1[i]);
-                        }
-                    } else {
-                        unsigned c = 0u;
-                        uint4 m = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                        for (int j = 0; j < CHUNKS; ++j) {
-                            const int jj = (chunk0 + j) % (COPIES / 4);
-                            const uint4 x = row[jj], z = row1[jj];
-                            c += (x.x + x.y) + (x.z + x.w);
-                            m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
-                        }
-                        // a component gains at most 1024 values below 2^22: less than 2^32
-                        const unsigned long long sum = ((unsigned long long)(m.x - was[i][0]) + (m.y - was[i][1])) +
-                                                       ((unsigned long long)(m.z - was[i][2]) + (m.w - was[i][3]));
-                        w0[i] += m2 * (double)(c - was0[i]);
-                        w1[i] += m2 * (double)sum;
-                        was0[i] = c;
-                        was[i][0] = m.x; was[i][1] = m.y; was[i][2] = m.z; was[i][3] = m.w;
+                    for (int j = 0; j < CHUNKS; ++j) {
+                        const int jj = (chunk0 + j) % (COPIES / 4);
+                        const uint4 x = row[jj], z = row1[jj];
+                        row[jj] = row1[jj] = make_uint4(0u, 0u, 0u, 0u);
+                        w0[i] = fma(weight[j][0].x, exact(x.x), w0[i]); w1[i] = fma(weight[j][0].x, exact(z.x), w1[i]);
+                        w0[i] = fma(weight[j][0].y, exact(x.y), w0[i]); w1[i] = fma(weight[j][0].y, exact(z.y), w1[i]);
+                        w0[i] = fma(weight[j][1].x, exact(x.z), w0[i]); w1[i] = fma(weight[j][1].x, exact(z.z), w1[i]);
+                        w0[i] = fma(weight[j][1].y, exact(x.w), w0[i]); w1[i] = fma(weight[j][1].y, exact(z.w), w1[i]);
                     }
                 }
             }
@@ -307,10 +287,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S->tempty[s]);
-                mb = __float_as_uint(HALVES == 1 ? fwht32_absmax(r) : fwht32_half_absmax(r, half ? -1.f : 1.f));
-                if (!GROUPED) mb = __reduce_max_sync(0xffffffffu, mb);
+                if constexpr (GROUPED) mb = __float_as_uint(HALVES == 1 ? fwht32_absmax(r) : fwht32_half_absmax(r, half ? -1.f : 1.f));
+                else mb = __reduce_max_sync(0xffffffffu, __float_as_uint(fwht32_absmax(r)));
             }
-            unsigned* slot = S->red[t][it & 1];
+            unsigned* slot = GROUPED ? S->lane_red[t][it & 1] : S->red[t][it & 1];
             if (GROUPED) slot[wt * 32 + lane] = mb;
             else if (lane == 0) slot[q] = mb;
             // The barrier also keeps this token's atomics behind the adding up of the token before.
@@ -359,9 +339,36 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
                 }
             }
             asm volatile("bar.sync %0, %1;" ::"r"(1 + t), "n"(32 * TOKEN_WARPS) : "memory");
-            m2 = (double)M * (double)M;
+            const double m2 = (double)M * (double)M;
             square += m2 * (double)sq;
-            add_up(it);
+            if constexpr (GROUPED) {
+                add_up_groups(it);
+            } else {
+#pragma unroll
+                for (int i = 0; i < PER; ++i) {
+                    const int bin = bin0 + BIN_LANES * i;
+                    if (bin < P.n_thr) {
+                        const uint4* row = reinterpret_cast<const uint4*>(hist + bin * COPIES);
+                        const uint4* row1 = reinterpret_cast<const uint4*>(hist + SUM_OFF / 4 + bin * COPIES);
+                        unsigned c = 0u;
+                        uint4 m = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                        for (int j = 0; j < CHUNKS; ++j) {
+                            const int jj = (chunk0 + j) % (COPIES / 4);
+                            const uint4 x = row[jj], z = row1[jj];
+                            c += (x.x + x.y) + (x.z + x.w);
+                            m.x += z.x; m.y += z.y; m.z += z.z; m.w += z.w;
+                        }
+                        // a component gains at most 1024 values below 2^22: less than 2^32
+                        const unsigned long long sum = ((unsigned long long)(m.x - was[i][0]) + (m.y - was[i][1])) +
+                                                       ((unsigned long long)(m.z - was[i][2]) + (m.w - was[i][3]));
+                        w0[i] += m2 * (double)(c - was0[i]);
+                        w1[i] += m2 * (double)sum;
+                        was0[i] = c;
+                        was[i][0] = m.x; was[i][1] = m.y; was[i][2] = m.z; was[i][3] = m.w;
+                    }
+                }
+            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) square += __shfl_xor_sync(0xffffffffu, square, o);
@@ -391,9 +398,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_uv_clip(const __grid_constant
     __syncthreads();
     for (int i = threadIdx.x; i < 2 * P.n_thr; i += THREADS) {
         double* d = tot + (i < P.n_thr ? i : BINS + i - P.n_thr);
-        double sum = d[0];
-        for (int part = 1; part < PARTS; ++part) sum += d[part * 2 * BINS];
-        d[0] = sum;
+        if constexpr (GROUPED) {
+            double sum = d[0];
+            for (int part = 1; part < PARTS; ++part) sum += d[part * 2 * BINS];
+            d[0] = sum;
+        } else {
+            d[0] = (d[0] + d[2 * BINS]) + (d[4 * BINS] + d[6 * BINS]);
+        }
     }
     __syncthreads();
     double* suf = tot + PARTS * 2 * BINS;                          // [2][BINS]: sum over bins b, b + 1, ..
