@@ -285,15 +285,7 @@ __device__ __forceinline__ unsigned peer_addr(unsigned smem_addr, unsigned rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
     return a;
 }
-__device__ __forceinline__ void peer_store(unsigned addr, float v)
-{
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void peer_arrive(unsigned bar_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
-}
-// bounded wait on a barrier that other CTAs of the cluster arrive at, behind their stores
+// bounded wait on a barrier of this CTA whose phase other CTAs of the cluster complete with what they store here
 __device__ __forceinline__ bool cluster_wait(volatile int* abort_flag, void* bar, unsigned parity, int* status, int code)
 {
     const unsigned long long t0 = global_ns();
