@@ -247,9 +247,10 @@ int gbs_dequantize(const gbs_plan_t* plan, const void* codes, const float* scale
  *   err_sum       device, K doubles, ACCUMULATED into (the caller zeroes them)
  *   err_rows_opt  NULL, or device n_rows * K floats receiving the per-row sums
  * Which kernel scores a call depends on its shape, its list and whether per-row sums are asked for: one histogram for all
- * candidates (d' <= 4096, group 0 or 128 and more, bf16) or a pass per eight.  Both round each residual to about 2^-23 max|y| (of the
- * token or group), so one alpha's sum from two calls agrees to about 1e-7 of the sum where the rows are ordinary, and to 2^-22 max|y| sqrt(n err) where the
- * candidate fits n values almost exactly; a search that compares sums from different calls decides closer ties by chance.
+ * candidates (d' <= 4096, group 0 or 128 and more, bf16) or a pass per eight.  The histogram rounds each
+ * residual to at most 1.5 x 2^-23 max|y| (of the token or group), the passes round each candidate's Delta to 2^-24 of itself, so one alpha's sum from two
+ * calls agrees to about 2e-7 of the sum where the rows are ordinary, and to 1.5 x 2^-22 max|y| sqrt(n err) where the candidate fits n values almost
+ * exactly (2e-5 of the sum where they are a thousandth off); a search that compares sums from different calls decides closer ties by chance.
  */
 int gbs_clip_error(const gbs_plan_t* plan, const void* x, int x_dtype, int64_t n_rows,
                    int64_t x_row_stride, const float* alphas_host, int K, double* err_sum,

@@ -24,9 +24,9 @@
 // What bounds it: the tensor pipe, 2 d m flops per token, and what stands around it.  4096 x 1536, b = 4: 176 us with two sweeps
 // over streamed chunks of H on 32 SMs; 27.4 us with one sweep over the Toeplitz operand, of which 13.9 were the MMAs (a poll and
 // a commit per 64 columns cost 217 of 1050 cycles: hence 128 columns per stage); 21.0 with a piece of its own for every warp and one
-// issuing warp; 18.3 now: first stage 1.0, MMAs 11.7 (0.94 per 128 input coordinates, 0.85 of them the tensor pipe's), maxima and
+// issuing warp; 18.3 now: first stage 1.0, MMAs 11.7 (0.94 per 128 input coordinates; 9.7 in all, 19 000 cycles, by the tensor pipe's counter), maxima and
 // exchange 0.8, quantizer 1.2, stores 1.4.  The number of CTAs per cluster is chosen by cost (pick_split): few wide shares when the batch
-// fills the chip, more and narrower ones when it does not.  1 row: 13.4 -> 8.9 us (of which 13 CTAs instead of 7: 4), 772: 14.6 -> 10.9.
+// fills the chip, more and narrower ones when it does not.  1 row: 13.4 -> 8.8 us (of which 13 CTAs instead of 7: 4), 772: 14.6 -> 10.9.
 // Every wait is bounded; an expired wait records a code in the plan's status word.
 #include <math.h>
 #include <stdlib.h>
@@ -447,8 +447,8 @@ struct Split {
 
 // How many CTAs share a token's coordinates.  An MMA of N columns takes N / 2 cycles (at least about 52), a stage's poll and commit 180 where
 // one warp issues and 40 where two do, a tile's exchange and epilogue a few thousand, and the clusters that fit at once take the tiles in
-// waves: the split with the least total is taken.  n_rows = 0 only asks whether a split exists.  1544, in us per launch of a graph of ten, with
-// 13, 10, 6 and 4 CTAs, 4 bits and, in brackets, 3: 1 row 8.8, 9.4, 12.1, 16.0 (9.0, 9.6, 12.2, 16.3); 772: 10.9, 11.0, 13.5, 17.3 (11.7, 11.9, 14.3,
+// waves: the split with the least total is taken.  n_rows = 0 only asks whether a split exists.  1544, in us per launch of a graph of ten (calls one by
+// one: 4096 rows 18.3), with 13, 10, 6 and 4 CTAs, 4 bits and, in brackets, 3: 1 row 8.8, 9.4, 12.1, 16.0 (9.0, 9.6, 12.2, 16.3); 772: 10.9, 11.0, 13.5, 17.3 (11.7, 11.9, 14.3,
 // 18.4); 1400: 16.7, 12.0, 13.7, 17.3 (17.7, 12.8, 14.4, 18.4), with the nine taken 11.4 (12.3); 2600: 24.3, 19.2, 15.0, 18.3 (25.5, 20.2, 15.6, 19.4);
 // 4096: 36.4, 26.7, 24.0, 19.4 (37.9, 28.0, 24.5, 20.5); 5500: 48.3, 34.1, 25.2, 31.7 (50.2, 35.6, 25.8, 32.8); 6854: 56.1, 41.3, 34.1, 32.1 (58.1,
 // 43.2, 34.8, 33.2).

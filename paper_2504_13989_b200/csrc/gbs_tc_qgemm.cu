@@ -289,9 +289,10 @@ int pick_tokens(long long n_tok, long long n_out, int kblocks, bool three, int s
 // per SM (4736 on 148): 300 cycles each up to 32 tokens, 600 up to 64.  So 32 tokens go to the tiles beyond two such waves and 64 beyond one.
 // Up to 16 tokens, and up to 32 with three bits on a side, the time was measured to grow with the channels of an SM.  Four bits: up to 8
 // tokens never go to the tiles, up to 16 beyond 18 200 channels until the tiles' second wave begins (18 944), and so on in every wave.
-// Three bits: up to 8 tokens likewise beyond 17 100, 16 beyond 8800, 32 beyond 7800.  4096 wide, few-token kernel and tiles, four bits: 32 tokens ->
-// 8704: 11.3 and 12.0 us, 10 240: 15.0 and 12.4; 64 tokens -> 4096: 8.4 and 11.4, 5760: 15.1 and 11.9; three bits: 32 -> 7168: 12.7 and
-// 11.9, 20 -> 7168: 11.6 and 12.0, 64 -> 4096: 11.0 and 12.0, 5760: 20.0 and 12.7.
+// Three bits: up to 8 tokens likewise beyond 17 100, 16 beyond 8800, 32 beyond 7800.  4096 wide, weights not in L2, few-token kernel and tiles, four
+// bits: 20 tokens -> 9472: 10.6 and 11.7 us, 10 240: 14.1 and 11.8; 32 -> 8704: 10.3 and 11.6, 9472: 10.6 and 11.7, 10 240: 14.0 and 11.8; 64 -> 4736:
+// 8.1 and 11.6, 5760: 14.1 and 11.6; three bits: 20 -> 7168: 11.2 and 12.5, 10 240: 16.0 and 12.7; 32 -> 7168: 12.3 and 12.5, 9472: 12.0 and 12.6,
+// 10 240: 17.3 and 12.7; 64 -> 4736: 10.1 and 12.4, 5760: 18.8 and 12.5.
 bool few_tokens(long long n_tok, long long n_out, bool three, int sm_count)
 {
     if (n_tok > GBS_QGEMV_MAX_TOKENS) return false;

@@ -27,12 +27,14 @@
 //     lane, each taking half of H_32's outputs.
 //   * The t^2 term is the sum of the same integers' squares, in 64 bits, so the three parts of the error belong to one and the same t and
 //     may cancel down to the 16 digits of fp64: a candidate that fits a batch exactly is as accurate as the others, wherever it stands in the list.
-//     t's rounding is the only approximation: at most 2^-23, so that an error E over n values moves by at most
-//     2^-22 M sqrt(n E) + n 2^-46 M^2 -- the size of Delta's rounding in the per-candidate kernel -- and, where the values differ,
-//     by the square root of n less.
+//     t's rounding is the only approximation.  The integer is within half a unit (2^-23) of the product, and the multiplier, one float per token or
+//     group, within 2^-24 of its own size: together at most 1.5 x 2^-23, so that an error E over n values moves by at most 1.5 x 2^-22 M sqrt(n E) +
+//     2.25 n 2^-46 M^2.  The integers' part differs from value to value and grows with the square root of n only; the multiplier's is common to a
+//     token or group.  Against 64 bits the sums are closer than the per-candidate kernel's, whose Delta is rounded once for all: groups of 128,
+//     4096 rows, K = 32, largest relative error 2e-9 - 5e-8 against 6e-8 - 2e-7 on ordinary rows, up to 4e-7 against 2e-5 where a candidate nearly fits.
 //   * A stands in tensor memory, so that an MMA reads one operand from shared memory and the table has the other's room.
-// What bounds it: the chain of a token's four warps, with the shared-memory port 62 - 66 % busy (per token about 130 cycles of lookups, 330 of
-// atomics, 200 of adding up, 450 with groups, 65 of the MMA's operand) and 50 - 66 % of the issue slots taken.  Neither count and sum in one
+// What bounds it: the chain of a token's four warps, with the shared-memory port 56 - 63 % busy (per token about 130 cycles of lookups, 330 of
+// atomics, 200 of adding up, 450 with groups, 65 of the MMA's operand) and 54 - 65 % of the issue slots taken.  Neither count and sum in one
 // atomic (2^24 + t, taken apart again when added up; two histograms in turn and one barrier per token: 148 us where this takes 135)
 // nor barriers that warps arrive at early and wait for late (154) nor fewer instructions per value (no change) make it faster.
 // 32 768 x 4096, K = 32, 3 bits: 829 us with five fp32 operations per value and candidate; 171.4 with one copy of the table, histograms
@@ -447,10 +449,11 @@ typedef void (*ClipKernel)(const CUtensorMap, const ClipParams);
 }  // namespace
 
 // Scores K clip ratios, or returns GBS_UVCLIP_NOT_SERVED where this path does not apply (groups of 32 or 64, per-row sums, thresholds
-// too close to one another): the caller then takes the per-candidate kernel.  So it does where that is the faster one, with candidates for
+// too close to one another, more than 224 of them with groups): the caller then takes the per-candidate kernel.  So it does where that is the faster one, with candidates for
 // one of its passes (eight) and few tiles per block, where building the table is what counts.  One scale per token: up to one (64 x 4096, K = 8:
 // 6.8 us there, 7.0 here at 3 bits, 7.4 at 4; 600 rows, 4 bits: 11.2 and 10.1).  Groups: up to three (700 rows: 16.5 and 16.7 at 3 bits,
-// 18.5 at 4; 2000: 24.9 and 22.8, 24.7).
+// 18.5 at 4; 2000: 24.9 and 22.8, 24.7).  More candidates take two passes or more there: groups, 1 row, K = 9: 10.2 and 7.2 us at 3 bits, 7.8 at 4, K = 16:
+// 10.2 and 7.8, 8.7; 591 rows, K = 16: 12.1 and 10.8, 11.9.
 int gbs_tc_uv_clip_histogram(const gbs_plan* p, const void* x, int64_t n_rows, int64_t stride, const float* alphas, int K,
                              double* err_sum, cudaStream_t stream)
 {
